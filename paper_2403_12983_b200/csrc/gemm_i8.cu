@@ -1,0 +1,627 @@
+// C = beta * C0 + alpha * A * B to (nearly) fp64 accuracy on the int8 tensor cores: error-free splitting of the operands
+// into 8-bit digits, exact integer products and sums (the scheme of Ootomo, Ozaki and Yokota, "DGEMM on integer matrix
+// multiplication unit", 2024, with balanced radix-256 digits).
+//
+// What it replaces and why.  The residuals of the refinement steps, R = G_J - H_JI V and the Schur products have to be
+// summed far beyond fp32 (see dgemm.cu).  On the fp64 pipe they run at 29-30 TFLOP/s, which was 218 of the 306 ms of the
+// state build of a d1 = 28672 layer.  kind::i8 multiplies at twice the bf16 rate and adds without any rounding: 2.6 POPS here,
+// so 21 or 15 digit products replace an fp64 product 6 to 9 times faster.  At d1 = 28672, m = 7168, k = 8602 the two residuals
+// take 18.4 ms, R 14.3 ms and the Schur products with their dot products 10.7 ms (230 ms for all on the fp64 pipe, and
+// 1.4 GB of fp64 panels written and read again); at d1 = 8192, m = 2048, k = 4096 2.9 ms against 12.7 ms.
+//
+// Splitting.  Row i of A and column j of B are scaled by powers of two so that their largest entry is below one; the
+// contraction index k is first balanced by 2^(-+ck), ck = half the exponent of H_kk, so that channels of very different
+// scale do not cost digits.  An entry becomes a fixed-point number of 8 S - 1 bits, cut into S signed digits
+// d_1 .. d_S (weight 2^(1 - 8 i)).  Digit products of order o = i + j <= S + 1 are kept, S (S + 1) / 2 of them; all
+// products of one order have one weight and accumulate in ONE int32 TMEM chain over the whole of K, exactly:
+// S * K * 2^14 < 2^31 (max_k).  What is dropped is below 2^(-8 S + 5) sqrt(K) of (row maximum x column maximum):
+// S = 6 for the residual of the inverse (its error enters the fp64 inverse of the swap loop), S = 5 elsewhere.
+//
+// Per output tile (128 x 256) the orders run from the smallest products to the largest; orders above 3 are added up in
+// fp32 registers as they finish (their weight is 2^-16 of the leading one and less), the last two stay in the two TMEM
+// buffers until the epilogue forms the sum in fp64.  Bound: the int8 tensor pipe; per 128-wide k-block of a digit pair a
+// CTA moves 48 KB from L2 for 512 cycles of MMA, the ratio of the Gram kernel.
+//   warp 0: TMA producer     warp 1: MMA issuer     warps 2-9: TMEM -> registers -> C
+#include "osscar_internal.cuh"
+#include "tc_common.cuh"
+#include <math.h>
+
+namespace osscar {
+namespace {
+
+using namespace tc;
+
+constexpr int I8_TM = 128, I8_BK = 128, I8_UK = 32;           // rows per tile; bytes (= digits) per k-block and per MMA
+constexpr int I8_A_BYTES = I8_TM * I8_BK;
+constexpr int I8_RING = 196608;                               // bytes of the operand ring
+constexpr int I8_STG = 32 * 16 * 8;                           // staging block of one accumulate warp: 32 rows x 16 doubles
+constexpr int I8_SMEM = I8_RING + 1024 + 256 + 8 * I8_STG;
+constexpr int I8_THREADS = 320;
+constexpr int64_t max_k(int S) { return 131071 / S; }         // S products of 2^14 per k in one int32 sum
+constexpr int I8_BAND = 8;
+
+enum { EPI_F32 = 0, EPI_F64 = 1, EPI_DOT = 2 };
+
+__device__ __forceinline__ double pow2d(int e) {              // 2^e, |e| <= 1000
+    e = e < -1000 ? -1000 : (e > 1000 ? 1000 : e);
+    return __hiloint2double((e + 1023) << 20, 0);
+}
+// Exponent e with m < 0.99 * 2^e (0 for m = 0): the top digit of a value scaled by it, carry included, stays below 128.
+__device__ __forceinline__ int scale_exponent(double m) {
+    if (m == 0.0) return 0;
+    int e;
+    const double f = frexp(m, &e);
+    return f > 0.99 ? e + 1 : e;
+}
+__device__ __forceinline__ unsigned long long abs_bits(double x) {      // orders like |x|; NaN above everything
+    return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ bool finite_bits(unsigned long long b) { return b < 0x7ff0000000000000ull; }
+
+// Balanced radix-256 digits of q: byte i of q + 0x80..80, with its top bit flipped, is the digit of weight 256^i.
+template <int S> __device__ __forceinline__ uint64_t digit_bytes(long long q) {
+    constexpr uint64_t kBias = S == 6 ? 0x808080808080ull : 0x8080808080ull;
+    return ((uint64_t)q + kBias) ^ kBias;
+}
+
+// ck[k] = half the binary exponent of the k-th diagonal entry of H_II.
+__global__ void k_i8_balance(const float* __restrict__ diag, int64_t stride, int64_t K, int32_t* __restrict__ ck)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= K) return;
+    const float d = diag[k * stride];
+    int e = 0;
+    if (d > 0.f && isfinite(d)) frexpf(d, &e);
+    ck[k] = e >> 1;
+}
+
+// Digits of the rows of A (rows x K, row stride lda): plane s holds digit s + 1, rows ldk bytes apart.  One block per
+// row: a pass for the largest entry, a second one (from L1 / L2) for the digits, 16 per thread and plane store.
+template <int S>
+__global__ void __launch_bounds__(256) k_i8_slice_rows(const float* __restrict__ A, int64_t lda, int64_t K, const int32_t* __restrict__ ck,
+                                int8_t* __restrict__ planes, int64_t plane, int64_t ldk, double* __restrict__ scale,
+                                int vec, const int32_t* __restrict__ done)
+{
+    if (done && *done) return;
+    __shared__ unsigned long long red[8];
+    const int64_t row = blockIdx.x;
+    const float* a = A + row * lda;
+    unsigned long long mx = 0;
+    for (int64_t k = threadIdx.x; k < K; k += 256) {
+        const unsigned long long b = abs_bits((double)a[k] * pow2d(-ck[k]));
+        mx = b > mx ? b : mx;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) { const unsigned long long b = __shfl_xor_sync(0xffffffffu, mx, o); mx = b > mx ? b : mx; }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) mx = red[w] > mx ? red[w] : mx;
+    const bool fin = finite_bits(mx);
+    const int e = fin ? scale_exponent(__longlong_as_double((long long)mx)) : 0;
+    if (threadIdx.x == 0) scale[row] = fin ? pow2d(e) : __longlong_as_double(0x7ff8000000000000ll);
+    for (int64_t k0 = (int64_t)threadIdx.x * 16; k0 < ldk; k0 += 256 * 16) {
+        uint32_t w[S][4];
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {
+            float x[4];
+            int c[4];
+            if (vec && k0 + q4 * 4 + 4 <= K) {
+                const float4 v = *reinterpret_cast<const float4*>(a + k0 + q4 * 4);
+                const int4 cv = *reinterpret_cast<const int4*>(ck + k0 + q4 * 4);
+                x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+                c[0] = cv.x; c[1] = cv.y; c[2] = cv.z; c[3] = cv.w;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int64_t k = k0 + q4 * 4 + i;
+                    x[i] = k < K ? a[k] : 0.f;
+                    c[i] = k < K ? ck[k] : 0;
+                }
+            }
+            uint64_t d[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) d[i] = fin ? digit_bytes<S>(__double2ll_rn((double)x[i] * pow2d(8 * S - 1 - e - c[i]))) : 0ull;
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+                uint32_t p = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) p |= (uint32_t)((d[i] >> (8 * (S - 1 - s))) & 0xff) << (8 * i);
+                w[s][q4] = p;
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < S; ++s)
+            *reinterpret_cast<uint4*>(planes + s * plane + row * ldk + k0) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+    }
+}
+
+// Largest entry of every column of B (K x N) after balancing, as ordered bits; grid (column tiles of 64, chunks of 256 rows).
+template <typename T>
+__global__ void __launch_bounds__(256) k_i8_colmax(const T* __restrict__ B, int64_t ldb, int64_t K, int64_t N, const int32_t* __restrict__ ck,
+                            unsigned long long* __restrict__ cmax, const int32_t* __restrict__ done)
+{
+    if (done && *done) return;
+    __shared__ unsigned long long red[4][64];
+    const int64_t n = (int64_t)blockIdx.x * 64 + (threadIdx.x & 63);
+    const int64_t k1 = min(K, ((int64_t)blockIdx.y + 1) * 256);
+    unsigned long long mx = 0;
+    if (n < N)
+        for (int64_t k = (int64_t)blockIdx.y * 256 + (threadIdx.x >> 6); k < k1; k += 4) {
+            const unsigned long long b = abs_bits((double)B[k * ldb + n] * pow2d(ck[k]));
+            mx = b > mx ? b : mx;
+        }
+    red[threadIdx.x >> 6][threadIdx.x & 63] = mx;
+    __syncthreads();
+    if (threadIdx.x < 64 && n < N) {
+#pragma unroll
+        for (int i = 1; i < 4; ++i) mx = red[i][threadIdx.x] > mx ? red[i][threadIdx.x] : mx;
+        atomicMax(&cmax[n], mx);
+    }
+}
+
+// Digits of the columns of B, stored transposed (column n of B = row n of the planes): tiles of 128 k x 32 columns turned
+// in shared memory.  tri_block > 0: entries of the diagonal blocks of that width are halved (column n is column col0 + n
+// of the whole matrix).
+template <int S, typename T>
+__global__ void __launch_bounds__(256) k_i8_slice_cols(const T* __restrict__ B, int64_t ldb, int64_t K, int64_t N, const int32_t* __restrict__ ck,
+                                const unsigned long long* __restrict__ cmax, int8_t* __restrict__ planes, int64_t plane, int64_t ldk,
+                                double* __restrict__ scale, int tri_block, int64_t col0, const int32_t* __restrict__ done)
+{
+    if (done && *done) return;
+    __shared__ T tile[128][33];
+    const int64_t n0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 128;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const int64_t k = k0 + ty + 8 * i, n = n0 + tx;
+        tile[ty + 8 * i][tx] = (k < K && n < N) ? B[k * ldb + n] : (T)0;
+    }
+    __syncthreads();
+    const int nl = threadIdx.x >> 3, kg = (threadIdx.x & 7) * 16;
+    const int64_t n = n0 + nl;
+    if (n >= N) return;
+    const unsigned long long mb = cmax[n];
+    const bool fin = finite_bits(mb);
+    const int e = fin ? scale_exponent(__longlong_as_double((long long)mb)) : 0;
+    if (blockIdx.y == 0 && kg == 0) scale[n] = fin ? pow2d(e) : __longlong_as_double(0x7ff8000000000000ll);
+    if (k0 + kg >= ldk) return;
+    uint32_t w[S][4];
+#pragma unroll
+    for (int q4 = 0; q4 < 4; ++q4) {
+        uint64_t d[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int64_t k = k0 + kg + q4 * 4 + i;
+            const int half = tri_block > 0 && k / tri_block == (col0 + n) / tri_block ? 1 : 0;
+            const int c = k < K ? ck[k] : 0;
+            d[i] = fin ? digit_bytes<S>(__double2ll_rn((double)tile[kg + q4 * 4 + i][nl] * pow2d(8 * S - 1 - e + c - half))) : 0ull;
+        }
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            uint32_t p = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) p |= (uint32_t)((d[i] >> (8 * (S - 1 - s))) & 0xff) << (8 * i);
+            w[s][q4] = p;
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+        *reinterpret_cast<uint4*>(planes + s * plane + n * ldk + k0 + kg) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
+}
+
+// K-major operand tile, SWIZZLE_128B: rows of 128 bytes, 8-row atoms 1024 bytes apart.
+__device__ __forceinline__ uint64_t i8_desc(uint32_t saddr) {
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr) : "memory");
+}
+
+struct I8Maps { CUtensorMap a, b; };
+struct I8Epi {
+    const double *sa, *sb;        // scales of the rows of A and of the columns of B
+    double alpha, beta;
+    const float* C0; int64_t ldc0;
+    void* C; int64_t ldc;         // EPI_F32: float, EPI_F64: double, EPI_DOT: partial sums [row][2 * TN]
+    int identity, vec;
+    int64_t row0, col0;           // position of this panel in the whole product (identity)
+};
+
+// TNC columns per tile.  tri = 1 + k-blocks left of this column panel: a tile reads only the k-range down to its own
+// diagonal block (0: the whole range).
+template <int S, int TNC, int EPI>
+__global__ void __launch_bounds__(I8_THREADS, 1)
+k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_constant__ I8Epi ep, int tri,
+         SearchCtl* __restrict__ ctl, const int32_t* __restrict__ done)
+{
+    constexpr int B_BYTES = TNC * I8_BK, STAGE = I8_A_BYTES + B_BYTES, STAGES = I8_RING / STAGE;
+    constexpr int HALF = TNC / 2, TMEM_COLS = 2 * TNC;
+    constexpr uint32_t kIdesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TNC >> 3) << 17) | ((uint32_t)(I8_TM >> 4) << 24);
+    if (done && *done) return;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t tiles_base = (raw + 1023u) & ~1023u;
+    uint8_t* bar_ptr = smem_raw + (tiles_base - raw) + I8_RING;
+    const uint32_t bars = tiles_base + I8_RING;
+    auto full_bar = [&](int s) { return bars + 8u * s; };
+    auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
+    auto tfull_bar = [&](int b) { return bars + 8u * (2 * STAGES + b); };
+    auto tempty_bar = [&](int b) { return bars + 8u * (2 * STAGES + 2 + b); };
+    const uint32_t drain_bar = bars + 8u * (2 * STAGES + 4);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_ptr + 8 * (2 * STAGES + 5));
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_ptr + 8 * (2 * STAGES + 5) + 8);
+    const long long wl = ctl->wait_limit;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int TM = (M + I8_TM - 1) / I8_TM, TN = (N + TNC - 1) / TNC;
+    const int num_ids = TM * TN;
+    const int nkb_all = (K + I8_BK - 1) / I8_BK;
+    auto tile_of = [&](int id, int* tm, int* tn, int* nkb) {
+        if (tri) {                       // longest columns first, so that the persistent CTAs end together
+            *tn = TN - 1 - id / TM; *tm = id % TM;
+            *nkb = min(nkb_all, tri - 1 + (*tn + 1) * (TNC / I8_BK));
+        } else {
+            const int per_band = I8_BAND * TN, b = id / per_band, r = id % per_band, rows = min(I8_BAND, TM - b * I8_BAND);
+            *tn = r / rows; *tm = b * I8_BAND + r % rows;
+            *nkb = nkb_all;
+        }
+    };
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 8); }
+        mbar_init(drain_bar, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            uint32_t it = 0;
+            bool ok = true;
+            for (int id = blockIdx.x; id < num_ids && ok; id += gridDim.x) {
+                int tm, tn, nkb;
+                tile_of(id, &tm, &tn, &nkb);
+                for (int o = S + 1; o >= 2 && ok; --o)
+                    for (int kb = 0; kb < nkb && ok; ++kb)
+                        for (int i = max(1, o - S); i <= min(S, o - 1); ++i, ++it) {
+                            const int s = it % STAGES;
+                            if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, wl)) { ok = false; break; }
+                            mbar_expect_tx(full_bar(s), STAGE);
+                            const uint32_t a_dst = tiles_base + s * STAGE;
+                            // the planes of an operand are stacked: rows past its end are another plane's and only feed
+                            // rows or columns of the tile that are never written
+                            tma_load_2d(a_dst, &maps.a, full_bar(s), kb * I8_BK, (i - 1) * M + tm * I8_TM);
+                            tma_load_2d(a_dst + I8_A_BYTES, &maps.b, full_bar(s), kb * I8_BK, (o - i - 1) * N + tn * TNC);
+                        }
+            }
+            if (*abort_flag) {                    // the copies still in flight must land before the CTA exits
+                const uint32_t first = it > STAGES ? it - STAGES : 0;
+                for (uint32_t j = first; j < it; ++j) mbar_drain(full_bar(j % STAGES), (j / STAGES) & 1);
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            uint32_t it = 0, fl = 0;
+            bool ok = true;
+            for (int id = blockIdx.x; id < num_ids && ok; id += gridDim.x) {
+                int tm, tn, nkb;
+                tile_of(id, &tm, &tn, &nkb);
+                for (int o = S + 1; o >= 2 && ok; --o, ++fl) {
+                    const int buf = fl & 1;
+                    if (!mbar_wait(tempty_bar(buf), ((fl >> 1) & 1) ^ 1, abort_flag, wl)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t d_tmem = tmem_base + (uint32_t)(buf * TNC);
+                    const int np = min(S, o - 1) - max(1, o - S) + 1;
+                    const int steps = nkb * np;
+                    for (int t = 0; t < steps; ++t, ++it) {
+                        const int s = it % STAGES;
+                        if (!mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, wl)) { ok = false; break; }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t a_src = tiles_base + s * STAGE, b_src = a_src + I8_A_BYTES;
+#pragma unroll
+                        for (int j = 0; j < I8_BK / I8_UK; ++j)
+                            umma_i8(d_tmem, i8_desc(a_src + j * I8_UK), i8_desc(b_src + j * I8_UK), kIdesc, (t | j) ? 1u : 0u);
+                        umma_commit(empty_bar(s));
+                    }
+                    if (ok) umma_commit(tfull_bar(buf));
+                }
+            }
+            if (!ok) {            // MMAs already issued keep running: they must finish before TMEM and the tiles are released
+                umma_commit(drain_bar);
+                mbar_drain(drain_bar, 0);
+            }
+        }
+    } else {
+        const int lg = warp & 3, half = (warp - 2) >> 2;
+        double* stg = reinterpret_cast<double*>(bar_ptr + 256) + (warp - 2) * (32 * 16);
+        const int rsub = lane >> 2, c4 = (lane & 3) * 4;
+        uint32_t fl = 0;
+        bool ok = true;
+        for (int id = blockIdx.x; id < num_ids && ok; id += gridDim.x) {
+            int tm, tn, nkb;
+            tile_of(id, &tm, &tn, &nkb);
+            float lo[HALF];               // orders above 3, in units of order 4
+#pragma unroll
+            for (int j = 0; j < HALF; ++j) lo[j] = 0.f;
+            for (int o = S + 1; o >= 4 && ok; --o, ++fl) {
+                const int buf = fl & 1;
+                if (!mbar_wait(tfull_bar(buf), (fl >> 1) & 1, abort_flag, wl)) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+                for (int c = 0; c < HALF / 32; ++c) {
+                    uint32_t r[32];
+                    tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(buf * TNC + half * HALF + c * 32), r);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) lo[c * 32 + j] = fmaf(lo[c * 32 + j], 0.00390625f, (float)(int)r[j]);
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tempty_bar(buf));
+            }
+            if (!ok) break;
+            const int b3 = fl & 1, b2 = b3 ^ 1;       // orders 3 and 2 wait in the two buffers
+            if (!mbar_wait(tfull_bar(b3), (fl >> 1) & 1, abort_flag, wl)) break;
+            if (!mbar_wait(tfull_bar(b2), ((fl + 1) >> 1) & 1, abort_flag, wl)) break;
+            fl += 2;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int64_t grow0 = (int64_t)tm * I8_TM + lg * 32;
+            const int64_t gcol0 = (int64_t)tn * TNC + half * HALF;
+            double sa[4], dot[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int64_t gr = grow0 + q * 8 + rsub;
+                sa[q] = gr < M ? ep.alpha * ep.sa[gr] : 0.0;
+                dot[q] = 0.0;
+            }
+#pragma unroll
+            for (int c = 0; c < HALF / 16; ++c) {
+                uint32_t r3[16], r2[16];
+                const uint32_t ta = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(half * HALF + c * 16);
+                tmem_ld16(ta + b3 * TNC, r3);
+                tmem_ld16(ta + b2 * TNC, r2);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (c == HALF / 16 - 1) {             // TMEM is read out: the next tile may start
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) { mbar_arrive(tempty_bar(b3)); mbar_arrive(tempty_bar(b2)); }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    // order 2 + order 3 / 256 + ..., an exact integer part and a small fp32 tail
+                    const double v = fma((double)(int)r2[j], 256.0, (double)(int)r3[j]) * 256.0 + (double)lo[c * 16 + j];
+                    stg[lane * 16 + (j ^ (lane & 15))] = v;
+                }
+                __syncwarp();
+                const int64_t gc = gcol0 + c * 16 + c4;
+                double sb[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) sb[i] = gc + i < N ? ep.sb[gc + i] * (1.0 / 1073741824.0) : 0.0;      // 2^-30: weight of order 4
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int r = q * 8 + rsub;
+                    const int64_t gr = grow0 + r;
+                    double v[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v[i] = stg[r * 16 + ((c4 + i) ^ (r & 15))] * sa[q] * sb[i];
+                    if (gr >= M || gc >= N) continue;
+                    const bool full = ep.vec && gc + 3 < N;
+                    if (EPI == EPI_DOT) {
+                        const float* h = ep.C0 + gr * ep.ldc0 + gc;
+                        if (full) {
+                            const float4 x = *reinterpret_cast<const float4*>(h);
+                            dot[q] += (v[0] * (double)x.x + v[1] * (double)x.y) + (v[2] * (double)x.z + v[3] * (double)x.w);
+                        } else {
+                            for (int i = 0; i < 4; ++i) if (gc + i < N) dot[q] += v[i] * (double)h[i];
+                        }
+                    } else if (EPI == EPI_F64) {
+                        double* cp = (double*)ep.C + gr * ep.ldc + gc;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) if (gc + i < N) cp[i] = v[i];
+                    } else {
+                        float* cp = (float*)ep.C + gr * ep.ldc + gc;
+                        if (ep.identity) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) v[i] += ep.row0 + gr == ep.col0 + gc + i ? 1.0 : 0.0;
+                        } else if (ep.beta != 0.0) {
+                            const float* c0 = ep.C0 + gr * ep.ldc0 + gc;
+                            if (full) {
+                                const float4 x = *reinterpret_cast<const float4*>(c0);
+                                v[0] += ep.beta * (double)x.x; v[1] += ep.beta * (double)x.y;
+                                v[2] += ep.beta * (double)x.z; v[3] += ep.beta * (double)x.w;
+                            } else {
+                                for (int i = 0; i < 4; ++i) if (gc + i < N) v[i] += ep.beta * (double)c0[i];
+                            }
+                        }
+                        if (full) *reinterpret_cast<float4*>(cp) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+                        else for (int i = 0; i < 4; ++i) if (gc + i < N) cp[i] = (float)v[i];
+                    }
+                }
+            }
+            if (EPI == EPI_DOT) {                 // partial sum of this tile half for each of the warp's rows
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    double v = dot[q];
+                    v += __shfl_xor_sync(0xffffffffu, v, 1);
+                    v += __shfl_xor_sync(0xffffffffu, v, 2);
+                    const int64_t gr = grow0 + q * 8 + rsub;
+                    if ((lane & 3) == 0 && gr < M) ((double*)ep.C)[gr * ep.ldc + 2 * tn + half] = v;
+                }
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(TMEM_COLS) : "memory");
+    }
+    if (threadIdx.x == 0 && *abort_flag) ctl->status = OSSCAR_E_TIMEOUT;
+}
+
+bool encode_planes(PFN_encodeTiled enc, CUtensorMap* map, const void* base, uint64_t K, uint64_t rows, uint64_t ldk, uint32_t box_rows)
+{
+    const cuuint64_t dims[2] = {K, rows};
+    const cuuint64_t strides[1] = {ldk};
+    const cuuint32_t box[2] = {(cuuint32_t)I8_BK, box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
+
+// Panel sizes of one product: `mp` rows of A and `np` columns of B at a time.
+struct I8Panels { int64_t mp, np, ldk; bool ok; };
+I8Panels plan(int64_t M, int64_t N, int64_t K, int S, size_t a_bytes, size_t b_bytes, int tn)
+{
+    I8Panels p;
+    p.ldk = round_up(K, 16);
+    const size_t per_a = (size_t)S * p.ldk + sizeof(double), per_b = (size_t)S * p.ldk + sizeof(double) + sizeof(unsigned long long);
+    const size_t fix_a = 1024, fix_b = 4 * (size_t)K + 2048;
+    int64_t mp = a_bytes > fix_a ? (int64_t)((a_bytes - fix_a) / per_a) : 0;
+    int64_t np = b_bytes > fix_b ? (int64_t)((b_bytes - fix_b) / per_b) : 0;
+    // whole tiles; planes are addressed with 32-bit coordinates
+    p.mp = mp >= M ? M : mp / I8_TM * I8_TM;
+    p.np = np >= N ? N : np / tn * tn;
+    p.ok = p.mp > 0 && p.np > 0 && K > 0 && K <= max_k(S) && M < (1 << 28) && N < (1 << 28);
+    return p;
+}
+
+template <int S, int TNC, int EPI>
+cudaError_t launch_mma(cudaStream_t st, const I8Maps& maps, int64_t M, int64_t N, int64_t K, const I8Epi& ep, int tri, int sms,
+                       SearchCtl* ctl, const int32_t* done)
+{
+    const cudaError_t e = cudaFuncSetAttribute(k_mma_i8<S, TNC, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, I8_SMEM);
+    if (e != cudaSuccess) return e;
+    const int64_t tiles = ((M + I8_TM - 1) / I8_TM) * ((N + TNC - 1) / TNC);
+    k_mma_i8<S, TNC, EPI><<<(unsigned)(tiles < sms ? tiles : sms), I8_THREADS, I8_SMEM, st>>>(maps, (int)M, (int)N, (int)K, ep, tri, ctl, done);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// Whether the product is worth its digits and fits the scratch.  The fp64 pipe keeps products of less than 2^29 multiply-adds
+// (its tiles are smaller, and it needs one launch instead of six) and contractions longer than max_k.
+bool gemm_i8_usable(int64_t M, int64_t N, int64_t K, int S, const I8Scratch& sc)
+{
+    if (!sc.a || !sc.b || ((uintptr_t)sc.a & 255) || ((uintptr_t)sc.b & 255)) return false;
+    if (M <= 0 || N <= 0 || K < 256) return false;
+    if ((double)M * (double)N * (double)K < 536870912.0) return false;
+    return plan(M, N, K, S, sc.a_bytes, sc.b_bytes, 256).ok;
+}
+
+template <int S>
+static cudaError_t gemm_i8_run(cudaStream_t st, const I8Gemm& p, I8Scratch& sc, SearchCtl* ctl, const int32_t* done)
+{
+    PFN_encodeTiled enc = get_encode();
+    if (!enc) return cudaErrorNotSupported;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int64_t M = p.M, N = p.N, K = p.K;
+    // 128-column tiles where 256-column ones would leave SMs without work
+    const int tn = ((M + I8_TM - 1) / I8_TM) * ((N + 255) / 256) < sms ? 128 : 256;
+    const I8Panels pl = plan(M, N, K, S, sc.a_bytes, sc.b_bytes, tn);
+    if (!pl.ok) return cudaErrorInvalidValue;
+    char* b = (char*)sc.b;
+    int32_t* ck = (int32_t*)b;                                 b += up256(4 * (size_t)K);
+    unsigned long long* cmax = (unsigned long long*)b;         b += up256(8 * (size_t)pl.np);
+    double* sb = (double*)b;                                   b += up256(8 * (size_t)pl.np);
+    int8_t* bp = (int8_t*)b;
+    char* a = (char*)sc.a;
+    double* sa = (double*)a;                                   a += up256(8 * (size_t)pl.mp);
+    int8_t* ap = (int8_t*)a;
+    const int vecA = (((uintptr_t)p.A & 15) == 0 && (p.lda % 4) == 0) ? 1 : 0;
+    k_i8_balance<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(p.diag, p.diag_stride, K, ck);
+    count_launches(1);
+    for (int64_t n0 = 0; n0 < N; n0 += pl.np) {
+        const int64_t nw = N - n0 < pl.np ? N - n0 : pl.np;
+        e = cudaMemsetAsync(cmax, 0, 8 * (size_t)nw, st);
+        if (e != cudaSuccess) return e;
+        const dim3 gm((unsigned)((nw + 63) / 64), (unsigned)((K + 255) / 256)), gs((unsigned)((nw + 31) / 32), (unsigned)((pl.ldk + 127) / 128));
+        const int tri_block = p.tri ? tn : 0;
+        if (p.Bd) {
+            k_i8_colmax<double><<<gm, 256, 0, st>>>(p.Bd + n0, p.ldb, K, nw, ck, cmax, done);
+            k_i8_slice_cols<S, double><<<gs, 256, 0, st>>>(p.Bd + n0, p.ldb, K, nw, ck, cmax, bp, nw * pl.ldk, pl.ldk, sb, tri_block, n0, done);
+        } else {
+            k_i8_colmax<float><<<gm, 256, 0, st>>>(p.B + n0, p.ldb, K, nw, ck, cmax, done);
+            k_i8_slice_cols<S, float><<<gs, 256, 0, st>>>(p.B + n0, p.ldb, K, nw, ck, cmax, bp, nw * pl.ldk, pl.ldk, sb, tri_block, n0, done);
+        }
+        count_launches(2);
+        for (int64_t m0 = 0; m0 < M; m0 += pl.mp) {
+            const int64_t mw = M - m0 < pl.mp ? M - m0 : pl.mp;
+            // the digits of A from the product before serve again when the whole of A is there
+            const bool have = pl.mp >= M && sc.have_A == p.A && sc.have_rows == M && sc.have_K == K && sc.have_S == S;
+            if (!have) {
+                sc.have_A = nullptr;
+                k_i8_slice_rows<S><<<(unsigned)mw, 256, 0, st>>>(p.A + m0 * p.lda, p.lda, K, ck, ap, mw * pl.ldk, pl.ldk, sa, vecA, done);
+                count_launches(1);
+                if (pl.mp >= M) { sc.have_A = p.A; sc.have_rows = M; sc.have_K = K; sc.have_S = S; }
+            }
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+            I8Maps maps;
+            if (!encode_planes(enc, &maps.a, ap, (uint64_t)K, (uint64_t)(S * mw), (uint64_t)pl.ldk, I8_TM)) return cudaErrorInvalidValue;
+            if (!encode_planes(enc, &maps.b, bp, (uint64_t)K, (uint64_t)(S * nw), (uint64_t)pl.ldk, (uint32_t)tn)) return cudaErrorInvalidValue;
+            I8Epi ep = {};
+            ep.sa = sa; ep.sb = sb; ep.alpha = p.alpha; ep.beta = p.beta; ep.identity = p.identity ? 1 : 0;
+            ep.row0 = m0; ep.col0 = n0; ep.ldc0 = p.ldc0; ep.ldc = p.ldc;
+            ep.C0 = p.C0 ? p.C0 + m0 * p.ldc0 + n0 : nullptr;
+            if (p.dot) {
+                ep.ldc = p.ldc;
+                ep.C = (double*)p.C + m0 * p.ldc + 2 * (n0 / tn);
+            } else if (p.out64) ep.C = (double*)p.C + m0 * p.ldc + n0;
+            else ep.C = (float*)p.C + m0 * p.ldc + n0;
+            ep.vec = (!ep.C0 || (((uintptr_t)ep.C0 & 15) == 0 && (p.ldc0 % 4) == 0)) && (p.dot || p.out64 || (((uintptr_t)ep.C & 15) == 0 && (p.ldc % 4) == 0)) ? 1 : 0;
+            const int tri = p.tri ? 1 + (int)(n0 / I8_BK) : 0;
+            if (p.dot) e = tn == 256 ? launch_mma<S, 256, EPI_DOT>(st, maps, mw, nw, K, ep, tri, sms, ctl, done)
+                                     : launch_mma<S, 128, EPI_DOT>(st, maps, mw, nw, K, ep, tri, sms, ctl, done);
+            else if (p.out64) e = tn == 256 ? launch_mma<S, 256, EPI_F64>(st, maps, mw, nw, K, ep, tri, sms, ctl, done)
+                                            : launch_mma<S, 128, EPI_F64>(st, maps, mw, nw, K, ep, tri, sms, ctl, done);
+            else e = tn == 256 ? launch_mma<S, 256, EPI_F32>(st, maps, mw, nw, K, ep, tri, sms, ctl, done)
+                               : launch_mma<S, 128, EPI_F32>(st, maps, mw, nw, K, ep, tri, sms, ctl, done);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    return cudaSuccess;
+}
+
+cudaError_t gemm_i8(cudaStream_t st, const I8Gemm& p, int S, I8Scratch& sc, SearchCtl* ctl, const int32_t* done)
+{
+    return S == 6 ? gemm_i8_run<6>(st, p, sc, ctl, done) : gemm_i8_run<5>(st, p, sc, ctl, done);
+}
+
+size_t gemm_i8_operand_bytes(int64_t rows, int64_t K, int S)
+{
+    return (size_t)rows * ((size_t)S * round_up(K, 16) + 16) + 4 * (size_t)K + 2048;
+}
+
+// columns of partial sums a `dot` product leaves per row
+int64_t gemm_i8_dot_cols(int64_t N) { return 2 * ((N + 127) / 128); }
+
+}  // namespace osscar

@@ -122,6 +122,30 @@ cudaError_t gemm_f64acc(cudaStream_t st, int64_t M, int64_t N, int64_t K, double
 cudaError_t gemm_f64out(cudaStream_t st, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
                         const float* B, int64_t ldb, double* C, int64_t ldc, const int32_t* done = nullptr, bool tri = false);
 
+// ---- gemm_i8.cu: the same products from 8-bit digits of the operands on the int8 tensor cores (exact integer sums)
+struct I8Scratch {                 // device memory for the digits of A and of B (256-byte aligned), and what A's part holds
+    void* a = nullptr; size_t a_bytes = 0;
+    void* b = nullptr; size_t b_bytes = 0;
+    const float* have_A = nullptr; int64_t have_rows = 0, have_K = 0; int have_S = 0;
+};
+struct I8Gemm {                    // C = beta * C0 + alpha * A * B, A (M x K) and B (K x N) row-major
+    int64_t M, N, K;
+    double alpha, beta;
+    const float* A; int64_t lda;
+    const float* B; const double* Bd; int64_t ldb;     // fp32 B, or fp64 Bd
+    const float* C0; int64_t ldc0;
+    void* C; int64_t ldc;
+    bool identity;                 // I + alpha A B instead of beta C0 + alpha A B
+    bool out64;                    // C in fp64
+    bool tri;                      // B symmetric, K = N: its block upper triangle with halved diagonal blocks (see dgemm.cu)
+    bool dot;                      // C (doubles, gemm_i8_dot_cols(N) per row) = partial sums of rows of A B times rows of C0
+    const float* diag; int64_t diag_stride;            // diagonal of H_II: balances the contraction index
+};
+bool gemm_i8_usable(int64_t M, int64_t N, int64_t K, int S, const I8Scratch& sc);
+cudaError_t gemm_i8(cudaStream_t st, const I8Gemm& p, int S, I8Scratch& sc, SearchCtl* ctl_dev, const int32_t* done);
+int64_t gemm_i8_dot_cols(int64_t N);
+size_t gemm_i8_operand_bytes(int64_t rows, int64_t K, int S);      // scratch that holds the digits of a whole operand
+
 // ---- panel_tc.cu: Y[i*so_row + e*so_col] = sum_k A[i][k] * P[e][k] on the tensor cores; A (M x K, streamed once) is split
 // into bf16 terms on the way (fp32-accurate); P is an N x K panel
 // A 16-byte aligned with lda % 4 == 0; scratch at least panel_dot_tc_scratch bytes.
@@ -160,6 +184,8 @@ cudaError_t gram_mirror(cudaStream_t st, float* H, int64_t d1);   // copy upper 
 // ---- state.cu: support selection and state construction --------------------------------------
 int select_support(osscar_ctx* ctx, int mode, int32_t* support);
 int build_state(osscar_ctx* ctx, bool guarded);
+// E = I - H_II Hinv summed beyond fp32; `v_free`: V and R hold nothing yet, so their memory may take operand digits
+cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32_t* done);
 int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref, const int32_t* done,
                        bool tensor_updates);
 cudaError_t gather_rows(cudaStream_t st, const float* src, int64_t m, int g, const int32_t* perm,
@@ -176,7 +202,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* p, int32_t* support_
                double* obj_trace, int32_t* swap_trace, osscar_search_result* res);
 cudaError_t score_pass(osscar_ctx* ctx);   // full scoring pass from the current state (fills D, A)
 // fp64 copy of the inverse from the fp32 one by a Newton-Schulz step summed in fp64 (single-row groups; uses `big`)
-int build_hinv64(osscar_ctx* ctx, bool guarded);
+int build_hinv64(osscar_ctx* ctx, bool guarded, bool v_free);
 // column shards: sum `count` values of `buf` (inside the workspace) over all shards through the context's hook
 int shard_reduce(osscar_ctx* ctx, void* buf, int64_t count, int dtype);
 

@@ -1077,12 +1077,11 @@ int persistent_grid(const Layout& L)
 
 }  // namespace
 
-int build_hinv64(osscar_ctx* ctx, bool guarded)
+int build_hinv64(osscar_ctx* ctx, bool guarded, bool v_free)
 {
     const Layout& L = ctx->L;
     cudaStream_t st = ctx->stream;
     char* ws = (char*)ctx->ws;
-    float* Hp = (float*)(ws + L.off_Hp);
     float* Hinv = (float*)(ws + L.off_Hinv);
     double* Hd = (double*)(ws + L.off_Hd);
     float* E = (float*)(ws + L.off_big);
@@ -1093,7 +1092,7 @@ int build_hinv64(osscar_ctx* ctx, bool guarded)
     // H_II^-1 = X0 (I + E + E^2 + ...): E is formed once with fp64 sums, the series is cut after E^2 (its products are
     // corrections of corrections: the tensor-core split product is ample), and the sum X0 + X0 (E + E^2) is taken in fp64.
     // The error left is E^3 (below 1e-9 for any start within 1e-3), against E^2 for a single Newton-Schulz step.
-    if (gemm_f64acc(st, L.nI, L.nI, L.nI, -1.0, Hp, L.ldp, Hinv, L.ldh, 0.0, nullptr, 0, E, L.ldh, true, done) != cudaSuccess) return OSSCAR_E_CUDA;
+    if (inverse_residual(ctx, E, v_free, done) != cudaSuccess) return OSSCAR_E_CUDA;
     if (cudaMemcpyAsync(T, E, sizeof(float) * L.nI * L.ldh, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return OSSCAR_E_CUDA;
     if (gemm_tc(st, L.nI, L.nI, L.nI, 1.f, E, L.ldh, E, L.ldh, 1.f, T, L.ldh, tc, L.tc_bytes, ctx->ctl, done) != cudaSuccess) return OSSCAR_E_CUDA;
     if (gemm_tc(st, L.nI, L.nI, L.nI, 1.f, Hinv, L.ldh, T, L.ldh, 0.f, E, L.ldh, tc, L.tc_bytes, ctx->ctl, done) != cudaSuccess) return OSSCAR_E_CUDA;
@@ -1197,7 +1196,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     };
     if (g == 1 && !fast) ctx->hd_valid = false;          // these drivers move the fp32 inverse only
     if (max_swaps > 0 && fast) {
-        if (!ctx->hd_valid) { const int rcd = build_hinv64(ctx, false); if (rcd != OSSCAR_OK) return rcd; }
+        if (!ctx->hd_valid) { const int rcd = build_hinv64(ctx, false, false); if (rcd != OSSCAR_OK) return rcd; }
         CK(bootstrap_g1());
     }
 

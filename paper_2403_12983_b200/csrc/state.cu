@@ -267,6 +267,20 @@ __global__ void k_schur(const float* __restrict__ Hp, int64_t ldp, const double*
     }
 }
 
+// c_t = Hp[J_t][J_t] - 2 * (partial sums of the quadratic form, in column order); one warp per pruned row.
+__global__ void k_schur_sum(const float* __restrict__ Hp, int64_t ldp, const double* __restrict__ part, int64_t ldpart, int np,
+                            int64_t nI, int64_t nJ, double* __restrict__ c, const int32_t* __restrict__ done)
+{
+    if (done && *done) return;
+    const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (t >= nJ) return;
+    double s = 0.0;
+    for (int i = lane; i < np; i += 32) s += part[t * ldpart + i];
+    s = warp_sum(s);
+    if (lane == 0) c[t] = (double)Hp[(nI + t) * ldp + nI + t] - 2.0 * s;
+}
+
 // Two deterministic stages: per-block partial sums, then one block adds them in a fixed order.
 __global__ void k_trace_product(const float* __restrict__ A, int64_t lda, const float* __restrict__ B, int64_t ldb,
                                 int64_t rows, int64_t cols, double* __restrict__ partial)
@@ -491,6 +505,45 @@ int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const 
     return OSSCAR_OK;
 }
 
+// Scratch for a product of `rows` x K digits against N columns: B's digits go to the front of the tensor-core region, A's
+// into what is left of it or into [other, other + bytes), whichever is larger.
+static I8Scratch i8_scratch(osscar_ctx* ctx, int64_t N, int64_t K, int S, void* other, size_t other_bytes)
+{
+    const Layout& L = ctx->L;
+    I8Scratch sc;
+    char* tc = (char*)ctx->ws + L.off_tc;
+    const size_t need_b = (gemm_i8_operand_bytes(N, K, S) + 255) / 256 * 256;
+    sc.b = tc; sc.b_bytes = L.tc_bytes;
+    sc.a = (void*)(((uintptr_t)other + 255) & ~(uintptr_t)255);
+    sc.a_bytes = other_bytes > 256 ? other_bytes - 256 : 0;
+    if (need_b < L.tc_bytes && L.tc_bytes - need_b > sc.a_bytes) {
+        sc.b_bytes = need_b;
+        sc.a = tc + need_b; sc.a_bytes = L.tc_bytes - need_b;
+    }
+    return sc;
+}
+
+constexpr int kResidualDigits = 6, kDirectDigits = 5;      // see gemm_i8.cu
+
+cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32_t* done)
+{
+    const Layout& L = ctx->L;
+    char* ws = (char*)ctx->ws;
+    const float* Hp = (const float*)(ws + L.off_Hp);
+    const float* Hinv = (const float*)(ws + L.off_Hinv);
+    // the fp64 inverse is made from this residual, so its place (and, before V exists, the ones behind it) is free
+    const size_t free_end = v_free ? L.off_y : L.off_V;
+    I8Scratch sc = i8_scratch(ctx, L.nI, L.nI, kResidualDigits, ws + L.off_Hd, free_end - L.off_Hd);
+    if (gemm_i8_usable(L.nI, L.nI, L.nI, kResidualDigits, sc)) {
+        I8Gemm p = {};
+        p.M = p.N = p.K = L.nI; p.alpha = -1.0; p.identity = true;
+        p.A = Hp; p.lda = L.ldp; p.B = Hinv; p.ldb = L.ldh; p.C = E; p.ldc = L.ldh;
+        p.diag = Hp; p.diag_stride = L.ldp + 1;
+        return gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, done);
+    }
+    return gemm_f64acc(ctx->stream, L.nI, L.nI, L.nI, -1.0, Hp, L.ldp, Hinv, L.ldh, 0.0, nullptr, 0, E, L.ldh, true, done);
+}
+
 // Rebuilds every piece of the search state from H, G and the current slot permutation.
 // With `guarded`, the kernels that can be skipped return at once when the loop has stopped.
 int build_state(osscar_ctx* ctx, bool guarded)
@@ -518,19 +571,20 @@ int build_state(osscar_ctx* ctx, bool guarded)
     count_launches(2);
     CK(cudaGetLastError());
     { const int rc_inv = invert_spd_inplace(ctx, Hinv, L.ldh, nI, Hp, L.ldp, done, true); if (rc_inv != OSSCAR_OK) return rc_inv; }
-    // Every product below that forms a small difference of large sums is accumulated in fp64 (gemm_f64acc): the scores
-    // of Eq. impact are compared at 1e-5 relative, and fp32 accumulation leaves cond(H_II) * 2^-24 in them.
+    // Every product below that forms a small difference of large sums is summed far beyond fp32 (digit products on the
+    // int8 tensor cores, gemm_i8; small ones on the fp64 pipe, gemm_f64acc): the scores of Eq. impact are compared at 1e-5
+    // relative, and fp32 accumulation leaves cond(H_II) * 2^-24 in them.
     // (1) the inverse.  Single-row groups: fp64 copy by a third-order correction from one fp64 residual, and the fp32
     //     inverse rounded from it (build_hinv64).  Groups of several rows: one Newton-Schulz step, E = I - H_II Hinv in
     //     fp64, Hinv := sym(Hinv + Hinv E) (E is tiny: any product will do)
     ctx->hd_valid = false;
     if (L.g == 1) {
-        const int rc_d = build_hinv64(ctx, guarded);
+        const int rc_d = build_hinv64(ctx, guarded, true);
         if (rc_d != OSSCAR_OK) return rc_d;
     } else {
         float* E = big;
         float* Dlt = big + nI * L.ldh;
-        CK(gemm_f64acc(st, nI, nI, nI, -1.0, Hp, L.ldp, Hinv, L.ldh, 0.0, nullptr, 0, E, L.ldh, true, done));
+        CK(inverse_residual(ctx, E, true, done));
         CK(gemm_tc(st, nI, nI, nI, 1.f, Hinv, L.ldh, E, L.ldh, 0.f, Dlt, L.ldh, tc, L.tc_bytes, ctx->ctl, done));
         k_add_sym<<<dim3((unsigned)((nI + 31) / 32), (unsigned)((nI + 31) / 32)), dim3(32, 8), 0, st>>>(Hinv, L.ldh, Dlt, L.ldh, nI, done);
         count_launches(1);
@@ -542,7 +596,22 @@ int build_state(osscar_ctx* ctx, bool guarded)
     count_launches(1);
     if (L.ldm != L.m) CK(cudaMemsetAsync(V, 0, sizeof(float) * nI * L.ldm, st));     // padding columns stay zero
     CK(gemm_tc(st, nI, L.m, nI, 1.f, Hinv, L.ldh, GI, L.ldm, 0.f, V, L.ldm, tc, L.tc_bytes, ctx->ctl, done));
-    CK(gemm_f64acc(st, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false, done));
+    const int64_t big_floats = (int64_t)((L.off_Hp - L.off_big) / sizeof(float));
+    {   // digits beside GI and rV, or in the place of R
+        const size_t used = sizeof(float) * 2 * (size_t)nI * L.ldm, tail = sizeof(float) * (size_t)big_floats - used;
+        const size_t rbytes = L.off_y - L.off_R;
+        I8Scratch sc = tail > rbytes ? i8_scratch(ctx, L.m, nI, kResidualDigits, (char*)big + used, tail)
+                                     : i8_scratch(ctx, L.m, nI, kResidualDigits, R, rbytes);
+        if (gemm_i8_usable(nI, L.m, nI, kResidualDigits, sc)) {
+            I8Gemm p = {};
+            p.M = nI; p.N = L.m; p.K = nI; p.alpha = -1.0; p.beta = 1.0;
+            p.A = Hp; p.lda = L.ldp; p.B = V; p.ldb = L.ldm; p.C0 = GI; p.ldc0 = L.ldm; p.C = rV; p.ldc = L.ldm;
+            p.diag = Hp; p.diag_stride = L.ldp + 1;
+            CK(gemm_i8(st, p, kResidualDigits, sc, ctx->ctl, done));
+        } else
+            CK(gemm_f64acc(st, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false, done));
+        // gemm_i8 leaves the pad columns of rV alone; they meet no valid column of V below
+    }
     CK(gemm_tc(st, nI, L.m, nI, 1.f, Hinv, L.ldh, rV, L.ldm, 1.f, V, L.ldm, tc, L.tc_bytes, ctx->ctl, done));
     // obj = Tr(W^T G) - Tr(G_I^T V)
     if (ctx->have_const) CK(set_device_double(st, &ctx->ctl->acc[0], ctx->user_const));
@@ -560,22 +629,59 @@ int build_state(osscar_ctx* ctx, bool guarded)
     k_set_obj<<<1, 1, 0, st>>>(ctx->ctl);
     count_launches(1);
     if (nJ > 0) {
-        // (3) R_J = G_J - Hp[J, I] V, accumulated in fp64
+        // (3) R_J = G_J - Hp[J, I] V
         k_gather_rows<<<(unsigned)nJ, 256, 0, st>>>(ctx->G, L.m, L.g, perm, nI, R, L.ldm);
-        CK(gemm_f64acc(st, nJ, L.m, nI, -1.0, Hp + nI * L.ldp, L.ldp, V, L.ldm, 1.0, R, L.ldm, R, L.ldm, false, done));
-        // (4) Pm = Hp[J, I] Hinv kept in fp64, in panels of whole pruned groups that fit the scratch, then the Schur
-        // complements H_qq - Pm_q . H_qI as fp64 dot products
         count_launches(1);
-        double* Pm = (double*)big;
-        const int64_t big_floats = (int64_t)((L.off_Hp - L.off_big) / sizeof(float));
-        int64_t gpp = (big_floats / 2) / (L.ldh * L.g);                 // pruned groups per panel
-        if (gpp < 1) return OSSCAR_E_WORKSPACE;
-        for (int64_t t0 = 0; t0 < L.ng - L.k; t0 += gpp) {
-            const int64_t ngr = L.ng - L.k - t0 < gpp ? L.ng - L.k - t0 : gpp;
-            const bool tri = L.g == 1;         // one quadratic form per pruned row: half of the symmetric inverse is enough
-            CK(gemm_f64out(st, ngr * L.g, nI, nI, Hp + (nI + t0 * L.g) * L.ldp, L.ldp, Hinv, L.ldh, Pm, L.ldh, done, tri));
-            k_schur<<<(unsigned)ngr, 256, 0, st>>>(Hp, L.ldp, Pm, L.ldh, nI, L.g, c, t0, tri ? 2.0 : 1.0, done);
+        const float* HJI = Hp + nI * L.ldp;
+        // single-row groups: partial sums of the quadratic forms at the end of `big`, the digits of H_JI in front of them
+        // (used by both products); wider groups: Pm in `big`
+        const bool one = L.g == 1;
+        const size_t part_bytes = one ? sizeof(double) * (size_t)nJ * gemm_i8_dot_cols(nI) : 0;
+        const size_t big_bytes = (sizeof(float) * (size_t)big_floats) / 256 * 256;
+        const size_t room = big_bytes > part_bytes + 512 ? (big_bytes - part_bytes) / 256 * 256 : 0;
+        double* part = (double*)((char*)big + room);
+        I8Scratch scR;
+        scR.a = big; scR.a_bytes = room; scR.b = tc; scR.b_bytes = L.tc_bytes;
+        if (gemm_i8_usable(nJ, L.m, nI, kDirectDigits, scR)) {
+            I8Gemm p = {};
+            p.M = nJ; p.N = L.m; p.K = nI; p.alpha = -1.0; p.beta = 1.0;
+            p.A = HJI; p.lda = L.ldp; p.B = V; p.ldb = L.ldm; p.C0 = R; p.ldc0 = L.ldm; p.C = R; p.ldc = L.ldm;
+            p.diag = Hp; p.diag_stride = L.ldp + 1;
+            CK(gemm_i8(st, p, kDirectDigits, scR, ctx->ctl, done));
+        } else
+            CK(gemm_f64acc(st, nJ, L.m, nI, -1.0, HJI, L.ldp, V, L.ldm, 1.0, R, L.ldm, R, L.ldm, false, done));
+        // (4) Schur complements H_qq - H_qI Hinv H_Iq.  Single-row groups need one quadratic form per pruned row, for which
+        // half of the symmetric inverse is enough: from the fp64 inverse, with the dot products in the product's epilogue.
+        if (one && gemm_i8_usable(nJ, nI, nI, kDirectDigits, scR)) {
+            I8Gemm p = {};
+            p.M = nJ; p.N = nI; p.K = nI; p.alpha = 1.0; p.tri = true; p.dot = true;
+            p.A = HJI; p.lda = L.ldp; p.Bd = (const double*)(ws + L.off_Hd); p.ldb = L.ldh; p.C0 = HJI; p.ldc0 = L.ldp;
+            p.C = part; p.ldc = gemm_i8_dot_cols(nI);
+            p.diag = Hp; p.diag_stride = L.ldp + 1;
+            CK(cudaMemsetAsync(part, 0, part_bytes, st));        // 256-column tiles fill half of the columns
+            CK(gemm_i8(st, p, kDirectDigits, scR, ctx->ctl, done));
+            k_schur_sum<<<(unsigned)((nJ + 7) / 8), 256, 0, st>>>(Hp, L.ldp, part, p.ldc, (int)p.ldc, nI, nJ, c, done);
             count_launches(1);
+        } else {
+            // Pm = Hp[J, I] Hinv kept in fp64, in panels of whole pruned groups that fit the scratch, then fp64 dot products
+            double* Pm = (double*)big;
+            int64_t gpp = (big_floats / 2) / (L.ldh * L.g);                 // pruned groups per panel
+            if (gpp < 1) return OSSCAR_E_WORKSPACE;
+            for (int64_t t0 = 0; t0 < L.ng - L.k; t0 += gpp) {
+                const int64_t ngr = L.ng - L.k - t0 < gpp ? L.ng - L.k - t0 : gpp;
+                const float* At = Hp + (nI + t0 * L.g) * L.ldp;
+                I8Scratch sc = i8_scratch(ctx, nI, nI, kDirectDigits, nullptr, 0);
+                if (!one && gemm_i8_usable(ngr * L.g, nI, nI, kDirectDigits, sc)) {
+                    I8Gemm p = {};
+                    p.M = ngr * L.g; p.N = nI; p.K = nI; p.alpha = 1.0; p.out64 = true;
+                    p.A = At; p.lda = L.ldp; p.B = Hinv; p.ldb = L.ldh; p.C = Pm; p.ldc = L.ldh;
+                    p.diag = Hp; p.diag_stride = L.ldp + 1;
+                    CK(gemm_i8(st, p, kDirectDigits, sc, ctx->ctl, done));
+                } else
+                    CK(gemm_f64out(st, ngr * L.g, nI, nI, At, L.ldp, Hinv, L.ldh, Pm, L.ldh, done, one));
+                k_schur<<<(unsigned)ngr, 256, 0, st>>>(Hp, L.ldp, Pm, L.ldh, nI, L.g, c, t0, one ? 2.0 : 1.0, done);
+                count_launches(1);
+            }
         }
     }
     CK(cudaGetLastError());
