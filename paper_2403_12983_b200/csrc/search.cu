@@ -1056,22 +1056,20 @@ cudaError_t enqueue_scores(osscar_ctx* ctx, const Ptrs& p, bool norms, bool gene
 #include "search_block.cuh"
 #include "search_loop_g1.cuh"
 
-// Blocks of the persistent loop: every block the device can hold at once (cooperative launch), but no more than the
-// longest phase has passes to hand out.  0 when the device cannot launch cooperatively.
-int persistent_grid(const Layout& L)
+// Blocks of the persistent loop: one per SM (cooperative launch), fewer for layers with few rows: a barrier costs more the
+// more blocks meet at it.  0 when the device cannot launch cooperatively.
+int persistent_grid(const Layout& L, size_t* smem)
 {
     int dev = 0, coop = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_swap_loop_g1, PL_T, 0) != cudaSuccess || per_sm < 1) return 0;
-    int64_t grid = (int64_t)sms * per_sm;
-    const int rbm = pl_rows_per_pass(L.ldm / 4), rbh = pl_rows_per_pass(L.ldh / 4);
-    int64_t passes = (L.nI + rbm - 1) / rbm;
-    if ((L.nJ + rbm - 1) / rbm > passes) passes = (L.nJ + rbm - 1) / rbm;
-    if ((L.nJ + rbh) / rbh > passes) passes = (L.nJ + rbh) / rbh;
-    if (grid > passes) grid = passes;
-    if (grid > PL_MAX_BLOCKS) grid = PL_MAX_BLOCKS;
+    *smem = pl_smem_bytes(L) <= PL_SMEM_MAX ? pl_smem_bytes(L) : 0;
+    if (cudaFuncSetAttribute(k_swap_loop_g1, cudaFuncAttributeMaxDynamicSharedMemorySize, PL_SMEM_MAX) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_swap_loop_g1, PL_T, *smem) != cudaSuccess || per_sm < 1) return 0;
+    int64_t grid = (L.d1 + PL_ROWS_PER_BLOCK) / PL_ROWS_PER_BLOCK;
+    if (grid > sms) grid = sms;
+    if (grid > PL_CAND - 1) grid = PL_CAND - 1;
     return (int)(grid < 1 ? 1 : grid);
 }
 
@@ -1156,7 +1154,8 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     // against 0.71 of copy bandwidth on the OPT-30B-shaped FC2 layer)
     const double state_bytes = 8.0 * L.nI * L.ldh + 4.0 * (L.nI + L.nJ) * L.ldm + 4.0 * L.nJ * L.ldh;
     const bool want_persistent = sharded ? false : prm->loop_mode == OSSCAR_LOOP_PERSISTENT || (prm->loop_mode == OSSCAR_LOOP_AUTO && state_bytes <= 96.0e6);
-    const int pgrid = (fast && want_persistent && L.nJ > 0) ? persistent_grid(L) : 0;
+    size_t psmem = 0;
+    const int pgrid = (fast && want_persistent && L.nJ > 0) ? persistent_grid(L, &psmem) : 0;
     if (prm->loop_mode == OSSCAR_LOOP_PERSISTENT && pgrid == 0) return OSSCAR_E_ARG;
     const bool persistent = pgrid > 0;
     if (block) max_swaps /= bs;                   // from here on: iterations
@@ -1274,6 +1273,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         la.prof = loop_prof;
         la.obj_trace = obj_trace; la.swap_trace = swap_trace;
         la.tol = tol; la.accept_mode = prm->accept_mode; la.max_swaps = max_swaps;
+        la.smem_vectors = psmem > 0 ? 1 : 0;
         if (cudaMemsetAsync(loop_prof, 0, 8 * sizeof(unsigned long long), st) != cudaSuccess) rc = OSSCAR_E_CUDA;
         const int chunk = prm->refresh_every > 0 ? prm->refresh_every : max_swaps;
         for (int it0 = 0; it0 < max_swaps && rc == OSSCAR_OK; it0 += chunk) {
@@ -1287,7 +1287,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
             la.max_steps = max_swaps - it0 < chunk ? max_swaps - it0 : chunk;
             if (cudaMemsetAsync(&ctx->ctl->bar_count, 0, sizeof(unsigned long long) + sizeof(int32_t), st) != cudaSuccess) { rc = OSSCAR_E_CUDA; break; }
             void* kargs[] = { (void*)&la };
-            if (cudaLaunchCooperativeKernel((const void*)k_swap_loop_g1, dim3((unsigned)pgrid), dim3(PL_T), kargs, 0, st) != cudaSuccess) {
+            if (cudaLaunchCooperativeKernel((const void*)k_swap_loop_g1, dim3((unsigned)pgrid), dim3(PL_T), kargs, psmem, st) != cudaSuccess) {
                 rc = OSSCAR_E_CUDA; break;
             }
             count_launches(1);
