@@ -10,6 +10,7 @@ namespace osscar {
 constexpr int kTracePartials = 1184;   // blocks of a trace reduction; the context owns that many doubles
 constexpr int64_t kMaxPairs = 1 << 20;     // PAIR_EXACT scores at most this many (kept, pruned) pairs per step
 constexpr int kLoopMaxBlocks = 2048;   // most blocks the persistent swap loop is launched with (size of its candidate lists)
+constexpr size_t kFreeDynSmem = 40 * 1024;   // dynamic shared memory above which a kernel asks for more (48 KB less its static arrays)
 constexpr int kPadF = 32;   // leading dimensions of internal fp32 matrices are padded to this many floats
 
 extern unsigned long long g_launches;      // kernels launched by the library (host-side count)

@@ -1164,7 +1164,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     if (max_swaps > 0) CK(enqueue_scores(ctx, p, true, pair));
     if (max_swaps > 0 && sharded && shard_reduce(ctx, p.vnorm, L.d1, OSSCAR_FP32) != OSSCAR_OK) return OSSCAR_E_CUDA;
     const size_t inv_smem = ((size_t)g * g + 2 * (size_t)g) * sizeof(double);      // matrix under inversion + pivot row/column
-    if (inv_smem > 48 * 1024) {
+    if (inv_smem > kFreeDynSmem) {
         CK(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem));
         CK(cudaFuncSetAttribute(k_pair_delta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem));
     }
@@ -1202,10 +1202,10 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     if (block) {
         CK(cudaMemsetAsync((char*)ctx->ws + L.off_block, 0, block_bytes_for(L, bs * g), st));
         const size_t smem = 2 * (size_t)g * bs * g * sizeof(double);
-        if (smem > 48 * 1024) CK(cudaFuncSetAttribute(k_blk_update_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (smem > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_update_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         const size_t smem2 = 2 * (size_t)bs * g * bs * g * sizeof(double);
-        if (smem2 > 48 * 1024) CK(cudaFuncSetAttribute(k_blk_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
-        if (smem2 / 2 > 48 * 1024) CK(cudaFuncSetAttribute(k_blk_update_c_g1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem2 / 2)));
+        if (smem2 > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
+        if (smem2 / 2 > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_update_c_g1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem2 / 2)));
     }
     if (g > 1) CK(cudaFuncSetAttribute(k_update_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * (size_t)g * g * sizeof(double))));
 

@@ -16,13 +16,105 @@ static __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+// Inverse of the g x g SPD matrix M (ld g, shared memory where possible) by Gauss-Jordan elimination without pivoting, the
+// matrix in registers: of NW warps, warp w owns the rows w, w + NW, ... (A of them), a lane the columns lane, lane + 32, ...
+// (B of them; B = 1 or NW = 32).  A step is one shuffle per owned row (its entry of the pivot column), the scaled pivot row
+// through double-buffered shared memory and ONE barrier.  Out receives the symmetrised inverse, M is overwritten.  Returns
+// the smallest pivot, i.e. the smallest diagonal entry of the successive Schur complements = the squared diagonal of the
+// Cholesky factor (<= 0 when M is not positive definite).
+template <int NW, int A, int B>
+static __device__ double spd_inverse_reg(double* M, double* Out, int g)
+{
+    static_assert(B == 1 || (NW == 32 && A == B), "row and column of the pivot in the same register");
+    __shared__ double rows[2][32 * B];
+    __shared__ double s_pinv[2], s_piv[NW], s_min;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double x[A][B];
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < A; ++a)
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int i = w + NW * a, c = lane + 32 * b;
+            x[a][b] = i < g && c < g ? M[i * g + c] : 0.0;
+        }
+    double minpiv = DBL_MAX;                       // kept by the owner of each pivot row
+#pragma unroll
+    for (int kk = 0; kk < A; ++kk) {
+        constexpr int kB = B;
+        const int bk = kB == 1 ? 0 : kk;
+        for (int jj = 0; jj < NW; ++jj) {
+            const int j = kk * NW + jj;
+            if (j >= g) break;
+            double* rowj = rows[j & 1];
+            double col[A];
+#pragma unroll
+            for (int a = 0; a < A; ++a) col[a] = __shfl_sync(0xffffffffu, x[a][bk], j & 31);      // entry (row, j)
+            if (w == jj) {                         // row j is this warp's row kk
+                double d = col[kk];
+                const bool bad = !(d > 0.0);
+                if (bad) { minpiv = -1.0; d = 1.0; }
+                else if (d < minpiv) minpiv = d;
+                const double pinv = 1.0 / d;
+#pragma unroll
+                for (int b = 0; b < B; ++b) rowj[lane + 32 * b] = x[kk][b] * pinv;
+                if (lane == 0) s_pinv[j & 1] = pinv;
+            }
+            __syncthreads();
+            const double pinv = s_pinv[j & 1];
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int c = lane + 32 * b;
+                const double r = rowj[c];
+#pragma unroll
+                for (int a = 0; a < A; ++a) {
+                    double v;
+                    if (a == kk && w == jj) v = c == j ? pinv : r;
+                    else if (c == j) v = -col[a] * pinv;
+                    else v = x[a][b] - col[a] * r;
+                    x[a][b] = v;
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < A; ++a)
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int i = w + NW * a, c = lane + 32 * b;
+            if (i < g && c < g) M[i * g + c] = x[a][b];
+        }
+    if (lane == 0) s_piv[w] = minpiv;
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < A; ++a)                    // the two triangles differ by rounding only
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int i = w + NW * a, c = lane + 32 * b;
+            if (i < g && c < g) Out[i * g + c] = 0.5 * (x[a][b] + M[c * g + i]);
+        }
+    if (threadIdx.x == 0) {
+        double mp = s_piv[0];
+        for (int i = 1; i < NW; ++i) mp = s_piv[i] < mp ? s_piv[i] : mp;
+        s_min = mp;
+    }
+    __syncthreads();
+    return s_min;
+}
+
 // Block-cooperative inverse of the g x g SPD matrix M (ld g) by in-place Gauss-Jordan elimination without pivoting:
 // g steps of one rank-1 update over all g^2 entries, so every thread of the block works in every step.
 // M is overwritten (keep it in shared memory where possible); Out receives the symmetrised inverse; Lw: scratch of
 // at least 2 g doubles.  Returns the smallest pivot, i.e. the smallest diagonal entry of the successive Schur
 // complements = the squared diagonal of the Cholesky factor (<= 0 when M is not positive definite).
+// The register form takes over where its thread layouts fit (blocks of 32 warps up to g = 96, of 8 warps up to g = 32):
+// with the two-barrier form below the scores of 32 groups of 80 rows took 0.21 ms, now 0.094 ms; larger matrices (the nested phase's joint downdates) stay here.
 static __device__ double spd_inverse(double* M, double* Lw, double* Out, int g)
 {
+    if (blockDim.x == 1024 && g > 32 && g <= 64) return spd_inverse_reg<32, 2, 2>(M, Out, g);
+    if (blockDim.x == 1024 && g > 64 && g <= 96) return spd_inverse_reg<32, 3, 3>(M, Out, g);
+    if (blockDim.x == 1024 && g <= 32) return spd_inverse_reg<32, 1, 1>(M, Out, g);
+    if (blockDim.x == 256 && g <= 32) return spd_inverse_reg<8, 4, 1>(M, Out, g);
     __shared__ double minpiv;
     const int t = threadIdx.x, nt = blockDim.x;
     double* colj = Lw; double* rowj = Lw + g;

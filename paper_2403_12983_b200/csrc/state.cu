@@ -247,7 +247,8 @@ __global__ void k_gj_writeback(float* __restrict__ A, int64_t lda, int64_t n, in
     }
 }
 
-// c_t[a][b] = Hp[J_ta][J_tb] - twice * sum_s Pm[ta][s] * Hp[J_tb][s]  for pruned slot t; one block per t.
+// c_t[a][b] = Hp[J_ta][J_tb] - twice * sum_s Pm[ta][s] * Hp[J_tb][s]  for pruned slot t; grid (slots, shares of the g * g
+// entries): 16 slots of 80 rows on one block each kept 16 SMs busy for 3.26 ms.
 // Pm holds the rows of the pruned slots [t0, t0 + gridDim.x) in fp64 (row stride ldpm): H_JI Hinv (twice = 1), or, for
 // single-row groups, H_JI U with U the halved block upper triangle of Hinv (twice = 2: h^T Hinv h = 2 h^T U h).
 __global__ void k_schur(const float* __restrict__ Hp, int64_t ldp, const double* __restrict__ Pm, int64_t ldpm,
@@ -256,7 +257,7 @@ __global__ void k_schur(const float* __restrict__ Hp, int64_t ldp, const double*
     if (done && *done) return;
     const int64_t t = t0 + blockIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int pair = w; pair < g * g; pair += nw) {
+    for (int pair = blockIdx.y * nw + w; pair < g * g; pair += nw * gridDim.y) {
         const int a = pair / g, b = pair % g;
         const double* pr = Pm + ((t - t0) * g + a) * ldpm;
         const float* hr = Hp + (nI + t * g + b) * ldp;
@@ -523,6 +524,13 @@ static I8Scratch i8_scratch(osscar_ctx* ctx, int64_t N, int64_t K, int S, void* 
     return sc;
 }
 
+// blocks per pruned slot of k_schur: about eight blocks per SM in all, each warp with at least one entry
+static unsigned schur_shares(int64_t slots, int g)
+{
+    const int64_t want = (148 * 8 + slots - 1) / slots, most = ((int64_t)g * g + 7) / 8;
+    return (unsigned)(want < 1 ? 1 : (want < most ? want : most));
+}
+
 constexpr int kResidualDigits = 6, kDirectDigits = 5;      // see gemm_i8.cu
 
 cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32_t* done)
@@ -679,7 +687,7 @@ int build_state(osscar_ctx* ctx, bool guarded)
                     CK(gemm_i8(st, p, kDirectDigits, sc, ctx->ctl, done));
                 } else
                     CK(gemm_f64out(st, ngr * L.g, nI, nI, At, L.ldp, Hinv, L.ldh, Pm, L.ldh, done, one));
-                k_schur<<<(unsigned)ngr, 256, 0, st>>>(Hp, L.ldp, Pm, L.ldh, nI, L.g, c, t0, one ? 2.0 : 1.0, done);
+                k_schur<<<dim3((unsigned)ngr, schur_shares(ngr, L.g)), 256, 0, st>>>(Hp, L.ldp, Pm, L.ldh, nI, L.g, c, t0, one ? 2.0 : 1.0, done);
                 count_launches(1);
             }
         }
