@@ -12,7 +12,7 @@
 // K is processed in panels sized to the caller's scratch (the bf16 terms of one panel of A and B live there).
 //
 // The same pipeline, instantiated with an MN-major A operand and a single bf16 term, is the Gram kernel
-// H (+)= Xc^T Xc over the upper-triangle tiles (chains of 32 k-blocks between drains), and with B taken from a
+// H (+)= Xc^T Xc over the upper-triangle tiles (chains of 8 k-blocks between drains), and with B taken from a
 // second matrix the cross term G (+)= Xc^T Yc (Y in bf16, or fp32 split into three terms).
 #include "osscar_internal.cuh"
 #include <cuda_bf16.h>
@@ -47,8 +47,10 @@ template <int MODE> struct Traits {
     static constexpr bool kSixPairs = MODE == MODE_GEMM3 || MODE == MODE_GRAM3;
     static constexpr int kTerms = kSixPairs ? 6 : (MODE == MODE_CROSS3 ? 3 : 1);
     static constexpr bool kUpper = MODE == MODE_GRAM || MODE == MODE_GRAM3;
-    // k-blocks per TMEM accumulation chain: short where small terms ride on large ones, 32 (128 MMAs) for plain bf16
-    static constexpr int kFlush = kSixPairs ? 2 : (MODE == MODE_CROSS3 ? 4 : 32);
+    // k-blocks per TMEM accumulation chain: short where small terms ride on large ones, 8 (32 MMAs) for plain bf16.  The drain of
+    // one buffer (about a thousand cycles) hides behind the MMAs of the other even at one k-block of six pairs, and the
+    // truncation bias of the accumulator shrinks with the chain
+    static constexpr int kFlush = kSixPairs ? 1 : (MODE == MODE_CROSS3 ? 2 : 8);
     static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((kAMN ? 1u : 0u) << 15) | (1u << 16)
                                      | ((uint32_t)(TILE_N >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
 };
@@ -241,12 +243,12 @@ k_mma_pipe(const __grid_constant__ Maps maps, int64_t M, int64_t N, int64_t K, f
                 if (!mbar_wait(tfull_bar(buf), (fl >> 1) & 1, abort_flag, wl)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t r[32];
-                    tmem_ld32(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(buf * TILE_N + half * 128 + c * 32), r);
+                for (int c = 0; c < 8; ++c) {             // sixteen columns at a time: 128 sums and 16 new values fit the registers
+                    uint32_t r[16];
+                    tmem_ld16(tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(buf * TILE_N + half * 128 + c * 16), r);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) acc[c * 32 + j] += __uint_as_float(r[j]);
+                    for (int j = 0; j < 16; ++j) acc[c * 16 + j] += __uint_as_float(r[j]);
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
@@ -259,7 +261,7 @@ k_mma_pipe(const __grid_constant__ Maps maps, int64_t M, int64_t N, int64_t K, f
                 float* crow = C + grow * ldc;
                 if (vec_ok) {
                     // 32 x 32 blocks go through shared memory so that a warp touches whole 128-byte lines of C:
-                    // 8 lanes per row, 4 rows per instruction, the 8 row groups of a block in flight together
+                    // 8 lanes per row, 4 rows per instruction
                     float* stg = epi + (warp - 2) * 32 * EPI_LD;
                     const int64_t grow0 = (int64_t)tm * TILE_M + lg * 32;
                     const int rsub = lane >> 3, c4 = (lane & 7) * 4;
@@ -270,26 +272,29 @@ k_mma_pipe(const __grid_constant__ Maps maps, int64_t M, int64_t N, int64_t K, f
 #pragma unroll
                         for (int j = 0; j < 32; ++j) stg[lane * EPI_LD + j] = alpha * acc[c * 32 + j];
                         __syncwarp();
-                        float4 o[8];
-                        if (beta != 0.f) {
-#pragma unroll
-                            for (int q = 0; q < 8; ++q) {
-                                const int64_t gr = grow0 + q * 4 + rsub;
-                                o[q] = (gr < M && gc < N) ? __ldcs(reinterpret_cast<const float4*>(C + gr * ldc + gc))
-                                                          : make_float4(0.f, 0.f, 0.f, 0.f);
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            const int r = q * 4 + rsub;
-                            const int64_t gr = grow0 + r;
-                            const float* sp = stg + r * EPI_LD + c4;
-                            float4 v = make_float4(sp[0], sp[1], sp[2], sp[3]);
+#pragma unroll 1
+                        for (int q0 = 0; q0 < 8; q0 += 4) {          // four row groups at a time: more of them spill the sums
+                            float4 o[4];
                             if (beta != 0.f) {
-                                v.x = fmaf(beta, o[q].x, v.x); v.y = fmaf(beta, o[q].y, v.y);
-                                v.z = fmaf(beta, o[q].z, v.z); v.w = fmaf(beta, o[q].w, v.w);
+#pragma unroll
+                                for (int q = 0; q < 4; ++q) {
+                                    const int64_t gr = grow0 + (q0 + q) * 4 + rsub;
+                                    o[q] = (gr < M && gc < N) ? __ldcs(reinterpret_cast<const float4*>(C + gr * ldc + gc))
+                                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+                                }
                             }
-                            if (gr < M && gc < N) *reinterpret_cast<float4*>(C + gr * ldc + gc) = v;
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const int r = (q0 + q) * 4 + rsub;
+                                const int64_t gr = grow0 + r;
+                                const float* sp = stg + r * EPI_LD + c4;
+                                float4 v = make_float4(sp[0], sp[1], sp[2], sp[3]);
+                                if (beta != 0.f) {
+                                    v.x = fmaf(beta, o[q].x, v.x); v.y = fmaf(beta, o[q].y, v.y);
+                                    v.z = fmaf(beta, o[q].z, v.z); v.w = fmaf(beta, o[q].w, v.w);
+                                }
+                                if (gr < M && gc < N) *reinterpret_cast<float4*>(C + gr * ldc + gc) = v;
+                            }
                         }
                     }
                 } else {
@@ -376,13 +381,14 @@ static void launch_split3(cudaStream_t st, const float* src, int64_t lds, int64_
 // of U in shared memory (up to 96 KB) across a run of 128-column tiles and only the terms of W stream through a
 // two-stage ring (48 KB per 64-wide k-block).  One TMEM accumulator chain per tile (at most 48 MMAs), drained by
 // eight accumulate warps that do the read-modify-write of C through the shared-memory staging blocks.
+constexpr int RU_THREADS = 320;                              // 10 warps: TMA, MMA, eight accumulate warps
 constexpr int RU_TN = 128;                                   // columns per tile
 constexpr int RU_W_BYTES = 3 * (RU_TN / 64) * BOX_BYTES;     // 49152: three terms of a 64 x 128 block of W
 constexpr int RU_U_BYTES = 3 * 2 * A_BYTES;                  // 98304: three terms x two k-blocks of the U band
 constexpr int RU_SMEM = RU_U_BYTES + 2 * RU_W_BYTES + 1024 + 256 + EPI_BYTES;
 constexpr uint32_t kRuIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(RU_TN >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
 
-__global__ void __launch_bounds__(NUM_THREADS, 1)
+__global__ void __launch_bounds__(RU_THREADS, 1)
 k_rank_update(const __grid_constant__ Maps maps, int64_t M, int64_t N, int nkb, float alpha, float* __restrict__ C, int64_t ldc,
               int TN, int nchunk, int num_items, float* __restrict__ sq_part, SearchCtl* __restrict__ ctl,
               const int32_t* __restrict__ done)
@@ -674,6 +680,57 @@ __global__ void k_rownorm_sum(const float* __restrict__ part, int64_t rows, int 
 }
 }  // namespace
 
+// Where the bf16 terms of U (M x K, rows of round_up(K, 8)) and W (K x N, rows of round_up(N, 8)) lie in the scratch.
+bool rank_update_terms(int64_t M, int64_t N, int64_t K, void* scratch, size_t scratch_bytes, RankTerms* t)
+{
+    if ((uintptr_t)scratch & 255) return false;
+    t->k8 = round_up(K, 8); t->ldn = round_up(N, 8);
+    auto align_up = [](size_t x) { return (x + 1023) / 1024 * 1024; };
+    const size_t u_bytes = align_up((size_t)M * t->k8 * 2), w_bytes = align_up((size_t)K * t->ldn * 2);
+    if (3 * (u_bytes + w_bytes) > scratch_bytes) return false;
+    for (int i = 0; i < 3; ++i) {
+        t->u[i] = (char*)scratch + i * u_bytes;
+        t->w[i] = (char*)scratch + 3 * u_bytes + i * w_bytes;
+    }
+    return true;
+}
+
+// C += alpha * U * W from terms already in place (K <= 128, N and ldc multiples of 4, C 16-byte aligned); see rank_update_tc.
+cudaError_t rank_update_run(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alpha, const RankTerms& t, float* C, int64_t ldc,
+                            SearchCtl* ctl_dev, const int32_t* done, float* row_sq, float* sq_scratch)
+{
+    PFN_encodeTiled enc = get_encode();
+    if (!enc) return cudaErrorNotSupported;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_rank_update, cudaFuncAttributeMaxDynamicSharedMemorySize, RU_SMEM);
+    if (e != cudaSuccess) return e;
+    Maps maps;
+    for (int i = 0; i < 3; ++i) {
+        if (!encode_2d(enc, &maps.a[i], t.u[i], (uint64_t)K, (uint64_t)M, (uint64_t)t.k8, BLOCK_K, TILE_M)) return cudaErrorInvalidValue;
+        if (!encode_2d(enc, &maps.b[i], t.w[i], (uint64_t)N, (uint64_t)K, (uint64_t)t.ldn, 64, BLOCK_K)) return cudaErrorInvalidValue;
+    }
+    const int TM = (int)((M + TILE_M - 1) / TILE_M), TN = (int)((N + RU_TN - 1) / RU_TN);
+    int nchunk = (4 * sms + TM - 1) / TM;                 // runs of column tiles per band: about four items per SM
+    if (nchunk > TN) nchunk = TN;
+    if (nchunk < 1) nchunk = 1;
+    const int per = (TN + nchunk - 1) / nchunk;
+    nchunk = (TN + per - 1) / per;                        // no empty runs
+    const int num_items = TM * nchunk;
+    const int nkb = (int)((K + BLOCK_K - 1) / BLOCK_K);
+    k_rank_update<<<num_items < sms ? num_items : sms, RU_THREADS, RU_SMEM, st>>>(maps, M, N, nkb, alpha, C, ldc, TN, nchunk, num_items,
+                                                                                  row_sq ? sq_scratch : nullptr, ctl_dev, done);
+    count_launches(1);
+    if (row_sq) {
+        k_rownorm_sum<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(sq_scratch, M, 2 * TN, row_sq, done);
+        count_launches(1);
+    }
+    return cudaGetLastError();
+}
+
 // C += alpha * U * W for a short inner dimension (see k_rank_update); falls back to the generic product otherwise.
 // With `row_sq` (M floats) and `sq_scratch` (M * 2 * ceil(N / 128) floats) the squared norms of the updated rows come
 // out of the same pass (short-dimension path only; returns cudaErrorInvalidValue otherwise).
@@ -686,48 +743,13 @@ cudaError_t rank_update_tc(cudaStream_t st, int64_t M, int64_t N, int64_t K, flo
     const bool fits = K <= 2 * BLOCK_K && (N % 4) == 0 && (ldc % 4) == 0 && (((uintptr_t)C & 15) == 0);
     if (!fits && row_sq) return cudaErrorInvalidValue;
     if (!fits) return gemm_tc(st, M, N, K, alpha, U, ldu, W, ldw, 1.f, C, ldc, scratch, scratch_bytes, ctl_dev, done);
-    PFN_encodeTiled enc = get_encode();
-    if (!enc) return cudaErrorNotSupported;
-    if ((uintptr_t)scratch & 255) return cudaErrorInvalidValue;
-    const int64_t k8 = round_up(K, 8), ldn = round_up(N, 8);
-    auto align_up = [](size_t x) { return (x + 1023) / 1024 * 1024; };
-    const size_t u_bytes = align_up((size_t)M * k8 * 2), w_bytes = align_up((size_t)K * ldn * 2);
-    if (3 * (u_bytes + w_bytes) > scratch_bytes) return cudaErrorInvalidValue;
-    __nv_bfloat16* up[3]; __nv_bfloat16* wp[3];
-    for (int i = 0; i < 3; ++i) {
-        up[i] = (__nv_bfloat16*)((char*)scratch + i * u_bytes);
-        wp[i] = (__nv_bfloat16*)((char*)scratch + 3 * u_bytes + i * w_bytes);
-    }
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_rank_update, cudaFuncAttributeMaxDynamicSharedMemorySize, RU_SMEM);
-    if (e != cudaSuccess) return e;
-    launch_split3(st, U, ldu, M, K, up[0], up[1], up[2], k8, done);
-    launch_split3(st, W, ldw, K, N, wp[0], wp[1], wp[2], ldn, done);
-    Maps maps;
-    for (int i = 0; i < 3; ++i) {
-        if (!encode_2d(enc, &maps.a[i], up[i], (uint64_t)K, (uint64_t)M, (uint64_t)k8, BLOCK_K, TILE_M)) return cudaErrorInvalidValue;
-        if (!encode_2d(enc, &maps.b[i], wp[i], (uint64_t)N, (uint64_t)K, (uint64_t)ldn, 64, BLOCK_K)) return cudaErrorInvalidValue;
-    }
-    const int TM = (int)((M + TILE_M - 1) / TILE_M), TN = (int)((N + RU_TN - 1) / RU_TN);
-    int nchunk = (4 * sms + TM - 1) / TM;                 // runs of column tiles per band: about four items per SM
-    if (nchunk > TN) nchunk = TN;
-    if (nchunk < 1) nchunk = 1;
-    const int per = (TN + nchunk - 1) / nchunk;
-    nchunk = (TN + per - 1) / per;                        // no empty runs
-    const int num_items = TM * nchunk;
-    const int nkb = (int)((K + BLOCK_K - 1) / BLOCK_K);
-    k_rank_update<<<num_items < sms ? num_items : sms, NUM_THREADS, RU_SMEM, st>>>(maps, M, N, nkb, alpha, C, ldc, TN, nchunk, num_items,
-                                                                                  row_sq ? sq_scratch : nullptr, ctl_dev, done);
-    count_launches(3);
-    if (row_sq) {
-        k_rownorm_sum<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(sq_scratch, M, 2 * TN, row_sq, done);
-        count_launches(1);
-    }
-    return cudaGetLastError();
+    RankTerms t;
+    if (!rank_update_terms(M, N, K, scratch, scratch_bytes, &t)) return cudaErrorInvalidValue;
+    auto bf = [](void* p) { return (__nv_bfloat16*)p; };
+    launch_split3(st, U, ldu, M, K, bf(t.u[0]), bf(t.u[1]), bf(t.u[2]), t.k8, done);
+    launch_split3(st, W, ldw, K, N, bf(t.w[0]), bf(t.w[1]), bf(t.w[2]), t.ldn, done);
+    count_launches(2);
+    return rank_update_run(st, M, N, K, alpha, t, C, ldc, ctl_dev, done, row_sq, sq_scratch);
 }
 
 // H (+)= Xc^T Xc over the upper-triangle tiles (Yc == nullptr), or G (+)= Xc^T Yc over all tiles.

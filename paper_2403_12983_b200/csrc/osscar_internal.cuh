@@ -170,6 +170,12 @@ cudaError_t rank_update_tc(cudaStream_t st, int64_t M, int64_t N, int64_t K, flo
                            void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done = nullptr,
                            float* row_sq = nullptr, float* sq_scratch = nullptr);
 
+// The two halves of rank_update_tc for a caller that writes the bf16 terms itself.
+struct RankTerms { void *u[3], *w[3]; int64_t k8, ldn; };
+bool rank_update_terms(int64_t M, int64_t N, int64_t K, void* scratch, size_t scratch_bytes, RankTerms* t);
+cudaError_t rank_update_run(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alpha, const RankTerms& t, float* C, int64_t ldc,
+                            SearchCtl* ctl_dev, const int32_t* done = nullptr, float* row_sq = nullptr, float* sq_scratch = nullptr);
+
 // H (+)= Xc^T Xc (upper-triangle tiles; Y null) or G (+)= Xc^T Yc with the drained-accumulator pipeline of gemm_tc.cu.
 cudaError_t gram_tc2(cudaStream_t st, const void* X, int64_t n_rows, int64_t d1, const void* Y, int y_fp32, int64_t m,
                      float* C, bool accumulate, void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev);
