@@ -209,7 +209,8 @@ int osscar_gram(osscar_ctx* ctx, const void* X, int x_dtype, int64_t n_rows, int
             // overwritten), else (or when it cannot hold a 64-row panel of the terms) the fp32 pipes
             cudaError_t ge = cudaErrorMemoryAllocation;
             if (ctx->ws) {
-                ge = gram_tc3(st, (const float*)X, n_rows, d1, H, !begin, ctx->ws, ctx->ws_bytes, ctx->ctl);
+                ge = gram_i8(st, (const float*)X, n_rows, d1, H, !begin, ctx->ws, ctx->ws_bytes, ctx->ctl);
+                if (ge == cudaErrorMemoryAllocation) ge = gram_tc3(st, (const float*)X, n_rows, d1, H, !begin, ctx->ws, ctx->ws_bytes, ctx->ctl);
                 if (ge == cudaSuccess) ctx->have_state = false;
             }
             if (ge == cudaErrorMemoryAllocation)
@@ -230,7 +231,7 @@ int osscar_gram(osscar_ctx* ctx, const void* X, int x_dtype, int64_t n_rows, int
     if (ctx->ws && ctx->ws_bytes >= gemm_tc_min_scratch(d1, m)) {
         // tensor-core product with the operand terms staged in the lent workspace (its contents are overwritten)
         const size_t cap = ctx->ws_bytes < ((size_t)3 << 30) ? ctx->ws_bytes : ((size_t)3 << 30);
-        CKS(gemm_tc(st, d1, m, d1, 1.f, H, d1, W, m, 0.f, G, m, ctx->ws, cap, ctx->ctl));
+        CKS(cross_term_tc(st, H, d1, W, m, G, ctx->ws, cap, ctx->ctl));
         ctx->have_state = false;
     } else {
         CKS(sgemm(st, false, false, d1, m, d1, 1.f, H, d1, W, m, 0.f, G, m));
@@ -279,7 +280,8 @@ int osscar_gram_cross(osscar_ctx* ctx, const void* X, int x_dtype, const void* Y
             // H as in osscar_gram: on the tensor cores when a workspace can stage the bf16 terms, else the fp32 pipes
             cudaError_t ge = cudaErrorMemoryAllocation;
             if (ctx->ws) {
-                ge = gram_tc3(st, (const float*)X, n_rows, d1, H, !begin, ctx->ws, ctx->ws_bytes, ctx->ctl);
+                ge = gram_i8(st, (const float*)X, n_rows, d1, H, !begin, ctx->ws, ctx->ws_bytes, ctx->ctl);
+                if (ge == cudaErrorMemoryAllocation) ge = gram_tc3(st, (const float*)X, n_rows, d1, H, !begin, ctx->ws, ctx->ws_bytes, ctx->ctl);
                 if (ge == cudaSuccess) ctx->have_state = false;
             }
             if (ge == cudaErrorMemoryAllocation)
@@ -420,13 +422,19 @@ int osscar_objective(osscar_ctx* ctx, const float* H, const float* W, const floa
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return OSSCAR_E_CUDA;
     cudaStream_t st = ctx->stream;
-    float* E = (float*)ctx->ws;
-    float* HE = E + d1 * m;
     k_clear_status<<<1, 1, 0, st>>>(ctx->ctl);
-    k_sub<<<1184, 256, 0, st>>>(W, Wt, E, d1 * m);
-    count_launches(2);
-    CKS(sgemm(st, false, false, d1, m, d1, 1.f, H, d1, E, m, 0.f, HE, m));
-    CKS(trace_product(st, E, m, HE, m, d1, m, ctx->partials, &ctx->ctl->acc[0]));
+    count_launches(1);
+    // from digits on the int8 tensor cores (within the 2 * d1 * m floats); small layers on the fp32 pipes
+    cudaError_t oe = objective_i8(st, H, W, Wt, d1, m, ctx->ws, need / 256 * 256, ctx->partials, &ctx->ctl->acc[0], ctx->ctl);
+    if (oe == cudaErrorMemoryAllocation) {
+        float* E = (float*)ctx->ws;
+        float* HE = E + d1 * m;
+        k_sub<<<1184, 256, 0, st>>>(W, Wt, E, d1 * m);
+        count_launches(1);
+        CKS(sgemm(st, false, false, d1, m, d1, 1.f, H, d1, E, m, 0.f, HE, m));
+        oe = trace_product(st, E, m, HE, m, d1, m, ctx->partials, &ctx->ctl->acc[0]);
+    }
+    CKS(oe);
     CKS(cudaMemcpyAsync(ctx->ctl_host, ctx->ctl, sizeof(SearchCtl), cudaMemcpyDeviceToHost, st));
     CKS(cudaStreamSynchronize(st));
     ctx->have_state = false;      // the workspace start was overwritten

@@ -10,6 +10,7 @@ namespace osscar {
 constexpr int kTracePartials = 1184;   // blocks of a trace reduction; the context owns that many doubles
 constexpr int64_t kMaxPairs = 1 << 20;     // PAIR_EXACT scores at most this many (kept, pruned) pairs per step
 constexpr int kLoopMaxBlocks = 2048;   // most blocks the persistent swap loop is launched with (size of its candidate lists)
+constexpr double kTinyProduct = 16777216.0;   // multiply-adds (256^3) up to which a product is one launch on the fp64 pipe
 constexpr size_t kFreeDynSmem = 40 * 1024;   // dynamic shared memory above which a kernel asks for more (48 KB less its static arrays)
 constexpr int kPadF = 32;   // leading dimensions of internal fp32 matrices are padded to this many floats
 
@@ -133,18 +134,31 @@ struct I8Gemm {                    // C = beta * C0 + alpha * A * B, A (M x K) a
     int64_t M, N, K;
     double alpha, beta;
     const float* A; int64_t lda;
-    const float* B; const double* Bd; int64_t ldb;     // fp32 B, or fp64 Bd
-    const float* C0; int64_t ldc0;
+    const float *B, *Bsub; const double* Bd; int64_t ldb;     // fp32 B (minus Bsub), or fp64 Bd
+    const float* BT;               // or B transposed, N rows of K (without a balance: diag null)
+    const float *C0, *C0sub; int64_t ldc0;
     void* C; int64_t ldc;
     bool identity;                 // I + alpha A B instead of beta C0 + alpha A B
+    int64_t identity_col0;         // column of I that column 0 of the product is
     bool out64;                    // C in fp64
     bool tri;                      // B symmetric, K = N: its block upper triangle with halved diagonal blocks (see dgemm.cu)
-    bool dot;                      // C (doubles, gemm_i8_dot_cols(N) per row) = partial sums of rows of A B times rows of C0
-    const float* diag; int64_t diag_stride;            // diagonal of H_II: balances the contraction index
+    bool dot;                      // C (doubles, gemm_i8_dot_cols(N) per row) = partial sums of rows of A B times rows of C0 (- C0sub)
+    const float* diag; int64_t diag_stride;            // diagonal of H_II: balances the contraction index (null: none)
+    bool inverse_scale;            // the columns of A scale like those of the inverse of H, not like those of H
 };
 bool gemm_i8_usable(int64_t M, int64_t N, int64_t K, int S, const I8Scratch& sc);
 cudaError_t gemm_i8(cudaStream_t st, const I8Gemm& p, int S, I8Scratch& sc, SearchCtl* ctl_dev, const int32_t* done);
 int64_t gemm_i8_dot_cols(int64_t N);
+// H (+)= Xc^T Xc (upper-triangle tiles) for fp32 Xc; cudaErrorMemoryAllocation: too small a product or scratch, take another path
+cudaError_t gram_i8(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1, float* C, bool accumulate,
+                    void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev);
+// G = H W (H d1 x d1, W and G d1 x m, dense) from four digits of each operand, or as gemm_tc where they do not pay or fit
+cudaError_t cross_term_tc(cudaStream_t st, const float* H, int64_t d1, const float* W, int64_t m, float* G,
+                          void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev);
+// *out = sum of (W - Wt) o H (W - Wt) (H d1 x d1, W and Wt d1 x m, dense); `partials`: the context's reduction scratch.
+// cudaErrorMemoryAllocation when the product is too small for digits or the scratch too small for them.
+cudaError_t objective_i8(cudaStream_t st, const float* H, const float* W, const float* Wt, int64_t d1, int64_t m,
+                         void* scratch, size_t scratch_bytes, double* partials, double* out_dev, SearchCtl* ctl_dev);
 size_t gemm_i8_operand_bytes(int64_t rows, int64_t K, int S);      // scratch that holds the digits of a whole operand
 
 // ---- panel_tc.cu: Y[i*so_row + e*so_col] = sum_k A[i][k] * P[e][k] on the tensor cores; A (M x K, streamed once) is split
@@ -191,12 +205,16 @@ cudaError_t gram_mirror(cudaStream_t st, float* H, int64_t d1);   // copy upper 
 // ---- state.cu: support selection and state construction --------------------------------------
 int select_support(osscar_ctx* ctx, int mode, int32_t* support);
 int build_state(osscar_ctx* ctx, bool guarded);
+// C = A B + beta C0 for A = Hinv or E (nI x nI): digits on the int8 tensor cores, or split bf16 where they do not pay or fit
+cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const float* B, int64_t ldb, float beta, const float* C0, float* C,
+                            int64_t ldc, int digits, void* other, size_t other_bytes, const int32_t* done);
 // E = I - H_II Hinv summed beyond fp32; `v_free`: V and R hold nothing yet, so their memory may take operand digits
 cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32_t* done);
 int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref, const int32_t* done,
                        bool tensor_updates);
 cudaError_t gather_rows(cudaStream_t st, const float* src, int64_t m, int g, const int32_t* perm,
                         int64_t slot_row0, int64_t nrows, float* dst, int64_t ld);
+cudaError_t sum_partials(cudaStream_t st, const double* partials, int n, double* out_dev);   // *out = sum, fixed order
 cudaError_t trace_product(cudaStream_t st, const float* A, int64_t lda, const float* B, int64_t ldb,
                           int64_t rows, int64_t cols, double* partials, double* out_dev);   // *out = sum A.*B
 

@@ -1085,15 +1085,15 @@ int build_hinv64(osscar_ctx* ctx, bool guarded, bool v_free)
     float* E = (float*)(ws + L.off_big);
     float* T = E + L.nI * L.ldh;
     const int32_t* done = guarded ? &ctx->ctl->done : nullptr;
-    void* tc = ws + L.off_tc;
     // X0 = the fp32 inverse at hand (raw from the blocked inversion, or carried by an fp32 driver).  With E = I - H_II X0,
-    // H_II^-1 = X0 (I + E + E^2 + ...): E is formed once with fp64 sums, the series is cut after E^2 (its products are
-    // corrections of corrections: the tensor-core split product is ample), and the sum X0 + X0 (E + E^2) is taken in fp64.
+    // H_II^-1 = X0 (I + E + E^2 + ...): E is formed once with sums beyond fp32, the series is cut after E^2 (a correction of a
+    // correction: three digits are ample; four for X0 (E + E^2)), and the sum X0 + X0 (E + E^2) is taken in fp64.
     // The error left is E^3 (below 1e-9 for any start within 1e-3), against E^2 for a single Newton-Schulz step.
     if (inverse_residual(ctx, E, v_free, done) != cudaSuccess) return OSSCAR_E_CUDA;
-    if (cudaMemcpyAsync(T, E, sizeof(float) * L.nI * L.ldh, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return OSSCAR_E_CUDA;
-    if (gemm_tc(st, L.nI, L.nI, L.nI, 1.f, E, L.ldh, E, L.ldh, 1.f, T, L.ldh, tc, L.tc_bytes, ctx->ctl, done) != cudaSuccess) return OSSCAR_E_CUDA;
-    if (gemm_tc(st, L.nI, L.nI, L.nI, 1.f, Hinv, L.ldh, T, L.ldh, 0.f, E, L.ldh, tc, L.tc_bytes, ctx->ctl, done) != cudaSuccess) return OSSCAR_E_CUDA;
+    char* const other = ws + L.off_Hd;                                     // written only below: may hold digits
+    const size_t other_bytes = (v_free ? L.off_y : L.off_V) - L.off_Hd;
+    if (inverse_product(ctx, L.nI, E, E, L.ldh, 1.f, E, T, L.ldh, 3, other, other_bytes, done) != cudaSuccess) return OSSCAR_E_CUDA;
+    if (inverse_product(ctx, L.nI, Hinv, T, L.ldh, 0.f, nullptr, E, L.ldh, 4, other, other_bytes, done) != cudaSuccess) return OSSCAR_E_CUDA;
     k_hinv_to_d<<<(unsigned)L.nI, 256, 0, st>>>(Hinv, E, Hd, L.ldh, L.nI, done);
     k_hinv_from_d<<<(unsigned)L.nI, 256, 0, st>>>(Hd, Hinv, L.ldh, done);
     count_launches(2);
@@ -1172,10 +1172,29 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         float* Pm = (float*)((char*)ctx->ws + L.off_big);
         const int64_t ldj = round_up(L.nJ, kPadF);
         float* XG = Pm + L.nJ * L.ldh;
-        cudaError_t e = sgemm(st, false, false, L.nJ, L.nI, L.nI, 1.f, p.Hp + L.nI * L.ldp, L.ldp, p.Hinv, L.ldh, 0.f, Pm, L.ldh,
-                              &ctx->ctl->done);
+        // both from four digits on the int8 tensor cores where that pays (32 heads of 80 rows, m = 2560: scoring all
+        // pairs 938 -> 599 us against the fp32 pipes), the digits of B in the front half of the tensor-core region and those of A in the rest
+        auto digits = [&](I8Gemm& q, float* C, int64_t ldc) -> cudaError_t {
+            I8Scratch sc;
+            const size_t half = L.tc_bytes / 2 / 256 * 256;
+            sc.b = (char*)ctx->ws + L.off_tc; sc.b_bytes = half;
+            sc.a = (char*)ctx->ws + L.off_tc + half; sc.a_bytes = L.tc_bytes - half;
+            if (!gemm_i8_usable(q.M, q.N, q.K, 4, sc)) return cudaErrorMemoryAllocation;
+            q.alpha = 1.0; q.C = C; q.ldc = ldc;
+            return gemm_i8(st, q, 4, sc, ctx->ctl, &ctx->ctl->done);
+        };
+        I8Gemm q = {};
+        q.M = L.nJ; q.N = q.K = L.nI; q.A = p.Hp + L.nI * L.ldp; q.lda = L.ldp; q.B = p.Hinv; q.ldb = L.ldh;
+        q.diag = p.Hp; q.diag_stride = L.ldp + 1;
+        cudaError_t e = digits(q, Pm, L.ldh);
+        if (e == cudaErrorMemoryAllocation)
+            e = sgemm(st, false, false, L.nJ, L.nI, L.nI, 1.f, p.Hp + L.nI * L.ldp, L.ldp, p.Hinv, L.ldh, 0.f, Pm, L.ldh, &ctx->ctl->done);
         if (e != cudaSuccess) return e;
-        e = sgemm(st, false, true, L.nI, L.nJ, L.m, 1.f, p.V, L.ldm, p.R, L.ldm, 0.f, XG, ldj, &ctx->ctl->done);
+        q = I8Gemm{};
+        q.M = L.nI; q.N = L.nJ; q.K = L.m; q.A = p.V; q.lda = L.ldm; q.BT = p.R; q.ldb = L.ldm;
+        e = digits(q, XG, ldj);
+        if (e == cudaErrorMemoryAllocation)
+            e = sgemm(st, false, true, L.nI, L.nJ, L.m, 1.f, p.V, L.ldm, p.R, L.ldm, 0.f, XG, ldj, &ctx->ctl->done);
         if (e != cudaSuccess) return e;
         const size_t smem = 3 * (size_t)g * g * sizeof(double);
         e = cudaFuncSetAttribute(k_pair_slots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

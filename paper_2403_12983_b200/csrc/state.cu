@@ -359,6 +359,13 @@ cudaError_t trace_product(cudaStream_t st, const float* A, int64_t lda, const fl
     return cudaGetLastError();
 }
 
+cudaError_t sum_partials(cudaStream_t st, const double* partials, int n, double* out_dev)
+{
+    k_sum_partials<<<1, 256, 0, st>>>(partials, n, out_dev);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 int make_layout(int64_t d1, int64_t m, int32_t g, int32_t k, Layout* L)
 {
     if (d1 <= 0 || m <= 0 || g <= 0 || g > OSSCAR_MAX_GROUP || d1 % g != 0) return OSSCAR_E_SHAPE;
@@ -533,6 +540,33 @@ static unsigned schur_shares(int64_t slots, int g)
 
 constexpr int kResidualDigits = 6, kDirectDigits = 5;      // see gemm_i8.cu
 
+// The products that only have to be as good as fp32 ones: four digits of an operand (31 bits below the largest entry of a row or
+// column, balanced), three where the result is itself a small correction.  (Three for V left its error at d1 = 8192 at 3.8e-8
+// against the 2.5e-8 of its fp32 rounding.)
+cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const float* B, int64_t ldb, float beta, const float* C0, float* C,
+                            int64_t ldc, int digits, void* other, size_t other_bytes, const int32_t* done)
+{
+    const Layout& L = ctx->L;
+    char* ws = (char*)ctx->ws;
+    const float* Hp = (const float*)(ws + L.off_Hp);
+    I8Scratch sc = i8_scratch(ctx, N, L.nI, digits, other, other_bytes);
+    if (gemm_i8_usable(L.nI, N, L.nI, digits, sc)) {
+        I8Gemm p = {};
+        p.M = L.nI; p.N = N; p.K = L.nI; p.alpha = 1.0; p.beta = beta;
+        p.A = A; p.lda = L.ldh; p.B = B; p.ldb = ldb; p.C0 = beta != 0.f ? C0 : nullptr; p.ldc0 = ldc; p.C = C; p.ldc = ldc;
+        p.diag = Hp; p.diag_stride = L.ldp + 1; p.inverse_scale = true;
+        return gemm_i8(ctx->stream, p, digits, sc, ctx->ctl, done);
+    }
+    // the smallest layers: one launch on the fp64 pipe instead of three (two splits and a product with a handful of tiles)
+    if ((double)L.nI * L.nI * (double)N <= kTinyProduct)
+        return gemm_f64acc(ctx->stream, L.nI, N, L.nI, 1.0, A, L.ldh, B, ldb, (double)beta, C0, ldc, C, ldc, false, done);
+    if (beta != 0.f && C0 != C) {
+        const cudaError_t e = cudaMemcpyAsync(C, C0, sizeof(float) * L.nI * ldc, cudaMemcpyDeviceToDevice, ctx->stream);
+        if (e != cudaSuccess) return e;
+    }
+    return gemm_tc(ctx->stream, L.nI, N, L.nI, 1.f, A, L.ldh, B, ldb, beta, C, ldc, ws + L.off_tc, L.tc_bytes, ctx->ctl, done);
+}
+
 cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32_t* done)
 {
     const Layout& L = ctx->L;
@@ -593,23 +627,24 @@ int build_state(osscar_ctx* ctx, bool guarded)
         float* E = big;
         float* Dlt = big + nI * L.ldh;
         CK(inverse_residual(ctx, E, true, done));
-        CK(gemm_tc(st, nI, nI, nI, 1.f, Hinv, L.ldh, E, L.ldh, 0.f, Dlt, L.ldh, tc, L.tc_bytes, ctx->ctl, done));
+        CK(inverse_product(ctx, nI, Hinv, E, L.ldh, 0.f, nullptr, Dlt, L.ldh, 3, ws + L.off_Hd, L.off_y - L.off_Hd, done));
         k_add_sym<<<dim3((unsigned)((nI + 31) / 32), (unsigned)((nI + 31) / 32)), dim3(32, 8), 0, st>>>(Hinv, L.ldh, Dlt, L.ldh, nI, done);
         count_launches(1);
     }
-    // (2) V = Hinv G_I on the tensor cores, then one refinement step with the residual G_I - H_II V in fp64
+    // (2) V = Hinv G_I, then one refinement step with the residual G_I - H_II V
     float* GI = big;
     float* rV = big + nI * L.ldm;
     k_gather_rows<<<(unsigned)nI, 256, 0, st>>>(ctx->G, L.m, L.g, perm, 0, GI, L.ldm);
     count_launches(1);
     if (L.ldm != L.m) CK(cudaMemsetAsync(V, 0, sizeof(float) * nI * L.ldm, st));     // padding columns stay zero
-    CK(gemm_tc(st, nI, L.m, nI, 1.f, Hinv, L.ldh, GI, L.ldm, 0.f, V, L.ldm, tc, L.tc_bytes, ctx->ctl, done));
     const int64_t big_floats = (int64_t)((L.off_Hp - L.off_big) / sizeof(float));
     {   // digits beside GI and rV, or in the place of R
         const size_t used = sizeof(float) * 2 * (size_t)nI * L.ldm, tail = sizeof(float) * (size_t)big_floats - used;
         const size_t rbytes = L.off_y - L.off_R;
-        I8Scratch sc = tail > rbytes ? i8_scratch(ctx, L.m, nI, kResidualDigits, (char*)big + used, tail)
-                                     : i8_scratch(ctx, L.m, nI, kResidualDigits, R, rbytes);
+        void* other = tail > rbytes ? (void*)((char*)big + used) : (void*)R;
+        const size_t other_bytes = tail > rbytes ? tail : rbytes;
+        CK(inverse_product(ctx, L.m, Hinv, GI, L.ldm, 0.f, nullptr, V, L.ldm, 4, other, other_bytes, done));
+        I8Scratch sc = i8_scratch(ctx, L.m, nI, kResidualDigits, other, other_bytes);
         if (gemm_i8_usable(nI, L.m, nI, kResidualDigits, sc)) {
             I8Gemm p = {};
             p.M = nI; p.N = L.m; p.K = nI; p.alpha = -1.0; p.beta = 1.0;
@@ -618,9 +653,8 @@ int build_state(osscar_ctx* ctx, bool guarded)
             CK(gemm_i8(st, p, kResidualDigits, sc, ctx->ctl, done));
         } else
             CK(gemm_f64acc(st, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false, done));
-        // gemm_i8 leaves the pad columns of rV alone; they meet no valid column of V below
+        CK(inverse_product(ctx, L.m, Hinv, rV, L.ldm, 1.f, V, V, L.ldm, 4, other, other_bytes, done));
     }
-    CK(gemm_tc(st, nI, L.m, nI, 1.f, Hinv, L.ldh, rV, L.ldm, 1.f, V, L.ldm, tc, L.tc_bytes, ctx->ctl, done));
     // obj = Tr(W^T G) - Tr(G_I^T V)
     if (ctx->have_const) CK(set_device_double(st, &ctx->ctl->acc[0], ctx->user_const));
     else CK(trace_product(st, ctx->W, L.m, ctx->G, L.m, L.d1, L.m, ctx->partials, &ctx->ctl->acc[0]));
@@ -678,13 +712,13 @@ int build_state(osscar_ctx* ctx, bool guarded)
             for (int64_t t0 = 0; t0 < L.ng - L.k; t0 += gpp) {
                 const int64_t ngr = L.ng - L.k - t0 < gpp ? L.ng - L.k - t0 : gpp;
                 const float* At = Hp + (nI + t0 * L.g) * L.ldp;
-                I8Scratch sc = i8_scratch(ctx, nI, nI, kDirectDigits, nullptr, 0);
-                if (!one && gemm_i8_usable(ngr * L.g, nI, nI, kDirectDigits, sc)) {
+                I8Scratch sc = i8_scratch(ctx, nI, nI, kResidualDigits, nullptr, 0);
+                if (!one && gemm_i8_usable(ngr * L.g, nI, nI, kResidualDigits, sc)) {
                     I8Gemm p = {};
                     p.M = ngr * L.g; p.N = nI; p.K = nI; p.alpha = 1.0; p.out64 = true;
                     p.A = At; p.lda = L.ldp; p.B = Hinv; p.ldb = L.ldh; p.C = Pm; p.ldc = L.ldh;
                     p.diag = Hp; p.diag_stride = L.ldp + 1;
-                    CK(gemm_i8(st, p, kDirectDigits, sc, ctx->ctl, done));
+                    CK(gemm_i8(st, p, kResidualDigits, sc, ctx->ctl, done));
                 } else
                     CK(gemm_f64out(st, ngr * L.g, nI, nI, At, L.ldp, Hinv, L.ldh, Pm, L.ldh, done, one));
                 k_schur<<<dim3((unsigned)ngr, schur_shares(ngr, L.g)), 256, 0, st>>>(Hp, L.ldp, Pm, L.ldh, nI, L.g, c, t0, one ? 2.0 : 1.0, done);
