@@ -1,5 +1,5 @@
 // Starting support and construction of the search state for a given support:
-// slot-permuted copy of H, (H_II)^-1 by an in-place blocked exchange (Gauss-Jordan) inversion,
+// slot-permuted copy of H, (H_II)^-1 (invert.cu) and its correction,
 // V = (H_II)^-1 G_I (Eq. tmp5), residual R, Schur complements c (Case 2 of Proposition 1).
 #include "osscar_internal.cuh"
 #include <math.h>
@@ -50,18 +50,26 @@ __global__ void k_energy(const float* __restrict__ H, const float* __restrict__ 
     if (threadIdx.x == 0) e[q] = acc;
 }
 
-// kept[q] = 1 iff fewer than k groups beat q (larger energy, or equal energy and smaller id).
+__device__ __forceinline__ int warp_count(int v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// kept[q] = 1 iff fewer than k groups beat q (larger energy, or equal energy and smaller id); a warp per group.
 __global__ void k_rank_select(const double* __restrict__ e, int64_t ng, int k, int32_t* __restrict__ kept)
 {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (q >= ng) return;
     const double eq = e[q];
     int rank = 0;
-    for (int64_t p = 0; p < ng; ++p) {
+#pragma unroll 4
+    for (int64_t p = threadIdx.x & 31; p < ng; p += 32) {
         const double ep = e[p];
         rank += (ep > eq) || (ep == eq && p < q);
     }
-    kept[q] = rank < k;
+    rank = warp_count(rank);
+    if ((threadIdx.x & 31) == 0) kept[q] = rank < k;
 }
 
 __global__ void k_user_support(const int32_t* __restrict__ support, int k, int64_t ng,
@@ -91,15 +99,18 @@ __global__ void __launch_bounds__(1024) k_user_support_guard(int32_t* __restrict
     if (threadIdx.x == 0 && ctl->status == OSSCAR_OK) ctl->status = OSSCAR_E_ARG;
 }
 
-// Slots: kept groups in ascending id order take slots 0..k-1, pruned groups k..ng-1.
+// Slots: kept groups in ascending id order take slots 0..k-1, pruned groups k..ng-1; a warp per group.
 __global__ void k_build_perm(const int32_t* __restrict__ kept, int64_t ng, int k,
                              int32_t* __restrict__ perm, int32_t* __restrict__ slotof,
                              int32_t* __restrict__ support)
 {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (q >= ng) return;
     int before_kept = 0;
-    for (int64_t p = 0; p < q; ++p) before_kept += kept[p];
+#pragma unroll 4
+    for (int64_t p = threadIdx.x & 31; p < q; p += 32) before_kept += kept[p];
+    before_kept = warp_count(before_kept);
+    if ((threadIdx.x & 31) != 0) return;
     const int slot = kept[q] ? before_kept : k + (int)(q - before_kept);
     if (slot < 0 || slot >= ng || (kept[q] && slot >= k)) return;       // cannot happen with exactly k marks
     perm[slot] = (int32_t)q;
@@ -107,20 +118,33 @@ __global__ void k_build_perm(const int32_t* __restrict__ kept, int64_t ng, int k
     if (kept[q]) support[slot] = (int32_t)q;
 }
 
-// Hp[i][j] = H[row(i)][row(j)], row(i) = perm[i / g] * g + i % g.
-__global__ void k_gather_sym(const float* __restrict__ H, int64_t d1, int g, const int32_t* __restrict__ perm,
+// Hp[i][j] = H[row(i)][row(j)], row(i) = perm[i / g] * g + i % g.  A thread owns four columns, whose source columns it looks up
+// once for GS_R rows: 32 independent loads in flight and 16-byte stores.  Bound: HBM, 8 d1^2 bytes.  With one element and
+// one look-up (two 64-bit divisions) per thread and step this copy took 6.4 ms at d1 = 28672, now 1.3 ms.
+constexpr int GS_R = 8;
+__global__ void __launch_bounds__(256) k_gather_sym(const float* __restrict__ H, int64_t d1, int g, const int32_t* __restrict__ perm,
                              float* __restrict__ Hp, int64_t ldp)
 {
-    const int64_t i = blockIdx.x;
-    const int64_t ri = (int64_t)perm[i / g] * g + i % g;
-    for (int64_t j = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; j < ldp; j += (int64_t)gridDim.y * blockDim.x) {
-        float v = 0.f;
-        if (j < d1) {
-            const int64_t rj = (int64_t)perm[j / g] * g + j % g;
-            v = H[ri * d1 + rj];
-        }
-        Hp[i * ldp + j] = v;
+    const int64_t j0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4, i0 = (int64_t)blockIdx.y * GS_R;
+    if (j0 >= ldp) return;
+    const uint32_t ug = (uint32_t)g;
+    int64_t col[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t j = (uint32_t)j0 + k;
+        col[k] = j < d1 ? (int64_t)perm[j / ug] * g + j % ug : -1;
     }
+    float v[GS_R][4];
+#pragma unroll
+    for (int r = 0; r < GS_R; ++r) {
+        const uint32_t i = (uint32_t)i0 + r;
+        const float* row = H + (i < d1 ? (int64_t)perm[i / ug] * g + i % ug : 0) * d1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[r][k] = i < d1 && col[k] >= 0 ? row[col[k]] : 0.f;
+    }
+#pragma unroll
+    for (int r = 0; r < GS_R; ++r)
+        if (i0 + r < d1) *reinterpret_cast<float4*>(Hp + (i0 + r) * ldp + j0) = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
 }
 
 // dst[i][0..ld) = src[row(slot0*g + i)][0..m) zero-padded, for i in [0, nrows).
@@ -139,112 +163,6 @@ __global__ void k_copy_pad(const float* __restrict__ src, int64_t lds, int64_t r
 {
     const int64_t i = blockIdx.x;
     for (int64_t c = threadIdx.x; c < ldd; c += blockDim.x) dst[i * ldd + c] = c < cols ? src[i * lds + c] : 0.f;
-}
-
-// ---------------------------------------------------------------- blocked exchange inversion
-constexpr int NB = 64;
-constexpr double kPivotRelTol = 1e-7;
-
-// Inverse of the nb x nb pivot block A[p0:p0+nb, p0:p0+nb] in fp64 (one block of 1024 threads): Gauss-Jordan
-// elimination without pivoting with the block held in registers.  Thread (i, cb) = (t / 16, t % 16) owns the entries
-// (i, cb + 16 k), k = 0..3.  In step j every thread fetches its row's entry of column j by a shuffle inside its
-// half-warp, the threads of row j publish the scaled pivot row through shared memory (double-buffered: one barrier per
-// step), and every entry takes its rank-1 update.  The pivots are the diagonal of the successive Schur complements
-// (the squared diagonal of the Cholesky factor).  Raises OSSCAR_E_NOTPD in ctl->status when a pivot is not positive.
-__global__ void __launch_bounds__(1024)
-k_pivot_inverse(const float* __restrict__ A, int64_t lda, int64_t p0, int nb, float* __restrict__ Dinv,
-                const float* __restrict__ Hp, int64_t ldp, SearchCtl* ctl)
-{
-    static_assert(NB == 64, "thread layout of the pivot inverse");
-    __shared__ double rowj[2][NB];
-    __shared__ double pinv_s[2];
-    __shared__ double hdiag[NB];         // diagonal of the original matrix: scale of the pivot test
-    __shared__ double Ls[NB][NB + 1];    // the finished inverse, for the symmetrised write
-    __shared__ int bad;
-    const int t = threadIdx.x, i = t >> 4, cb = t & 15, lane = t & 31;
-    double Lr[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int c = cb + 16 * k;
-        // symmetrise: the two triangles can differ in the last bits
-        Lr[k] = (i < nb && c < nb) ? 0.5 * ((double)A[(p0 + i) * lda + p0 + c] + (double)A[(p0 + c) * lda + p0 + i]) : 0.0;
-    }
-    if (t == 0) bad = 0;
-    if (t < nb) hdiag[t] = (double)Hp[(p0 + t) * ldp + p0 + t];
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-        for (int jj = 0; jj < 16; ++jj) {
-            const int j = kk * 16 + jj;
-            if (j >= nb) break;
-            const int buf = j & 1;
-            const double x = __shfl_sync(0xffffffffu, Lr[kk], (lane & 16) | jj);     // entry (i, j) of this thread's row
-            if (i == j) {
-                double d = x;
-                // a pivot that fp32 data cannot tell from zero counts as not positive
-                if (!(d > kPivotRelTol * hdiag[j])) { if (cb == 0) bad = 1; d = 1.0; }
-                const double pinv = 1.0 / d;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) rowj[buf][cb + 16 * k] = Lr[k] * pinv;
-                if (cb == 0) pinv_s[buf] = pinv;
-            }
-            __syncthreads();
-            const double pinv = pinv_s[buf];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int c = cb + 16 * k;
-                const double r = rowj[buf][c];
-                double v;
-                if (i == j) v = (c == j) ? pinv : r;
-                else if (c == j) v = -x * pinv;
-                else v = Lr[k] - x * r;
-                Lr[k] = v;
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) Ls[i][cb + 16 * k] = Lr[k];
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {                  // the two triangles differ by rounding only
-        const int c = cb + 16 * k;
-        if (i < nb && c < nb) Dinv[i * NB + c] = (float)(0.5 * (Ls[i][c] + Ls[c][i]));
-    }
-    if (t == 0 && bad && ctl->status == OSSCAR_OK) ctl->status = OSSCAR_E_NOTPD;       // the first error is the one reported
-}
-
-// U = A[p0:p0+nb, 0:n) (copy of the pivot rows), and zero T's pivot rows afterwards is done in k_zero_rows.
-__global__ void k_copy_rows(const float* __restrict__ A, int64_t lda, int64_t p0, int nb, int64_t n,
-                            float* __restrict__ U, int64_t ldu)
-{
-    const int i = blockIdx.y;
-    if (i >= nb) return;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x)
-        U[i * ldu + c] = A[(p0 + i) * lda + c];
-}
-__global__ void k_zero_rows(float* __restrict__ T, int64_t ldt, int64_t p0, int nb, int ncols)
-{
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < nb * ncols) T[(p0 + idx / ncols) * ldt + idx % ncols] = 0.f;
-}
-// A[:, P] = T (rows outside P), A[P, :] = Un (columns outside P), A[P, P] = Dinv.
-__global__ void k_gj_writeback(float* __restrict__ A, int64_t lda, int64_t n, int64_t p0, int nb,
-                               const float* __restrict__ T, int64_t ldt, const float* __restrict__ Un, int64_t ldu,
-                               const float* __restrict__ Dinv)
-{
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * nb) return;
-    {   // column panel: element (row, p0 + j)
-        const int64_t row = idx / nb; const int j = (int)(idx % nb);
-        if (row < p0 || row >= p0 + nb) A[row * lda + p0 + j] = T[row * ldt + j];
-    }
-    {   // row panel: element (p0 + i, col)
-        const int i = (int)(idx / n); const int64_t col = idx % n;
-        float v;
-        if (col >= p0 && col < p0 + nb) v = Dinv[i * NB + (col - p0)];
-        else v = Un[i * ldu + col];
-        A[(p0 + i) * lda + col] = v;
-    }
 }
 
 // c_t[a][b] = Hp[J_ta][J_tb] - twice * sum_s Pm[ta][s] * Hp[J_tb][s]  for pruned slot t; grid (slots, shares of the g * g
@@ -418,6 +336,7 @@ int make_layout(int64_t d1, int64_t m, int32_t g, int32_t k, Layout* L)
     L->off_perm = take(sizeof(int32_t) * ng);
     L->off_slotof = take(sizeof(int32_t) * ng);
     L->off_energy = take(sizeof(double) * ng + sizeof(int32_t) * ng);
+    constexpr int64_t NB = 64;                              // pivot block of the inversion (invert.cu)
     L->off_panel = take(sizeof(float) * (d1 * NB + 2 * NB * L->ldp + NB * NB));
     L->off_loop = take(2 * (size_t)kLoopMaxBlocks * 16 + 64);
     const size_t gg8 = sizeof(double) * g * g;
@@ -456,7 +375,7 @@ int select_support(osscar_ctx* ctx, int mode, int32_t* support)
     int32_t* kept = (int32_t*)(e + L.ng);
     int32_t* perm = (int32_t*)(ws + L.off_perm);
     int32_t* slotof = (int32_t*)(ws + L.off_slotof);
-    const int nb = (int)((L.ng + 255) / 256);
+    const unsigned nb = (unsigned)((L.ng + 7) / 8);          // eight groups per block
     if (mode == OSSCAR_INIT_USER) {
         CK(cudaMemsetAsync(kept, 0, sizeof(int32_t) * L.ng, st));
         k_user_support<<<(L.k + 255) / 256, 256, 0, st>>>(support, L.k, L.ng, kept, ctx->ctl);
@@ -469,46 +388,6 @@ int select_support(osscar_ctx* ctx, int mode, int32_t* support)
     }
     k_build_perm<<<nb, 256, 0, st>>>(kept, L.ng, L.k, perm, slotof, support);
     count_launches(mode == OSSCAR_INIT_USER ? 2 : 3);
-    CK(cudaGetLastError());
-    return OSSCAR_OK;
-}
-
-// In-place inverse of the n x n SPD matrix A (row stride lda) by the blocked exchange (Gauss-Jordan) scheme:
-// per 64-wide pivot block an fp64 Gauss-Jordan inverse in shared memory, then one rank-64 update of the whole matrix in a GEMM.
-// `ref` (row stride ldref) supplies the original diagonal, the scale of the positive-definiteness test.
-// With `tensor_updates` the rank-64 updates of large matrices run on the tensor cores (three bf16 terms per operand,
-// k_rank_update): their accumulation chains are 64 products long, so the truncating accumulator costs nothing that
-// the correction of the inverse from an fp64 residual, which the caller then applies, does not remove.
-int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref, const int32_t* done,
-                       bool tensor_updates)
-{
-    const Layout& L = ctx->L;
-    cudaStream_t st = ctx->stream;
-    float* T = (float*)((char*)ctx->ws + L.off_panel);
-    float* U = T + L.d1 * NB;
-    float* Un = U + NB * L.ldp;
-    float* Dinv = Un + NB * L.ldp;
-    const bool tc_updates = tensor_updates && n >= 4096 && (lda % 4) == 0 && (((uintptr_t)A & 15) == 0);
-    if (tc_updates) CK(cudaMemsetAsync(U, 0, sizeof(float) * NB * lda, st));       // the pad columns of the row panel stay zero
-    for (int64_t p0 = 0; p0 < n; p0 += NB) {
-        const int nb = (int)(n - p0 < NB ? n - p0 : NB);
-        k_pivot_inverse<<<1, 1024, 0, st>>>(A, lda, p0, nb, Dinv, ref, ldref, ctx->ctl);
-        // T = A[:, P] * Dinv
-        CK(sgemm(st, false, false, n, nb, nb, 1.f, A + p0, lda, Dinv, NB, 0.f, T, NB, done));
-        k_zero_rows<<<(nb * nb + 255) / 256, 256, 0, st>>>(T, NB, p0, nb, nb);
-        {
-            dim3 grid((unsigned)((n + 255) / 256 < 32 ? (n + 255) / 256 : 32), (unsigned)nb);
-            k_copy_rows<<<grid, 256, 0, st>>>(A, lda, p0, nb, n, U, lda);
-        }
-        CK(sgemm(st, false, false, nb, n, nb, -1.f, Dinv, NB, U, lda, 0.f, Un, lda, done));
-        // the rank-64 update of the whole matrix
-        if (tc_updates)
-            CK(rank_update_tc(st, n, lda, nb, -1.f, T, NB, U, lda, A, lda, (char*)ctx->ws + L.off_tc, L.tc_bytes, ctx->ctl, done));
-        else
-            CK(sgemm(st, false, false, n, n, nb, -1.f, T, NB, U, lda, 1.f, A, lda, done));
-        k_gj_writeback<<<(unsigned)((n * nb + 255) / 256), 256, 0, st>>>(A, lda, n, p0, nb, T, NB, Un, lda, Dinv);
-        count_launches(4);     // pivot inverse, zero rows, copy rows, write-back (the GEMMs count themselves)
-    }
     CK(cudaGetLastError());
     return OSSCAR_OK;
 }
@@ -605,7 +484,7 @@ int build_state(osscar_ctx* ctx, bool guarded)
     const int64_t nI = L.nI, nJ = L.nJ;
 
     {   // slot-permuted copy of H
-        dim3 grid((unsigned)L.d1, (unsigned)((L.ldp + 255) / 256 < 64 ? (L.ldp + 255) / 256 : 64));
+        dim3 grid((unsigned)((L.ldp + 1023) / 1024), (unsigned)((L.d1 + GS_R - 1) / GS_R));
         k_gather_sym<<<grid, 256, 0, st>>>(ctx->H, L.d1, L.g, perm, Hp, L.ldp);
     }
     CK(cudaMemsetAsync(ws + L.off_vec_begin, 0, L.off_vec_end - L.off_vec_begin, st));
