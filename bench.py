@@ -108,9 +108,16 @@ def reduce_over_ranks(values: dict, world: int, backend_device):
     return out
 
 
-def swap_bytes(nI, nJ, m, fused_y=False):
+LAZY_ROUND = 4     # steps between two writes of the matrices in the launch chain of single-row groups
+
+
+def swap_bytes(nI, nJ, m, fused_y=False, lazy=False):
     """Algorithmic HBM bytes of one swap: V and R_J read+write and H[J,I] read once in fp32; the inverse read+write
-    in fp64 with the next y fused into that pass (single-row groups), or in fp32 with a separate y pass."""
+    in fp64 with the next y fused into that pass (single-row groups), or in fp32 with a separate y pass.  `lazy`: V, R and
+    the inverse are read in every step and written in every LAZY_ROUND-th."""
+    if lazy:
+        held = 8 * nI * nI + 4 * (nI + nJ) * m
+        return held + 4 * nJ * nI + held // LAZY_ROUND
     if fused_y:
         return 16 * nI * nI + 4 * (2 * nI * m + 2 * nJ * m + nJ * nI)
     return 4 * (3 * nI * nI + 2 * nI * m + 2 * nJ * m + nJ * nI)
@@ -123,9 +130,10 @@ KERNEL_BYTES = {   # algorithmic bytes per launch of the streaming kernels of a 
     "swap_loop": lambda nI, nJ, m: swap_bytes(nI, nJ, m, True),
     "update_v": lambda nI, nJ, m: 8 * nI * m,
     "update_r": lambda nI, nJ, m: 8 * nJ * m,
-    "l1_hpass_update_v": lambda nI, nJ, m: 4 * nJ * nI + 8 * nI * m,
-    "l2_update_r_swap": lambda nI, nJ, m: 8 * nJ * m,
-    "l4_update_hinv_y": lambda nI, nJ, m: 16 * nI * nI,
+    # launch chain of single-row groups: H pass; rows of V and R; y and, in every LAZY_ROUND-th step, the write of the inverse
+    "l1_hpass_update_v": lambda nI, nJ, m: 4 * nJ * nI,
+    "l2_update_r_swap": lambda nI, nJ, m: 4 * (nI + nJ) * m * (LAZY_ROUND + 1) // LAZY_ROUND,
+    "l4_update_hinv_y": lambda nI, nJ, m: 8 * nI * nI * (LAZY_ROUND + 1) // LAZY_ROUND,
 }
 
 
@@ -271,7 +279,7 @@ def other_configs(pkg, b, solver, dev, with_cpu):
         rec = {"workload": workload_label(wl, wl.max_swaps), "layer_solve_s": f0.elapsed_time(f1) / 1e3, "swaps": r.n_swaps,
                "stop_reason": r.stop_reason, "phases_ms": r.ms, "loop_driver": r.loop_driver,
                "swaps_per_s": r.n_swaps / max(loop_s, 1e-9) if r.n_swaps else 0.0,
-               "loop_gbs": swap_bytes(nI, nJ, wl.m, fused) * r.n_swaps / max(loop_s, 1e-9) / 1e9 if r.n_swaps else 0.0}
+               "loop_gbs": swap_bytes(nI, nJ, wl.m, fused, fused and r.loop_driver == "launches") * r.n_swaps / max(loop_s, 1e-9) / 1e9 if r.n_swaps else 0.0}
         if name == "c3":        # no improving swap from the energy start: the paper's fixed-iteration form gives the step time
             rf = pkg.solve_layer(solver, x, W, wl.g, wl.k, 8, accept_mode=b.ACCEPT_ALWAYS, **kw)
             rec["forced_swaps"] = {"swaps": rf.n_swaps, "ms_per_swap": rf.ms["search_loop"] / max(rf.n_swaps, 1)}
@@ -441,7 +449,7 @@ def run_ours(args):
         return
 
     pk = peaks()
-    # bf16 activations: one MMA per product; fp32 activations: three bf16 terms, six term pairs executed per product
+    # bf16 activations: one MMA per product; fp32 activations: three digits, six digit products executed per product
     gram_terms = 1 if wl.x_dtype == torch.bfloat16 else 6
     ms_step = red["max_total_ms"] / K
     search_s = red["max_search_ms"] / 1e3
@@ -455,21 +463,17 @@ def run_ours(args):
     fused_path = wl.g == 1 and wl.score_mode != "pair_exact" and args.block_pairs <= 1
     loop_ms = phase["search_loop"] / K
     if fused_path and loop_ms > 0 and loop_ms >= phase["gram"] / K:
-        # the swap loop is the dominant kernel: one cooperative launch per solve (or its five-launch-per-step form),
+        # the swap loop is the dominant kernel: one cooperative launch per solve (or its six-launch-per-step form),
         # timed by the library with CUDA events on its own stream around the loop
         persistent = res.loop_driver == "persistent"
-        bytes_per_launch = swap_bytes(nI, nJ, m, True) * (swaps / K)
+        bytes_per_launch = swap_bytes(nI, nJ, m, True, not persistent and not (shard and world > 1)) * (swaps / K)
         ach = bytes_per_launch / (loop_ms * 1e-3) / 1e9
         roof = {"kernel": "k_swap_loop_g1 (persistent cooperative loop, one launch per solve)" if persistent
-                          else "swap loop as five launches per step (k_decide_g1, k_l1_g1, k_l2_g1, k_select_in_g1, k_l4_g1)",
+                          else "swap loop as six launches per step (k_lz_decide, k_lz_hpass, k_lz_rows, k_lz_finish, k_lz_select, k_lz_y)",
                 "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": ach / pk["hbm_gbs"],
-                # DRAM bytes / algorithmic bytes of one step of the launch-chain kernels, measured with ncu on a mid-size case
-                # whose state exceeds L2 (1687.2 MB of traffic for 1795.2 MB); traffic grows in proportion to the rows streamed.
-                # The persistent loop has no such capture.
-                "traffic": None if persistent else int(0.940 * bytes_per_launch), "traffic_source": None if persistent else
-                "algorithmic bytes x 0.940 (ncu dram__bytes of k_l1_g1, k_l2_g1, k_l4_g1 on a 6 GB case, kernels as committed)",
+                "traffic": None,
                 "bytes_per_launch": int(bytes_per_launch), "ms_per_launch": loop_ms,
-                "bytes_per_swap": swap_bytes(nI, nJ, m, True), "peak_source": pk["source"]}
+                "bytes_per_swap": swap_bytes(nI, nJ, m, True, not persistent and not (shard and world > 1)), "peak_source": pk["source"]}
     elif dom in KERNEL_BYTES and kern_avg.get(dom, 0) > 0:
         bytes_per_launch = KERNEL_BYTES[dom](nI, nJ, m)
         ach = bytes_per_launch / (kern_avg[dom] * 1e-3) / 1e9
@@ -489,11 +493,12 @@ def run_ours(args):
     tiles = sum(tn_ - t // 2 for t in range(tm_))
     gram_exec_tflops = 2.0 * 128 * 256 * tiles * wl.n * gram_terms / max(phase["gram"] / K * 1e-3, 1e-12) / 1e12
     fused = wl.g == 1 and wl.score_mode != "pair_exact"
+    lazy = fused and args.block_pairs <= 1 and res.loop_driver == "launches" and not (shard and world > 1)
     if args.block_pairs > 1:     # one pass over every matrix per ITERATION, plus the read of V and R for the scores
         it_bytes = swap_bytes(nI, nJ, m, False) + 4 * (nI + nJ) * m
         loop_gbs = it_bytes * (per_step_swaps / args.block_pairs) / max(phase["search_loop"] / K * 1e-3, 1e-12) / 1e9
     else:
-        loop_gbs = swap_bytes(nI, nJ, m, fused) * per_step_swaps / max(phase["search_loop"] / K * 1e-3, 1e-12) / 1e9
+        loop_gbs = swap_bytes(nI, nJ, m, fused, lazy) * per_step_swaps / max(phase["search_loop"] / K * 1e-3, 1e-12) / 1e9
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_step, "higher_is_better": True, "scaling": "strong" if shard and world > 1 else "weak", "vs_baseline": None,
@@ -514,7 +519,7 @@ def run_ours(args):
                  "executed_mma_per_product": gram_terms,
                  "frac_of_bf16_peak": gram_exec_tflops / pk["bf16_tflops_sustained"], "peak": pk["bf16_tflops_sustained"],
                  "peak_source": pk["source"] + " (sustained)"},
-        "swap_loop": {"gbs": loop_gbs, "bytes_per_swap": swap_bytes(nI, nJ, m, fused), "frac_of_hbm": loop_gbs / pk["hbm_gbs"],
+        "swap_loop": {"gbs": loop_gbs, "bytes_per_swap": swap_bytes(nI, nJ, m, fused, lazy), "frac_of_hbm": loop_gbs / pk["hbm_gbs"],
                       "peak": pk["hbm_gbs"], "peak_source": pk["source"]},
         "roofline": roof,
         "gpu_launches": int(launches),
@@ -553,7 +558,7 @@ def main():
     ap.add_argument("--block-pairs", type=int, default=0, help="groups exchanged per iteration (t_hat = 2 s, p_hat = 0); 0 = single swaps")
     ap.add_argument("--no-block-extra", action="store_true", help="skip the extra solves with block exchanges of 16 and 50 groups")
     ap.add_argument("--accept-always", action="store_true", help="paper-literal fixed number of iterations")
-    ap.add_argument("--loop-mode", type=int, default=0, help="0 auto, 1 persistent cooperative loop, 2 five launches per step (single-row groups)")
+    ap.add_argument("--loop-mode", type=int, default=0, help="0 auto, 1 persistent cooperative loop, 2 a chain of launches per step (single-row groups)")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--shard", action="store_true", help="with --gpus N: ONE layer over all ranks (token-split Gram, column-sharded "
                     "swap search with two all-reduces per swap) instead of N independent replicas")

@@ -28,7 +28,7 @@ struct SearchCtl {
     int32_t n_refresh;
     int32_t sel_slot;        // kept slot leaving
     int32_t sel_t;           // pruned slot (0-based among pruned slots) entering
-    int32_t pad0;
+    int32_t pending;         // rank-two terms not yet written into the matrices (search_lazy_g1.cuh)
     double  obj;             // running objective
     double  sel_D;           // drop score of the chosen slot
     double  delta;           // exact change of obj of the chosen swap
@@ -37,7 +37,7 @@ struct SearchCtl {
     long long wait_limit;    // cycles a bounded device-side wait may spin before it raises OSSCAR_E_TIMEOUT
     unsigned long long bar_count;   // arrivals at the grid barrier of the persistent swap loop (monotone)
     int32_t abort;           // set by a wait that ran out: every block of the persistent loop returns
-    int32_t pad1;
+    int32_t y_due;           // the step in flight made a swap (search_lazy_g1.cuh)
 };
 
 // Geometry of one layer's search state inside the caller's workspace.

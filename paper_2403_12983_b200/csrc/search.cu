@@ -1055,6 +1055,7 @@ cudaError_t enqueue_scores(osscar_ctx* ctx, const Ptrs& p, bool norms, bool gene
 
 #include "search_block.cuh"
 #include "search_loop_g1.cuh"
+#include "search_lazy_g1.cuh"
 
 // Blocks of the persistent loop: one per SM (cooperative launch), fewer for layers with few rows: a barrier costs more the
 // more blocks meet at it.  0 when the device cannot launch cooperatively.
@@ -1158,6 +1159,11 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     const int pgrid = (fast && want_persistent && L.nJ > 0) ? persistent_grid(L, &psmem) : 0;
     if (prm->loop_mode == OSSCAR_LOOP_PERSISTENT && pgrid == 0) return OSSCAR_E_ARG;
     const bool persistent = pgrid > 0;
+    // launch chain of single-row groups: matrices written every few steps (its vectors and coefficients live in `big`, which is
+    // idle during a search); column shards keep the step that writes them every time
+    LazyPtrs lz = {};
+    const bool lazy = fast && !persistent && !sharded && L.nJ > 0;
+    if (lazy && lazy_layout(L, (char*)ctx->ws + L.off_big, &lz) > L.off_Hp - L.off_big) return OSSCAR_E_WORKSPACE;
     if (block) max_swaps /= bs;                   // from here on: iterations
     const int64_t npairs = (int64_t)L.k * (L.ng - L.k);
     if (sharded && !(g == 1 && !pair && !block)) return OSSCAR_E_ARG;
@@ -1205,7 +1211,18 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         count_launches(3);
         return cudaGetLastError();
     };
+    const unsigned lz_ty = (unsigned)g1_threads(L.ldh / 2);
     auto bootstrap_g1 = [&]() -> cudaError_t {       // score vectors, first entering group and its y from the current state
+        if (lazy) {
+            k_lz_reset<<<1, 1, 0, st>>>(ctx->ctl);
+            k_lz_finish<true><<<LZ_FB, 256, 0, st>>>(p, lz);
+            k_lz_select<<<LZ_CL, LZ_CT, 0, st>>>(p, lz, 0);
+            if (lz_ty == 64) k_lz_y<0, 64><<<(unsigned)L.nI, 64, 0, st>>>(p, lz);
+            else if (lz_ty == 128) k_lz_y<0, 128><<<(unsigned)L.nI, 128, 0, st>>>(p, lz);
+            else k_lz_y<0, 256><<<(unsigned)L.nI, 256, 0, st>>>(p, lz);
+            count_launches(4);
+            return cudaGetLastError();
+        }
         k_scores_g1<<<(unsigned)((L.d1 + 255) / 256), 256, 0, st>>>(p);
         k_select_in_g1<<<1, 1024, 0, st>>>(p);
         k_ypass_d<<<dim3((unsigned)((L.nI + 7) / 8), 1), 256, 0, st>>>(p);
@@ -1279,6 +1296,47 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         else if (t_l4 == 128) launch_pdl(dp, k_l4_g1<G1_RB4, 128>, dim3(nb), dim3(128), st, p);
         else launch_pdl(dp, k_l4_g1<G1_RB4, 256>, dim3(nb), dim3(256), st, p);
     };
+    // row tiles of k_lz_rows: enough blocks for several rounds on every SM, 16 to 128 rows each
+    int lz_rc = 16;
+    while (lazy && lz_rc < 128 && (L.d1 / (2 * lz_rc) + 1) * lz.tiles >= 1776) lz_rc *= 2;
+    auto lz_blocks = [&](int64_t rows) { return (unsigned)((rows + lz_rc - 1) / lz_rc * lz.tiles); };
+    auto launch_lz_rows = [&](int P) {
+        const unsigned nbV = lz_blocks(L.nI), nbR = lz_blocks(L.nJ);
+        const dim3 grid(nbV + nbR + 32), block(LZ_T);
+        const bool dp = dep();
+        static_assert(LZ_B == 4, "one instance per number of terms");
+        if (P == 0) launch_pdl(dp, k_lz_rows<1, false>, grid, block, st, p, lz, nbV, nbR, lz_rc);
+        else if (P == 1) launch_pdl(dp, k_lz_rows<2, false>, grid, block, st, p, lz, nbV, nbR, lz_rc);
+        else if (P == 2) launch_pdl(dp, k_lz_rows<3, false>, grid, block, st, p, lz, nbV, nbR, lz_rc);
+        else launch_pdl(dp, k_lz_rows<4, true>, grid, block, st, p, lz, nbV, nbR, lz_rc);
+    };
+    auto launch_lz_hpass = [&](int P) {            // as many rows per block as give a thread about eight pieces
+        const bool dp = dep();
+        const int64_t n4 = L.ldh / 4, items = L.nJ + 1;
+        if (n4 <= 512) launch_pdl(dp, k_lz_hpass<4, 2>, dim3((unsigned)((items + 3) / 4)), dim3(LZ_T), st, p, lz, P);
+        else if (n4 <= 1024) launch_pdl(dp, k_lz_hpass<2, 4>, dim3((unsigned)((items + 1) / 2)), dim3(LZ_T), st, p, lz, P);
+        else launch_pdl(dp, k_lz_hpass<1, 9>, dim3((unsigned)items), dim3(LZ_T), st, p, lz, P);
+    };
+    auto launch_lz_y = [&](int P) {
+        const bool dp = dep();
+        const dim3 grid((unsigned)L.nI);
+        if (P == LZ_B - 1) {
+            const int yt = (int)((L.ldh + LZ_YC - 1) / LZ_YC);
+            int rc = 16;
+            while (rc < 64 && (L.nI / (2 * rc) + 1) * yt >= 888) rc *= 2;       // several rounds of blocks on every SM
+            launch_pdl(dp, k_lz_y_write<LZ_B>, dim3((unsigned)((L.nI + rc - 1) / rc * yt)), dim3(LZ_T), st, p, lz, yt, rc);
+            launch_pdl(dep(), k_lz_y_sum, dim3((unsigned)((L.nI + 255) / 256)), dim3(256), st, p, lz, yt);
+            count_launches(1);
+            return;
+        }
+#define LZ_Y(TB) do { \
+        if (P == 0) launch_pdl(dp, k_lz_y<1, TB>, grid, dim3(TB), st, p, lz); \
+        else if (P == 1) launch_pdl(dp, k_lz_y<2, TB>, grid, dim3(TB), st, p, lz); \
+        else launch_pdl(dp, k_lz_y<3, TB>, grid, dim3(TB), st, p, lz); } while (0)
+        if (lz_ty == 64) LZ_Y(64); else if (lz_ty == 128) LZ_Y(128); else LZ_Y(256);
+#undef LZ_Y
+    };
+    int lz_it0 = 0;                 // step of the last state build: the matrices are written every LZ_B steps from there
     int next_prof = 0;
     int nmarks = 0;                 // events recorded per profiled step (depends on the step variant)
     unsigned long long* loop_prof = (unsigned long long*)((char*)ctx->ws + L.off_loop + 2 * (size_t)kLoopMaxBlocks * 16);
@@ -1330,6 +1388,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
             if (enqueue_scores(ctx, p, true, pair) != cudaSuccess) { rc = OSSCAR_E_CUDA; break; }
             if (sharded && shard_reduce(ctx, p.vnorm, L.d1, OSSCAR_FP32) != OSSCAR_OK) { rc = OSSCAR_E_CUDA; break; }
             if (fast && bootstrap_g1() != cudaSuccess) { rc = OSSCAR_E_CUDA; break; }
+            lz_it0 = it;
             after_kernel = false;
         }
         cudaEvent_t* pe = nullptr;
@@ -1356,16 +1415,15 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
             launch_l4();        mark();
             after_kernel = false;               // the next step opens with ordinary launches
             count_launches(7);
-        } else if (fast) {
-            // single-row groups: decide, {H pass || V}, {R || slot exchange}, next entering group, {Hinv + next y}
-            // G1_RB rows per block; the H pass has one more block for the leaving row
-            const unsigned nbV = (unsigned)((L.nI + G1_RB - 1) / G1_RB), nbR = (unsigned)((L.nJ + G1_RB - 1) / G1_RB), nbH = nbR + 1;
-            launch_pdl(dep(), k_decide_g1, dim3(1), dim3(1024), st, p, (int)prm->accept_mode, tol, obj_trace, swap_trace, 0);   mark();
-            launch_l1(nbV, nbH);                                                                 mark();
-            launch_l2(nbR);                                                                      mark();
-            launch_pdl(dep(), k_select_in_g1, dim3(1), dim3(1024), st, p);                              mark();
-            launch_l4();                                                     mark();
-            count_launches(5);
+        } else if (lazy) {
+            const int P = (it - lz_it0) % LZ_B;
+            launch_pdl(dep(), k_lz_decide, dim3(LZ_CL), dim3(LZ_CT), st, p, lz, P, (int)prm->accept_mode, tol, obj_trace, swap_trace);      mark();
+            launch_lz_hpass(P);                                                                  mark();
+            launch_lz_rows(P);                                                                   mark();
+            launch_pdl(dep(), k_lz_finish<false>, dim3(LZ_FB), dim3(256), st, p, lz);
+            launch_pdl(dep(), k_lz_select, dim3(LZ_CL), dim3(LZ_CT), st, p, lz, P + 1);               mark();
+            launch_lz_y(P);                                                                      mark();
+            count_launches(6);
         } else {
             if (pair) { if (pair_scores() != cudaSuccess) { rc = OSSCAR_E_CUDA; break; } after_kernel = false; }
             else launch_pdl(dep(), k_select, dim3(1), dim3(1024), st, p);
@@ -1437,6 +1495,10 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         cudaStreamSynchronize(st);
         for (int i = 0; i < nprof; ++i) for (int j = 0; j <= NK; ++j) cudaEventDestroy(evp[i][j]);
         return rc;
+    }
+    if (lazy && max_swaps > 0) {       // terms still pending go into the matrices
+        k_lz_flush<<<dim3((unsigned)(L.nI > L.nJ ? L.nI : L.nJ), 3), 256, 0, st>>>(p, lz);
+        count_launches(1);
     }
     CK(cudaEventRecord(ctx->ev1, st));
     if (fast && max_swaps > 0) {       // the fp32 inverse follows its fp64 copy (state reader, other drivers)
