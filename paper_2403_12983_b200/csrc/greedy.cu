@@ -13,6 +13,12 @@
 namespace osscar {
 namespace {
 
+__device__ __forceinline__ void wait_then_release() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+
 using namespace smallmat;
 
 constexpr int kMaxT = 256;          // rows removed per iteration (t_hat * g)
@@ -50,6 +56,7 @@ __global__ void k_copy_pad2(const float* __restrict__ src, int64_t lds, int64_t 
 // gram[grp][a][b] = V[grp*g+a,:] . V[grp*g+b,:]; grid (live groups, g).
 __global__ void k_gr_gram(GPtrs p)
 {
+    wait_then_release();
     const int g = p.g;
     const int64_t grp = blockIdx.x;
     const int a = blockIdx.y;
@@ -82,6 +89,7 @@ __global__ void k_gr_gram(GPtrs p)
 // D[grp] = Tr((Hinv_rr)^-1 Gram); one block per live group (dynamic smem 3 g^2 doubles).
 __global__ void k_gr_score(GPtrs p)
 {
+    wait_then_release();
     extern __shared__ double smd[];
     __shared__ double red[32];
     const int g = p.g, gg = g * g;
@@ -101,6 +109,7 @@ __global__ void k_gr_score(GPtrs p)
 // refill their holes.  One block.
 __global__ void __launch_bounds__(1024) k_gr_select(GPtrs p, int n_live, int t, int trace_pos)
 {
+    wait_then_release();
     __shared__ double sv[32]; __shared__ int sid[32], sidx[32];
     __shared__ int chosen[kMaxT];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -162,6 +171,7 @@ __global__ void __launch_bounds__(1024) k_gr_select(GPtrs p, int n_live, int t, 
 // B[e] = A[row r_e, :] (T rows), C = A[r, r] -> C^-1 (fp64), in one block for the small part.
 __global__ void k_gr_stage_b(GPtrs p, int n_live)
 {
+    wait_then_release();
     const int g = p.g, t = p.sel[0], T = t * g;
     const int e = blockIdx.x;
     if (e >= T) return;
@@ -171,6 +181,7 @@ __global__ void k_gr_stage_b(GPtrs p, int n_live)
 }
 __global__ void __launch_bounds__(1024) k_gr_cinv(GPtrs p, int in_smem)
 {
+    wait_then_release();
     extern __shared__ double smg[];           // T^2 + 2 T doubles when the matrix fits
     const int g = p.g, t = p.sel[0], T = t * g;
     double* C = in_smem ? smg : p.Cm; double* Lw = in_smem ? smg + T * T : p.Cm + kMaxT * kMaxT; double* Cinv = p.Cm + 2 * kMaxT * kMaxT;
@@ -186,6 +197,7 @@ __global__ void __launch_bounds__(1024) k_gr_cinv(GPtrs p, int in_smem)
 // BC[e][s] = sum_f Cinv[e][f] B[f][s]  and  KT[e][c] = sum_f Cinv[e][f] V[r_f][c];  obj += sum_e KT[e] . V[r_e].
 __global__ void k_gr_stage_bc(GPtrs p, int n_live)
 {
+    wait_then_release();
     const int g = p.g, t = p.sel[0], T = t * g;
     const double* Cinv = p.Cm + 2 * kMaxT * kMaxT;
     const int64_t nA = (int64_t)T * p.lda, nV = (int64_t)T * p.ldv;
@@ -208,8 +220,9 @@ __global__ void k_gr_stage_bc(GPtrs p, int n_live)
         }
     }
 }
-__global__ void __launch_bounds__(256) k_gr_obj(GPtrs p, double* __restrict__ partial)
+__global__ void __launch_bounds__(256) k_gr_obj(GPtrs p, double* partial)
 {
+    wait_then_release();
     __shared__ double red[32];
     const int g = p.g, t = p.sel[0], T = t * g;
     double acc = 0.0;
@@ -223,19 +236,22 @@ __global__ void __launch_bounds__(256) k_gr_obj(GPtrs p, double* __restrict__ pa
     __syncthreads();
     if (threadIdx.x == 0) { double s = 0.0; for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i]; partial[blockIdx.x] = s; }
 }
-__global__ void k_gr_obj_add(SearchCtl* ctl, const double* __restrict__ partial, int n)
+__global__ void k_gr_obj_add(SearchCtl* ctl, const double* partial, int n)
 {
+    wait_then_release();
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += partial[i];      // fixed order
-    ctl->obj += s;
+    for (int i = threadIdx.x; i < n; i += 32) s += partial[i];      // one warp, fixed order
+    s = warp_sum(s);
+    if (threadIdx.x == 0) ctl->obj += s;
 }
 
 // M[s][c] -= sum_e left[e][s] * right[e][c] for live rows s and columns c < ncols (M = A with right = B, or
 // M = V with right = KT).  Block: 1024 columns x 8 rows; the right-hand pieces of a thread are reused by its 8 rows.
 __global__ void __launch_bounds__(256)
-k_gr_update(float* __restrict__ M, int64_t ld, int64_t ncols4, int64_t nrows, const float* __restrict__ left, int64_t ldl,
-            const float* __restrict__ right, int64_t ldr, const int32_t* __restrict__ sel, int g)
+k_gr_update(float* M, int64_t ld, int64_t ncols4, int64_t nrows, const float* left, int64_t ldl,
+            const float* right, int64_t ldr, const int32_t* sel, int g)
 {
+    wait_then_release();
     const int T = sel[0] * g;
     const int64_t c4 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c4 >= ncols4) return;
@@ -247,11 +263,11 @@ k_gr_update(float* __restrict__ M, int64_t ld, int64_t ncols4, int64_t nrows, co
         acc[i] = s < nrows ? reinterpret_cast<const float4*>(M + s * ld)[c4] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     for (int e = 0; e < T; ++e) {
-        const float4 rv = __ldg(reinterpret_cast<const float4*>(right + (int64_t)e * ldr) + c4);
+        const float4 rv = *(reinterpret_cast<const float4*>(right + (int64_t)e * ldr) + c4);
 #pragma unroll
         for (int i = 0; i < UT_ROWS; ++i) {
             const int64_t s = row0 + i;
-            const float l = s < nrows ? -__ldg(left + (int64_t)e * ldl + s) : 0.f;
+            const float l = s < nrows ? -left[(int64_t)e * ldl + s] : 0.f;
             acc[i].x = fmaf(l, rv.x, acc[i].x); acc[i].y = fmaf(l, rv.y, acc[i].y);
             acc[i].z = fmaf(l, rv.z, acc[i].z); acc[i].w = fmaf(l, rv.w, acc[i].w);
         }
@@ -267,6 +283,7 @@ k_gr_update(float* __restrict__ M, int64_t ld, int64_t ncols4, int64_t nrows, co
 // permutation entries; phase 1 copies the matching columns of A for every remaining live row.
 __global__ void k_gr_compact(GPtrs p, int phase, int64_t n_new_rows /* live groups after the iteration */)
 {
+    wait_then_release();
     const int g = p.g, t = p.sel[0];
     for (int i = blockIdx.y; i < t; i += gridDim.y) {
         const int dst = p.sel[1 + i], src = p.sel[1 + kMaxT + i];
@@ -339,6 +356,20 @@ size_t greedy_scratch_bytes(int64_t d1, int64_t m, int g)
 
 // Runs the nested phase down to L.k groups; leaves the slot permutation (kept groups sorted in slots [0, k)) in the
 // workspace and the sorted kept ids in `support`.  The caller then builds the regular search state.
+// Every kernel of an iteration is a programmatic dependent of the one before it: it begins with wait_then_release, and what its
+// predecessor wrote is read with ordinary loads (see search.cu).
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_trace, int32_t* n_iters_out)
 {
     const Layout& L = ctx->L;
@@ -370,12 +401,15 @@ int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_t
     k_identity_perm<<<nbg, 256, 0, st>>>(p.perm, slotof, ng);
     k_copy_pad2<<<(unsigned)d1, 256, 0, st>>>(ctx->H, d1, d1, p.A, p.lda);
     count_launches(2);
-    // fp32 pipes for the rank-64 updates: no correction of the inverse follows here
-    int rc = invert_spd_inplace(ctx, p.A, p.lda, d1, ctx->H, d1, nullptr, false);
+    // large layers: rank-64 updates on the tensor cores and one Newton-Schulz step from digits; else the fp32 pipes
+    const bool corrected = dense_inverse_correctable(ctx);
+    int rc = invert_spd_inplace(ctx, p.A, p.lda, d1, ctx->H, d1, nullptr, corrected);
     if (rc != OSSCAR_OK) return rc;
+    if (corrected) CK(correct_dense_inverse(ctx, p.A, p.lda));
     // W* = H^-1 G (Algorithm 1, line 1)
     if (L.ldm != L.m) CK(cudaMemsetAsync(p.V, 0, sizeof(float) * d1 * L.ldm, st));
-    CK(sgemm(st, false, false, d1, L.m, d1, 1.f, p.A, p.lda, ctx->G, L.m, 0.f, p.V, L.ldm));
+    if (corrected) CK(dense_inverse_times(ctx, p.A, p.lda, ctx->G, p.V, L.ldm));
+    else CK(sgemm(st, false, false, d1, L.m, d1, 1.f, p.A, p.lda, ctx->G, L.m, 0.f, p.V, L.ldm));
     if (ctx->have_const) CK(set_device_double(st, &ctx->ctl->acc[0], ctx->user_const));
     else CK(trace_product(st, ctx->W, L.m, ctx->G, L.m, d1, L.m, ctx->partials, &ctx->ctl->acc[0]));
     CK(trace_product(st, ctx->G, L.m, p.V, L.ldm, d1, L.m, ctx->partials, &ctx->ctl->acc[1]));
@@ -389,18 +423,18 @@ int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_t
     while (n_live > L.k) {
         const int t = n_live - L.k < t_hat ? n_live - L.k : t_hat;
         const int64_t nrows = (int64_t)n_live * g;
-        k_gr_gram<<<dim3((unsigned)n_live, (unsigned)g), 128, 0, st>>>(p);
-        k_gr_score<<<(unsigned)n_live, g == 1 ? 32 : 256, smem_score, st>>>(p);
-        k_gr_select<<<1, 1024, 0, st>>>(p, n_live, t, trace_pos);
-        k_gr_stage_b<<<(unsigned)(t * g), 256, 0, st>>>(p, n_live);
+        CK(launch_chained(k_gr_gram, dim3((unsigned)n_live, (unsigned)g), dim3(128), 0, st, p));
+        CK(launch_chained(k_gr_score, dim3((unsigned)n_live), dim3(g == 1 ? 32 : 256), smem_score, st, p));
+        CK(launch_chained(k_gr_select, dim3(1), dim3(1024), 0, st, p, n_live, t, trace_pos));
+        CK(launch_chained(k_gr_stage_b, dim3((unsigned)(t * g)), dim3(256), 0, st, p, n_live));
         {
             const size_t cs = ((size_t)t * g * t * g + 2 * (size_t)t * g) * sizeof(double);
             const bool fits = cs <= 200 * 1024;
-            k_gr_cinv<<<1, fits ? 1024 : 256, fits ? cs : 0, st>>>(p, fits ? 1 : 0);
+            CK(launch_chained(k_gr_cinv, dim3(1), dim3(fits ? 1024 : 256), fits ? cs : 0, st, p, fits ? 1 : 0));
         }
-        k_gr_stage_bc<<<(unsigned)(((int64_t)t * g * (p.lda + p.ldv) + 255) / 256 < 2368 ? ((int64_t)t * g * (p.lda + p.ldv) + 255) / 256 : 2368), 256, 0, st>>>(p, n_live);
-        k_gr_obj<<<128, 256, 0, st>>>(p, ctx->partials);
-        k_gr_obj_add<<<1, 1, 0, st>>>(ctx->ctl, ctx->partials, 128);
+        CK(launch_chained(k_gr_stage_bc, dim3((unsigned)(((int64_t)t * g * (p.lda + p.ldv) + 255) / 256 < 2368 ? ((int64_t)t * g * (p.lda + p.ldv) + 255) / 256 : 2368)), dim3(256), 0, st, p, n_live));
+        CK(launch_chained(k_gr_obj, dim3(128), dim3(256), 0, st, p, ctx->partials));
+        CK(launch_chained(k_gr_obj_add, dim3(1), dim3(32), 0, st, ctx->ctl, ctx->partials, 128));
         const int64_t Tt = (int64_t)t * g;
         if (Tt >= 32) {
             // wide downdates: A -= BC^T B and V -= B^T KT as products with inner dimension T on the tensor cores
@@ -412,14 +446,14 @@ int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_t
         } else {
             const int64_t nc4 = (round_up(nrows, 4)) / 4;
             dim3 ga((unsigned)((nc4 + 255) / 256), (unsigned)((nrows + UT_ROWS - 1) / UT_ROWS));
-            k_gr_update<<<ga, 256, 0, st>>>(p.A, p.lda, nc4, nrows, p.BC, p.lda, p.B, p.lda, p.sel, g);
+            CK(launch_chained(k_gr_update, ga, dim3(256), 0, st, p.A, p.lda, nc4, nrows, p.BC, p.lda, p.B, p.lda, p.sel, g));
             const int64_t nv4 = p.ldv / 4;
             dim3 gv((unsigned)((nv4 + 255) / 256), (unsigned)((nrows + UT_ROWS - 1) / UT_ROWS));
-            k_gr_update<<<gv, 256, 0, st>>>(p.V, p.ldv, nv4, nrows, p.B, p.lda, p.KT, p.ldv, p.sel, g);     // V -= B (C^-1 V_r)
+            CK(launch_chained(k_gr_update, gv, dim3(256), 0, st, p.V, p.ldv, nv4, nrows, p.B, p.lda, p.KT, p.ldv, p.sel, g));     // V -= B (C^-1 V_r)
         }
         const int n_new = n_live - t;
-        k_gr_compact<<<dim3(64, (unsigned)t), 256, 0, st>>>(p, 0, (int64_t)n_new);
-        k_gr_compact<<<dim3(64, (unsigned)t), 256, 0, st>>>(p, 1, (int64_t)n_new);
+        CK(launch_chained(k_gr_compact, dim3(64, (unsigned)t), dim3(256), 0, st, p, 0, (int64_t)n_new));
+        CK(launch_chained(k_gr_compact, dim3(64, (unsigned)t), dim3(256), 0, st, p, 1, (int64_t)n_new));
         count_launches(12);
         CK(cudaGetLastError());
         n_live = n_new; trace_pos += t; ++iters;

@@ -213,6 +213,11 @@ cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32
 // ---- invert.cu
 int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref, const int32_t* done,
                        bool tensor_updates);
+// H^-1 of the whole layer in the place of Hp (nested phase): one Newton-Schulz step from digit products, in column panels, and
+// C = A B (d1 x d1 times d1 x m).  `correctable`: the layer is large enough and the free regions take the panels.
+bool dense_inverse_correctable(const osscar_ctx* ctx);
+cudaError_t correct_dense_inverse(osscar_ctx* ctx, float* A, int64_t lda);
+cudaError_t dense_inverse_times(osscar_ctx* ctx, const float* A, int64_t lda, const float* B, float* C, int64_t ldc);
 cudaError_t gather_rows(cudaStream_t st, const float* src, int64_t m, int g, const int32_t* perm,
                         int64_t slot_row0, int64_t nrows, float* dst, int64_t ld);
 cudaError_t sum_partials(cudaStream_t st, const double* partials, int n, double* out_dev);   // *out = sum, fixed order

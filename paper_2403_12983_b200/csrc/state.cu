@@ -219,7 +219,7 @@ __global__ void k_sum_partials(const double* __restrict__ partial, int n, double
     if (threadIdx.x == 0) *out = acc;
 }
 
-// A := sym(A + D) on the n x n leading block: the blocked inversion leaves its two triangles different in the last bits
+// A := sym(A + D) (D may be null) on the n x n leading block: the blocked inversion leaves its two triangles different in the last bits
 // times cond, and the correction of that difference is the antisymmetric part of D, so both are symmetrised together.
 // A thread owns the pair (r, c), (c, r) with c >= r; tiles below the diagonal have nothing to do.
 __global__ void k_add_sym(float* __restrict__ A, int64_t lda, const float* __restrict__ D, int64_t ldd, int64_t n,
@@ -230,7 +230,7 @@ __global__ void k_add_sym(float* __restrict__ A, int64_t lda, const float* __res
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
     for (int64_t r = (int64_t)blockIdx.y * 32 + threadIdx.y; r < (int64_t)blockIdx.y * 32 + 32 && r < n; r += 8) {
         if (c >= n || c < r) continue;
-        const float v = 0.5f * ((A[r * lda + c] + A[c * lda + r]) + (D[r * ldd + c] + D[c * ldd + r]));
+        const float v = 0.5f * ((A[r * lda + c] + A[c * lda + r]) + (D ? D[r * ldd + c] + D[c * ldd + r] : 0.f));
         A[r * lda + c] = v;
         A[c * lda + r] = v;
     }
@@ -463,6 +463,76 @@ cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32
         return gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, done);
     }
     return gemm_f64acc(ctx->stream, L.nI, L.nI, L.nI, -1.0, Hp, L.ldp, Hinv, L.ldh, 0.0, nullptr, 0, E, L.ldh, true, done);
+}
+
+// Free while the nested phase prepares H^-1 in the place of Hp: the regions behind it, up to the staged vectors, and the
+// tensor-core region.  A column panel of E and its digits go into the latter, the digits of H or of H^-1 into the former.
+struct DensePanels { int64_t np; float* E; I8Scratch sc; int digits; };
+static bool dense_panels(const osscar_ctx* ctx, DensePanels* d)
+{
+    const Layout& L = ctx->L;
+    char* ws = (char*)ctx->ws;
+    const int64_t n = L.d1;
+    d->digits = n <= 131071 / 5 ? 5 : 4;                             // contraction lengths that five (four) digits allow, see gemm_i8.cu
+    const size_t per_col = sizeof(float) * (size_t)n + (size_t)d->digits * round_up(n, 16) + 16, fixed = 4 * (size_t)n + 8192;
+    int64_t np = L.tc_bytes > fixed ? (int64_t)((L.tc_bytes - fixed) / per_col) / 256 * 256 : 0;
+    if (np > n) np = round_up(n, 4);
+    if (n < 4096 || np < 256) return false;
+    d->np = np;
+    const size_t e_bytes = (sizeof(float) * (size_t)n * np + 255) / 256 * 256;
+    if (e_bytes >= L.tc_bytes) return false;
+    d->E = (float*)(ws + L.off_tc);
+    d->sc.b = ws + L.off_tc + e_bytes; d->sc.b_bytes = L.tc_bytes - e_bytes;
+    d->sc.a = ws + L.off_Hinv; d->sc.a_bytes = L.off_y - L.off_Hinv;
+    return gemm_i8_usable(n, 256, n, d->digits, d->sc);
+}
+bool dense_inverse_correctable(const osscar_ctx* ctx) { DensePanels d; return dense_panels(ctx, &d); }
+
+cudaError_t correct_dense_inverse(osscar_ctx* ctx, float* A, int64_t lda)
+{
+    const int64_t n = ctx->L.d1;
+    DensePanels d;
+    if (!dense_panels(ctx, &d)) return cudaErrorInvalidValue;
+    cudaStream_t st = ctx->stream;
+    for (int64_t j0 = 0; j0 < n; j0 += d.np) {
+        const int64_t w = n - j0 < d.np ? n - j0 : d.np;
+        I8Gemm p = {};                       // E[:, j0:] = (I - H A)[:, j0:]
+        p.M = p.K = n; p.N = w; p.alpha = -1.0; p.identity = true; p.identity_col0 = j0;
+        p.A = ctx->H; p.lda = n; p.B = A + j0; p.ldb = lda; p.C = d.E; p.ldc = d.np;
+        p.diag = ctx->H; p.diag_stride = n + 1;
+        I8Scratch sc = d.sc;
+        cudaError_t e = gemm_i8(st, p, d.digits, sc, ctx->ctl, nullptr);
+        if (e != cudaSuccess) return e;
+        // A[:, j0:] += A E[:, j0:]: a row's digits are taken before the row changes, and the columns already corrected only help
+        p = {};
+        p.M = p.K = n; p.N = w; p.alpha = 1.0; p.beta = 1.0;
+        p.A = A; p.lda = lda; p.B = d.E; p.ldb = d.np; p.C0 = A + j0; p.ldc0 = lda; p.C = A + j0; p.ldc = lda;
+        p.diag = ctx->H; p.diag_stride = n + 1; p.inverse_scale = true;
+        sc = d.sc;
+        e = gemm_i8(st, p, 3, sc, ctx->ctl, nullptr);
+        if (e != cudaSuccess) return e;
+    }
+    k_add_sym<<<dim3((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32)), dim3(32, 8), 0, st>>>(A, lda, nullptr, 0, n, nullptr);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t dense_inverse_times(osscar_ctx* ctx, const float* A, int64_t lda, const float* B, float* C, int64_t ldc)
+{
+    const Layout& L = ctx->L;
+    const int64_t n = L.d1;
+    DensePanels d;
+    if (!dense_panels(ctx, &d)) return cudaErrorInvalidValue;
+    I8Scratch sc;
+    sc.a = d.sc.a; sc.a_bytes = d.sc.a_bytes;
+    sc.b = (char*)ctx->ws + L.off_tc; sc.b_bytes = L.tc_bytes;
+    if (!gemm_i8_usable(n, L.m, n, 4, sc))
+        return sgemm(ctx->stream, false, false, n, L.m, n, 1.f, A, lda, B, L.m, 0.f, C, ldc);
+    I8Gemm p = {};
+    p.M = p.K = n; p.N = L.m; p.alpha = 1.0;
+    p.A = A; p.lda = lda; p.B = B; p.ldb = L.m; p.C = C; p.ldc = ldc;
+    p.diag = ctx->H; p.diag_stride = n + 1; p.inverse_scale = true;
+    return gemm_i8(ctx->stream, p, 4, sc, ctx->ctl, nullptr);
 }
 
 // Rebuilds every piece of the search state from H, G and the current slot permutation.
