@@ -506,106 +506,91 @@ __global__ void __launch_bounds__(256) k_update_rows(Ptrs p, int kind)
     }
 }
 
-// Groups of more than one row: y = Hinv h and the H pass as warp tiles of TP_R rows x TP_E right-hand sides, so that a
-// streamed piece of a matrix row meets TP_E vectors and a piece of a vector TP_R rows (the per-(row, vector) kernels
-// above re-read every row g times from L2).  Blocks of TP_W warps; grid (row tiles, ceil(g / TP_E)); TP_R is chosen per
-// launch so that small layers still fill the machine.
-constexpr int TP_E = 4, TP_W = 4;
+// Groups of more than one row: y = Hinv h and the H pass.  A block of TP_W warps takes TP_W * TP_R rows (TP_R per warp) and
+// TP_E right-hand sides; pieces of TP_C float4 of the vectors are staged in shared memory, so that a piece of a vector is
+// read once per block instead of once per warp and row.  Bound before: the L1 reads of the vectors (nine 16-byte loads per
+// 16-byte piece of H at one row per warp): 43 -> 21 us for the H pass and 20 -> 16 us for y at 2304 + 2304 rows in groups of nine.  Grid (row tiles, ceil(g / TP_E)); TP_R is chosen per launch so that small
+// layers still fill the machine.
+constexpr int TP_E = 4, TP_W = 4, TP_C = 128;
 
-// y[e][s] = Hinv[s, :] . Hp[q_e, 0:n_I]
-template <int TP_R>
-__global__ void __launch_bounds__(32 * TP_W) k_ypass_g(Ptrs p)
+// HP: u_l = Hp[l, 0:n_I] b and d_l = Hp[l, q] - Hp[l, 0:n_I] u2 for the pruned rows and the g leaving rows; else
+// y[e][s] = Hinv[s, :] . Hp[q_e, 0:n_I].
+template <bool HP, int TP_R>
+__device__ __forceinline__ void row_dots_g(const Ptrs& p)
 {
+    constexpr int NV = HP ? 2 * TP_E : TP_E;
     pdl_wait_then_release();
     if (p.ctl->done) return;
+    __shared__ float4 sv[NV][TP_C];
     const int g = p.g, e0 = blockIdx.y * TP_E;
     const int lane = threadIdx.x & 31;
-    const int64_t s0 = ((int64_t)blockIdx.x * TP_W + (threadIdx.x >> 5)) * TP_R;
-    if (s0 >= p.nI) return;
-    const float4 *arow[TP_R], *hrow[TP_E];
-#pragma unroll
-    for (int i = 0; i < TP_R; ++i) arow[i] = reinterpret_cast<const float4*>(p.Hinv + (s0 + i < p.nI ? s0 + i : p.nI - 1) * p.ldh);
-#pragma unroll
-    for (int j = 0; j < TP_E; ++j)
-        hrow[j] = reinterpret_cast<const float4*>(p.Hp + (p.nI + (int64_t)p.ctl->sel_t * g + (e0 + j < g ? e0 + j : g - 1)) * p.ldp);
-    float acc[TP_R][TP_E];
-#pragma unroll
-    for (int i = 0; i < TP_R; ++i)
-#pragma unroll
-        for (int j = 0; j < TP_E; ++j) acc[i][j] = 0.f;
-    for (int64_t c = lane; c < p.ldh / 4; c += 32) {
-        float4 x[TP_R], h[TP_E];
-#pragma unroll
-        for (int i = 0; i < TP_R; ++i) x[i] = arow[i][c];
-#pragma unroll
-        for (int j = 0; j < TP_E; ++j) h[j] = *(hrow[j] + c);
-#pragma unroll
-        for (int i = 0; i < TP_R; ++i)
-#pragma unroll
-            for (int j = 0; j < TP_E; ++j) acc[i][j] += dot4f(x[i], h[j]);
-    }
-#pragma unroll
-    for (int i = 0; i < TP_R; ++i)
-#pragma unroll
-        for (int j = 0; j < TP_E; ++j) {
-            const float t = warp_sum(acc[i][j]);
-            if (lane == 0 && s0 + i < p.nI && e0 + j < g) p.y[(int64_t)(e0 + j) * p.ldh + s0 + i] = t;
-        }
-}
-
-// u_l = Hp[l, 0:n_I] b,  d_l = Hp[l, q] - Hp[l, 0:n_I] u2   for the pruned rows and the g leaving rows.
-template <int TP_R>
-__global__ void __launch_bounds__(32 * TP_W) k_hpass_g(Ptrs p)
-{
-    pdl_wait_then_release();
-    if (p.ctl->done) return;
-    const int g = p.g, e0 = blockIdx.y * TP_E;
-    const int lane = threadIdx.x & 31;
-    const int64_t nrows = p.nJ + g;
+    const int64_t nrows = HP ? p.nJ + g : p.nI;
     const int64_t l0 = ((int64_t)blockIdx.x * TP_W + (threadIdx.x >> 5)) * TP_R;
-    if (l0 >= nrows) return;
     const int64_t r0 = (int64_t)p.ctl->sel_slot * g;
-    const int64_t qcol0 = p.nI + (int64_t)p.ctl->sel_t * g;
-    const float4 *rows[TP_R], *bv[TP_E], *uv[TP_E];
+    const int64_t q0 = p.nI + (int64_t)p.ctl->sel_t * g;
+    const int n4 = (int)(p.ldh / 4);
+    const float* rows[TP_R];
 #pragma unroll
     for (int i = 0; i < TP_R; ++i) {
         const int64_t l = l0 + i < nrows ? l0 + i : nrows - 1;
-        rows[i] = reinterpret_cast<const float4*>(p.Hp + (l < p.nJ ? p.nI + l : r0 + (l - p.nJ)) * p.ldp);
+        rows[i] = HP ? p.Hp + (l < p.nJ ? p.nI + l : r0 + (l - p.nJ)) * p.ldp : p.Hinv + l * p.ldh;
     }
-#pragma unroll
-    for (int j = 0; j < TP_E; ++j) {
-        const int64_t e = e0 + j < g ? e0 + j : g - 1;
-        bv[j] = reinterpret_cast<const float4*>(p.b + e * p.ldh);
-        uv[j] = reinterpret_cast<const float4*>(p.u2 + e * p.ldh);
-    }
-    float au[TP_R][TP_E], ad[TP_R][TP_E];
+    auto vec = [&](int v) {                   // HP: b_e, u2_e in turn
+        const int64_t e = e0 + (HP ? v >> 1 : v) < g ? e0 + (HP ? v >> 1 : v) : g - 1;
+        return reinterpret_cast<const float4*>(HP ? ((v & 1) ? p.u2 : p.b) + e * p.ldh : p.Hp + (q0 + e) * p.ldp);
+    };
+    float acc[TP_R][NV];
 #pragma unroll
     for (int i = 0; i < TP_R; ++i)
 #pragma unroll
-        for (int j = 0; j < TP_E; ++j) { au[i][j] = 0.f; ad[i][j] = 0.f; }
-    for (int64_t c = lane; c < p.ldh / 4; c += 32) {
-        float4 x[TP_R];
+        for (int v = 0; v < NV; ++v) acc[i][v] = 0.f;
+    for (int c0 = 0; c0 < n4; c0 += TP_C) {
+        float4 x[TP_R][TP_C / 32];
 #pragma unroll
-        for (int i = 0; i < TP_R; ++i) x[i] = rows[i][c];
+        for (int i = 0; i < TP_R; ++i)
 #pragma unroll
-        for (int j = 0; j < TP_E; ++j) {
-            const float4 bb = *(bv[j] + c), uu = *(uv[j] + c);
+            for (int k = 0; k < TP_C / 32; ++k) {
+                const int c = c0 + lane + 32 * k;
+                x[i][k] = c < n4 ? reinterpret_cast<const float4*>(rows[i])[c] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        __syncthreads();                      // the previous piece has been read
 #pragma unroll
-            for (int i = 0; i < TP_R; ++i) { au[i][j] += dot4f(x[i], bb); ad[i][j] += dot4f(x[i], uu); }
+        for (int v = 0; v < NV; ++v) {
+            const int c = c0 + (int)threadIdx.x;
+            sv[v][threadIdx.x] = c < n4 ? vec(v)[c] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < TP_C / 32; ++k)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                const float4 w = sv[v][lane + 32 * k];
+#pragma unroll
+                for (int i = 0; i < TP_R; ++i) acc[i][v] += dot4f(x[i][k], w);
+            }
     }
 #pragma unroll
-    for (int i = 0; i < TP_R; ++i)
+    for (int i = 0; i < TP_R; ++i) {
+        const int64_t l = l0 + i;
 #pragma unroll
-        for (int j = 0; j < TP_E; ++j) {
-            const float su = warp_sum(au[i][j]), sd = warp_sum(ad[i][j]);
-            const int64_t l = l0 + i;
-            if (lane == 0 && l < nrows && e0 + j < g) {
-                p.u[l * g + e0 + j] = su;
-                p.d[l * g + e0 + j] = reinterpret_cast<const float*>(rows[i])[qcol0 + e0 + j] - sd;
+        for (int e = 0; e < TP_E; ++e) {
+            if (HP) {
+                const float su = warp_sum(acc[i][(2 * e) % NV]), sd = warp_sum(acc[i][(2 * e + 1) % NV]);
+                if (lane == 0 && l < nrows && e0 + e < g) {
+                    p.u[l * g + e0 + e] = su;
+                    p.d[l * g + e0 + e] = rows[i][q0 + e0 + e] - sd;
+                }
+            } else {
+                const float t = warp_sum(acc[i][e % NV]);
+                if (lane == 0 && l < nrows && e0 + e < g) p.y[(int64_t)(e0 + e) * p.ldh + l] = t;
             }
         }
+    }
 }
+template <int TP_R>
+__global__ void __launch_bounds__(32 * TP_W) k_ypass_g(Ptrs p) { static_assert(32 * TP_W == TP_C, "a thread stages one piece per vector"); row_dots_g<false, TP_R>(p); }
+template <int TP_R>
+__global__ void __launch_bounds__(32 * TP_W) k_hpass_g(Ptrs p) { row_dots_g<true, TP_R>(p); }
 
 // Groups of more than one row: the rank-2g updates as register tiles.  A block owns TG_RT rows x (TG_T float4) columns;
 // the 2 g coefficients of its rows sit in shared memory, every streamed piece of the g-row panels (b, u2 / K, Vq) is
@@ -1267,8 +1252,8 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     const unsigned hblocks = (unsigned)((L.nJ + g + 8 * RPW - 1) / (8 * RPW));
     const unsigned gtiles = (unsigned)((g + TP_E - 1) / TP_E);
     auto tile_blocks = [](int64_t rows, int R) { return (unsigned)((rows + TP_W * R - 1) / (TP_W * R)); };
-    auto tile_rows = [&](int64_t rows) {           // rows per warp: as many as still leave about 4096 warps in flight
-        for (int R = 4; R > 1; R >>= 1) if ((rows + R - 1) / R * gtiles >= 4096) return R;
+    auto tile_rows = [&](int64_t rows) {           // rows per warp: as many as still leave two blocks per SM
+        for (int R = 4; R > 1; R >>= 1) if ((int64_t)tile_blocks(rows, R) * gtiles >= 296) return R;
         return 1;
     };
     const unsigned prep_blocks = (unsigned)(((L.nI + L.ldm) * g + 255) / 256);
