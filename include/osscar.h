@@ -51,8 +51,8 @@ enum { OSSCAR_SCORE_INDEPENDENT = 0, OSSCAR_SCORE_PAIR_EXACT = 1 };
 enum { OSSCAR_ACCEPT_IMPROVING = 0, OSSCAR_ACCEPT_ALWAYS = 1 };
 enum { OSSCAR_STOP_MAX_SWAPS = 0, OSSCAR_STOP_NO_IMPROVEMENT = 1, OSSCAR_STOP_GUARD = 2 };
 /* Swap loop of single-row groups.  PERSISTENT = one cooperative kernel that runs all steps with bounded grid-wide
- * barriers between their phases (OSSCAR_E_ARG if the device cannot launch cooperatively); LAUNCHES = five dependent
- * launches per step, enqueued ahead of the device; AUTO = PERSISTENT for states that fit the L2 cache (under 96 MB),
+ * barriers between their phases (OSSCAR_E_ARG if the device cannot launch cooperatively); LAUNCHES = a chain of
+ * dependent launches per step, enqueued ahead of the device; AUTO = PERSISTENT for states that fit the L2 cache (under 96 MB),
  * LAUNCHES for states streamed from HBM. */
 enum { OSSCAR_LOOP_AUTO = 0, OSSCAR_LOOP_PERSISTENT = 1, OSSCAR_LOOP_LAUNCHES = 2 };
 
@@ -104,12 +104,13 @@ int osscar_set_workspace(osscar_ctx* ctx, void* dev_ptr, size_t bytes);
  *   flags & BEGIN : H := Xc^T Xc, otherwise H += Xc^T Xc   (split over calibration rows);
  *   flags & END   : H += damp * mean(diag H) * I (damp = 0: none; not in the paper),
  *                   G := H W_hat, *const_term := Tr(W_hat^T G), then one stream sync.
- *                   With a workspace set, G is formed on the tensor cores (three-term bf16 split, fp32-accurate)
- *                   and the workspace contents are overwritten; without one it runs on the fp32 pipes.
+ *                   With a workspace set, G is formed on the tensor cores (8-bit digits with exact integer sums, or a
+ *                   three-term bf16 split where those do not fit; fp32-accurate) and the workspace
+ *                   contents are overwritten; without one it runs on the fp32 pipes.
  * X: device, n_rows x d1, bf16 (tensor cores, fp32 accumulation) or fp32.  For bf16 the
- * pointer must be 16-byte aligned and d1 a multiple of 8.  fp32 X with a workspace set is split into three bf16
- * terms there (row panels of 6 * round_up(d1, 8) bytes per row, workspace contents overwritten) and accumulated on
- * the tensor cores to fp32 accuracy; without a workspace it runs on the fp32 pipes.
+ * pointer must be 16-byte aligned and d1 a multiple of 8.  fp32 X with a workspace set is split there into three
+ * 8-bit digits (small products or workspaces: three bf16 terms, row panels of 6 * round_up(d1, 8) bytes per row;
+ * workspace contents overwritten) and accumulated on the tensor cores to fp32 accuracy; without a workspace it runs on the fp32 pipes.
  * W: device d1 x m fp32 (read on END).
  * H: device d1 x d1 fp32, G: device d1 x m fp32, const_term: host (written on END).
  * n_rows may be 0 (nothing is added).

@@ -41,7 +41,8 @@ class SearchResult(C.Structure):
 
 STEP_KERNELS = ["select", "pair_grams", "y_pass", "small_algebra", "staging", "h_pass", "update_hinv", "update_v",
                 "update_r", "group_scores", "h_swap_rows", "h_swap_cols"]
-# single-row groups run a fused five-launch step
+# single-row groups run a fused step: decide, H pass, rows of V and R, finish + select, inverse + next y (column shards and
+# the persistent loop: decide, H pass || V, R || slot exchange, select, inverse + next y)
 STEP_KERNELS_G1 = ["decide", "l1_hpass_update_v", "l2_update_r_swap", "select_in", "l4_update_hinv_y"]
 # block exchanges (block_pairs > 1): stages of one iteration
 STEP_KERNELS_BLOCK = ["select", "gather_y", "grams_algebra_staging", "h_pass", "update_hinv", "update_v", "update_r",

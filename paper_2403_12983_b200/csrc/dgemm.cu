@@ -6,7 +6,8 @@
 // relative.  Products accumulated in fp32 leave errors of cond(H_II) * 2^-24 in them (measured 4e-4 in the add scores of
 // an OPT-1.3B-shaped FC2 layer), enough to change the selected group.  With the residuals of one refinement step
 // (I - H_II Hinv, G_I - H_II V) and the two differences themselves accumulated in fp64, the state that is then stored
-// in fp32 is correct to the rounding of its entries.
+// in fp32 is correct to the rounding of its entries.  The larger of these products run as digit products on the int8 tensor
+// cores (gemm_i8.cu); this kernel takes those that are too small for them or whose digits do not fit the workspace.
 //
 // Tiling: block 128 x 64, k-step 16, 8 warps of 32 x 32 (4 x 4 mma tiles, 32 fp64 accumulators per lane).  Operands
 // are converted to fp64 once, on their way into shared memory; fragments are 8-byte shared loads without bank conflicts

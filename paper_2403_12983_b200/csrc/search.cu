@@ -1145,7 +1145,8 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     if (prm->loop_mode == OSSCAR_LOOP_PERSISTENT && pgrid == 0) return OSSCAR_E_ARG;
     const bool persistent = pgrid > 0;
     // launch chain of single-row groups: matrices written every few steps (its vectors and coefficients live in `big`, which is
-    // idle during a search); column shards keep the step that writes them every time
+    // idle during a search and, with the staged rows of the nested phase, larger than they are at every size); column shards
+    // keep the step that writes them every time
     LazyPtrs lz = {};
     const bool lazy = fast && !persistent && !sharded && L.nJ > 0;
     if (lazy && lazy_layout(L, (char*)ctx->ws + L.off_big, &lz) > L.off_Hp - L.off_big) return OSSCAR_E_WORKSPACE;

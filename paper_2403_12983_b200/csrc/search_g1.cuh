@@ -1,4 +1,5 @@
-// Swap step for single-row groups (g = 1): five launches per swap, each matrix streamed once.
+// Swap step of column shards of single-row groups (g = 1): five launches and two sums over shards per swap, each matrix
+// streamed once (search_lazy_g1.cuh is the step of one device, which writes the matrices only every few steps).
 // Included by search.cu (same translation unit: uses its Ptrs, reductions and small-matrix slots).
 //
 //   decide      one block: i* = argmin D, exact change of obj, accept test, staged vectors b, u2, K, Vq
