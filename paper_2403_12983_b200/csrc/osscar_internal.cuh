@@ -210,6 +210,8 @@ cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const fl
                             int64_t ldc, int digits, void* other, size_t other_bytes, const int32_t* done);
 // E = I - H_II Hinv summed beyond fp32; `v_free`: V and R hold nothing yet, so their memory may take operand digits
 cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32_t* done);
+// V += Hinv (G_I - H_II V), the residual summed beyond fp32.  GI: G_I in slot order (ldm), rV: as large, `other`: room for digits
+cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes, const int32_t* done);
 // ---- invert.cu
 int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref, const int32_t* done,
                        bool tensor_updates);

@@ -1491,16 +1491,24 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         k_hinv_from_d<<<(unsigned)L.nI, 256, 0, st>>>(p.Hd, p.Hinv, L.ldh, nullptr);
         count_launches(1);
     }
+    if (own_limit) { k_search_wait_limit<<<1, 1, 0, st>>>(ctx->ctl, ctx->wait_limit); count_launches(1); }
 
     // results: weights, support, objective recomputed from the final state
+    float* GI = (float*)((char*)ctx->ws + L.off_big);                  // G_I in slot order
+    CK(gather_rows(st, ctx->G, L.m, L.g, p.perm, 0, L.nI, GI, L.ldm));
+    if (g > 1 && max_swaps > 0) {
+        // The fp32 updates of wide groups leave 3e-5 to 8e-5 in the weights of a 3 x 3 convolution of 512 channels after 24
+        // swaps (the single-row drivers, with their fp64 inverse, 2e-6): one refinement step, 0.3 ms there, and the weights
+        // are within 2e-6 as well.  After the caller's wait budget has been put back: the products wait on barriers of their own.
+        float* rV = GI + L.nI * L.ldm;
+        char* tail = (char*)(rV + L.nI * L.ldm);
+        CK(refine_v(ctx, GI, rV, tail, (size_t)((char*)ctx->ws + L.off_Hp - tail), nullptr));
+    }
     CK(cudaMemsetAsync(W_out, 0, sizeof(float) * L.d1 * L.m, st));
     k_scatter_rows<<<(unsigned)L.nI, 256, 0, st>>>(p, W_out);
     k_sorted_support<<<(L.k + 255) / 256, 256, 0, st>>>(p, support_out);
     {
-        float* big = (float*)((char*)ctx->ws + L.off_big);
-        // G_I in slot order, then Tr(G_I^T V)
-        CK(gather_rows(st, ctx->G, L.m, L.g, p.perm, 0, L.nI, big, L.ldm));
-        CK(trace_product(st, big, L.ldm, p.V, L.ldm, L.nI, L.m, ctx->partials, &ctx->ctl->acc[1]));
+        CK(trace_product(st, GI, L.ldm, p.V, L.ldm, L.nI, L.m, ctx->partials, &ctx->ctl->acc[1]));
         if (sharded) {      // Tr(G_I^T V) is a sum over this shard's columns
             k_shard_scalar<<<1, 1, 0, st>>>(ctx->ctl, p.shard, 0);
             if (shard_reduce(ctx, p.shard, 1, OSSCAR_FP64) != OSSCAR_OK) return OSSCAR_E_CUDA;
@@ -1510,7 +1518,6 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         k_final_obj<<<1, 1, 0, st>>>(ctx->ctl);
         count_launches(3);
     }
-    if (own_limit) { k_search_wait_limit<<<1, 1, 0, st>>>(ctx->ctl, ctx->wait_limit); count_launches(1); }
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(ctx->ctl_host, ctx->ctl, sizeof(SearchCtl), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));

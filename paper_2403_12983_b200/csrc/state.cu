@@ -465,6 +465,27 @@ cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32
     return gemm_f64acc(ctx->stream, L.nI, L.nI, L.nI, -1.0, Hp, L.ldp, Hinv, L.ldh, 0.0, nullptr, 0, E, L.ldh, true, done);
 }
 
+cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes, const int32_t* done)
+{
+    const Layout& L = ctx->L;
+    char* ws = (char*)ctx->ws;
+    const float* Hp = (const float*)(ws + L.off_Hp);
+    float* V = (float*)(ws + L.off_V);
+    const int64_t nI = L.nI;
+    I8Scratch sc = i8_scratch(ctx, L.m, nI, kResidualDigits, other, other_bytes);
+    cudaError_t e;
+    if (gemm_i8_usable(nI, L.m, nI, kResidualDigits, sc)) {
+        I8Gemm p = {};
+        p.M = nI; p.N = L.m; p.K = nI; p.alpha = -1.0; p.beta = 1.0;
+        p.A = Hp; p.lda = L.ldp; p.B = V; p.ldb = L.ldm; p.C0 = GI; p.ldc0 = L.ldm; p.C = rV; p.ldc = L.ldm;
+        p.diag = Hp; p.diag_stride = L.ldp + 1;
+        e = gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, done);
+    } else
+        e = gemm_f64acc(ctx->stream, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false, done);
+    if (e != cudaSuccess) return e;
+    return inverse_product(ctx, L.m, (const float*)(ws + L.off_Hinv), rV, L.ldm, 1.f, V, V, L.ldm, 4, other, other_bytes, done);
+}
+
 // Free while the nested phase prepares H^-1 in the place of Hp: the regions behind it, up to the staged vectors, and the
 // tensor-core region.  A column panel of E and its digits go into the latter, the digits of H or of H^-1 into the former.
 struct DensePanels { int64_t np; float* E; I8Scratch sc; int digits; };
@@ -593,16 +614,7 @@ int build_state(osscar_ctx* ctx, bool guarded)
         void* other = tail > rbytes ? (void*)((char*)big + used) : (void*)R;
         const size_t other_bytes = tail > rbytes ? tail : rbytes;
         CK(inverse_product(ctx, L.m, Hinv, GI, L.ldm, 0.f, nullptr, V, L.ldm, 4, other, other_bytes, done));
-        I8Scratch sc = i8_scratch(ctx, L.m, nI, kResidualDigits, other, other_bytes);
-        if (gemm_i8_usable(nI, L.m, nI, kResidualDigits, sc)) {
-            I8Gemm p = {};
-            p.M = nI; p.N = L.m; p.K = nI; p.alpha = -1.0; p.beta = 1.0;
-            p.A = Hp; p.lda = L.ldp; p.B = V; p.ldb = L.ldm; p.C0 = GI; p.ldc0 = L.ldm; p.C = rV; p.ldc = L.ldm;
-            p.diag = Hp; p.diag_stride = L.ldp + 1;
-            CK(gemm_i8(st, p, kResidualDigits, sc, ctx->ctl, done));
-        } else
-            CK(gemm_f64acc(st, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false, done));
-        CK(inverse_product(ctx, L.m, Hinv, rV, L.ldm, 1.f, V, V, L.ldm, 4, other, other_bytes, done));
+        CK(refine_v(ctx, GI, rV, other, other_bytes, done));
     }
     // obj = Tr(W^T G) - Tr(G_I^T V)
     if (ctx->have_const) CK(set_device_double(st, &ctx->ctl->acc[0], ctx->user_const));

@@ -1,0 +1,29 @@
+"""Weights of a swap search with groups of several rows solve their normal equations to fp32 rounding, not to its drift."""
+import pytest
+import torch
+
+import paper_2403_12983_b200 as pkg
+from paper_2403_12983_b200 import binding as b
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d1,m,g,k", [(36, 5, 2, 7), (1152, 130, 9, 70), (1600, 512, 80, 9), (2304, 513, 9, 128)])
+def test_weights_after_swaps(d1, m, g, k):
+    gen = torch.Generator(device="cuda").manual_seed(d1 + m)
+    X = torch.randn(3 * d1, d1, generator=gen, device="cuda", dtype=torch.float64) + 0.3 * torch.randn(3 * d1, 1, generator=gen, device="cuda")
+    X *= torch.exp(0.5 * torch.randn(d1 // g, generator=gen, device="cuda")).repeat_interleave(g)
+    W = 0.05 * torch.randn(d1, m, generator=gen, device="cuda")
+    H = (X.t() @ X).float()
+    H = 0.5 * (H + H.t())
+    G = (H.double() @ W.double()).float()
+    s = pkg.Solver(0)
+    s.init_support(H, G, W, g, k, b.INIT_ENERGY)
+    out = s.local_search(6, accept_mode=b.ACCEPT_ALWAYS)
+    I = (out.support.long()[:, None] * g + torch.arange(g, device="cuda")).reshape(-1)
+    ref = torch.linalg.solve(H.double()[I][:, I], G.double()[I])
+    got = out.W[I].double()
+    # entries rounded to fp32 (2^-25 on average in the norm) plus the residual of one step: drift x cond(H_II) 2^-24, both far
+    # below 1e-3 here, so their product stays below 4 roundings
+    assert (got - ref).norm() <= 4 * 2.0 ** -24 * ref.norm()
+    s.close()
