@@ -154,7 +154,7 @@ cudaError_t gemm_f64acc(cudaStream_t st, int64_t M, int64_t N, int64_t K, double
 // The plain product with the result kept in fp64: C (M x N doubles, row stride ldc) = A * B; with `tri` (B symmetric,
 // K == N) C = A * U for the halved block upper triangle U of B (see the kernel).
 cudaError_t gemm_f64out(cudaStream_t st, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
-                        const float* B, int64_t ldb, double* C, int64_t ldc, const int32_t* done, bool tri)
+                        const float* B, int64_t ldb, double* C, int64_t ldc, bool tri)
 {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (tri && K != N) return cudaErrorInvalidValue;
@@ -164,7 +164,7 @@ cudaError_t gemm_f64out(cudaStream_t st, int64_t M, int64_t N, int64_t K, const 
     constexpr int smem = (2 * DG_BM * DG_AS + 2 * DG_BK * DG_BS) * (int)sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_gemm_f64acc<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k_gemm_f64acc<double><<<grid, DG_T, smem, st>>>(M, N, K, 1.0, A, lda, B, ldb, 0.0, nullptr, 0, C, ldc, 0, vecA, vecB, tri ? 1 : 0, done);
+    k_gemm_f64acc<double><<<grid, DG_T, smem, st>>>(M, N, K, 1.0, A, lda, B, ldb, 0.0, nullptr, 0, C, ldc, 0, vecA, vecB, tri ? 1 : 0, nullptr);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -403,7 +403,7 @@ int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_t
     count_launches(2);
     // large layers: rank-64 updates on the tensor cores and one Newton-Schulz step from digits; else the fp32 pipes
     const bool corrected = dense_inverse_correctable(ctx);
-    int rc = invert_spd_inplace(ctx, p.A, p.lda, d1, ctx->H, d1, nullptr, corrected);
+    int rc = invert_spd_inplace(ctx, p.A, p.lda, d1, ctx->H, d1, corrected);
     if (rc != OSSCAR_OK) return rc;
     if (corrected) CK(correct_dense_inverse(ctx, p.A, p.lda));
     // W* = H^-1 G (Algorithm 1, line 1)

@@ -136,10 +136,9 @@ __device__ __forceinline__ void split3(float x, __nv_bfloat16& a, __nv_bfloat16&
 template <bool TERMS>
 __global__ void __launch_bounds__(GJ_T)
 k_gj_panels(const float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* Dinv, float* T, float* U, float* Un, int64_t ldu,
-            float* next, RankTerms terms, const int32_t* done)
+            float* next, RankTerms terms)
 {
     wait_then_release();
-    if (done && *done) return;
     __shared__ float sD[NB][NB];
     __shared__ float sA[NB][33];          // A[row, P] transposed: [k][row]
     __shared__ float sU[NB][33];          // A[P, col]: [k][col]
@@ -253,10 +252,9 @@ __device__ __forceinline__ float gj_entry(int64_t row, int64_t col, int64_t p0, 
 // pivot block instead (its tile-mates are the blocks 1, 2, ...).
 __global__ void __launch_bounds__(GJ_T)
 k_gj_update(float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* T, const float* U, const float* Un, int64_t ldu,
-            const float* Dinv, const float* next, float* Dnext, const float* ref, int64_t ldref, int tiles_n, SearchCtl* ctl, const int32_t* done)
+            const float* Dinv, const float* next, float* Dnext, const float* ref, int64_t ldref, int tiles_n, SearchCtl* ctl)
 {
     wait_then_release();
-    if (done && *done) return;
     extern __shared__ __align__(16) float up_smem[];
     const int t = threadIdx.x;
     if (blockIdx.x == 0) {
@@ -407,10 +405,9 @@ k_gj_update(float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* T
 // panels do not touch.
 __global__ void __launch_bounds__(GJ_T)
 k_gj_writeback(float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* T, const float* Un, int64_t ldu, const float* Dinv,
-               float* Dnext, const float* ref, int64_t ldref, SearchCtl* ctl, const int32_t* done)
+               float* Dnext, const float* ref, int64_t ldref, SearchCtl* ctl)
 {
     wait_then_release();
-    if (done && *done) return;
     if (blockIdx.x == 0) {
         if (p0 + NB < n) pivot_block(A, lda, p0 + NB, (int)(n - p0 - NB < NB ? n - p0 - NB : NB), Dnext, ref, ldref, ctl);
         return;
@@ -450,7 +447,7 @@ cudaError_t launch_dependent(bool dependent, void (*kernel)(KArgs...), unsigned 
 // With `tensor_updates` the rank-64 updates of large matrices run on the tensor cores (three bf16 terms per operand,
 // k_rank_update): their accumulation chains are 64 products long, so the truncating accumulator costs nothing that
 // the correction of the inverse from a residual summed beyond fp32, which the caller then applies, does not remove.
-int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref, const int32_t* done,
+int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref,
                        bool tensor_updates)
 {
     const Layout& L = ctx->L;
@@ -472,10 +469,10 @@ int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const 
         for (int64_t p0 = 0, s = 0; p0 < n; p0 += NB, ++s) {
             const int nb = (int)(n - p0 < NB ? n - p0 : NB);
             const float* D = Dbuf[s & 1];
-            CK(launch_dependent(p0 > 0, k_gj_panels<true>, pgrid, 0, st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, (float*)nullptr, terms, done));
-            CK(rank_update_run(st, n, lda, NB, -1.f, terms, A, lda, ctx->ctl, done));
+            CK(launch_dependent(p0 > 0, k_gj_panels<true>, pgrid, 0, st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, (float*)nullptr, terms));
+            CK(rank_update_run(st, n, lda, NB, -1.f, terms, A, lda, ctx->ctl));
             CK(launch_dependent(true, k_gj_writeback, 1 + 4 * 148, 0, st, A, lda, n, p0, nb, (const float*)T, (const float*)Un, lda, D,
-                                Dbuf[(s & 1) ^ 1], ref, ldref, ctx->ctl, done));
+                                Dbuf[(s & 1) ^ 1], ref, ldref, ctx->ctl));
         }
         CK(cudaGetLastError());
         return OSSCAR_OK;
@@ -489,9 +486,9 @@ int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const 
     for (int64_t p0 = 0, s = 0; p0 < n; p0 += NB, ++s) {
         const int nb = (int)(n - p0 < NB ? n - p0 : NB);
         const float* D = Dbuf[s & 1];
-        CK(launch_dependent(true, k_gj_panels<false>, pgrid, 0, st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, next, RankTerms{}, done));
+        CK(launch_dependent(true, k_gj_panels<false>, pgrid, 0, st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, next, RankTerms{}));
         CK(launch_dependent(true, k_gj_update, ugrid, UP_SMEM, st, A, lda, n, p0, nb, (const float*)T, (const float*)U, (const float*)Un, lda,
-                            D, (const float*)next, Dbuf[(s & 1) ^ 1], ref, ldref, tiles_n, ctx->ctl, done));
+                            D, (const float*)next, Dbuf[(s & 1) ^ 1], ref, ldref, tiles_n, ctx->ctl));
     }
     CK(cudaGetLastError());
     return OSSCAR_OK;

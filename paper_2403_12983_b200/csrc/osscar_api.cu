@@ -343,7 +343,7 @@ int osscar_init_support(osscar_ctx* ctx, const float* H, const float* G, const f
         CKS(cudaStreamSynchronize(st));
         if (ctx->ctl_host->status != OSSCAR_OK) return ctx->ctl_host->status;
     }
-    if (rc == OSSCAR_OK) rc = build_state(ctx, false);
+    if (rc == OSSCAR_OK) rc = build_state(ctx);
     if (rc == OSSCAR_OK && score_pass(ctx) != cudaSuccess) rc = OSSCAR_E_CUDA;
     if (rc != OSSCAR_OK) { cudaStreamSynchronize(st); return rc; }
     CKC(cudaMemcpyAsync(ctx->ctl_host, ctx->ctl, sizeof(SearchCtl), cudaMemcpyDeviceToHost, st));
@@ -373,7 +373,7 @@ int osscar_init_support_greedy(osscar_ctx* ctx, const float* H, const float* G, 
     count_launches(1);
     int iters = 0;
     int rc = greedy_support(ctx, t_hat, support, drop_trace, &iters);
-    if (rc == OSSCAR_OK) rc = build_state(ctx, false);
+    if (rc == OSSCAR_OK) rc = build_state(ctx);
     if (rc == OSSCAR_OK && score_pass(ctx) != cudaSuccess) rc = OSSCAR_E_CUDA;
     if (rc != OSSCAR_OK) { cudaStreamSynchronize(st); return rc; }
     CKC(cudaMemcpyAsync(ctx->ctl_host, ctx->ctl, sizeof(SearchCtl), cudaMemcpyDeviceToHost, st));

@@ -122,7 +122,7 @@ cudaError_t gemm_f64acc(cudaStream_t st, int64_t M, int64_t N, int64_t K, double
                         const float* B, int64_t ldb, double beta, const float* C0, int64_t ldc0, float* C, int64_t ldc,
                         bool identity_plus, const int32_t* done = nullptr);
 cudaError_t gemm_f64out(cudaStream_t st, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
-                        const float* B, int64_t ldb, double* C, int64_t ldc, const int32_t* done = nullptr, bool tri = false);
+                        const float* B, int64_t ldb, double* C, int64_t ldc, bool tri = false);
 
 // ---- gemm_i8.cu: the same products from 8-bit digits of the operands on the int8 tensor cores (exact integer sums)
 struct I8Scratch {                 // device memory for the digits of A and of B (256-byte aligned), and what A's part holds
@@ -204,16 +204,16 @@ cudaError_t gram_mirror(cudaStream_t st, float* H, int64_t d1);   // copy upper 
 
 // ---- state.cu: support selection and state construction --------------------------------------
 int select_support(osscar_ctx* ctx, int mode, int32_t* support);
-int build_state(osscar_ctx* ctx, bool guarded);
+int build_state(osscar_ctx* ctx);
 // C = A B + beta C0 for A = Hinv or E (nI x nI): digits on the int8 tensor cores, or split bf16 where they do not pay or fit
 cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const float* B, int64_t ldb, float beta, const float* C0, float* C,
-                            int64_t ldc, int digits, void* other, size_t other_bytes, const int32_t* done);
+                            int64_t ldc, int digits, void* other, size_t other_bytes);
 // E = I - H_II Hinv summed beyond fp32; `v_free`: V and R hold nothing yet, so their memory may take operand digits
-cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32_t* done);
+cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free);
 // V += Hinv (G_I - H_II V), the residual summed beyond fp32.  GI: G_I in slot order (ldm), rV: as large, `other`: room for digits
-cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes, const int32_t* done);
+cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes);
 // ---- invert.cu
-int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref, const int32_t* done,
+int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref,
                        bool tensor_updates);
 // H^-1 of the whole layer in the place of Hp (nested phase): one Newton-Schulz step from digit products, in column panels, and
 // C = A B (d1 x d1 times d1 x m).  `correctable`: the layer is large enough and the free regions take the panels.
@@ -235,7 +235,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* p, int32_t* support_
                double* obj_trace, int32_t* swap_trace, osscar_search_result* res);
 cudaError_t score_pass(osscar_ctx* ctx);   // full scoring pass from the current state (fills D, A)
 // fp64 copy of the inverse from the fp32 one by a Newton-Schulz step summed in fp64 (single-row groups; uses `big`)
-int build_hinv64(osscar_ctx* ctx, bool guarded, bool v_free);
+int build_hinv64(osscar_ctx* ctx, bool v_free);
 // column shards: sum `count` values of `buf` (inside the workspace) over all shards through the context's hook
 int shard_reduce(osscar_ctx* ctx, void* buf, int64_t count, int dtype);
 

@@ -847,7 +847,7 @@ __global__ void k_begin(SearchCtl* ctl, double* obj_trace, int32_t* done_host)
     ctl->acc[2] = ctl->obj;
     *done_host = 0;
 }
-__global__ void k_count_refresh(SearchCtl* ctl) { if (!ctl->done) ctl->n_refresh += 1; }
+__global__ void k_count_refresh(SearchCtl* ctl) { ctl->n_refresh += 1; }
 __global__ void k_search_wait_limit(SearchCtl* ctl, long long cycles) { ctl->wait_limit = cycles; }
 __global__ void k_shard_scalar(SearchCtl* ctl, double* sh, int back) { if (back) ctl->acc[1] = sh[0]; else sh[0] = ctl->acc[1]; }
 __global__ void k_final_obj(SearchCtl* ctl) { ctl->acc[3] = ctl->const_term - ctl->acc[1]; }
@@ -1061,7 +1061,7 @@ int persistent_grid(const Layout& L, size_t* smem)
 
 }  // namespace
 
-int build_hinv64(osscar_ctx* ctx, bool guarded, bool v_free)
+int build_hinv64(osscar_ctx* ctx, bool v_free)
 {
     const Layout& L = ctx->L;
     cudaStream_t st = ctx->stream;
@@ -1070,18 +1070,17 @@ int build_hinv64(osscar_ctx* ctx, bool guarded, bool v_free)
     double* Hd = (double*)(ws + L.off_Hd);
     float* E = (float*)(ws + L.off_big);
     float* T = E + L.nI * L.ldh;
-    const int32_t* done = guarded ? &ctx->ctl->done : nullptr;
     // X0 = the fp32 inverse at hand (raw from the blocked inversion, or carried by an fp32 driver).  With E = I - H_II X0,
     // H_II^-1 = X0 (I + E + E^2 + ...): E is formed once with sums beyond fp32, the series is cut after E^2 (a correction of a
     // correction: three digits are ample; four for X0 (E + E^2)), and the sum X0 + X0 (E + E^2) is taken in fp64.
     // The error left is E^3 (below 1e-9 for any start within 1e-3), against E^2 for a single Newton-Schulz step.
-    if (inverse_residual(ctx, E, v_free, done) != cudaSuccess) return OSSCAR_E_CUDA;
+    if (inverse_residual(ctx, E, v_free) != cudaSuccess) return OSSCAR_E_CUDA;
     char* const other = ws + L.off_Hd;                                     // written only below: may hold digits
     const size_t other_bytes = (v_free ? L.off_y : L.off_V) - L.off_Hd;
-    if (inverse_product(ctx, L.nI, E, E, L.ldh, 1.f, E, T, L.ldh, 3, other, other_bytes, done) != cudaSuccess) return OSSCAR_E_CUDA;
-    if (inverse_product(ctx, L.nI, Hinv, T, L.ldh, 0.f, nullptr, E, L.ldh, 4, other, other_bytes, done) != cudaSuccess) return OSSCAR_E_CUDA;
-    k_hinv_to_d<<<(unsigned)L.nI, 256, 0, st>>>(Hinv, E, Hd, L.ldh, L.nI, done);
-    k_hinv_from_d<<<(unsigned)L.nI, 256, 0, st>>>(Hd, Hinv, L.ldh, done);
+    if (inverse_product(ctx, L.nI, E, E, L.ldh, 1.f, E, T, L.ldh, 3, other, other_bytes) != cudaSuccess) return OSSCAR_E_CUDA;
+    if (inverse_product(ctx, L.nI, Hinv, T, L.ldh, 0.f, nullptr, E, L.ldh, 4, other, other_bytes) != cudaSuccess) return OSSCAR_E_CUDA;
+    k_hinv_to_d<<<(unsigned)L.nI, 256, 0, st>>>(Hinv, E, Hd, L.ldh, L.nI);
+    k_hinv_from_d<<<(unsigned)L.nI, 256, 0, st>>>(Hd, Hinv, L.ldh);
     count_launches(2);
     if (cudaGetLastError() != cudaSuccess) return OSSCAR_E_CUDA;
     ctx->hd_valid = true;
@@ -1217,9 +1216,29 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     };
     if (g == 1 && !fast) ctx->hd_valid = false;          // these drivers move the fp32 inverse only
     if (max_swaps > 0 && fast) {
-        if (!ctx->hd_valid) { const int rcd = build_hinv64(ctx, false, false); if (rcd != OSSCAR_OK) return rcd; }
+        if (!ctx->hd_valid) { const int rcd = build_hinv64(ctx, false); if (rcd != OSSCAR_OK) return rcd; }
         CK(bootstrap_g1());
     }
+
+    // Rebuild of the state inside a search.  It overwrites what a finished search still needs (pending terms, the inverse, V, R),
+    // and the host runs ahead of the device: it is enqueued only for a loop that is known to go on.  The flag is copied
+    // in stream order, so all shards of a layer read the same value; beside a rebuild the wait is short.
+    bool stopped = false;
+    auto rebuild = [&]() -> int {
+        volatile int32_t* flag = ctx->done_flag_host + 3;
+        CK(cudaMemcpyAsync((void*)flag, &ctx->ctl->done, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        stopped = *flag != 0;
+        if (stopped) return OSSCAR_OK;
+        const int rb = build_state(ctx);
+        if (rb != OSSCAR_OK) return rb;
+        k_count_refresh<<<1, 1, 0, st>>>(ctx->ctl);
+        count_launches(1);
+        CK(enqueue_scores(ctx, p, true, pair));
+        if (sharded && shard_reduce(ctx, p.vnorm, L.d1, OSSCAR_FP32) != OSSCAR_OK) return OSSCAR_E_CUDA;
+        if (fast) CK(bootstrap_g1());
+        return OSSCAR_OK;
+    };
 
     if (block) {
         CK(cudaMemsetAsync((char*)ctx->ws + L.off_block, 0, block_bytes_for(L, bs * g), st));
@@ -1327,8 +1346,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     int nmarks = 0;                 // events recorded per profiled step (depends on the step variant)
     unsigned long long* loop_prof = (unsigned long long*)((char*)ctx->ws + L.off_loop + 2 * (size_t)kLoopMaxBlocks * 16);
     if (persistent && max_swaps > 0) {
-        // chunks of steps between rebuilds of the state (one chunk when the state is only ever updated); a stopped loop
-        // makes the remaining launches return at once, so no host round trip is needed in between
+        // chunks of steps between rebuilds of the state (one chunk when the state is only ever updated)
         LoopArgs la;
         la.p = p;
         la.candD = (LoopCand*)((char*)ctx->ws + L.off_loop);
@@ -1341,11 +1359,8 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         const int chunk = prm->refresh_every > 0 ? prm->refresh_every : max_swaps;
         for (int it0 = 0; it0 < max_swaps && rc == OSSCAR_OK; it0 += chunk) {
             if (it0 > 0) {
-                rc = build_state(ctx, true);
-                if (rc != OSSCAR_OK) break;
-                k_count_refresh<<<1, 1, 0, st>>>(ctx->ctl);
-                count_launches(1);
-                if (enqueue_scores(ctx, p, true, false) != cudaSuccess || bootstrap_g1() != cudaSuccess) { rc = OSSCAR_E_CUDA; break; }
+                rc = rebuild();
+                if (rc != OSSCAR_OK || stopped) break;
             }
             la.max_steps = max_swaps - it0 < chunk ? max_swaps - it0 : chunk;
             if (cudaMemsetAsync(&ctx->ctl->bar_count, 0, sizeof(unsigned long long) + sizeof(int32_t), st) != cudaSuccess) { rc = OSSCAR_E_CUDA; break; }
@@ -1367,13 +1382,8 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
             }
         }
         if (prm->refresh_every > 0 && it > 0 && it % prm->refresh_every == 0) {
-            rc = build_state(ctx, true);
-            if (rc != OSSCAR_OK) break;
-            k_count_refresh<<<1, 1, 0, st>>>(ctx->ctl);
-            count_launches(1);
-            if (enqueue_scores(ctx, p, true, pair) != cudaSuccess) { rc = OSSCAR_E_CUDA; break; }
-            if (sharded && shard_reduce(ctx, p.vnorm, L.d1, OSSCAR_FP32) != OSSCAR_OK) { rc = OSSCAR_E_CUDA; break; }
-            if (fast && bootstrap_g1() != cudaSuccess) { rc = OSSCAR_E_CUDA; break; }
+            rc = rebuild();
+            if (rc != OSSCAR_OK || stopped) break;
             lz_it0 = it;
             after_kernel = false;
         }
@@ -1488,7 +1498,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     }
     CK(cudaEventRecord(ctx->ev1, st));
     if (fast && max_swaps > 0) {       // the fp32 inverse follows its fp64 copy (state reader, other drivers)
-        k_hinv_from_d<<<(unsigned)L.nI, 256, 0, st>>>(p.Hd, p.Hinv, L.ldh, nullptr);
+        k_hinv_from_d<<<(unsigned)L.nI, 256, 0, st>>>(p.Hd, p.Hinv, L.ldh);
         count_launches(1);
     }
     if (own_limit) { k_search_wait_limit<<<1, 1, 0, st>>>(ctx->ctl, ctx->wait_limit); count_launches(1); }
@@ -1502,7 +1512,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         // are within 2e-6 as well.  After the caller's wait budget has been put back: the products wait on barriers of their own.
         float* rV = GI + L.nI * L.ldm;
         char* tail = (char*)(rV + L.nI * L.ldm);
-        CK(refine_v(ctx, GI, rV, tail, (size_t)((char*)ctx->ws + L.off_Hp - tail), nullptr));
+        CK(refine_v(ctx, GI, rV, tail, (size_t)((char*)ctx->ws + L.off_Hp - tail)));
     }
     CK(cudaMemsetAsync(W_out, 0, sizeof(float) * L.d1 * L.m, st));
     k_scatter_rows<<<(unsigned)L.nI, 256, 0, st>>>(p, W_out);

@@ -544,10 +544,8 @@ __global__ void __launch_bounds__(256) k_ypass_d(Ptrs p)
 }
 
 // Hd := (double) Hinv + (double) Dlt, symmetrised (second Newton-Schulz step, summed in fp64), and the reverse copy.
-__global__ void k_hinv_to_d(const float* __restrict__ Hinv, const float* __restrict__ Dlt, double* __restrict__ Hd, int64_t ldh, int64_t n,
-                            const int32_t* __restrict__ done)
+__global__ void k_hinv_to_d(const float* __restrict__ Hinv, const float* __restrict__ Dlt, double* __restrict__ Hd, int64_t ldh, int64_t n)
 {
-    if (done && *done) return;
     const int64_t r = blockIdx.x;
     for (int64_t c = threadIdx.x; c < ldh; c += blockDim.x) {
         double v = 0.0;
@@ -555,9 +553,8 @@ __global__ void k_hinv_to_d(const float* __restrict__ Hinv, const float* __restr
         Hd[r * ldh + c] = v;
     }
 }
-__global__ void k_hinv_from_d(const double* __restrict__ Hd, float* __restrict__ Hinv, int64_t ldh, const int32_t* __restrict__ done)
+__global__ void k_hinv_from_d(const double* __restrict__ Hd, float* __restrict__ Hinv, int64_t ldh)
 {
-    if (done && *done) return;
     const int64_t r = blockIdx.x;
     for (int64_t c = threadIdx.x; c < ldh; c += blockDim.x) Hinv[r * ldh + c] = (float)Hd[r * ldh + c];
 }

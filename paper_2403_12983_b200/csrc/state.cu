@@ -170,9 +170,8 @@ __global__ void k_copy_pad(const float* __restrict__ src, int64_t lds, int64_t r
 // Pm holds the rows of the pruned slots [t0, t0 + gridDim.x) in fp64 (row stride ldpm): H_JI Hinv (twice = 1), or, for
 // single-row groups, H_JI U with U the halved block upper triangle of Hinv (twice = 2: h^T Hinv h = 2 h^T U h).
 __global__ void k_schur(const float* __restrict__ Hp, int64_t ldp, const double* __restrict__ Pm, int64_t ldpm,
-                        int64_t nI, int g, double* __restrict__ c, int64_t t0, double twice, const int32_t* __restrict__ done)
+                        int64_t nI, int g, double* __restrict__ c, int64_t t0, double twice)
 {
-    if (done && *done) return;
     const int64_t t = t0 + blockIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int pair = blockIdx.y * nw + w; pair < g * g; pair += nw * gridDim.y) {
@@ -188,9 +187,8 @@ __global__ void k_schur(const float* __restrict__ Hp, int64_t ldp, const double*
 
 // c_t = Hp[J_t][J_t] - 2 * (partial sums of the quadratic form, in column order); one warp per pruned row.
 __global__ void k_schur_sum(const float* __restrict__ Hp, int64_t ldp, const double* __restrict__ part, int64_t ldpart, int np,
-                            int64_t nI, int64_t nJ, double* __restrict__ c, const int32_t* __restrict__ done)
+                            int64_t nI, int64_t nJ, double* __restrict__ c)
 {
-    if (done && *done) return;
     const int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (t >= nJ) return;
@@ -222,10 +220,8 @@ __global__ void k_sum_partials(const double* __restrict__ partial, int n, double
 // A := sym(A + D) (D may be null) on the n x n leading block: the blocked inversion leaves its two triangles different in the last bits
 // times cond, and the correction of that difference is the antisymmetric part of D, so both are symmetrised together.
 // A thread owns the pair (r, c), (c, r) with c >= r; tiles below the diagonal have nothing to do.
-__global__ void k_add_sym(float* __restrict__ A, int64_t lda, const float* __restrict__ D, int64_t ldd, int64_t n,
-                          const int32_t* __restrict__ done)
+__global__ void k_add_sym(float* __restrict__ A, int64_t lda, const float* __restrict__ D, int64_t ldd, int64_t n)
 {
-    if (done && *done) return;
     if (blockIdx.x < blockIdx.y) return;
     const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.x;
     for (int64_t r = (int64_t)blockIdx.y * 32 + threadIdx.y; r < (int64_t)blockIdx.y * 32 + 32 && r < n; r += 8) {
@@ -423,7 +419,7 @@ constexpr int kResidualDigits = 6, kDirectDigits = 5;      // see gemm_i8.cu
 // column, balanced), three where the result is itself a small correction.  (Three for V left its error at d1 = 8192 at 3.8e-8
 // against the 2.5e-8 of its fp32 rounding.)
 cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const float* B, int64_t ldb, float beta, const float* C0, float* C,
-                            int64_t ldc, int digits, void* other, size_t other_bytes, const int32_t* done)
+                            int64_t ldc, int digits, void* other, size_t other_bytes)
 {
     const Layout& L = ctx->L;
     char* ws = (char*)ctx->ws;
@@ -434,19 +430,19 @@ cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const fl
         p.M = L.nI; p.N = N; p.K = L.nI; p.alpha = 1.0; p.beta = beta;
         p.A = A; p.lda = L.ldh; p.B = B; p.ldb = ldb; p.C0 = beta != 0.f ? C0 : nullptr; p.ldc0 = ldc; p.C = C; p.ldc = ldc;
         p.diag = Hp; p.diag_stride = L.ldp + 1; p.inverse_scale = true;
-        return gemm_i8(ctx->stream, p, digits, sc, ctx->ctl, done);
+        return gemm_i8(ctx->stream, p, digits, sc, ctx->ctl, nullptr);
     }
     // the smallest layers: one launch on the fp64 pipe instead of three (two splits and a product with a handful of tiles)
     if ((double)L.nI * L.nI * (double)N <= kTinyProduct)
-        return gemm_f64acc(ctx->stream, L.nI, N, L.nI, 1.0, A, L.ldh, B, ldb, (double)beta, C0, ldc, C, ldc, false, done);
+        return gemm_f64acc(ctx->stream, L.nI, N, L.nI, 1.0, A, L.ldh, B, ldb, (double)beta, C0, ldc, C, ldc, false);
     if (beta != 0.f && C0 != C) {
         const cudaError_t e = cudaMemcpyAsync(C, C0, sizeof(float) * L.nI * ldc, cudaMemcpyDeviceToDevice, ctx->stream);
         if (e != cudaSuccess) return e;
     }
-    return gemm_tc(ctx->stream, L.nI, N, L.nI, 1.f, A, L.ldh, B, ldb, beta, C, ldc, ws + L.off_tc, L.tc_bytes, ctx->ctl, done);
+    return gemm_tc(ctx->stream, L.nI, N, L.nI, 1.f, A, L.ldh, B, ldb, beta, C, ldc, ws + L.off_tc, L.tc_bytes, ctx->ctl);
 }
 
-cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32_t* done)
+cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free)
 {
     const Layout& L = ctx->L;
     char* ws = (char*)ctx->ws;
@@ -460,12 +456,12 @@ cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free, const int32
         p.M = p.N = p.K = L.nI; p.alpha = -1.0; p.identity = true;
         p.A = Hp; p.lda = L.ldp; p.B = Hinv; p.ldb = L.ldh; p.C = E; p.ldc = L.ldh;
         p.diag = Hp; p.diag_stride = L.ldp + 1;
-        return gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, done);
+        return gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, nullptr);
     }
-    return gemm_f64acc(ctx->stream, L.nI, L.nI, L.nI, -1.0, Hp, L.ldp, Hinv, L.ldh, 0.0, nullptr, 0, E, L.ldh, true, done);
+    return gemm_f64acc(ctx->stream, L.nI, L.nI, L.nI, -1.0, Hp, L.ldp, Hinv, L.ldh, 0.0, nullptr, 0, E, L.ldh, true);
 }
 
-cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes, const int32_t* done)
+cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes)
 {
     const Layout& L = ctx->L;
     char* ws = (char*)ctx->ws;
@@ -479,11 +475,11 @@ cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, s
         p.M = nI; p.N = L.m; p.K = nI; p.alpha = -1.0; p.beta = 1.0;
         p.A = Hp; p.lda = L.ldp; p.B = V; p.ldb = L.ldm; p.C0 = GI; p.ldc0 = L.ldm; p.C = rV; p.ldc = L.ldm;
         p.diag = Hp; p.diag_stride = L.ldp + 1;
-        e = gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, done);
+        e = gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, nullptr);
     } else
-        e = gemm_f64acc(ctx->stream, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false, done);
+        e = gemm_f64acc(ctx->stream, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false);
     if (e != cudaSuccess) return e;
-    return inverse_product(ctx, L.m, (const float*)(ws + L.off_Hinv), rV, L.ldm, 1.f, V, V, L.ldm, 4, other, other_bytes, done);
+    return inverse_product(ctx, L.m, (const float*)(ws + L.off_Hinv), rV, L.ldm, 1.f, V, V, L.ldm, 4, other, other_bytes);
 }
 
 // Free while the nested phase prepares H^-1 in the place of Hp: the regions behind it, up to the staged vectors, and the
@@ -533,7 +529,7 @@ cudaError_t correct_dense_inverse(osscar_ctx* ctx, float* A, int64_t lda)
         e = gemm_i8(st, p, 3, sc, ctx->ctl, nullptr);
         if (e != cudaSuccess) return e;
     }
-    k_add_sym<<<dim3((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32)), dim3(32, 8), 0, st>>>(A, lda, nullptr, 0, n, nullptr);
+    k_add_sym<<<dim3((unsigned)((n + 31) / 32), (unsigned)((n + 31) / 32)), dim3(32, 8), 0, st>>>(A, lda, nullptr, 0, n);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -556,9 +552,8 @@ cudaError_t dense_inverse_times(osscar_ctx* ctx, const float* A, int64_t lda, co
     return gemm_i8(ctx->stream, p, 4, sc, ctx->ctl, nullptr);
 }
 
-// Rebuilds every piece of the search state from H, G and the current slot permutation.
-// With `guarded`, the kernels that can be skipped return at once when the loop has stopped.
-int build_state(osscar_ctx* ctx, bool guarded)
+// Builds every piece of the search state from H, G and the current slot permutation.
+int build_state(osscar_ctx* ctx)
 {
     const Layout& L = ctx->L;
     cudaStream_t st = ctx->stream;
@@ -570,7 +565,6 @@ int build_state(osscar_ctx* ctx, bool guarded)
     float* big = (float*)(ws + L.off_big);
     double* c = (double*)(ws + L.off_c);
     const int32_t* perm = (const int32_t*)(ws + L.off_perm);
-    const int32_t* done = guarded ? &ctx->ctl->done : nullptr;
     void* tc = ws + L.off_tc;
     const int64_t nI = L.nI, nJ = L.nJ;
 
@@ -582,7 +576,7 @@ int build_state(osscar_ctx* ctx, bool guarded)
     k_copy_pad<<<(unsigned)nI, 256, 0, st>>>(Hp, L.ldp, nI, nI, Hinv, L.ldh);
     count_launches(2);
     CK(cudaGetLastError());
-    { const int rc_inv = invert_spd_inplace(ctx, Hinv, L.ldh, nI, Hp, L.ldp, done, true); if (rc_inv != OSSCAR_OK) return rc_inv; }
+    { const int rc_inv = invert_spd_inplace(ctx, Hinv, L.ldh, nI, Hp, L.ldp, true); if (rc_inv != OSSCAR_OK) return rc_inv; }
     // Every product below that forms a small difference of large sums is summed far beyond fp32 (digit products on the
     // int8 tensor cores, gemm_i8; small ones on the fp64 pipe, gemm_f64acc): the scores of Eq. impact are compared at 1e-5
     // relative, and fp32 accumulation leaves cond(H_II) * 2^-24 in them.
@@ -591,14 +585,14 @@ int build_state(osscar_ctx* ctx, bool guarded)
     //     fp64, Hinv := sym(Hinv + Hinv E) (E is tiny: any product will do)
     ctx->hd_valid = false;
     if (L.g == 1) {
-        const int rc_d = build_hinv64(ctx, guarded, true);
+        const int rc_d = build_hinv64(ctx, true);
         if (rc_d != OSSCAR_OK) return rc_d;
     } else {
         float* E = big;
         float* Dlt = big + nI * L.ldh;
-        CK(inverse_residual(ctx, E, true, done));
-        CK(inverse_product(ctx, nI, Hinv, E, L.ldh, 0.f, nullptr, Dlt, L.ldh, 3, ws + L.off_Hd, L.off_y - L.off_Hd, done));
-        k_add_sym<<<dim3((unsigned)((nI + 31) / 32), (unsigned)((nI + 31) / 32)), dim3(32, 8), 0, st>>>(Hinv, L.ldh, Dlt, L.ldh, nI, done);
+        CK(inverse_residual(ctx, E, true));
+        CK(inverse_product(ctx, nI, Hinv, E, L.ldh, 0.f, nullptr, Dlt, L.ldh, 3, ws + L.off_Hd, L.off_y - L.off_Hd));
+        k_add_sym<<<dim3((unsigned)((nI + 31) / 32), (unsigned)((nI + 31) / 32)), dim3(32, 8), 0, st>>>(Hinv, L.ldh, Dlt, L.ldh, nI);
         count_launches(1);
     }
     // (2) V = Hinv G_I, then one refinement step with the residual G_I - H_II V
@@ -613,8 +607,8 @@ int build_state(osscar_ctx* ctx, bool guarded)
         const size_t rbytes = L.off_y - L.off_R;
         void* other = tail > rbytes ? (void*)((char*)big + used) : (void*)R;
         const size_t other_bytes = tail > rbytes ? tail : rbytes;
-        CK(inverse_product(ctx, L.m, Hinv, GI, L.ldm, 0.f, nullptr, V, L.ldm, 4, other, other_bytes, done));
-        CK(refine_v(ctx, GI, rV, other, other_bytes, done));
+        CK(inverse_product(ctx, L.m, Hinv, GI, L.ldm, 0.f, nullptr, V, L.ldm, 4, other, other_bytes));
+        CK(refine_v(ctx, GI, rV, other, other_bytes));
     }
     // obj = Tr(W^T G) - Tr(G_I^T V)
     if (ctx->have_const) CK(set_device_double(st, &ctx->ctl->acc[0], ctx->user_const));
@@ -650,9 +644,9 @@ int build_state(osscar_ctx* ctx, bool guarded)
             p.M = nJ; p.N = L.m; p.K = nI; p.alpha = -1.0; p.beta = 1.0;
             p.A = HJI; p.lda = L.ldp; p.B = V; p.ldb = L.ldm; p.C0 = R; p.ldc0 = L.ldm; p.C = R; p.ldc = L.ldm;
             p.diag = Hp; p.diag_stride = L.ldp + 1;
-            CK(gemm_i8(st, p, kDirectDigits, scR, ctx->ctl, done));
+            CK(gemm_i8(st, p, kDirectDigits, scR, ctx->ctl, nullptr));
         } else
-            CK(gemm_f64acc(st, nJ, L.m, nI, -1.0, HJI, L.ldp, V, L.ldm, 1.0, R, L.ldm, R, L.ldm, false, done));
+            CK(gemm_f64acc(st, nJ, L.m, nI, -1.0, HJI, L.ldp, V, L.ldm, 1.0, R, L.ldm, R, L.ldm, false));
         // (4) Schur complements H_qq - H_qI Hinv H_Iq.  Single-row groups need one quadratic form per pruned row, for which
         // half of the symmetric inverse is enough: from the fp64 inverse, with the dot products in the product's epilogue.
         if (one && gemm_i8_usable(nJ, nI, nI, kDirectDigits, scR)) {
@@ -662,8 +656,8 @@ int build_state(osscar_ctx* ctx, bool guarded)
             p.C = part; p.ldc = gemm_i8_dot_cols(nI);
             p.diag = Hp; p.diag_stride = L.ldp + 1;
             CK(cudaMemsetAsync(part, 0, part_bytes, st));        // 256-column tiles fill half of the columns
-            CK(gemm_i8(st, p, kDirectDigits, scR, ctx->ctl, done));
-            k_schur_sum<<<(unsigned)((nJ + 7) / 8), 256, 0, st>>>(Hp, L.ldp, part, p.ldc, (int)p.ldc, nI, nJ, c, done);
+            CK(gemm_i8(st, p, kDirectDigits, scR, ctx->ctl, nullptr));
+            k_schur_sum<<<(unsigned)((nJ + 7) / 8), 256, 0, st>>>(Hp, L.ldp, part, p.ldc, (int)p.ldc, nI, nJ, c);
             count_launches(1);
         } else {
             // Pm = Hp[J, I] Hinv kept in fp64, in panels of whole pruned groups that fit the scratch, then fp64 dot products
@@ -679,10 +673,10 @@ int build_state(osscar_ctx* ctx, bool guarded)
                     p.M = ngr * L.g; p.N = nI; p.K = nI; p.alpha = 1.0; p.out64 = true;
                     p.A = At; p.lda = L.ldp; p.B = Hinv; p.ldb = L.ldh; p.C = Pm; p.ldc = L.ldh;
                     p.diag = Hp; p.diag_stride = L.ldp + 1;
-                    CK(gemm_i8(st, p, kResidualDigits, sc, ctx->ctl, done));
+                    CK(gemm_i8(st, p, kResidualDigits, sc, ctx->ctl, nullptr));
                 } else
-                    CK(gemm_f64out(st, ngr * L.g, nI, nI, At, L.ldp, Hinv, L.ldh, Pm, L.ldh, done, one));
-                k_schur<<<dim3((unsigned)ngr, schur_shares(ngr, L.g)), 256, 0, st>>>(Hp, L.ldp, Pm, L.ldh, nI, L.g, c, t0, one ? 2.0 : 1.0, done);
+                    CK(gemm_f64out(st, ngr * L.g, nI, nI, At, L.ldp, Hinv, L.ldh, Pm, L.ldh, one));
+                k_schur<<<dim3((unsigned)ngr, schur_shares(ngr, L.g)), 256, 0, st>>>(Hp, L.ldp, Pm, L.ldh, nI, L.g, c, t0, one ? 2.0 : 1.0);
                 count_launches(1);
             }
         }
