@@ -56,16 +56,18 @@ __device__ __forceinline__ int warp_count(int v) {
     return v;
 }
 
-// kept[q] = 1 iff fewer than k groups beat q (larger energy, or equal energy and smaller id); a warp per group.
+// kept[q] = 1 iff fewer than k groups beat q (larger energy, or equal energy and smaller id); a warp per group.  NaN ranks
+// below every number: exactly k groups are marked whatever the energies are, and the slot permutation is complete.
 __global__ void k_rank_select(const double* __restrict__ e, int64_t ng, int k, int32_t* __restrict__ kept)
 {
     const int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (q >= ng) return;
-    const double eq = e[q];
+    auto ordered = [](double x) { return x == x ? x : -INFINITY; };
+    const double eq = ordered(e[q]);
     int rank = 0;
 #pragma unroll 4
     for (int64_t p = threadIdx.x & 31; p < ng; p += 32) {
-        const double ep = e[p];
+        const double ep = ordered(e[p]);
         rank += (ep > eq) || (ep == eq && p < q);
     }
     rank = warp_count(rank);
