@@ -137,7 +137,11 @@ __global__ void __launch_bounds__(1024) k_gr_select(GPtrs p, int n_live, int t, 
         if (tid == 0) {
             for (int i = 1; i < (int)(blockDim.x >> 5); ++i)
                 if (sv[i] < best || (sv[i] == best && sid[i] < bid)) { best = sv[i]; bid = sid[i]; bidx = sidx[i]; }
-            if (bidx < 0 || !isfinite(best)) { p.ctl->status = OSSCAR_E_NOTPD; bidx = n_live - 1 - round; }
+            if (bidx < 0 || !isfinite(best)) {            // fewer than t groups can leave: any others, each once
+                p.ctl->status = OSSCAR_E_NOTPD;
+                auto taken = [&](int slot) { for (int i = 0; i < round; ++i) if (chosen[i] == slot) return true; return false; };
+                for (bidx = n_live - 1; taken(bidx);) --bidx;
+            }
             chosen[round] = bidx;
             if (p.drop_trace) p.drop_trace[trace_pos + round] = p.perm[bidx];
             p.D[bidx] = INFINITY;                 // not again in this iteration

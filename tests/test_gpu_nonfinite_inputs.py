@@ -35,3 +35,21 @@ def test_groups_with_nan_weights_rank_last(g, mode):
         solver.init_support(torch.full_like(H, float("nan")), G, W, g, ng // 2, mode)
     assert len(solver.init_support(H, G, W, g, ng // 2, mode)[0]) == ng // 2
     solver.close()
+
+
+@pytest.mark.parametrize("g,t_hat", [(1, 10), (1, 1), (4, 5)])
+def test_nested_phase_of_a_singular_layer_is_an_error(g, t_hat):
+    H, G, W = _problem()
+    gen = torch.Generator().manual_seed(4)
+    X = torch.randn(40, 96, generator=gen)           # fewer rows than inputs: H has rank 40
+    Hs = (X.t() @ X).cuda()
+    Hz = H.clone()
+    Hz[:, ::3] = 0                                   # a third of the groups cannot be scored
+    Hz[::3] = 0
+    solver = pkg.Solver(0)
+    for bad in (Hs, Hz, -H, torch.full_like(H, float("nan"))):
+        with pytest.raises(pkg.OsscarError, match="positive definite"):
+            solver.init_support_greedy(bad, bad @ W, W, g, 5, t_hat)
+        S, drops = solver.init_support_greedy(H, G, W, g, 5, t_hat)[:2]
+        assert sorted(S.tolist() + drops.tolist()) == list(range(96 // g))
+    solver.close()
