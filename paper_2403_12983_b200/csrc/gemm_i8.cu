@@ -164,11 +164,13 @@ __global__ void __launch_bounds__(256) k_i8_colmax(const T* __restrict__ B, cons
 
 // Digits of the columns of B, stored transposed (column n of B = row n of the planes): tiles of 128 k x 32 columns turned
 // in shared memory.  tri_block > 0: entries of the diagonal blocks of that width are halved (column n is column col0 + n
-// of the whole matrix).
-template <int S, typename T>
+// of the whole matrix).  spread (or null): sums over a column of the squares of its entries, each rounded to 15 bits below the
+// column's scale; as whole numbers they do not depend on the order of the additions.
+template <int S, typename T, bool SPREAD = false>
 __global__ void __launch_bounds__(256) k_i8_slice_cols(const T* __restrict__ B, const T* __restrict__ sub, int64_t ldb, int64_t K, int64_t N, const int32_t* __restrict__ ck,
                                 const unsigned long long* __restrict__ cmax, int8_t* __restrict__ planes, int64_t plane, int64_t ldk,
-                                double* __restrict__ scale, int tri_block, int64_t col0, const int32_t* __restrict__ done)
+                                double* __restrict__ scale, int tri_block, int64_t col0, const int32_t* __restrict__ done,
+                                unsigned long long* __restrict__ spread = nullptr)
 {
     if (done && *done) return;
     __shared__ T tile[128][33];
@@ -182,13 +184,14 @@ __global__ void __launch_bounds__(256) k_i8_slice_cols(const T* __restrict__ B, 
     __syncthreads();
     const int nl = threadIdx.x >> 3, kg = (threadIdx.x & 7) * 16;
     const int64_t n = n0 + nl;
-    if (n >= N) return;
-    const unsigned long long mb = cmax[n];
+    if (!SPREAD && n >= N) return;
+    const unsigned long long mb = n < N ? cmax[n] : 0ull;
     const bool fin = finite_bits(mb);
     const int e = fin ? scale_exponent(__longlong_as_double((long long)mb)) : 0;
-    if (blockIdx.y == 0 && kg == 0) scale[n] = fin ? pow2d(e) : __longlong_as_double(0x7ff8000000000000ll);
-    if (k0 + kg >= ldk) return;
+    if (blockIdx.y == 0 && kg == 0 && n < N) scale[n] = fin ? pow2d(e) : __longlong_as_double(0x7ff8000000000000ll);
+    if (!SPREAD && k0 + kg >= ldk) return;
     uint32_t w[S][4];
+    unsigned long long sq = 0;                     // entries beyond the matrix are zero in the tile
 #pragma unroll
     for (int q4 = 0; q4 < 4; ++q4) {
         uint64_t d[4];
@@ -197,7 +200,9 @@ __global__ void __launch_bounds__(256) k_i8_slice_cols(const T* __restrict__ B, 
             const int64_t k = k0 + kg + q4 * 4 + i;
             const int half = tri_block > 0 && k / tri_block == (col0 + n) / tri_block ? 1 : 0;
             const int c = k < K ? ck[k] : 0;
-            d[i] = fin ? digit_bytes<S>(__double2ll_rn((double)tile[kg + q4 * 4 + i][nl] * pow2d(8 * S - 1 - e + c - half))) : 0ull;
+            const long long q = fin ? __double2ll_rn((double)tile[kg + q4 * 4 + i][nl] * pow2d(8 * S - 1 - e + c - half)) : 0ll;
+            if (SPREAD) { const long long t = q >> (8 * S - 16); sq += (unsigned long long)(t * t); }
+            d[i] = digit_bytes<S>(q);
         }
 #pragma unroll
         for (int s = 0; s < S; ++s) {
@@ -206,6 +211,11 @@ __global__ void __launch_bounds__(256) k_i8_slice_cols(const T* __restrict__ B, 
             for (int i = 0; i < 4; ++i) p |= (uint32_t)((d[i] >> (8 * (S - 1 - s))) & 0xff) << (8 * i);
             w[s][q4] = p;
         }
+    }
+    if (SPREAD) {                                  // eight neighbouring threads share a column
+        for (int o = 4; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        if (n < N && kg == 0) atomicAdd(&spread[n], sq);
+        if (n >= N || k0 + kg >= ldk) return;
     }
 #pragma unroll
     for (int s = 0; s < S; ++s)
@@ -674,9 +684,22 @@ size_t gemm_i8_operand_bytes(int64_t rows, int64_t K, int S)
     return (size_t)rows * ((size_t)S * round_up(K, 16) + 16) + 4 * (size_t)K + 2048;
 }
 
-// C (upper-triangle tiles) = beta C + sum of `slices` partial products, in slice order; block rows of tiles as in the product.
-__global__ void __launch_bounds__(256) k_i8_add_slices(float* __restrict__ C, int64_t d1, const float* __restrict__ part, int slices, int64_t stride, int add, int per)
+// Whether some column of a panel of `rows` rows has its scale above 32 times its root mean square (see gram_i8): skip[0] = 1 and
+// skip[1] = 0 then, the other way round otherwise.  Columns of zeros or with entries that are not finite do not count.
+__global__ void __launch_bounds__(1024) k_i8_outliers(const unsigned long long* __restrict__ cmax, const unsigned long long* __restrict__ spread,
+                                                      int64_t rows, int64_t d1, int32_t* __restrict__ skip)
 {
+    bool out = false;
+    for (int64_t j = threadIdx.x; j < d1; j += 1024) out |= cmax[j] != 0 && finite_bits(cmax[j]) && spread[j] < ((unsigned long long)rows << 20);
+    const int any = __syncthreads_or(out);
+    if (threadIdx.x == 0) { skip[0] = any ? 1 : 0; skip[1] = any ? 0 : 1; }
+}
+
+// C (upper-triangle tiles) = beta C + sum of `slices` partial products, in slice order; block rows of tiles as in the product.
+__global__ void __launch_bounds__(256) k_i8_add_slices(float* __restrict__ C, int64_t d1, const float* __restrict__ part, int slices, int64_t stride, int add, int per,
+                                                       const int32_t* __restrict__ done)
+{
+    if (*done) return;
     const int64_t row = blockIdx.y;
     const int64_t c0 = (row / I8_TM / per) * (I8_TM * per);
     for (int64_t c = c0 + (int64_t)blockIdx.x * 256 + threadIdx.x; c < d1; c += (int64_t)gridDim.x * 256) {
@@ -686,18 +709,25 @@ __global__ void __launch_bounds__(256) k_i8_add_slices(float* __restrict__ C, in
     }
 }
 
-// H (+)= Xc^T Xc over the upper-triangle tiles for fp32 Xc (n_rows x d1): three digits per entry, 23 bits below the largest of
-// its column in the panel, six products at twice the bf16 rate.  Both operands are the same transposed digits.  A layer with
-// fewer tiles than SMs splits the rows of a panel over CTAs, whose fp32 partial sums are added in order.  Measured at 24500 x 1024 in
-// five chunks: 0.97 -> 0.55 ms with the splitting, at 6272 x 4608: 1.2 -> 0.95 ms.
+// H (+)= Xc^T Xc over the upper-triangle tiles for fp32 Xc (n_rows x d1): four digits per entry, ten products at twice the bf16
+// rate.  Both operands are the same transposed digits.  A layer with fewer tiles than SMs splits the rows of a panel over
+// CTAs, whose fp32 partial sums are added in order.
+// Digits are fixed-point below the scale s_j of a column (a power of two, less than twice its largest entry), and the products
+// of order 6 are left out: at most 3 * 2^-32 s_i s_j a row, which repeated values (pixels, padding) add up with one sign.  A
+// column whose scale is at most 32 times its root mean square keeps that below 3 * 2^-22 sqrt(H_ii H_jj), less than the
+// sums of the bf16 terms lose.  A panel with a column beyond it (single large entries) goes through the bf16 terms, whose bits are
+// relative to every entry: both paths are enqueued, one returns at once.  (Three digits without this test left 2e-5 of
+// sqrt(H_ii H_jj), and 1e-3 of an entry, where one entry of a column was 300 times the rest.)
+// One chunk, ms, bf16 terms -> digits: 0.171 -> 0.119 at 4900 x 256, 0.187 -> 0.132 at 4900 x 1024, 0.087 -> 0.091 at 2048 x 1024, 0.051 -> 0.085
+// at 1024 x 1024, 0.80 -> 0.74 at 6272 x 4608, 0.196 -> 0.27 at 1500 x 4608: short chunks, and those whose tiles fill the SMs anyway, stay on the terms.
 // cudaErrorMemoryAllocation where the scratch is too small or the product too small to pay: the caller takes another path.
 cudaError_t gram_i8(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1, float* C, bool accumulate,
                     void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev)
 {
-    constexpr int S = 3;
+    constexpr int S = 4;
     if (n_rows <= 0) return cudaSuccess;
     if (!scratch || ((uintptr_t)scratch & 255) || d1 >= (1 << 28)) return cudaErrorMemoryAllocation;
-    if (n_rows < 256 || (double)n_rows * (double)d1 * (double)d1 < 536870912.0) return cudaErrorMemoryAllocation;
+    if (n_rows < (d1 < 1536 ? 2048 : 4096) || (double)n_rows * (double)d1 * (double)d1 < 268435456.0) return cudaErrorMemoryAllocation;
     PFN_encodeTiled enc = get_encode();
     if (!enc) return cudaErrorNotSupported;
     int dev = 0, sms = 0;
@@ -706,11 +736,11 @@ cudaError_t gram_i8(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1,
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int64_t TM = (d1 + I8_TM - 1) / I8_TM;
-    auto upper_tiles = [&](int tnc) { int64_t n = 0; for (int64_t r = 0; r < TM; ++r) n += (d1 + tnc - 1) / tnc - r / (tnc / I8_TM); return n; };
-    const int tn = 256;
-    const int64_t tiles = upper_tiles(tn);
-    // rows of a panel: digits, balance exponents and column scales
-    const size_t fixed = 16 * (size_t)d1 + 4096;
+    constexpr int tn = 256;
+    int64_t tiles = 0;
+    for (int64_t r = 0; r < TM; ++r) tiles += (d1 + tn - 1) / tn - r / (tn / I8_TM);
+    // rows of a panel: digits, balance exponents, column scales and sums
+    const size_t fixed = 24 * (size_t)d1 + 4096;
     if (scratch_bytes <= fixed) return cudaErrorMemoryAllocation;
     auto panel_rows = [&](size_t bytes) {
         int64_t r = (int64_t)(bytes / ((size_t)S * d1 + 4)) / 16 * 16 - 16;
@@ -726,29 +756,36 @@ cudaError_t gram_i8(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1,
         const int64_t most = (panel < n_rows ? panel : n_rows) / (8 * I8_BK);
         if (ks > most) ks = most;
         const size_t pb = up256(sizeof(float) * (size_t)d1 * d1);
-        while (ks > 1 && fixed + pb * (size_t)ks >= scratch_bytes) --ks;
-        if (ks > 1) {
-            const int64_t left = panel_rows(scratch_bytes - fixed - pb * (size_t)ks);
-            if (left >= n_rows || left >= 4096) { ksplit = (int)ks; if (panel > left) panel = left; }
+        for (; ks > 1; --ks) {
+            const int64_t left = fixed + pb * (size_t)ks < scratch_bytes ? panel_rows(scratch_bytes - fixed - pb * (size_t)ks) : 0;
+            if (left < n_rows && left < 1024) continue;
+            ksplit = (int)ks;
+            if (panel > left) panel = left;
+            break;
         }
     }
-    if (panel < 256 && panel < n_rows) return cudaErrorMemoryAllocation;
+    if (panel < n_rows) {                // panels of equal height
+        if (panel < 1024) return cudaErrorMemoryAllocation;
+        const int64_t np = (n_rows + panel - 1) / panel;
+        panel = round_up((n_rows + np - 1) / np, 16);
+    }
     char* b = (char*)scratch;
     float* part = (float*)b;                                   if (ksplit > 1) b += up256(sizeof(float) * (size_t)d1 * d1) * ksplit;
     int32_t* ck = (int32_t*)b;                                 b += up256(4 * (size_t)round_up(panel, 16));
     unsigned long long* cmax = (unsigned long long*)b;         b += up256(8 * (size_t)d1);
+    unsigned long long* spread = (unsigned long long*)b;       b += up256(8 * (size_t)d1);
     double* sc = (double*)b;                                   b += up256(8 * (size_t)d1);
     int8_t* planes = (int8_t*)b;
-    e = cudaMemsetAsync(ck, 0, 4 * (size_t)panel, st);
-    if (e != cudaSuccess) return e;
+    const int32_t *skip_digits = &ctl_dev->gram_skip[0], *skip_terms = &ctl_dev->gram_skip[1];
     for (int64_t r0 = 0; r0 < n_rows; r0 += panel) {
         const int64_t rows = n_rows - r0 < panel ? n_rows - r0 : panel, ldk = round_up(rows, 16);
-        e = cudaMemsetAsync(cmax, 0, 8 * (size_t)d1, st);
+        e = cudaMemsetAsync(ck, 0, (size_t)((char*)sc - (char*)ck), st);           // and the column maxima and sums behind it
         if (e != cudaSuccess) return e;
         k_i8_colmax<float><<<dim3((unsigned)((d1 + 63) / 64), (unsigned)((rows + 255) / 256)), 256, 0, st>>>(X + r0 * d1, nullptr, d1, rows, d1, ck, cmax, nullptr);
-        k_i8_slice_cols<S, float><<<dim3((unsigned)((d1 + 31) / 32), (unsigned)((ldk + 127) / 128)), 256, 0, st>>>(
-            X + r0 * d1, nullptr, d1, rows, d1, ck, cmax, planes, d1 * ldk, ldk, sc, 0, 0, nullptr);
-        count_launches(2);
+        k_i8_slice_cols<S, float, true><<<dim3((unsigned)((d1 + 31) / 32), (unsigned)((ldk + 127) / 128)), 256, 0, st>>>(
+            X + r0 * d1, nullptr, d1, rows, d1, ck, cmax, planes, d1 * ldk, ldk, sc, 0, 0, nullptr, spread);
+        k_i8_outliers<<<1, 1024, 0, st>>>(cmax, spread, rows, d1, ctl_dev->gram_skip);
+        count_launches(3);
         I8Maps maps;
         if (!encode_planes(enc, &maps.a, planes, (uint64_t)rows, (uint64_t)(S * d1), (uint64_t)ldk, I8_TM)) return cudaErrorInvalidValue;
         if (!encode_planes(enc, &maps.b, planes, (uint64_t)rows, (uint64_t)(S * d1), (uint64_t)ldk, (uint32_t)tn)) return cudaErrorInvalidValue;
@@ -759,12 +796,14 @@ cudaError_t gram_i8(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1,
         ep.C = ks > 1 ? part : C; ep.C0 = C; ep.beta = ks == 1 && add ? 1.0 : 0.0;
         ep.vec = ((uintptr_t)ep.C & 15) == 0 && ((uintptr_t)C & 15) == 0 && (d1 % 4) == 0 ? 1 : 0;
         const I8Cover cov = { 0, 1, ks, (int64_t)(up256(sizeof(float) * (size_t)d1 * d1) / sizeof(float)) };
-        e = launch_mma<S, 256, EPI_F32>(st, maps, d1, d1, rows, ep, cov, sms, ctl_dev, nullptr);
+        e = launch_mma<S, 256, EPI_F32>(st, maps, d1, d1, rows, ep, cov, sms, ctl_dev, skip_digits);
         if (e != cudaSuccess) return e;
         if (ks > 1) {
-            k_i8_add_slices<<<dim3((unsigned)((d1 + 1023) / 1024), (unsigned)d1), 256, 0, st>>>(C, d1, part, ks, cov.slice_stride, add ? 1 : 0, tn / I8_TM);
+            k_i8_add_slices<<<dim3((unsigned)((d1 + 1023) / 1024), (unsigned)d1), 256, 0, st>>>(C, d1, part, ks, cov.slice_stride, add ? 1 : 0, tn / I8_TM, skip_digits);
             count_launches(1);
         }
+        e = gram_tc3(st, X + r0 * d1, rows, d1, C, add, scratch, scratch_bytes, ctl_dev, skip_terms);
+        if (e != cudaSuccess) return e;
     }
     return cudaGetLastError();
 }

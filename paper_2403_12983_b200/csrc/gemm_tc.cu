@@ -820,7 +820,7 @@ cudaError_t gram_tc2(cudaStream_t st, const void* X, int64_t n_rows, int64_t d1,
 // sized to the scratch (each panel needs 6 * rows * round_up(d1, 8) bytes).  Returns cudaErrorMemoryAllocation when
 // the scratch cannot hold a panel of 64 rows, so that the caller can take another path.
 cudaError_t gram_tc3(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1, float* C, bool accumulate,
-                     void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev)
+                     void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done)
 {
     if (n_rows <= 0) return cudaSuccess;
     const int64_t ldn = round_up(d1, 8);
@@ -847,14 +847,14 @@ cudaError_t gram_tc3(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1
     const int vec_ok = (((uintptr_t)C & 15) == 0 && (d1 % 4) == 0) ? 1 : 0;
     for (int64_t r0 = 0; r0 < n_rows; r0 += panel) {
         const int64_t rows = n_rows - r0 < panel ? n_rows - r0 : panel;
-        launch_split3(st, X + r0 * d1, d1, rows, d1, xp[0], xp[1], xp[2], ldn, nullptr);
+        launch_split3(st, X + r0 * d1, d1, rows, d1, xp[0], xp[1], xp[2], ldn, done);
         Maps maps;
         for (int i = 0; i < 3; ++i) {
             if (!encode_2d(enc, &maps.a[i], xp[i], (uint64_t)d1, (uint64_t)rows, (uint64_t)ldn, 64, BLOCK_K)) return cudaErrorInvalidValue;
             maps.b[i] = maps.a[i];
         }
         k_mma_pipe<MODE_GRAM3><<<num_ids < sms ? num_ids : sms, NUM_THREADS, SMEM_BYTES, st>>>(
-            maps, d1, d1, rows, 1.f, (accumulate || r0 > 0) ? 1.f : 0.f, C, d1, vec_ok, num_ids, ctl_dev, nullptr);
+            maps, d1, d1, rows, 1.f, (accumulate || r0 > 0) ? 1.f : 0.f, C, d1, vec_ok, num_ids, ctl_dev, done);
         count_launches(2);
     }
     return cudaGetLastError();

@@ -205,8 +205,8 @@ int osscar_gram(osscar_ctx* ctx, const void* X, int x_dtype, int64_t n_rows, int
             // upper-triangle tiles only; the lower triangle is filled on END
             CKS(gram_tc2(st, X, n_rows, d1, nullptr, 0, 0, H, !begin, nullptr, 0, ctx->ctl));
         } else {
-            // fp32 activations: three-term bf16 split on the tensor cores when a workspace is lent (its contents are
-            // overwritten), else (or when it cannot hold a 64-row panel of the terms) the fp32 pipes
+            // fp32 activations: digits or the three-term bf16 split on the tensor cores when a workspace is lent (its contents
+            // are overwritten), else (or when it cannot hold a 64-row panel of the terms) the fp32 pipes
             cudaError_t ge = cudaErrorMemoryAllocation;
             if (ctx->ws) {
                 ge = gram_i8(st, (const float*)X, n_rows, d1, H, !begin, ctx->ws, ctx->ws_bytes, ctx->ctl);

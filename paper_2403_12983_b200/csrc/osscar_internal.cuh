@@ -38,6 +38,7 @@ struct SearchCtl {
     unsigned long long bar_count;   // arrivals at the grid barrier of the persistent swap loop (monotone)
     int32_t abort;           // set by a wait that ran out: every block of the persistent loop returns
     int32_t y_due;           // the step in flight made a swap (search_lazy_g1.cuh)
+    int32_t gram_skip[2];    // Gram of fp32 activations: the panel in flight skips the digits / the bf16 terms (gemm_i8.cu)
 };
 
 // Geometry of one layer's search state inside the caller's workspace.
@@ -196,7 +197,7 @@ cudaError_t gram_tc2(cudaStream_t st, const void* X, int64_t n_rows, int64_t d1,
 // H (+)= Xc^T Xc for fp32 Xc on the tensor cores (three-term bf16 split staged in `scratch`, row panels sized to it);
 // cudaErrorMemoryAllocation when the scratch is too small for one panel.
 cudaError_t gram_tc3(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1, float* C, bool accumulate,
-                     void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev);
+                     void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done = nullptr);
 
 // ---- gram_tc.cu ---------------------------------------------------------------------------------------------
 cudaError_t set_device_double(cudaStream_t st, double* dst, double v);          // *dst = v on the stream

@@ -47,3 +47,37 @@ def test_gram_and_cross_term_fp32(rows, d1, m, ws):
     gb = 48 * 2.0 ** -24 * (Hd.abs() @ W.double().abs())
     assert bool(((G.double().cpu() - G64).abs() <= gb).all())
     assert const == pytest.approx(float((W.double() * G64).sum()), rel=1e-5)
+
+
+# entries far above the rest of their column, values that repeat (their roundings do not average out), and both in one chunk
+@pytest.mark.parametrize("rows,d1", [([4900, 2100], 384), ([4100], 1600), ([2500], 777)])
+@pytest.mark.parametrize("kind,height", [("relu", 30), ("relu", 300), ("relu", 1000), ("relu", 1e6), ("pixels", 1), ("pixels", 8), ("constant", 6), ("constant", 40)])
+def test_gram_of_columns_with_outliers(rows, d1, kind, height):
+    import torch
+    import paper_2403_12983_b200 as pkg
+    from paper_2403_12983_b200 import binding as b
+    gen = torch.Generator(device="cuda").manual_seed(d1)
+    X = []
+    for i, r in enumerate(rows):
+        x = torch.relu(torch.randn(r, d1, generator=gen, device="cuda"))
+        if kind == "pixels":
+            x = torch.randint(0, 256, (r, d1), generator=gen, device="cuda").float() / 255
+        if kind == "constant":
+            x = (0.5 + torch.rand(1, d1, generator=gen, device="cuda")).expand(r, d1).contiguous()
+        if height > 1 and i == 0:                    # the second chunk has none
+            j = torch.arange(0, d1, 3, device="cuda")
+            x[j * 37 % r, j] = height * x.square().mean(0).sqrt()[j]
+        X.append(x)
+    solver = pkg.Solver(0)
+    solver.ensure_workspace(d1, 64, 1, d1 // 2)
+    H, G, W = torch.empty(d1, d1, device="cuda"), torch.empty(d1, 64, device="cuda"), torch.randn(d1, 64, generator=gen, device="cuda")
+    for i, x in enumerate(X):
+        solver.gram_chunk(x, H, (b.GRAM_BEGIN if i == 0 else 0) | (b.GRAM_END if i == len(X) - 1 else 0), W, G, 0.0)
+    solver.close()
+    X = torch.cat(X).double()
+    H64 = X.t() @ X                                  # no cancellation: nothing is negative
+    # bf16 terms: chains of 24 truncating additions per 64 rows and one fp32 addition per drain, at most 24 x 2^-23 in all;
+    # digits: 3 x 2^-22 sqrt(H_ii H_jj) left out
+    assert float(((H.double() - H64).abs() / H64).max()) < 24 * 2.0 ** -23
+    d = H64.diagonal().sqrt()
+    assert float(((H.double() - H64).abs() / (d[:, None] * d[None, :])).max()) < 24 * 2.0 ** -23
