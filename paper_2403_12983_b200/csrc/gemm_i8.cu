@@ -445,14 +445,13 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
                     const bool full = ep.vec && gc + 3 < N;
                     if (EPI == EPI_DOT) {
                         const float* h = ep.C0 + gr * ep.ldc0 + gc;
-                        if (ep.C0sub) {
-                            const float* hs = ep.C0sub + gr * ep.ldc0 + gc;
-                            for (int i = 0; i < 4; ++i) if (gc + i < N) dot[q] += v[i] * (double)(h[i] - hs[i]);
-                        } else if (full) {
-                            const float4 x = *reinterpret_cast<const float4*>(h);
+                        const float* hs = ep.C0sub ? ep.C0sub + gr * ep.ldc0 + gc : nullptr;
+                        if (full) {
+                            float4 x = *reinterpret_cast<const float4*>(h);
+                            if (hs) { const float4 y = *reinterpret_cast<const float4*>(hs); x.x -= y.x; x.y -= y.y; x.z -= y.z; x.w -= y.w; }
                             dot[q] += (v[0] * (double)x.x + v[1] * (double)x.y) + (v[2] * (double)x.z + v[3] * (double)x.w);
                         } else {
-                            for (int i = 0; i < 4; ++i) if (gc + i < N) dot[q] += v[i] * (double)h[i];
+                            for (int i = 0; i < 4; ++i) if (gc + i < N) dot[q] += v[i] * (double)(hs ? h[i] - hs[i] : h[i]);
                         }
                     } else if (EPI == EPI_F64) {
                         double* cp = (double*)ep.C + gr * ep.ldc + gc;
@@ -646,10 +645,10 @@ static cudaError_t gemm_i8_run(cudaStream_t st, const I8Gemm& p, I8Scratch& sc, 
                 ep.C = (double*)p.C + m0 * p.ldc + 2 * (n0 / tn);
             } else if (p.out64) ep.C = (double*)p.C + m0 * p.ldc + n0;
             else ep.C = (float*)p.C + m0 * p.ldc + n0;
-            ep.vec = (!ep.C0 || (((uintptr_t)ep.C0 & 15) == 0 && (p.ldc0 % 4) == 0)) && (p.dot || p.out64 || (((uintptr_t)ep.C & 15) == 0 && (p.ldc % 4) == 0)) ? 1 : 0;
+            ep.vec = (!ep.C0 || ((((uintptr_t)ep.C0 | (uintptr_t)ep.C0sub) & 15) == 0 && (p.ldc0 % 4) == 0)) && (p.dot || p.out64 || (((uintptr_t)ep.C & 15) == 0 && (p.ldc % 4) == 0)) ? 1 : 0;
             const I8Cover cov = { p.tri ? 1 + (int)(n0 / I8_BK) : 0, 0, 1, 0 };
             // the combinations of digits and epilogues that the callers use
-            if constexpr (S == 3 || S == 5) {
+            if constexpr (S == 4 || S == 5) {
                 if (p.dot) e = tn == 256 ? launch_mma<S, 256, EPI_DOT>(st, maps, mw, nw, K, ep, cov, sms, ctl, done)
                                          : launch_mma<S, 128, EPI_DOT>(st, maps, mw, nw, K, ep, cov, sms, ctl, done);
             }
@@ -657,7 +656,7 @@ static cudaError_t gemm_i8_run(cudaStream_t st, const I8Gemm& p, I8Scratch& sc, 
                 if (p.out64) e = tn == 256 ? launch_mma<S, 256, EPI_F64>(st, maps, mw, nw, K, ep, cov, sms, ctl, done)
                                            : launch_mma<S, 128, EPI_F64>(st, maps, mw, nw, K, ep, cov, sms, ctl, done);
             }
-            if (p.dot ? (S != 3 && S != 5) : (p.out64 && S != 6)) return cudaErrorInvalidValue;
+            if (p.dot ? (S != 4 && S != 5) : (p.out64 && S != 6)) return cudaErrorInvalidValue;
             if (!p.dot && !p.out64)
                 e = tn == 256 ? launch_mma<S, 256, EPI_F32>(st, maps, mw, nw, K, ep, cov, sms, ctl, done)
                               : launch_mma<S, 128, EPI_F32>(st, maps, mw, nw, K, ep, cov, sms, ctl, done);
@@ -830,8 +829,8 @@ cudaError_t cross_term_tc(cudaStream_t st, const float* H, int64_t d1, const flo
     return gemm_i8(st, p, S, sc, ctl_dev, nullptr);
 }
 
-// Fixed-order sum of n doubles in two stages, the first over 256 blocks.
-__global__ void __launch_bounds__(256) k_i8_sum(const double* __restrict__ x, int64_t n, double* __restrict__ part)
+// Fixed-order sum of n doubles in two stages, the first over 256 blocks (added to what the blocks already have, if `add`).
+__global__ void __launch_bounds__(256) k_i8_sum(const double* __restrict__ x, int64_t n, double* __restrict__ part, int add)
 {
     __shared__ double red[8];
     double s = 0.0;
@@ -842,40 +841,48 @@ __global__ void __launch_bounds__(256) k_i8_sum(const double* __restrict__ x, in
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int i = 1; i < 8; ++i) s += red[i];
-        part[blockIdx.x] = s;
+        part[blockIdx.x] = add ? part[blockIdx.x] + s : s;
     }
 }
 
-// *out = sum of D o (H D), D = W - Wt (fp32 differences), as one digit product with the sum in its epilogue: neither D nor H D
-// is ever stored.  Three digits (six products): the 2^-24 roundings of the entries below the largest of a row of H or column of
-// D are independent of each other and average out in the sum of d1 m terms.  On the fp32 pipes (38 TFLOP/s) the product
-// alone took 6.93 ms at d1 = 8192, m = 2048; a call now takes 1.04 ms.
-// The scratch takes the digits of D and of a row panel of H, and one partial sum per row and half tile.
+// *out = sum of D o (H D), D = W - Wt (fp32 differences), as digit products with the sum in their epilogue: neither D nor H D
+// is ever stored.  Four digits (ten products): 1e-9 of the result, least-squares refits and columns with single large
+// weights included.  (Three digits left up to 5e-7 there, the fp32 pipes 9e-8.)
+// The scratch takes one partial sum per row and half tile and the digits of a slab of the contraction: some columns of H
+// and as many rows of D, whose sums add up.  A slab has all tiles of the result, whatever m is.
+// A call takes 1.64 ms at d1 = 8192, m = 2048 and 0.24 ms at 2048, 512, on the fp32 pipes 6.99 and 0.32 ms.  Bound: the int8 tensor pipe (1.3 of the 1.64 ms),
+// then the slicing of H.
 cudaError_t objective_i8(cudaStream_t st, const float* H, const float* W, const float* Wt, int64_t d1, int64_t m,
                          void* scratch, size_t scratch_bytes, double* partials, double* out_dev, SearchCtl* ctl_dev)
 {
-    constexpr int S = 3;
+    constexpr int S = 4;
     const int64_t pc = gemm_i8_dot_cols(m);
     const size_t part_bytes = up256(sizeof(double) * (size_t)d1 * pc);
-    if (!scratch || ((uintptr_t)scratch & 255) || scratch_bytes <= part_bytes) return cudaErrorMemoryAllocation;
-    I8Scratch sc;
-    size_t need_b = up256(gemm_i8_operand_bytes(m, d1, S));
-    const size_t room = (scratch_bytes - part_bytes) / 256 * 256;
-    if (need_b > room / 5 * 3) need_b = room / 2 / 256 * 256;
+    if (!scratch || ((uintptr_t)scratch & 255) || (double)d1 * (double)d1 * (double)m < 536870912.0) return cudaErrorMemoryAllocation;
+    auto b_bytes = [&](int64_t w) { return up256(gemm_i8_operand_bytes(m, w, S)); };
+    auto a_bytes = [&](int64_t w) { return up256(gemm_i8_operand_bytes(d1, w, S)); };
+    int64_t w = round_up(d1, I8_BK) < max_k(S) ? round_up(d1, I8_BK) : max_k(S) / I8_BK * I8_BK;
+    while (w >= 256 && part_bytes + a_bytes(w) + b_bytes(w) > scratch_bytes) w -= I8_BK;
+    if (w < 256) return cudaErrorMemoryAllocation;
+    const int64_t slabs = (d1 + w - 1) / w;
+    w = round_up((d1 + slabs - 1) / slabs, I8_BK);
     double* part = (double*)scratch;
-    sc.b = (char*)scratch + part_bytes; sc.b_bytes = need_b;
-    sc.a = (char*)scratch + part_bytes + need_b; sc.a_bytes = room - need_b;
-    if (!gemm_i8_usable(d1, m, d1, S, sc)) return cudaErrorMemoryAllocation;
-    I8Gemm p = {};
-    p.M = d1; p.N = m; p.K = d1; p.alpha = 1.0; p.dot = true;
-    p.A = H; p.lda = d1; p.B = W; p.Bsub = Wt; p.ldb = m; p.C0 = W; p.C0sub = Wt; p.ldc0 = m; p.C = part; p.ldc = pc;
-    p.diag = H; p.diag_stride = d1 + 1;
     cudaError_t e = cudaMemsetAsync(part, 0, sizeof(double) * (size_t)d1 * pc, st);       // 256-column tiles fill half of the columns
     if (e != cudaSuccess) return e;
-    e = gemm_i8(st, p, S, sc, ctl_dev, nullptr);
-    if (e != cudaSuccess) return e;
-    k_i8_sum<<<256, 256, 0, st>>>(part, d1 * pc, partials);
-    count_launches(1);
+    for (int64_t k0 = 0; k0 < d1; k0 += w) {
+        I8Scratch sc;
+        sc.b = (char*)scratch + part_bytes; sc.b_bytes = b_bytes(w);
+        sc.a = (char*)sc.b + sc.b_bytes; sc.a_bytes = a_bytes(w);
+        I8Gemm p = {};
+        p.M = d1; p.N = m; p.K = d1 - k0 < w ? d1 - k0 : w; p.alpha = 1.0; p.dot = true;
+        p.A = H + k0; p.lda = d1; p.B = W + k0 * m; p.Bsub = Wt + k0 * m; p.ldb = m;
+        p.C0 = W; p.C0sub = Wt; p.ldc0 = m; p.C = part; p.ldc = pc;
+        p.diag = H + k0 * (d1 + 1); p.diag_stride = d1 + 1;
+        e = gemm_i8(st, p, S, sc, ctl_dev, nullptr);
+        if (e != cudaSuccess) return e;
+        k_i8_sum<<<256, 256, 0, st>>>(part, d1 * pc, partials, k0 > 0 ? 1 : 0);
+        count_launches(1);
+    }
     return sum_partials(st, partials, 256, out_dev);
 }
 
