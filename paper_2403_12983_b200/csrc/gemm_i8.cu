@@ -851,14 +851,16 @@ __global__ void __launch_bounds__(256) k_i8_sum(const double* __restrict__ x, in
 // The scratch takes one partial sum per row and half tile and the digits of a slab of the contraction: some columns of H
 // and as many rows of D, whose sums add up.  A slab has all tiles of the result, whatever m is.
 // A call takes 1.64 ms at d1 = 8192, m = 2048 and 0.24 ms at 2048, 512, on the fp32 pipes 6.99 and 0.32 ms.  Bound: the int8 tensor pipe (1.3 of the 1.64 ms),
-// then the slicing of H.
+// then the slicing of H.  Narrow results stay on the fp32 pipes: the scratch shrinks with m, and every slab costs its launches and the
+// slicing of d1 rows (about 90 us at d1 = 8192).  Pipes against digits, ms: 3.15 / 3.78 at 12288, 384, 4.68 / 2.96 at 12288, 512, 1.28 / 1.92
+// at 8192, 256, 2.11 / 1.34 at 8192, 512, 0.32 / 0.38 at 2048, 256, 0.33 / 0.24 at 2048, 512.
 cudaError_t objective_i8(cudaStream_t st, const float* H, const float* W, const float* Wt, int64_t d1, int64_t m,
                          void* scratch, size_t scratch_bytes, double* partials, double* out_dev, SearchCtl* ctl_dev)
 {
     constexpr int S = 4;
     const int64_t pc = gemm_i8_dot_cols(m);
     const size_t part_bytes = up256(sizeof(double) * (size_t)d1 * pc);
-    if (!scratch || ((uintptr_t)scratch & 255) || (double)d1 * (double)d1 * (double)m < 536870912.0) return cudaErrorMemoryAllocation;
+    if (!scratch || ((uintptr_t)scratch & 255) || m <= 384 || (double)d1 * (double)d1 * (double)m < 536870912.0) return cudaErrorMemoryAllocation;
     auto b_bytes = [&](int64_t w) { return up256(gemm_i8_operand_bytes(m, w, S)); };
     auto a_bytes = [&](int64_t w) { return up256(gemm_i8_operand_bytes(d1, w, S)); };
     int64_t w = round_up(d1, I8_BK) < max_k(S) ? round_up(d1, I8_BK) : max_k(S) / I8_BK * I8_BK;

@@ -1,4 +1,4 @@
-"""osscar_objective against fp64: below 2^29 multiply-adds on the fp32 pipes, above from digits, in slabs of the contraction that
+"""osscar_objective against fp64: below 2^29 multiply-adds and up to 384 columns on the fp32 pipes, above from digits, in slabs of the contraction that
 the 2 * d1 * m floats of scratch take; sizes around the tiles (128 rows, 256 or 128 columns) and the 128-wide k-blocks."""
 import pytest
 
@@ -16,7 +16,8 @@ def _call(H, W, Wt):
     return got, launches
 
 
-@pytest.mark.parametrize("d1,m", [(128, 256), (1000, 333), (129, 257), (515, 1030), (2050, 64), (700, 1), (64, 40), (1, 1), (1153, 100)])
+@pytest.mark.parametrize("d1,m", [(128, 256), (1000, 333), (129, 257), (515, 1030), (2050, 64), (700, 1), (64, 40), (1, 1), (1153, 100),
+                                  (2100, 130), (1200, 384)])      # large, but too narrow for digits
 def test_objective_matches_fp64(d1, m):
     import torch
     gen = torch.Generator().manual_seed(d1 + m)
