@@ -52,8 +52,8 @@ enum { OSSCAR_ACCEPT_IMPROVING = 0, OSSCAR_ACCEPT_ALWAYS = 1 };
 enum { OSSCAR_STOP_MAX_SWAPS = 0, OSSCAR_STOP_NO_IMPROVEMENT = 1, OSSCAR_STOP_GUARD = 2 };
 /* Swap loop of single-row groups.  PERSISTENT = one cooperative kernel that runs all steps with bounded grid-wide
  * barriers between their phases (OSSCAR_E_ARG if the device cannot launch cooperatively); LAUNCHES = a chain of
- * dependent launches per step, enqueued ahead of the device; AUTO = PERSISTENT for states that fit the L2 cache (under 96 MB),
- * LAUNCHES for states streamed from HBM. */
+ * dependent launches per step, enqueued ahead of the device; AUTO = PERSISTENT for states that fit the L2 cache (under 96 MB)
+ * and have up to 8192 columns, LAUNCHES for wider ones and for states streamed from HBM. */
 enum { OSSCAR_LOOP_AUTO = 0, OSSCAR_LOOP_PERSISTENT = 1, OSSCAR_LOOP_LAUNCHES = 2 };
 
 #define OSSCAR_MAX_GROUP 96   /* largest supported group size g */

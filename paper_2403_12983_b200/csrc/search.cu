@@ -1138,7 +1138,11 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     // resident blocks per SM of one-row kernels keep more loads in flight than the loop's blocks do (measured 0.81
     // against 0.71 of copy bandwidth on the OPT-30B-shaped FC2 layer)
     const double state_bytes = 8.0 * L.nI * L.ldh + 4.0 * (L.nI + L.nJ) * L.ldm + 4.0 * L.nJ * L.ldh;
-    const bool want_persistent = sharded ? false : prm->loop_mode == OSSCAR_LOOP_PERSISTENT || (prm->loop_mode == OSSCAR_LOOP_AUTO && state_bytes <= 96.0e6);
+    // Wide results (rows of V and R past 8192 floats) go to the chain as well: it deals a row to several blocks, the loop to one
+    // warp.  Loop against chain, us a swap: 21.5 / 26.5 at d1 = 256, m = 4096, 27.7 / 27.8 at 256, 8192, 40.0 / 28.5 at 256, 16384, 181 / 34.9 at 256, 32768,
+    // 31.2 / 34.3 at 1024, 8192, 53.1 / 42.1 at 1024, 16384.
+    const bool want_persistent = sharded ? false : prm->loop_mode == OSSCAR_LOOP_PERSISTENT ||
+                                 (prm->loop_mode == OSSCAR_LOOP_AUTO && state_bytes <= 96.0e6 && L.ldm <= 8192);
     size_t psmem = 0;
     const int pgrid = (fast && want_persistent && L.nJ > 0) ? persistent_grid(L, &psmem) : 0;
     if (prm->loop_mode == OSSCAR_LOOP_PERSISTENT && pgrid == 0) return OSSCAR_E_ARG;
