@@ -133,6 +133,68 @@ k_gemm_f64acc(int64_t M, int64_t N, int64_t K, double alpha, const float* __rest
     }
 }
 
+// The same product (float result) where the tiles above would leave most SMs idle: 32 x 32 tiles, the k-range of a tile dealt to
+// the eight warps of its block in pieces of 16, whose fp64 sums are added in warp order.  Bound: latency; fragments come straight
+// from global memory (L2), 32 loads in flight per thread.  G = H W with 128 x 64 tiles and with these, ms a call (45 us of it around the
+// product): 0.071 / 0.054 at 256, 256, 0.150 / 0.069 at 1024, 4, 0.518 / 0.146 at 4096, 1 (32 tiles); state of a layer 0.367 / 0.272 at
+// d1 = m = 256, 2.95 / 2.68 at 5000, 1283 with 1777 rows kept.
+constexpr int DS_TILES = 74;             // 128 x 64 tiles up to which the split is taken: half of the SMs
+constexpr int DS_T = 32, DS_W = 8, DS_SMEM = DS_W * DS_T * DS_T * (int)sizeof(double);
+__global__ void __launch_bounds__(32 * DS_W)
+k_gemm_f64_split(int64_t M, int64_t N, int64_t K, double alpha, const float* __restrict__ A, int64_t lda, const float* __restrict__ B, int64_t ldb,
+                 double beta, const float* C0, int64_t ldc0, float* C, int64_t ldc, int identity, const int32_t* __restrict__ done)
+{
+    if (done && *done) return;
+    extern __shared__ double dg_smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int fr = lane >> 2, fk = lane & 3;                   // fragment row / column index, k index inside a k4 step
+    const int64_t m0 = (int64_t)blockIdx.y * DS_T, n0 = (int64_t)blockIdx.x * DS_T;
+    double acc[4][4][2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { acc[i][j][0] = 0.0; acc[i][j][1] = 0.0; }
+    for (int64_t k0 = warp * 16; k0 < K; k0 += DS_W * 16) {
+        float a[4][4], b[4][4];                                // [k4 step][tile]
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const int64_t k = k0 + 4 * s + fk;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int64_t r = m0 + i * 8 + fr, c = n0 + i * 8 + fr;
+                a[s][i] = r < M && k < K ? A[r * lda + k] : 0.f;
+                b[s][i] = c < N && k < K ? B[k * ldb + c] : 0.f;
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (n0 + j * 8 < N) {                          // narrow results: the same in the whole block
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) dmma(acc[i][j][0], acc[i][j][1], (double)a[s][i], (double)b[s][j]);
+                }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) dg_smem[(warp * DS_T + i * 8 + fr) * DS_T + j * 8 + 2 * fk + e] = acc[i][j][e];
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < DS_T * DS_T; idx += 32 * DS_W) {
+        const int64_t row = m0 + idx / DS_T, col = n0 + idx % DS_T;
+        if (row >= M || col >= N) continue;
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < DS_W; ++w) v += dg_smem[w * DS_T * DS_T + idx];
+        v *= alpha;
+        if (identity) v += row == col ? 1.0 : 0.0;
+        else if (beta != 0.0) v += beta * (double)C0[row * ldc0 + col];
+        C[row * ldc + col] = (float)v;
+    }
+}
+
 }  // namespace
 
 cudaError_t gemm_f64acc(cudaStream_t st, int64_t M, int64_t N, int64_t K, double alpha, const float* A, int64_t lda,
@@ -143,6 +205,14 @@ cudaError_t gemm_f64acc(cudaStream_t st, int64_t M, int64_t N, int64_t K, double
     const int vecA = (((uintptr_t)A & 15) == 0 && (lda % 4) == 0) ? 1 : 0;
     const int vecB = (((uintptr_t)B & 15) == 0 && (ldb % 4) == 0) ? 1 : 0;
     dim3 grid((unsigned)((N + DG_BN - 1) / DG_BN), (unsigned)((M + DG_BM - 1) / DG_BM));
+    if ((int64_t)grid.x * grid.y <= DS_TILES) {
+        const dim3 gs((unsigned)((N + DS_T - 1) / DS_T), (unsigned)((M + DS_T - 1) / DS_T));
+        const cudaError_t es = cudaFuncSetAttribute(k_gemm_f64_split, cudaFuncAttributeMaxDynamicSharedMemorySize, DS_SMEM);
+        if (es != cudaSuccess) return es;
+        k_gemm_f64_split<<<gs, 32 * DS_W, DS_SMEM, st>>>(M, N, K, alpha, A, lda, B, ldb, beta, C0, ldc0, C, ldc, identity_plus ? 1 : 0, done);
+        count_launches(1);
+        return cudaGetLastError();
+    }
     constexpr int smem = (2 * DG_BM * DG_AS + 2 * DG_BK * DG_BS) * (int)sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(k_gemm_f64acc<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
