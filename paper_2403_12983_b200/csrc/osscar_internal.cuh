@@ -38,6 +38,7 @@ struct SearchCtl {
     unsigned long long bar_count;   // arrivals at the grid barrier of the persistent swap loop (monotone)
     int32_t abort;           // set by a wait that ran out: every block of the persistent loop returns
     int32_t y_due;           // the step in flight made a swap (search_lazy_g1.cuh)
+    int32_t settled;         // the search made no swap: V is as refined as it was
     int32_t gram_skip[2];    // Gram of fp32 activations: the panel in flight skips the digits / the bf16 terms (gemm_i8.cu)
 };
 
@@ -208,11 +209,12 @@ int select_support(osscar_ctx* ctx, int mode, int32_t* support);
 int build_state(osscar_ctx* ctx);
 // C = A B + beta C0 for A = Hinv or E (nI x nI): digits on the int8 tensor cores, or split bf16 where they do not pay or fit
 cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const float* B, int64_t ldb, float beta, const float* C0, float* C,
-                            int64_t ldc, int digits, void* other, size_t other_bytes);
+                            int64_t ldc, int digits, void* other, size_t other_bytes, const int32_t* skip = nullptr);
 // E = I - H_II Hinv summed beyond fp32; `v_free`: V and R hold nothing yet, so their memory may take operand digits
 cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free);
-// V += Hinv (G_I - H_II V), the residual summed beyond fp32.  GI: G_I in slot order (ldm), rV: as large, `other`: room for digits
-cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes);
+// V += Hinv (G_I - H_II V), the residual summed beyond fp32.  GI: G_I in slot order (ldm), rV: as large, `other`: room for digits;
+// nothing happens where *skip (device, may be null) is set
+cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes, const int32_t* skip = nullptr);
 // ---- invert.cu
 int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref,
                        bool tensor_updates);

@@ -847,6 +847,7 @@ __global__ void k_begin(SearchCtl* ctl, double* obj_trace, int32_t* done_host)
     ctl->acc[2] = ctl->obj;
     *done_host = 0;
 }
+__global__ void k_settled(SearchCtl* ctl) { ctl->settled = ctl->n_swaps == 0; }
 __global__ void k_count_refresh(SearchCtl* ctl) { ctl->n_refresh += 1; }
 __global__ void k_search_wait_limit(SearchCtl* ctl, long long cycles) { ctl->wait_limit = cycles; }
 __global__ void k_shard_scalar(SearchCtl* ctl, double* sh, int back) { if (back) ctl->acc[1] = sh[0]; else sh[0] = ctl->acc[1]; }
@@ -1516,7 +1517,9 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         // are within 2e-6 as well.  After the caller's wait budget has been put back: the products wait on barriers of their own.
         float* rV = GI + L.nI * L.ldm;
         char* tail = (char*)(rV + L.nI * L.ldm);
-        CK(refine_v(ctx, GI, rV, tail, (size_t)((char*)ctx->ws + L.off_Hp - tail)));
+        k_settled<<<1, 1, 0, st>>>(ctx->ctl);          // a start that no swap improved has been refined by the state build
+        count_launches(1);
+        CK(refine_v(ctx, GI, rV, tail, (size_t)((char*)ctx->ws + L.off_Hp - tail), &ctx->ctl->settled));
     }
     CK(cudaMemsetAsync(W_out, 0, sizeof(float) * L.d1 * L.m, st));
     k_scatter_rows<<<(unsigned)L.nI, 256, 0, st>>>(p, W_out);

@@ -421,7 +421,7 @@ constexpr int kResidualDigits = 6, kDirectDigits = 5;      // see gemm_i8.cu
 // column, balanced), three where the result is itself a small correction.  (Three for V left its error at d1 = 8192 at 3.8e-8
 // against the 2.5e-8 of its fp32 rounding.)
 cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const float* B, int64_t ldb, float beta, const float* C0, float* C,
-                            int64_t ldc, int digits, void* other, size_t other_bytes)
+                            int64_t ldc, int digits, void* other, size_t other_bytes, const int32_t* skip)
 {
     const Layout& L = ctx->L;
     char* ws = (char*)ctx->ws;
@@ -432,16 +432,16 @@ cudaError_t inverse_product(osscar_ctx* ctx, int64_t N, const float* A, const fl
         p.M = L.nI; p.N = N; p.K = L.nI; p.alpha = 1.0; p.beta = beta;
         p.A = A; p.lda = L.ldh; p.B = B; p.ldb = ldb; p.C0 = beta != 0.f ? C0 : nullptr; p.ldc0 = ldc; p.C = C; p.ldc = ldc;
         p.diag = Hp; p.diag_stride = L.ldp + 1; p.inverse_scale = true;
-        return gemm_i8(ctx->stream, p, digits, sc, ctx->ctl, nullptr);
+        return gemm_i8(ctx->stream, p, digits, sc, ctx->ctl, skip);
     }
     // the smallest layers: one launch on the fp64 pipe instead of three (two splits and a product with a handful of tiles)
     if ((double)L.nI * L.nI * (double)N <= kTinyProduct)
-        return gemm_f64acc(ctx->stream, L.nI, N, L.nI, 1.0, A, L.ldh, B, ldb, (double)beta, C0, ldc, C, ldc, false);
+        return gemm_f64acc(ctx->stream, L.nI, N, L.nI, 1.0, A, L.ldh, B, ldb, (double)beta, C0, ldc, C, ldc, false, skip);
     if (beta != 0.f && C0 != C) {
         const cudaError_t e = cudaMemcpyAsync(C, C0, sizeof(float) * L.nI * ldc, cudaMemcpyDeviceToDevice, ctx->stream);
         if (e != cudaSuccess) return e;
     }
-    return gemm_tc(ctx->stream, L.nI, N, L.nI, 1.f, A, L.ldh, B, ldb, beta, C, ldc, ws + L.off_tc, L.tc_bytes, ctx->ctl);
+    return gemm_tc(ctx->stream, L.nI, N, L.nI, 1.f, A, L.ldh, B, ldb, beta, C, ldc, ws + L.off_tc, L.tc_bytes, ctx->ctl, skip);
 }
 
 cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free)
@@ -463,7 +463,7 @@ cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free)
     return gemm_f64acc(ctx->stream, L.nI, L.nI, L.nI, -1.0, Hp, L.ldp, Hinv, L.ldh, 0.0, nullptr, 0, E, L.ldh, true);
 }
 
-cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes)
+cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes, const int32_t* skip)
 {
     const Layout& L = ctx->L;
     char* ws = (char*)ctx->ws;
@@ -477,11 +477,11 @@ cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, s
         p.M = nI; p.N = L.m; p.K = nI; p.alpha = -1.0; p.beta = 1.0;
         p.A = Hp; p.lda = L.ldp; p.B = V; p.ldb = L.ldm; p.C0 = GI; p.ldc0 = L.ldm; p.C = rV; p.ldc = L.ldm;
         p.diag = Hp; p.diag_stride = L.ldp + 1;
-        e = gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, nullptr);
+        e = gemm_i8(ctx->stream, p, kResidualDigits, sc, ctx->ctl, skip);
     } else
-        e = gemm_f64acc(ctx->stream, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false);
+        e = gemm_f64acc(ctx->stream, nI, L.m, nI, -1.0, Hp, L.ldp, V, L.ldm, 1.0, GI, L.ldm, rV, L.ldm, false, skip);
     if (e != cudaSuccess) return e;
-    return inverse_product(ctx, L.m, (const float*)(ws + L.off_Hinv), rV, L.ldm, 1.f, V, V, L.ldm, 4, other, other_bytes);
+    return inverse_product(ctx, L.m, (const float*)(ws + L.off_Hinv), rV, L.ldm, 1.f, V, V, L.ldm, 4, other, other_bytes, skip);
 }
 
 // Free while the nested phase prepares H^-1 in the place of Hp: the regions behind it, up to the staged vectors, and the

@@ -27,3 +27,21 @@ def test_weights_after_swaps(d1, m, g, k):
     # below 1e-3 here, so their product stays below 4 roundings
     assert (got - ref).norm() <= 4 * 2.0 ** -24 * ref.norm()
     s.close()
+
+
+@pytest.mark.parametrize("d1,m,g,k", [(36, 5, 2, 7), (1152, 130, 9, 70), (2304, 513, 9, 128)])
+def test_weights_of_a_start_that_no_swap_improves(d1, m, g, k):
+    gen = torch.Generator(device="cuda").manual_seed(d1)
+    X = torch.randn(3 * d1, d1, generator=gen, device="cuda") * torch.exp(0.5 * torch.randn(d1 // g, generator=gen, device="cuda")).repeat_interleave(g)
+    W = 0.05 * torch.randn(d1, m, generator=gen, device="cuda")
+    H = X.t() @ X
+    H = 0.5 * (H + H.t())
+    G = H @ W
+    s = pkg.Solver(0)
+    support, obj0 = s.init_support(H, G, W, g, k, b.INIT_ENERGY)
+    V = s.debug_state(1)
+    out = s.local_search(6, accept_rel_tol=1.0)
+    assert out.n_swaps == 0
+    I = (support.long()[:, None] * g + torch.arange(g, device="cuda")).reshape(-1)
+    assert torch.equal(out.W[I], V)                 # as the state build left them: no further pass over them
+    s.close()
