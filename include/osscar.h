@@ -108,7 +108,7 @@ int osscar_set_workspace(osscar_ctx* ctx, void* dev_ptr, size_t bytes);
  *                   three-term bf16 split where those do not fit; fp32-accurate) and the workspace
  *                   contents are overwritten; without one it runs on the fp32 pipes.
  * X: device, n_rows x d1, bf16 (tensor cores, fp32 accumulation) or fp32.  For bf16 the
- * pointer must be 16-byte aligned and d1 a multiple of 8.  fp32 X with a workspace set is split there into four
+ * pointer must be 16-byte aligned and d1 a multiple of 8.  fp32 X with a workspace set is split there into three
  * 8-bit digits (small products or workspaces, and blocks with single entries far above the rest of their column: three bf16
  * terms, row panels of 6 * round_up(d1, 8) bytes per row; workspace contents overwritten) and accumulated on the tensor
  * cores to fp32 accuracy; without a workspace it runs on the fp32 pipes.

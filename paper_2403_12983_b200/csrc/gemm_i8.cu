@@ -247,8 +247,8 @@ struct I8Epi {
 // (EPI_F32 only): the k-range of a tile is dealt to that many CTAs, slice s writes to C + s * slice_stride.
 struct I8Cover { int tri, upper, ksplit; int64_t slice_stride; };
 
-// TNC columns per tile.
-template <int S, int TNC, int EPI>
+// TNC columns per tile; digit products up to order OM.
+template <int S, int TNC, int EPI, int OM = S + 1>
 __global__ void __launch_bounds__(I8_THREADS, 1)
 k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_constant__ I8Epi ep, const I8Cover cov, int num_ids,
          SearchCtl* __restrict__ ctl, const int32_t* __restrict__ done)
@@ -317,7 +317,7 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
             for (int id = blockIdx.x; id < num_ids && ok; id += gridDim.x) {
                 int tm, tn, kb0, kb1;
                 tile_of(id, &tm, &tn, &kb0, &kb1);
-                for (int o = S + 1; o >= 2 && ok; --o)
+                for (int o = OM; o >= 2 && ok; --o)
                     for (int kb = kb0; kb < kb1 && ok; ++kb)
                         for (int i = max(1, o - S); i <= min(S, o - 1); ++i, ++it) {
                             const int s = it % STAGES;
@@ -342,7 +342,7 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
             for (int id = blockIdx.x; id < num_ids && ok; id += gridDim.x) {
                 int tm, tn, kb0, kb1;
                 tile_of(id, &tm, &tn, &kb0, &kb1);
-                for (int o = S + 1; o >= 2 && ok; --o, ++fl) {
+                for (int o = OM; o >= 2 && ok; --o, ++fl) {
                     const int buf = fl & 1;
                     if (!mbar_wait(tempty_bar(buf), ((fl >> 1) & 1) ^ 1, abort_flag, wl)) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -379,7 +379,7 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
             float lo[HALF];               // orders above 3, in units of order 4
 #pragma unroll
             for (int j = 0; j < HALF; ++j) lo[j] = 0.f;
-            for (int o = S + 1; o >= 4 && ok; --o, ++fl) {
+            for (int o = OM; o >= 4 && ok; --o, ++fl) {
                 const int buf = fl & 1;
                 if (!mbar_wait(tfull_bar(buf), (fl >> 1) & 1, abort_flag, wl)) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -537,17 +537,17 @@ I8Panels plan(int64_t M, int64_t N, int64_t K, int S, size_t a_bytes, size_t b_b
     return p;
 }
 
-template <int S, int TNC, int EPI>
+template <int S, int TNC, int EPI, int OM = S + 1>
 cudaError_t launch_mma(cudaStream_t st, const I8Maps& maps, int64_t M, int64_t N, int64_t K, const I8Epi& ep, const I8Cover& cov, int sms,
                        SearchCtl* ctl, const int32_t* done)
 {
-    const cudaError_t e = cudaFuncSetAttribute(k_mma_i8<S, TNC, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, I8_SMEM);
+    const cudaError_t e = cudaFuncSetAttribute(k_mma_i8<S, TNC, EPI, OM>, cudaFuncAttributeMaxDynamicSharedMemorySize, I8_SMEM);
     if (e != cudaSuccess) return e;
     const int64_t TM = (M + I8_TM - 1) / I8_TM, TN = (N + TNC - 1) / TNC;
     int64_t ids = TM * TN;
     if (cov.upper) { ids = 0; for (int64_t r = 0; r < TM; ++r) ids += TN - r / (TNC / I8_TM); }
     ids *= cov.ksplit > 1 ? cov.ksplit : 1;
-    k_mma_i8<S, TNC, EPI><<<(unsigned)(ids < sms ? ids : sms), I8_THREADS, I8_SMEM, st>>>(maps, (int)M, (int)N, (int)K, ep, cov, (int)ids, ctl, done);
+    k_mma_i8<S, TNC, EPI, OM><<<(unsigned)(ids < sms ? ids : sms), I8_THREADS, I8_SMEM, st>>>(maps, (int)M, (int)N, (int)K, ep, cov, (int)ids, ctl, done);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -684,13 +684,13 @@ size_t gemm_i8_operand_bytes(int64_t rows, int64_t K, int S)
     return (size_t)rows * ((size_t)S * round_up(K, 16) + 16) + 4 * (size_t)K + 2048;
 }
 
-// Whether some column of a panel of `rows` rows has its scale above 32 times its root mean square (see gram_i8): skip[0] = 1 and
+// Whether some column of a panel of `rows` rows has its scale above 16 times its root mean square (see gram_i8): skip[0] = 1 and
 // skip[1] = 0 then, the other way round otherwise.  Columns of zeros or with entries that are not finite do not count.
 __global__ void __launch_bounds__(1024) k_i8_outliers(const unsigned long long* __restrict__ cmax, const unsigned long long* __restrict__ spread,
                                                       int64_t rows, int64_t d1, int32_t* __restrict__ skip)
 {
     bool out = false;
-    for (int64_t j = threadIdx.x; j < d1; j += 1024) out |= cmax[j] != 0 && finite_bits(cmax[j]) && spread[j] < ((unsigned long long)rows << 20);
+    for (int64_t j = threadIdx.x; j < d1; j += 1024) out |= cmax[j] != 0 && finite_bits(cmax[j]) && spread[j] < ((unsigned long long)rows << 22);
     const int any = __syncthreads_or(out);
     if (threadIdx.x == 0) { skip[0] = any ? 1 : 0; skip[1] = any ? 0 : 1; }
 }
@@ -709,22 +709,24 @@ __global__ void __launch_bounds__(256) k_i8_add_slices(float* __restrict__ C, in
     }
 }
 
-// H (+)= Xc^T Xc over the upper-triangle tiles for fp32 Xc (n_rows x d1): four digits per entry, ten products at twice the bf16
-// rate.  Both operands are the same transposed digits.  A layer with fewer tiles than SMs splits the rows of a panel over
-// CTAs, whose fp32 partial sums are added in order.
-// Digits are fixed-point below the scale s_j of a column (a power of two, less than twice its largest entry), and the products
-// of order 6 are left out: at most 3 * 2^-32 s_i s_j a row, which repeated values (pixels, padding) add up with one sign.  A
-// column whose scale is at most 32 times its root mean square keeps that below 3 * 2^-22 sqrt(H_ii H_jj), less than the
-// sums of the bf16 terms lose.  A panel with a column beyond it (single large entries) goes through the bf16 terms, whose bits are
-// relative to every entry: both paths are enqueued, one returns at once.  (Three digits without this test left 2e-5 of
-// sqrt(H_ii H_jj), and 1e-3 of an entry, where one entry of a column was 300 times the rest.)
-// One chunk, ms, bf16 terms -> digits: 0.171 -> 0.119 at 4900 x 256, 0.187 -> 0.132 at 4900 x 1024, 0.087 -> 0.091 at 2048 x 1024, 0.051 -> 0.085
-// at 1024 x 1024, 0.80 -> 0.74 at 6272 x 4608, 0.196 -> 0.27 at 1500 x 4608: short chunks, and those whose tiles fill the SMs anyway, stay on the terms.
+// H (+)= Xc^T Xc over the upper-triangle tiles for fp32 Xc (n_rows x d1): three digits per entry, the eight digit products of orders
+// 2 to 5 at twice the bf16 rate.  Both operands are the same transposed digits.  A layer with fewer tiles than SMs splits the
+// rows of a panel over CTAs, whose fp32 partial sums are added in order.
+// Digits are fixed-point below the scale s_j of a column (a power of two, less than 2.1 times its largest entry): an entry is rounded
+// by up to 2^-24 s_j, and values that repeat (pixels, padding) add that up with one sign.  Where the scale is at most 16 times
+// the column's root mean square it stays below 2^-19 sqrt(H_ii H_jj) in the worst case (1e-7 measured on pixels and on
+// rectified Gaussians), less than the truncating sums of the bf16 terms lose.  A panel with a column beyond it (single large
+// entries) goes through the bf16 terms, whose bits are relative to every entry: both paths are enqueued, one returns at once.
+// (Six products without this test left 2e-5 of sqrt(H_ii H_jj), and 1e-3 of an entry, where one entry of a column was 300 times
+// the rest; four digits, ten products, 0.74 ms at 6272 x 4608.)
+// One chunk, ms, bf16 terms -> digits: 0.171 -> 0.108 at 4900 x 256, 0.187 -> 0.117 at 4900 x 1024, 0.087 -> 0.087 at 2048 x 1024, 0.80 -> 0.62
+// at 6272 x 4608, 0.22 -> 0.23 at 4900 x 2048; before the row thresholds 0.034 -> 0.056 at 512 x 1024 and 0.072 -> 0.081 at 1500 x 2304: short
+// chunks stay on the terms.
 // cudaErrorMemoryAllocation where the scratch is too small or the product too small to pay: the caller takes another path.
 cudaError_t gram_i8(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1, float* C, bool accumulate,
                     void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev)
 {
-    constexpr int S = 4;
+    constexpr int S = 3;
     if (n_rows <= 0) return cudaSuccess;
     if (!scratch || ((uintptr_t)scratch & 255) || d1 >= (1 << 28)) return cudaErrorMemoryAllocation;
     if (n_rows < (d1 < 1536 ? 2048 : 4096) || (double)n_rows * (double)d1 * (double)d1 < 268435456.0) return cudaErrorMemoryAllocation;
@@ -796,7 +798,7 @@ cudaError_t gram_i8(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1,
         ep.C = ks > 1 ? part : C; ep.C0 = C; ep.beta = ks == 1 && add ? 1.0 : 0.0;
         ep.vec = ((uintptr_t)ep.C & 15) == 0 && ((uintptr_t)C & 15) == 0 && (d1 % 4) == 0 ? 1 : 0;
         const I8Cover cov = { 0, 1, ks, (int64_t)(up256(sizeof(float) * (size_t)d1 * d1) / sizeof(float)) };
-        e = launch_mma<S, 256, EPI_F32>(st, maps, d1, d1, rows, ep, cov, sms, ctl_dev, skip_digits);
+        e = launch_mma<S, 256, EPI_F32, S + 2>(st, maps, d1, d1, rows, ep, cov, sms, ctl_dev, skip_digits);
         if (e != cudaSuccess) return e;
         if (ks > 1) {
             k_i8_add_slices<<<dim3((unsigned)((d1 + 1023) / 1024), (unsigned)d1), 256, 0, st>>>(C, d1, part, ks, cov.slice_stride, add ? 1 : 0, tn / I8_TM, skip_digits);

@@ -77,7 +77,7 @@ def test_gram_of_columns_with_outliers(rows, d1, kind, height):
     X = torch.cat(X).double()
     H64 = X.t() @ X                                  # no cancellation: nothing is negative
     # bf16 terms: chains of 24 truncating additions per 64 rows and one fp32 addition per drain, at most 24 x 2^-23 in all;
-    # digits: 3 x 2^-22 sqrt(H_ii H_jj) left out
+    # digits: 2^-19 sqrt(H_ii H_jj) at most
     assert float(((H.double() - H64).abs() / H64).max()) < 24 * 2.0 ** -23
     d = H64.diagonal().sqrt()
     assert float(((H.double() - H64).abs() / (d[:, None] * d[None, :])).max()) < 24 * 2.0 ** -23
