@@ -15,11 +15,13 @@
 // d_1 .. d_S (weight 2^(1 - 8 i)).  Digit products of order o = i + j <= S + 1 are kept, S (S + 1) / 2 of them; all
 // products of one order have one weight and accumulate in ONE int32 TMEM chain over the whole of K, exactly:
 // S * K * 2^14 < 2^31 (max_k).  What is dropped is below 2^(-8 S + 5) sqrt(K) of (row maximum x column maximum):
-// S = 6 for the residual of the inverse (its error enters the fp64 inverse of the swap loop), S = 5 elsewhere.
+// S = 6 for the residuals of the inverse and of V and for the Schur panels of wide groups, 5 for R and the Schur products of single
+// rows, 4 for products that have to be as good as fp32 ones (V, G = H W, X0 T, pair scores, the objective), 3 for corrections
+// and, with the products of order 5 as well, for the Gram of fp32 activations.
 //
 // Per output tile (128 x 256) the orders run from the smallest products to the largest; orders above 3 are added up in
 // fp32 registers as they finish (their weight is 2^-16 of the leading one and less), the last two stay in the two TMEM
-// buffers until the epilogue forms the sum in fp64.  Bound: the int8 tensor pipe; per 128-wide k-block of a digit pair a
+// buffers until the epilogue forms the sum in fp64.  Tiles of 128 columns where those of 256 leave SMs idle.  Bound: the int8 tensor pipe; per 128-wide k-block of a digit pair a
 // CTA moves 48 KB from L2 for 512 cycles of MMA, the ratio of the Gram kernel.
 //   warp 0: TMA producer     warp 1: MMA issuer     warps 2-9: TMEM -> registers -> C
 #include "osscar_internal.cuh"
@@ -670,7 +672,6 @@ static cudaError_t gemm_i8_run(cudaStream_t st, const I8Gemm& p, I8Scratch& sc, 
 cudaError_t gemm_i8(cudaStream_t st, const I8Gemm& p, int S, I8Scratch& sc, SearchCtl* ctl, const int32_t* done)
 {
     switch (S) {
-        case 2: return gemm_i8_run<2>(st, p, sc, ctl, done);
         case 3: return gemm_i8_run<3>(st, p, sc, ctl, done);
         case 4: return gemm_i8_run<4>(st, p, sc, ctl, done);
         case 5: return gemm_i8_run<5>(st, p, sc, ctl, done);

@@ -13,12 +13,6 @@
 namespace osscar {
 namespace {
 
-__device__ __forceinline__ void wait_then_release() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-
 using namespace smallmat;
 
 constexpr int kMaxT = 256;          // rows removed per iteration (t_hat * g)
@@ -56,7 +50,7 @@ __global__ void k_copy_pad2(const float* __restrict__ src, int64_t lds, int64_t 
 // gram[grp][a][b] = V[grp*g+a,:] . V[grp*g+b,:]; grid (live groups, g).
 __global__ void k_gr_gram(GPtrs p)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     const int g = p.g;
     const int64_t grp = blockIdx.x;
     const int a = blockIdx.y;
@@ -89,7 +83,7 @@ __global__ void k_gr_gram(GPtrs p)
 // D[grp] = Tr((Hinv_rr)^-1 Gram); one block per live group (dynamic smem 3 g^2 doubles).
 __global__ void k_gr_score(GPtrs p)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     extern __shared__ double smd[];
     __shared__ double red[32];
     const int g = p.g, gg = g * g;
@@ -109,7 +103,7 @@ __global__ void k_gr_score(GPtrs p)
 // refill their holes.  One block.
 __global__ void __launch_bounds__(1024) k_gr_select(GPtrs p, int n_live, int t, int trace_pos)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     __shared__ double sv[32]; __shared__ int sid[32], sidx[32];
     __shared__ int chosen[kMaxT];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -175,7 +169,7 @@ __global__ void __launch_bounds__(1024) k_gr_select(GPtrs p, int n_live, int t, 
 // B[e] = A[row r_e, :] (T rows), C = A[r, r] -> C^-1 (fp64), in one block for the small part.
 __global__ void k_gr_stage_b(GPtrs p, int n_live)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     const int g = p.g, t = p.sel[0], T = t * g;
     const int e = blockIdx.x;
     if (e >= T) return;
@@ -185,7 +179,7 @@ __global__ void k_gr_stage_b(GPtrs p, int n_live)
 }
 __global__ void __launch_bounds__(1024) k_gr_cinv(GPtrs p, int in_smem)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     extern __shared__ double smg[];           // T^2 + 2 T doubles when the matrix fits
     const int g = p.g, t = p.sel[0], T = t * g;
     double* C = in_smem ? smg : p.Cm; double* Lw = in_smem ? smg + T * T : p.Cm + kMaxT * kMaxT; double* Cinv = p.Cm + 2 * kMaxT * kMaxT;
@@ -201,7 +195,7 @@ __global__ void __launch_bounds__(1024) k_gr_cinv(GPtrs p, int in_smem)
 // BC[e][s] = sum_f Cinv[e][f] B[f][s]  and  KT[e][c] = sum_f Cinv[e][f] V[r_f][c];  obj += sum_e KT[e] . V[r_e].
 __global__ void k_gr_stage_bc(GPtrs p, int n_live)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     const int g = p.g, t = p.sel[0], T = t * g;
     const double* Cinv = p.Cm + 2 * kMaxT * kMaxT;
     const int64_t nA = (int64_t)T * p.lda, nV = (int64_t)T * p.ldv;
@@ -226,7 +220,7 @@ __global__ void k_gr_stage_bc(GPtrs p, int n_live)
 }
 __global__ void __launch_bounds__(256) k_gr_obj(GPtrs p, double* partial)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     __shared__ double red[32];
     const int g = p.g, t = p.sel[0], T = t * g;
     double acc = 0.0;
@@ -242,7 +236,7 @@ __global__ void __launch_bounds__(256) k_gr_obj(GPtrs p, double* partial)
 }
 __global__ void k_gr_obj_add(SearchCtl* ctl, const double* partial, int n)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     double s = 0.0;
     for (int i = threadIdx.x; i < n; i += 32) s += partial[i];      // one warp, fixed order
     s = warp_sum(s);
@@ -255,7 +249,7 @@ __global__ void __launch_bounds__(256)
 k_gr_update(float* M, int64_t ld, int64_t ncols4, int64_t nrows, const float* left, int64_t ldl,
             const float* right, int64_t ldr, const int32_t* sel, int g)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     const int T = sel[0] * g;
     const int64_t c4 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c4 >= ncols4) return;
@@ -287,7 +281,7 @@ k_gr_update(float* M, int64_t ld, int64_t ncols4, int64_t nrows, const float* le
 // permutation entries; phase 1 copies the matching columns of A for every remaining live row.
 __global__ void k_gr_compact(GPtrs p, int phase, int64_t n_new_rows /* live groups after the iteration */)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     const int g = p.g, t = p.sel[0];
     for (int i = blockIdx.y; i < t; i += gridDim.y) {
         const int dst = p.sel[1 + i], src = p.sel[1 + kMaxT + i];
@@ -360,20 +354,7 @@ size_t greedy_scratch_bytes(int64_t d1, int64_t m, int g)
 
 // Runs the nested phase down to L.k groups; leaves the slot permutation (kept groups sorted in slots [0, k)) in the
 // workspace and the sorted kept ids in `support`.  The caller then builds the regular search state.
-// Every kernel of an iteration is a programmatic dependent of the one before it: it begins with wait_then_release, and what its
-// predecessor wrote is read with ordinary loads (see search.cu).
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
+// Every kernel of an iteration is a programmatic dependent of the one before it.
 int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_trace, int32_t* n_iters_out)
 {
     const Layout& L = ctx->L;
@@ -427,18 +408,18 @@ int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_t
     while (n_live > L.k) {
         const int t = n_live - L.k < t_hat ? n_live - L.k : t_hat;
         const int64_t nrows = (int64_t)n_live * g;
-        CK(launch_chained(k_gr_gram, dim3((unsigned)n_live, (unsigned)g), dim3(128), 0, st, p));
-        CK(launch_chained(k_gr_score, dim3((unsigned)n_live), dim3(g == 1 ? 32 : 256), smem_score, st, p));
-        CK(launch_chained(k_gr_select, dim3(1), dim3(1024), 0, st, p, n_live, t, trace_pos));
-        CK(launch_chained(k_gr_stage_b, dim3((unsigned)(t * g)), dim3(256), 0, st, p, n_live));
+        CK(launch_pdl_smem(true, k_gr_gram, dim3((unsigned)n_live, (unsigned)g), dim3(128), 0, st, p));
+        CK(launch_pdl_smem(true, k_gr_score, dim3((unsigned)n_live), dim3(g == 1 ? 32 : 256), smem_score, st, p));
+        CK(launch_pdl_smem(true, k_gr_select, dim3(1), dim3(1024), 0, st, p, n_live, t, trace_pos));
+        CK(launch_pdl_smem(true, k_gr_stage_b, dim3((unsigned)(t * g)), dim3(256), 0, st, p, n_live));
         {
             const size_t cs = ((size_t)t * g * t * g + 2 * (size_t)t * g) * sizeof(double);
             const bool fits = cs <= 200 * 1024;          // else in global memory: 160 rows 4.1 -> 1.8 ms with 1024 threads instead of 256
-            CK(launch_chained(k_gr_cinv, dim3(1), dim3(1024), fits ? cs : 0, st, p, fits ? 1 : 0));
+            CK(launch_pdl_smem(true, k_gr_cinv, dim3(1), dim3(1024), fits ? cs : 0, st, p, fits ? 1 : 0));
         }
-        CK(launch_chained(k_gr_stage_bc, dim3((unsigned)(((int64_t)t * g * (p.lda + p.ldv) + 255) / 256 < 2368 ? ((int64_t)t * g * (p.lda + p.ldv) + 255) / 256 : 2368)), dim3(256), 0, st, p, n_live));
-        CK(launch_chained(k_gr_obj, dim3(128), dim3(256), 0, st, p, ctx->partials));
-        CK(launch_chained(k_gr_obj_add, dim3(1), dim3(32), 0, st, ctx->ctl, ctx->partials, 128));
+        CK(launch_pdl_smem(true, k_gr_stage_bc, dim3((unsigned)(((int64_t)t * g * (p.lda + p.ldv) + 255) / 256 < 2368 ? ((int64_t)t * g * (p.lda + p.ldv) + 255) / 256 : 2368)), dim3(256), 0, st, p, n_live));
+        CK(launch_pdl_smem(true, k_gr_obj, dim3(128), dim3(256), 0, st, p, ctx->partials));
+        CK(launch_pdl_smem(true, k_gr_obj_add, dim3(1), dim3(32), 0, st, ctx->ctl, ctx->partials, 128));
         const int64_t Tt = (int64_t)t * g;
         if (Tt >= 32) {
             // wide downdates: A -= BC^T B and V -= B^T KT as products with inner dimension T on the tensor cores
@@ -450,14 +431,14 @@ int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_t
         } else {
             const int64_t nc4 = (round_up(nrows, 4)) / 4;
             dim3 ga((unsigned)((nc4 + 255) / 256), (unsigned)((nrows + UT_ROWS - 1) / UT_ROWS));
-            CK(launch_chained(k_gr_update, ga, dim3(256), 0, st, p.A, p.lda, nc4, nrows, p.BC, p.lda, p.B, p.lda, p.sel, g));
+            CK(launch_pdl_smem(true, k_gr_update, ga, dim3(256), 0, st, p.A, p.lda, nc4, nrows, p.BC, p.lda, p.B, p.lda, p.sel, g));
             const int64_t nv4 = p.ldv / 4;
             dim3 gv((unsigned)((nv4 + 255) / 256), (unsigned)((nrows + UT_ROWS - 1) / UT_ROWS));
-            CK(launch_chained(k_gr_update, gv, dim3(256), 0, st, p.V, p.ldv, nv4, nrows, p.B, p.lda, p.KT, p.ldv, p.sel, g));     // V -= B (C^-1 V_r)
+            CK(launch_pdl_smem(true, k_gr_update, gv, dim3(256), 0, st, p.V, p.ldv, nv4, nrows, p.B, p.lda, p.KT, p.ldv, p.sel, g));     // V -= B (C^-1 V_r)
         }
         const int n_new = n_live - t;
-        CK(launch_chained(k_gr_compact, dim3(64, (unsigned)t), dim3(256), 0, st, p, 0, (int64_t)n_new));
-        CK(launch_chained(k_gr_compact, dim3(64, (unsigned)t), dim3(256), 0, st, p, 1, (int64_t)n_new));
+        CK(launch_pdl_smem(true, k_gr_compact, dim3(64, (unsigned)t), dim3(256), 0, st, p, 0, (int64_t)n_new));
+        CK(launch_pdl_smem(true, k_gr_compact, dim3(64, (unsigned)t), dim3(256), 0, st, p, 1, (int64_t)n_new));
         count_launches(12);
         CK(cudaGetLastError());
         n_live = n_new; trace_pos += t; ++iters;

@@ -22,12 +22,6 @@ constexpr int64_t kTensorRows = 4096;
 constexpr int GJ_T = 256;
 constexpr int UP_M = 64, UP_N = 128;                     // tile of the update
 
-// see search.cu: what the kernel before wrote is read after this, with ordinary loads
-__device__ __forceinline__ void wait_then_release() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 struct PivotSmem {
     double rowj[2][NB];
     double hdiag[NB];
@@ -138,7 +132,7 @@ __global__ void __launch_bounds__(GJ_T)
 k_gj_panels(const float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* Dinv, float* T, float* U, float* Un, int64_t ldu,
             float* next, RankTerms terms)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     __shared__ float sD[NB][NB];
     __shared__ float sA[NB][33];          // A[row, P] transposed: [k][row]
     __shared__ float sU[NB][33];          // A[P, col]: [k][col]
@@ -254,7 +248,7 @@ __global__ void __launch_bounds__(GJ_T)
 k_gj_update(float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* T, const float* U, const float* Un, int64_t ldu,
             const float* Dinv, const float* next, float* Dnext, const float* ref, int64_t ldref, int tiles_n, SearchCtl* ctl)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     extern __shared__ __align__(16) float up_smem[];
     const int t = threadIdx.x;
     if (blockIdx.x == 0) {
@@ -407,7 +401,7 @@ __global__ void __launch_bounds__(GJ_T)
 k_gj_writeback(float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* T, const float* Un, int64_t ldu, const float* Dinv,
                float* Dnext, const float* ref, int64_t ldref, SearchCtl* ctl)
 {
-    wait_then_release();
+    pdl_wait_then_release();
     if (blockIdx.x == 0) {
         if (p0 + NB < n) pivot_block(A, lda, p0 + NB, (int)(n - p0 - NB < NB ? n - p0 - NB : NB), Dnext, ref, ldref, ctl);
         return;
@@ -423,19 +417,6 @@ k_gj_writeback(float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float
             A[(p0 + i) * lda + col] = col >= p0 && col < p0 + nb ? Dinv[i * NB + (col - p0)] : Un[i * ldu + col];
         }
     }
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_dependent(bool dependent, void (*kernel)(KArgs...), unsigned grid, size_t smem, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(GJ_T); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = dependent ? 1 : 0;
-    count_launches(1);
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 #define CK(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return OSSCAR_E_CUDA; } while (0)
@@ -469,10 +450,11 @@ int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const 
         for (int64_t p0 = 0, s = 0; p0 < n; p0 += NB, ++s) {
             const int nb = (int)(n - p0 < NB ? n - p0 : NB);
             const float* D = Dbuf[s & 1];
-            CK(launch_dependent(p0 > 0, k_gj_panels<true>, pgrid, 0, st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, (float*)nullptr, terms));
+            CK(launch_pdl(p0 > 0, k_gj_panels<true>, dim3(pgrid), dim3(GJ_T), st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, (float*)nullptr, terms));
             CK(rank_update_run(st, n, lda, NB, -1.f, terms, A, lda, ctx->ctl));
-            CK(launch_dependent(true, k_gj_writeback, 1 + 4 * 148, 0, st, A, lda, n, p0, nb, (const float*)T, (const float*)Un, lda, D,
-                                Dbuf[(s & 1) ^ 1], ref, ldref, ctx->ctl));
+            CK(launch_pdl(true, k_gj_writeback, dim3(1 + 4 * 148), dim3(GJ_T), st, A, lda, n, p0, nb, (const float*)T, (const float*)Un, lda, D,
+                          Dbuf[(s & 1) ^ 1], ref, ldref, ctx->ctl));
+            count_launches(2);
         }
         CK(cudaGetLastError());
         return OSSCAR_OK;
@@ -486,9 +468,10 @@ int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const 
     for (int64_t p0 = 0, s = 0; p0 < n; p0 += NB, ++s) {
         const int nb = (int)(n - p0 < NB ? n - p0 : NB);
         const float* D = Dbuf[s & 1];
-        CK(launch_dependent(true, k_gj_panels<false>, pgrid, 0, st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, next, RankTerms{}));
-        CK(launch_dependent(true, k_gj_update, ugrid, UP_SMEM, st, A, lda, n, p0, nb, (const float*)T, (const float*)U, (const float*)Un, lda,
+        CK(launch_pdl(true, k_gj_panels<false>, dim3(pgrid), dim3(GJ_T), st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, next, RankTerms{}));
+        CK(launch_pdl_smem(true, k_gj_update, dim3(ugrid), dim3(GJ_T), UP_SMEM, st, A, lda, n, p0, nb, (const float*)T, (const float*)U, (const float*)Un, lda,
                             D, (const float*)next, Dbuf[(s & 1) ^ 1], ref, ldref, tiles_n, ctx->ctl));
+        count_launches(2);
     }
     CK(cudaGetLastError());
     return OSSCAR_OK;

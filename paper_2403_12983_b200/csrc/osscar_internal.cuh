@@ -111,6 +111,39 @@ struct osscar_ctx {
 
 namespace osscar {
 
+// ---- dependent launches.  The kernels of a chain (swap steps, iterations of the nested phase, steps of the inversion) are
+// launched so that the next one may start while the current one is still running.  A kernel of single-row groups first
+// requests the rows it streams (written by kernels that finished long ago), all others begin with the wait; a kernel waits here for
+// the kernel before it to complete before it reads anything that kernel wrote (staged vectors, scalars, the control
+// block), and only then lets its own successor start: a successor's early part can thus overlap only the late part of its
+// immediate predecessor, and its blocks are already resident when the predecessor drains.  Without the launch attribute both
+// instructions do nothing.  What the predecessor wrote is read with ordinary loads only: the read-only (non-coherent)
+// path may still hold a line from the step before, since no kernel boundary separates the two any more.
+static __device__ __forceinline__ void pdl_wait_then_release() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch, with `dependent` set, as a programmatic dependent of the kernel before it on the stream.  Only a launch that directly
+// follows another kernel launch of the chain may be one: behind an event record, a copy or a reduction by the caller's
+// hook the launch is an ordinary, fully ordered one.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pdl_smem(bool dependent, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pdl(bool dependent, void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args)
+{
+    return launch_pdl_smem(dependent, kernel, grid, block, 0, st, args...);
+}
+
 // ---- sgemm.cu: C = alpha * op(A) * B + beta * C on the fp32 pipes ----------------------------
 // A is M x K (lda) or, with transA, stored K x M; B is K x N (ldb) or, with transB, stored N x K.
 // `done` (may be null): device flag; when non-zero the kernel returns without touching C.

@@ -52,19 +52,6 @@ struct Ptrs {
 // layout of the `small` region (doubles, each g*g): indices of the matrices
 enum { S_CINV = 0, S_C1INV, S_Q1, S_Q1C, S_M2, S_GV, S_GX, S_GR, S_C, S_P, S_T1, S_T2, S_T3, S_C1, S_L, S_LI };
 
-// Programmatic dependent launch: the kernels of a swap step are launched so that the next one may start while the
-// current one is still running.  A kernel of single-row groups first requests the rows it streams (written by kernels
-// that finished long ago), the kernels of wider groups begin with the wait; a kernel waits here for the kernel before
-// it to complete before it reads anything that kernel wrote (staged vectors, scalars, the control block), and only then
-// lets its own successor start: a successor's early part can thus overlap only the late part of its immediate
-// predecessor, and its blocks are already resident when the predecessor drains.  Without the launch attribute both
-// instructions do nothing.  What the predecessor wrote is read with ordinary loads only: the read-only (non-coherent)
-// path may still hold a line from the step before, since no kernel boundary separates the two any more.
-__device__ __forceinline__ void pdl_wait_then_release() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // ------------------------------------------------------------------ row norms / group Grams
 // norm[i] = ||M[i, 0:ld)||^2 (pads are zero); one block per row.
 __global__ void k_row_norms(const float* __restrict__ M, int64_t ld, float* __restrict__ norm, const SearchCtl* ctl)
@@ -963,27 +950,6 @@ __global__ void __launch_bounds__(1024) k_pair_select(Ptrs p, int64_t npairs)
         if (bx < 0 || !isfinite(best)) { ctl->done = 1; ctl->stop_reason = OSSCAR_STOP_GUARD; *p.done_host = 1; }
         else { ctl->sel_slot = (int)(bx / npr); ctl->sel_t = (int)(bx % npr); ctl->sel_D = p.D[bx / npr]; }
     }
-}
-
-// Launch, with `dependent` set, as a programmatic dependent of the kernel before it on the stream (see
-// pdl_wait_then_release).  Only a launch that directly follows another kernel launch of the step may be one: behind an
-// event record, a copy or a reduction by the caller's hook the launch is an ordinary, fully ordered one.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_smem(bool dependent, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = dependent ? 1 : 0;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(bool dependent, void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args... args)
-{
-    return launch_pdl_smem(dependent, kernel, grid, block, 0, st, args...);
 }
 
 #include "search_g1.cuh"

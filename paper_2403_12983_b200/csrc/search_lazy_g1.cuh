@@ -282,22 +282,22 @@ __global__ void __launch_bounds__(LZ_T) k_lz_hpass(Ptrs p, LazyPtrs z, int P)
 }
 
 // Sums over the warp of eight values at once: after the call lane 4 i + (0..3) holds the sum of v[i'], i' = lz_row8(lane).
-__device__ __forceinline__ float lz_sum8(const float (&v)[8])
+template <typename T> __device__ __forceinline__ T lz_sum8(const T (&v)[8])
 {
     const int lane = threadIdx.x & 31;
-    float a[4], b[2];
+    T a[4], b[2];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const float keep = lane & 16 ? v[i + 4] : v[i], give = lane & 16 ? v[i] : v[i + 4];
+        const T keep = lane & 16 ? v[i + 4] : v[i], give = lane & 16 ? v[i] : v[i + 4];
         a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        const float keep = lane & 8 ? a[i + 2] : a[i], give = lane & 8 ? a[i] : a[i + 2];
+        const T keep = lane & 8 ? a[i + 2] : a[i], give = lane & 8 ? a[i] : a[i + 2];
         b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
     }
-    const float keep = lane & 4 ? b[1] : b[0], give = lane & 4 ? b[0] : b[1];
-    float s = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+    const T keep = lane & 4 ? b[1] : b[0], give = lane & 4 ? b[0] : b[1];
+    T s = keep + __shfl_xor_sync(0xffffffffu, give, 4);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     return s;
@@ -568,27 +568,6 @@ __global__ void __launch_bounds__(TB) k_lz_y(Ptrs p, LazyPtrs z)
         for (int e = 0; e < NE; ++e) sum = fma(z.scal[LZ_E + e], z.bu[(int64_t)e * p.ldh + s], sum);
         p.y[s] = (float)sum;
     }
-}
-
-__device__ __forceinline__ double lz_sum8(const double (&v)[8])         // as for floats
-{
-    const int lane = threadIdx.x & 31;
-    double a[4], b[2];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const double keep = lane & 16 ? v[i + 4] : v[i], give = lane & 16 ? v[i] : v[i + 4];
-        a[i] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const double keep = lane & 8 ? a[i + 2] : a[i], give = lane & 8 ? a[i] : a[i + 2];
-        b[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
-    }
-    const double keep = lane & 4 ? b[1] : b[0], give = lane & 4 ? b[0] : b[1];
-    double s = keep + __shfl_xor_sync(0xffffffffu, give, 4);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    return s;
 }
 
 // The last step of a round: the NT terms are added to the rows of the inverse, which are written, and y = Hinv' h in the same
