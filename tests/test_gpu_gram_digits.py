@@ -1,18 +1,27 @@
 """Gram and cross term from digits at sizes around their tiles (128 rows, 256 columns, 128-wide k-blocks, 16-byte digit rows),
-with chunks that accumulate, row splits for layers of few tiles, and panels cut by a small workspace."""
+with chunks that accumulate, row splits for layers of few tiles, and panels cut by a small workspace; by the number of launches
+each case is seen to take the path that it names."""
 import pytest
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("rows,d1,m,ws", [
-    ([4900, 4900], 1024, 300, None),         # 20 tiles: rows split over CTAs, second chunk added
-    ([700], 1001, 70, None),                 # nothing divides
-    ([300, 513], 1500, 400, None),           # short chunks
-    ([2000], 1152, 512, 1 << 23),            # panels of about two thousand rows at most
-    ([4096], 2600, 128, None),               # more tiles than SMs would be: no split
+def _panels(rows, n):
+    h = -(-(-(-rows // n)) // 16) * 16 if n > 1 else rows
+    return [min(h, rows - i) for i in range(0, rows, h)]
+
+
+@pytest.mark.parametrize("rows,d1,m,ws,panels,split", [
+    ([4900, 4900], 1024, 300, None, [1, 1], True),         # 20 tiles: rows split over CTAs, second chunk added
+    ([700], 1001, 70, None, [0], False),                   # nothing divides; short chunks stay on the bf16 terms
+    ([300, 513], 1500, 400, None, [0, 0], False),
+    ([2051], 1001, 70, None, [1], True),
+    ([5003], 1152, 512, 1 << 23, [3], False),              # panels of 1680 rows, the last of 1643
+    ([5003, 2048], 1152, 512, 1 << 24, [3, 2], True),      # panels whose rows are split as well
+    ([2500], 1152, 512, 3499776, [0], False),              # no room for a thousand rows
+    ([4096], 2600, 128, None, [1], False),                 # a tile for every SM: no split
 ])
-def test_gram_and_cross_term_fp32(rows, d1, m, ws):
+def test_gram_and_cross_term_fp32(rows, d1, m, ws, panels, split):
     import torch
     import paper_2403_12983_b200 as pkg
     from paper_2403_12983_b200 import binding as b
@@ -29,9 +38,17 @@ def test_gram_and_cross_term_fp32(rows, d1, m, ws):
     G = torch.empty(d1, m, device="cuda")
     Wd = W.cuda()
     const = None
+    before = b.launch_count()
     for i, x in enumerate(X):
-        flags = (b.GRAM_BEGIN if i == 0 else 0) | (b.GRAM_END if i == len(X) - 1 else 0)
-        const = solver.gram_chunk(x.cuda(), H, flags, Wd, G, 0.0)
+        solver.gram_chunk(x.cuda(), H, b.GRAM_BEGIN if i == 0 else 0)
+    terms = solver._ws.numel() - 4096                                    # panels of the bf16 terms, two launches each
+    rows_t = terms // (6 * ((d1 + 7) // 8 * 8))
+    count = lambda n: 2 * -(-n // (n if rows_t >= n else rows_t // 64 * 64))  # noqa: E731
+    launches = b.launch_count() - before
+    # digits: maxima, digits, outliers, product (and its sum), and the terms that a panel with outliers takes instead
+    want = sum(sum((5 if split else 4) + count(h) for h in _panels(r, n)) if n else count(r) for r, n in zip(rows, panels))
+    assert launches == 1 + want
+    const = solver.gram_chunk(torch.empty(0, d1, device="cuda"), H, b.GRAM_END, Wd, G, 0.0)
     solver.close()
     X64 = [x.double() for x in X]
     H64 = sum(x.t() @ x for x in X64)

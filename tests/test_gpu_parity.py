@@ -653,7 +653,7 @@ def test_guard_stop_when_every_candidate_is_dependent(solver, osscar, g, pairs):
     ("c5", dict(n=8192, d1=4200, m=2300, k=2100, chunk_rows=4096), 1, 8),            # one row per pass, two passes per row of V
 ])
 def test_persistent_loop_and_launch_chain_follow_the_oracle(solver, osscar, name, over, seed, max_swaps):
-    """Single-row groups have two drivers: one cooperative kernel with grid-wide barriers, or five launches per step.
+    """Single-row groups have two drivers: one cooperative kernel with grid-wide barriers, or a chain of launches per step.
     Both must follow the strict oracle; where no choice is a near-tie they make the same swaps."""
     b = osscar.binding
     wl = workloads.config(name, seed=seed, **over)
