@@ -449,8 +449,8 @@ def run_ours(args):
         return
 
     pk = peaks()
-    # bf16 activations: one MMA per product; fp32 activations: three digits, six digit products executed per product
-    gram_terms = 1 if wl.x_dtype == torch.bfloat16 else 6
+    # bf16 activations: one MMA per product; fp32 activations: three digits, eight digit products executed per product
+    gram_terms = 1 if wl.x_dtype == torch.bfloat16 else 8
     ms_step = red["max_total_ms"] / K
     search_s = red["max_search_ms"] / 1e3
     value = red["sum_swaps"] / max(search_s, 1e-9)

@@ -9,7 +9,7 @@
 // at d1 = 28672, m = 7168, k = 8602 2.46 GB a step against 3.52 GB.  The rows of V and R are formed in registers in every
 // step, so norms and scores come from the same fp32 values as before (with fewer roundings on the way); y = Hinv h takes the
 // pending terms as 2 LZ_B scalars.  The row and column of the leaving slot are replaced in the base at once, and the pending
-// coefficients of that slot are cleared.  Per swap: 628 -> 502 us there, 107 -> 98 us at d1 = 8192, m = 2048, k = 4096.
+// coefficients of that slot are cleared.  Per swap: 628 -> 490 us there, 107 -> 97 us at d1 = 8192, m = 2048, k = 4096.
 //
 //   decide   one cluster of blocks: i* from the candidates, exact change of obj, accept test, the new vectors and coefficients
 //   hpass    u_l, d_l for every pruned row and the leaving row

@@ -55,8 +55,8 @@ def test_state_matches_fp64_algebra(d1, m, g, k, spread):
     assert np.max(np.abs(Hinv - inv) / (s[:, None] * s[None, :])) <= (2 if g == 1 else 8) * U24
     V64 = inv @ G[I]
     R64 = G[J] - HJI @ V64
-    # V: its own fp32 rounding, and a split-bf16 product (chains of 48 truncating additions) that corrects a first V made
-    # by another one
+    # V: its own fp32 rounding, and a product (four digits, fp64, or split bf16 with chains of 48 truncating additions, the
+    # loosest of the three) that corrects a first V made by another one
     vb = np.abs(inv) @ (np.abs(HII) @ (np.abs(inv) @ np.abs(G[I])))
     assert np.all(np.abs(V - V64) <= 2 * U24 * np.abs(V64) + (48 * U24) ** 2 * vb + 1e-30)
     # R: the error of V carried through H_JI, and its own rounding; given the device's V, only the latter
