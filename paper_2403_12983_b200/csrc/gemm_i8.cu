@@ -21,9 +21,16 @@
 //
 // Per output tile (128 x 256) the orders run from the smallest products to the largest; orders above 3 are added up in
 // fp32 registers as they finish (their weight is 2^-16 of the leading one and less), the last two stay in the two TMEM
-// buffers until the epilogue forms the sum in fp64.  Tiles of 128 columns where those of 256 leave SMs idle.  Bound: the int8 tensor pipe; per 128-wide k-block of a digit pair a
-// CTA moves 48 KB from L2 for 512 cycles of MMA, the ratio of the Gram kernel.
-//   warp 0: TMA producer     warp 1: MMA issuer     warps 2-9: TMEM -> registers -> C
+// buffers until the epilogue forms the sum in fp64.  Tiles of 128 columns where those of 256 leave SMs idle.
+//
+// Two orders o and o - 1 share one pass over the operands, one TMEM buffer each: in step i of a k-block, A_i B_(o-i) of the one order
+// is followed by A_i B_(o-1-i) of the other, whose digit of B is the one the next step has loaded.  A step moves 48 KB from
+// L2 for 1024 cycles of MMA; a pass per order moved them for 512.  MMAs issued back to back reach 4.3 Pop/s here; what the kernel
+// lost against that were the L2 requests of its loads and an epilogue that held both TMEM buffers for 50000 to 75000 cycles per tile,
+// spent on instruction fetches (it was unrolled over the chunks of a row), on conversions to 64 bits, on C0 and on spills.  Now
+// 28000 to 40000.  The objective at d1 = 8192, m = 2048: 1.69 -> 1.53 ms; a layer of d1 = 28672, m = 7168, k = 8602 with its products
+// 197 -> 164 ms under the power cap; G = H W at 5000 x 1283 (240 tiles) 0.30 -> 0.25 ms.
+//   warp 0: TMA producer     warp 1: MMA issuer     warps 4-11: TMEM -> registers -> C
 #include "osscar_internal.cuh"
 #include "tc_common.cuh"
 #include <math.h>
@@ -38,9 +45,10 @@ constexpr int I8_A_BYTES = I8_TM * I8_BK;
 constexpr int I8_RING = 196608;                               // bytes of the operand ring
 constexpr int I8_STG = 32 * 16 * 8;                           // staging block of one accumulate warp: 32 rows x 16 doubles
 constexpr int I8_SMEM = I8_RING + 1024 + 256 + 8 * I8_STG;
-constexpr int I8_THREADS = 320;
+constexpr int I8_THREADS = 384;                               // warps 2 and 3 idle: registers are dealt by groups of four warps
 constexpr int64_t max_k(int S) { return 131071 / S; }         // S products of 2^14 per k in one int32 sum
 constexpr int I8_BAND = 8;
+constexpr int64_t digit_stride(int64_t K) { return K >= 1024 ? (K + 127) / 128 * 128 : (K + 15) / 16 * 16; }      // bytes from row to row of a digit plane
 
 enum { EPI_F32 = 0, EPI_F64 = 1, EPI_DOT = 2 };
 
@@ -55,6 +63,10 @@ __device__ __forceinline__ int scale_exponent(double m) {
     const double f = frexp(m, &e);
     return f > 0.99 ? e + 1 : e;
 }
+// (double)t of a whole number below 2^51 by one addition: conversions to 64 bits run at a quarter of the rate of fp64 additions.
+__device__ __forceinline__ double whole_double(long long t) { return __longlong_as_double(t + 0x4338000000000000ll) - 6755399441055744.0; }
+__device__ __forceinline__ void sts64(uint32_t a, double v) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
+__device__ __forceinline__ double lds64(uint32_t a) { double v; asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory"); return v; }
 __device__ __forceinline__ unsigned long long abs_bits(double x) {      // orders like |x|; NaN above everything
     return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
 }
@@ -312,6 +324,9 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
 
+    // 384 x 168 registers at launch = 128 x 72 + 256 x 216: the accumulate warps hold 128 sums each, which spilled within 168
+    if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (warp == 0) {
         if (lane == 0) {
             uint32_t it = 0;
@@ -319,9 +334,10 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
             for (int id = blockIdx.x; id < num_ids && ok; id += gridDim.x) {
                 int tm, tn, kb0, kb1;
                 tile_of(id, &tm, &tn, &kb0, &kb1);
-                for (int o = OM; o >= 2 && ok; --o)
+                for (int o = OM; o >= 2 && ok; o -= 2) {
+                    const int sum = min(o, S + 1), n = sum - 1;          // step i: digit i of A, digit sum - i of B
                     for (int kb = kb0; kb < kb1 && ok; ++kb)
-                        for (int i = max(1, o - S); i <= min(S, o - 1); ++i, ++it) {
+                        for (int i = 1; i <= n; ++i, ++it) {
                             const int s = it % STAGES;
                             if (!mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1, abort_flag, wl)) { ok = false; break; }
                             mbar_expect_tx(full_bar(s), STAGE);
@@ -329,8 +345,9 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
                             // the planes of an operand are stacked: rows past its end are another plane's and only feed
                             // rows or columns of the tile that are never written
                             tma_load_2d(a_dst, &maps.a, full_bar(s), kb * I8_BK, (i - 1) * M + tm * I8_TM);
-                            tma_load_2d(a_dst + I8_A_BYTES, &maps.b, full_bar(s), kb * I8_BK, (o - i - 1) * N + tn * TNC);
+                            tma_load_2d(a_dst + I8_A_BYTES, &maps.b, full_bar(s), kb * I8_BK, (sum - i - 1) * N + tn * TNC);
                         }
+                }
             }
             if (*abort_flag) {                    // the copies still in flight must land before the CTA exits
                 const uint32_t first = it > STAGES ? it - STAGES : 0;
@@ -344,24 +361,36 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
             for (int id = blockIdx.x; id < num_ids && ok; id += gridDim.x) {
                 int tm, tn, kb0, kb1;
                 tile_of(id, &tm, &tn, &kb0, &kb1);
-                for (int o = OM; o >= 2 && ok; --o, ++fl) {
-                    const int buf = fl & 1;
-                    if (!mbar_wait(tempty_bar(buf), ((fl >> 1) & 1) ^ 1, abort_flag, wl)) { ok = false; break; }
+                for (int o = OM; o >= 2 && ok; o -= 2) {
+                    const int sum = min(o, S + 1), n = sum - 1, pair = o > 2 ? 2 : 1;
+                    for (int b = 0; b < pair && ok; ++b) ok = mbar_wait(tempty_bar((fl + b) & 1), (((fl + b) >> 1) & 1) ^ 1, abort_flag, wl);
+                    if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t d_tmem = tmem_base + (uint32_t)(buf * TNC);
-                    const int np = min(S, o - 1) - max(1, o - S) + 1;
-                    const int steps = (kb1 - kb0) * np;
-                    for (int t = 0; t < steps; ++t, ++it) {
-                        const int s = it % STAGES;
-                        if (!mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, wl)) { ok = false; break; }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t a_src = tiles_base + s * STAGE, b_src = a_src + I8_A_BYTES;
+                    const uint32_t d_hi = tmem_base + (uint32_t)((fl & 1) * TNC), d_lo = tmem_base + (uint32_t)(((fl + 1) & 1) * TNC);
+                    const bool wide = o > S + 1;            // step i belongs to the lower order of the pair
+                    for (int kb = kb0; kb < kb1 && ok; ++kb)
+                        for (int i = 1; i <= n; ++i, ++it) {
+                            const int s = it % STAGES, s1 = (it + 1) % STAGES;
+                            // of the k-block's steps only the first is not waited for by the step before it
+                            if (i == 1 && !mbar_wait(full_bar(s), (it / STAGES) & 1, abort_flag, wl)) { ok = false; break; }
+                            if (i < n && !mbar_wait(full_bar(s1), ((it + 1) / STAGES) & 1, abort_flag, wl)) { ok = false; break; }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint32_t a_src = tiles_base + s * STAGE, b_src = a_src + I8_A_BYTES;
+                            const uint32_t a_next = tiles_base + s1 * STAGE, b_next = a_next + I8_A_BYTES;
+                            const uint32_t go_on = kb > kb0 || i > 1 ? 1u : 0u;
 #pragma unroll
-                        for (int j = 0; j < I8_BK / I8_UK; ++j)
-                            umma_i8(d_tmem, i8_desc(a_src + j * I8_UK), i8_desc(b_src + j * I8_UK), kIdesc, (t | j) ? 1u : 0u);
-                        umma_commit(empty_bar(s));
-                    }
-                    if (ok) umma_commit(tfull_bar(buf));
+                            for (int j = 0; j < I8_BK / I8_UK; ++j)
+                                umma_i8(wide ? d_lo : d_hi, i8_desc(a_src + j * I8_UK), i8_desc(b_src + j * I8_UK), kIdesc, go_on | (j ? 1u : 0u));
+                            if (i < n)
+#pragma unroll
+                                for (int j = 0; j < I8_BK / I8_UK; ++j)
+                                    umma_i8(wide ? d_hi : d_lo, i8_desc((wide ? a_next : a_src) + j * I8_UK), i8_desc((wide ? b_src : b_next) + j * I8_UK),
+                                            kIdesc, go_on | (j ? 1u : 0u));
+                            umma_commit(empty_bar(s));
+                        }
+                    if (ok)
+                        for (int b = 0; b < pair; ++b) umma_commit(tfull_bar((fl + b) & 1));
+                    fl += pair;
                 }
             }
             if (!ok) {            // MMAs already issued keep running: they must finish before TMEM and the tiles are released
@@ -369,15 +398,28 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
                 mbar_drain(drain_bar, 0);
             }
         }
+    }
     } else {
-        const int lg = warp & 3, half = (warp - 2) >> 2;
-        double* stg = reinterpret_cast<double*>(bar_ptr + 256) + (warp - 2) * (32 * 16);
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+        const int lg = warp & 3, half = (warp - 4) >> 2;
         const int rsub = lane >> 2, c4 = (lane & 3) * 4;
+        // staging block: entry (row, j) at row * 16 + (j ^ (row & 15)).  This lane writes row `lane` and reads rows q * 8 + rsub, columns c4 ...
+        const uint32_t stg = bars + 256 + (warp - 4) * I8_STG;
+        const uint32_t st_w = stg + lane * 128 + (lane & 15) * 8;
+        const uint32_t st_r[2] = { stg + rsub * 128 + ((rsub ^ c4) * 8), stg + (rsub + 8) * 128 + (((rsub + 8) ^ c4) * 8) };
         uint32_t fl = 0;
         bool ok = true;
         for (int id = blockIdx.x; id < num_ids && ok; id += gridDim.x) {
             int tm, tn, kb0, kb1;
             const int slice = tile_of(id, &tm, &tn, &kb0, &kb1);
+            const int64_t grow0 = (int64_t)tm * I8_TM + lg * 32;
+            const int64_t gcol0 = (int64_t)tn * TNC + half * HALF;
+            const bool with_c0 = EPI == EPI_DOT || (EPI == EPI_F32 && !ep.identity && ep.beta != 0.0);
+            if (with_c0 && grow0 + lane < M)          // the tile's part of C0 comes to L2 while its products run
+                for (int64_t gc = gcol0; gc < gcol0 + HALF && gc < N; gc += 32) {
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(ep.C0 + (grow0 + lane) * ep.ldc0 + gc));
+                    if (EPI == EPI_DOT && ep.C0sub) asm volatile("prefetch.global.L2 [%0];" ::"l"(ep.C0sub + (grow0 + lane) * ep.ldc0 + gc));
+                }
             float lo[HALF];               // orders above 3, in units of order 4
 #pragma unroll
             for (int j = 0; j < HALF; ++j) lo[j] = 0.f;
@@ -398,22 +440,54 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
                 if (lane == 0) mbar_arrive(tempty_bar(buf));
             }
             if (!ok) break;
+            // whole pieces of C0 are requested a chunk ahead: the two TMEM buffers are held until the last chunk has been read out
+            float4 pre[4], pre_sub[4];
+            auto request = [&](int c) {
+                const int64_t gc = gcol0 + c * 16 + c4;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int64_t gr = grow0 + q * 8 + rsub;
+                    if (with_c0 && ep.vec && gr < M && gcol0 + c * 16 + 16 <= N) {
+                        pre[q] = *reinterpret_cast<const float4*>(ep.C0 + gr * ep.ldc0 + gc);
+                        if (EPI == EPI_DOT && ep.C0sub) pre_sub[q] = *reinterpret_cast<const float4*>(ep.C0sub + gr * ep.ldc0 + gc);
+                    }
+                }
+            };
+            if (EPI != EPI_F64) request(0);
             const int b3 = fl & 1, b2 = b3 ^ 1;       // orders 3 and 2 wait in the two buffers
             if (!mbar_wait(tfull_bar(b3), (fl >> 1) & 1, abort_flag, wl)) break;
             if (!mbar_wait(tfull_bar(b2), ((fl + 1) >> 1) & 1, abort_flag, wl)) break;
             fl += 2;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int64_t grow0 = (int64_t)tm * I8_TM + lg * 32;
-            const int64_t gcol0 = (int64_t)tn * TNC + half * HALF;
             double sa[4], dot[4];
+            bool row_in[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int64_t gr = grow0 + q * 8 + rsub;
-                sa[q] = gr < M ? ep.alpha * ep.sa[gr] : 0.0;
+                row_in[q] = gr < M;
+                sa[q] = row_in[q] ? ep.alpha * ep.sa[gr] : 0.0;
                 dot[q] = 0.0;
             }
+            int sbx[HALF / 32];               // column scales, one column in 32 per lane: powers of two (or NaN), their low word is zero
 #pragma unroll
+            for (int i = 0; i < HALF / 32; ++i) {
+                const int64_t gc = gcol0 + i * 32 + lane;
+                sbx[i] = gc < N ? __double2hiint(ep.sb[gc] * (1.0 / 1073741824.0)) : 0;            // 2^-30: weight of order 4
+            }
+            float* const out = (float*)ep.C + (int64_t)slice * cov.slice_stride + (grow0 + rsub) * ep.ldc + gcol0 + c4;       // EPI_F32
+            const int64_t step8 = 8 * ep.ldc;
+            // A loop that is not unrolled, with the sums moved down by sixteen registers after each chunk: as straight code (60 KB,
+            // run once per tile) it spent its time on instruction fetches, 55000 to 75000 cycles per tile.
+#pragma unroll 1
             for (int c = 0; c < HALF / 16; ++c) {
+                if (c > 0) {
+#pragma unroll
+                    for (int j = 0; j < HALF - 16; ++j) lo[j] = lo[j + 16];
+                    if (!(c & 1)) {
+#pragma unroll
+                        for (int i = 0; i < HALF / 32 - 1; ++i) sbx[i] = sbx[i + 1];
+                    }
+                }
                 uint32_t r3[16], r2[16];
                 const uint32_t ta = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(half * HALF + c * 16);
                 tmem_ld16(ta + b3 * TNC, r3);
@@ -424,60 +498,67 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
                     __syncwarp();
                     if (lane == 0) { mbar_arrive(tempty_bar(b3)); mbar_arrive(tempty_bar(b2)); }
                 }
+                const int64_t gc = gcol0 + c * 16 + c4;
+                if (gcol0 + c * 16 >= N) continue;                    // the same in the whole warp
+                const bool whole = ep.vec && gcol0 + c * 16 + 16 <= N;
                 __syncwarp();
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    // order 2 + order 3 / 256 + ..., an exact integer part and a small fp32 tail
-                    const double v = fma((double)(int)r2[j], 256.0, (double)(int)r3[j]) * 256.0 + (double)lo[c * 16 + j];
-                    stg[lane * 16 + (j ^ (lane & 15))] = v;
-                }
+                for (int j = 0; j < 16; ++j)          // order 2 + order 3 / 256 + ..., an exact integer part and a small fp32 tail
+                    sts64(st_w ^ (j * 8), fma(whole_double((long long)(int)r2[j] * 256 + (int)r3[j]), 256.0, (double)lo[j]));
                 __syncwarp();
-                const int64_t gc = gcol0 + c * 16 + c4;
+                float4 cur[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cur[q] = pre[q];
+                if (EPI == EPI_F32 && c + 1 < HALF / 16) request(c + 1);
                 double sb[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) sb[i] = gc + i < N ? ep.sb[gc + i] * (1.0 / 1073741824.0) : 0.0;      // 2^-30: weight of order 4
+                for (int i = 0; i < 4; ++i) sb[i] = __hiloint2double(__shfl_sync(0xffffffffu, sbx[0], (c & 1) * 16 + c4 + i), 0);
+                const bool diagonal = EPI == EPI_F32 && ep.identity && ep.row0 + grow0 < ep.col0 + gcol0 + c * 16 + 16 && ep.col0 + gcol0 + c * 16 < ep.row0 + grow0 + 32;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const int r = q * 8 + rsub;
-                    const int64_t gr = grow0 + r;
                     double v[4];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) v[i] = stg[r * 16 + ((c4 + i) ^ (r & 15))] * sa[q] * sb[i];
-                    if (gr >= M || gc >= N) continue;
-                    const bool full = ep.vec && gc + 3 < N;
+                    for (int i = 0; i < 4; ++i) v[i] = lds64((st_r[q & 1] + (q >> 1) * 2048) ^ (i * 8)) * (EPI == EPI_DOT ? sb[i] : sa[q] * sb[i]);
+                    const int64_t gr = grow0 + q * 8 + rsub;
                     if (EPI == EPI_DOT) {
-                        const float* h = ep.C0 + gr * ep.ldc0 + gc;
-                        const float* hs = ep.C0sub ? ep.C0sub + gr * ep.ldc0 + gc : nullptr;
-                        if (full) {
-                            float4 x = *reinterpret_cast<const float4*>(h);
-                            if (hs) { const float4 y = *reinterpret_cast<const float4*>(hs); x.x -= y.x; x.y -= y.y; x.z -= y.z; x.w -= y.w; }
+                        if (!row_in[q]) continue;
+                        if (whole) {
+                            float4 x = cur[q];
+                            if (ep.C0sub) { const float4 y = pre_sub[q]; x.x -= y.x; x.y -= y.y; x.z -= y.z; x.w -= y.w; }
                             dot[q] += (v[0] * (double)x.x + v[1] * (double)x.y) + (v[2] * (double)x.z + v[3] * (double)x.w);
                         } else {
-                            for (int i = 0; i < 4; ++i) if (gc + i < N) dot[q] += v[i] * (double)(hs ? h[i] - hs[i] : h[i]);
+                            const float* h = ep.C0 + gr * ep.ldc0 + gc;
+                            const float* hs = ep.C0sub + gr * ep.ldc0 + gc;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) if (gc + i < N) dot[q] += v[i] * (double)(ep.C0sub ? h[i] - hs[i] : h[i]);
                         }
                     } else if (EPI == EPI_F64) {
+                        if (!row_in[q]) continue;
                         double* cp = (double*)ep.C + gr * ep.ldc + gc;
 #pragma unroll
                         for (int i = 0; i < 4; ++i) if (gc + i < N) cp[i] = v[i];
                     } else {
-                        float* cp = (float*)ep.C + (int64_t)slice * cov.slice_stride + gr * ep.ldc + gc;
-                        if (ep.identity) {
+                        if (diagonal) {
 #pragma unroll
                             for (int i = 0; i < 4; ++i) v[i] += ep.row0 + gr == ep.col0 + gc + i ? 1.0 : 0.0;
-                        } else if (ep.beta != 0.0) {
-                            const float* c0 = ep.C0 + gr * ep.ldc0 + gc;
-                            if (full) {
-                                const float4 x = *reinterpret_cast<const float4*>(c0);
+                        }
+                        if (!row_in[q]) continue;
+                        float* cp = out + q * step8 + c * 16;
+                        if (whole) {
+                            if (with_c0) {
+                                const float4 x = cur[q];
                                 v[0] += ep.beta * (double)x.x; v[1] += ep.beta * (double)x.y;
                                 v[2] += ep.beta * (double)x.z; v[3] += ep.beta * (double)x.w;
-                            } else {
-                                for (int i = 0; i < 4; ++i) if (gc + i < N) v[i] += ep.beta * (double)c0[i];
                             }
+                            *reinterpret_cast<float4*>(cp) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+                        } else {
+                            const float* c0 = ep.C0 + gr * ep.ldc0 + gc;
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) if (gc + i < N) cp[i] = (float)(with_c0 ? v[i] + ep.beta * (double)c0[i] : v[i]);
                         }
-                        if (full) *reinterpret_cast<float4*>(cp) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
-                        else for (int i = 0; i < 4; ++i) if (gc + i < N) cp[i] = (float)v[i];
                     }
                 }
+                if (EPI == EPI_DOT && c + 1 < HALF / 16) request(c + 1);       // two matrices: no room for a second set of registers
             }
             if (EPI == EPI_DOT) {                 // partial sum of this tile half for each of the warp's rows
 #pragma unroll
@@ -486,7 +567,7 @@ k_mma_i8(const __grid_constant__ I8Maps maps, int M, int N, int K, const __grid_
                     v += __shfl_xor_sync(0xffffffffu, v, 1);
                     v += __shfl_xor_sync(0xffffffffu, v, 2);
                     const int64_t gr = grow0 + q * 8 + rsub;
-                    if ((lane & 3) == 0 && gr < M) ((double*)ep.C)[gr * ep.ldc + 2 * tn + half] = v;
+                    if ((lane & 3) == 0 && gr < M) ((double*)ep.C)[gr * ep.ldc + 2 * tn + half] = sa[q] * v;
                 }
             }
         }
@@ -515,10 +596,10 @@ inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Panel sizes of one product: `mp` rows of A and `np` columns of B at a time.
 struct I8Panels { int64_t mp, np, ldk; bool ok; };
-I8Panels plan(int64_t M, int64_t N, int64_t K, int S, size_t a_bytes, size_t b_bytes, int tn, int sms = 148)
+I8Panels plan_stride(int64_t M, int64_t N, int64_t K, int S, size_t a_bytes, size_t b_bytes, int tn, int sms, int64_t ldk)
 {
     I8Panels p;
-    p.ldk = round_up(K, 16);
+    p.ldk = ldk;
     const size_t per_a = (size_t)S * p.ldk + sizeof(double), per_b = (size_t)S * p.ldk + sizeof(double) + sizeof(unsigned long long);
     const size_t fix_a = 1024, fix_b = 4 * (size_t)K + 2048;
     int64_t mp = a_bytes > fix_a ? (int64_t)((a_bytes - fix_a) / per_a) : 0;
@@ -537,6 +618,14 @@ I8Panels plan(int64_t M, int64_t N, int64_t K, int S, size_t a_bytes, size_t b_b
     }
     p.ok = p.mp > 0 && p.np > 0 && K > 0 && K <= max_k(S) && M < (1 << 28) && N < (1 << 28);
     return p;
+}
+// Rows of digits start on cache lines where that costs no panel: the 128 bytes of a row in a tile are then one line in L2 instead
+// of two, and requests to L2 are what the loads of large products wait for: two tiles of K = 5000 took 566000 cycles with rows of 5008 bytes,
+// 486000 with 5120.
+I8Panels plan(int64_t M, int64_t N, int64_t K, int S, size_t a_bytes, size_t b_bytes, int tn, int sms = 148)
+{
+    const I8Panels p = plan_stride(M, N, K, S, a_bytes, b_bytes, tn, sms, digit_stride(K));
+    return p.ok && p.mp >= M && p.np >= N ? p : plan_stride(M, N, K, S, a_bytes, b_bytes, tn, sms, round_up(K, 16));
 }
 
 template <int S, int TNC, int EPI, int OM = S + 1>
@@ -682,7 +771,7 @@ cudaError_t gemm_i8(cudaStream_t st, const I8Gemm& p, int S, I8Scratch& sc, Sear
 
 size_t gemm_i8_operand_bytes(int64_t rows, int64_t K, int S)
 {
-    return (size_t)rows * ((size_t)S * round_up(K, 16) + 16) + 4 * (size_t)K + 2048;
+    return (size_t)rows * ((size_t)S * digit_stride(K) + 16) + 4 * (size_t)K + 2048;
 }
 
 // Whether some column of a panel of `rows` rows has its scale above 16 times its root mean square (see gram_i8): skip[0] = 1 and
@@ -781,7 +870,9 @@ cudaError_t gram_i8(cudaStream_t st, const float* X, int64_t n_rows, int64_t d1,
     int8_t* planes = (int8_t*)b;
     const int32_t *skip_digits = &ctl_dev->gram_skip[0], *skip_terms = &ctl_dev->gram_skip[1];
     for (int64_t r0 = 0; r0 < n_rows; r0 += panel) {
-        const int64_t rows = n_rows - r0 < panel ? n_rows - r0 : panel, ldk = round_up(rows, 16);
+        const int64_t rows = n_rows - r0 < panel ? n_rows - r0 : panel;
+        const bool lines = (size_t)S * d1 * digit_stride(rows) <= scratch_bytes - (size_t)((char*)planes - (char*)scratch);       // see plan()
+        const int64_t ldk = lines ? digit_stride(rows) : round_up(rows, 16);
         e = cudaMemsetAsync(ck, 0, (size_t)((char*)sc - (char*)ck), st);           // and the column maxima and sums behind it
         if (e != cudaSuccess) return e;
         k_i8_colmax<float><<<dim3((unsigned)((d1 + 63) / 64), (unsigned)((rows + 255) / 256)), 256, 0, st>>>(X + r0 * d1, nullptr, d1, rows, d1, ck, cmax, nullptr);
