@@ -1008,6 +1008,7 @@ cudaError_t enqueue_scores(osscar_ctx* ctx, const Ptrs& p, bool norms, bool gene
 #include "search_block.cuh"
 #include "search_loop_g1.cuh"
 #include "search_lazy_g1.cuh"
+#include "search_delayed_g1.cuh"
 
 // Blocks of the persistent loop: one per SM (cooperative launch), fewer for layers with few rows: a barrier costs more the
 // more blocks meet at it.  0 when the device cannot launch cooperatively.
@@ -1072,6 +1073,48 @@ cudaError_t score_pass(osscar_ctx* ctx)
     return cudaGetLastError();
 }
 
+// The delayed loop: batches of base columns and swaps, at most two of them ahead of the device, until the search ends; rewrites of the
+// matrices where the terms are full, rebuilds of the state every refresh_every swaps, and a rewrite at the end.
+static int delayed_search(osscar_ctx* ctx, const Ptrs& p, const DlPlan& dl, const osscar_search_params* prm, double tol, int max_swaps,
+                          double* obj_trace, int32_t* swap_trace, cudaEvent_t* ev)
+{
+    cudaStream_t st = ctx->stream;
+    int made = 0, next_refresh = prm->refresh_every > 0 ? prm->refresh_every : INT_MAX;
+    for (;;) {
+        DlArgs a;
+        a.p = p; a.z = dl.z; a.obj_trace = obj_trace; a.swap_trace = swap_trace; a.tol = tol; a.accept_mode = prm->accept_mode;
+        a.max_swaps = next_refresh < max_swaps ? next_refresh : max_swaps;
+        a.rows = dl.rows; a.kb = dl.kb;
+        CK(dl_prepare(ctx, p, dl));
+        const int least = (a.max_swaps - made + dl.kb / 2 - 1) / (dl.kb / 2);        // batches that the swaps take at least
+        volatile int32_t* rep = nullptr;
+        for (int fed = 0;; ++fed) {
+            const int seen = fed < least ? fed - 2 : fed - 1;
+            if (seen >= 0) {
+                CK(cudaEventSynchronize(ev[seen & 1]));
+                rep = ctx->done_flag_host + 4 + 4 * (seen & 1);
+                if (rep[0]) break;
+            }
+            CK(dl_batch(ctx, p, dl, a));
+            k_dl_report<<<1, 1, 0, st>>>(ctx->ctl, ctx->done_flag_dev + 4 + 4 * (fed & 1));
+            count_launches(1);
+            CK(cudaEventRecord(ev[fed & 1], st));
+        }
+        const int stop = rep[0], terms = rep[1], n = rep[2];
+        if (rep[3] != OSSCAR_OK) return OSSCAR_OK;            // reported at the end of the call
+        const bool refresh = stop == 1 && n == next_refresh && n < max_swaps;
+        CK(dl_rewrite(ctx, p, dl, terms, swap_trace + 2 * made, !refresh));
+        made = n;
+        if (refresh) {
+            const int rb = build_state(ctx);
+            if (rb != OSSCAR_OK) return rb;
+            k_count_refresh<<<1, 1, 0, st>>>(ctx->ctl);
+            count_launches(1);
+            next_refresh += prm->refresh_every;
+        } else if (stop == 1) return OSSCAR_OK;
+    }
+}
+
 int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* support_out, float* W_out,
                double* obj_trace, int32_t* swap_trace, osscar_search_result* res)
 {
@@ -1099,17 +1142,14 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     }
     BlockPtrs bp = make_block_ptrs(ctx, bs);
     const bool fast = g == 1 && !pair && !block;  // fused step for single-row groups
-    // one cooperative kernel for the whole loop, unless asked otherwise or the device cannot hold such a grid
-    // AUTO: the cooperative loop for states that stay in L2 (its barriers cost less than five launches per step: 2-8 x
-    // the swaps per second measured on the small layers); the launch chain for states streamed from HBM, where four
-    // resident blocks per SM of one-row kernels keep more loads in flight than the loop's blocks do (measured 0.81
-    // against 0.71 of copy bandwidth on the OPT-30B-shaped FC2 layer)
+    // AUTO: delayed updates (search_delayed_g1.cuh).  Asked for by name, or where that one does not fit: the cooperative loop for
+    // states that stay in L2, the launch chain for states streamed from HBM and for wide results (rows of V and R past 8192 floats: the
+    // chain deals a row to several blocks, the loop to one warp).  Column shards: their own chain.
+    DlPlan dl = {};
+    const bool delayed = fast && !sharded && prm->loop_mode == OSSCAR_LOOP_AUTO && max_swaps > 0 && dl_plan(ctx, &dl);
     const double state_bytes = 8.0 * L.nI * L.ldh + 4.0 * (L.nI + L.nJ) * L.ldm + 4.0 * L.nJ * L.ldh;
-    // Wide results (rows of V and R past 8192 floats) go to the chain as well: it deals a row to several blocks, the loop to one
-    // warp.  Loop against chain, us a swap: 21.5 / 26.5 at d1 = 256, m = 4096, 27.7 / 27.8 at 256, 8192, 40.0 / 28.5 at 256, 16384, 181 / 34.9 at 256, 32768,
-    // 31.2 / 34.3 at 1024, 8192, 53.1 / 42.1 at 1024, 16384.
-    const bool want_persistent = sharded ? false : prm->loop_mode == OSSCAR_LOOP_PERSISTENT ||
-                                 (prm->loop_mode == OSSCAR_LOOP_AUTO && state_bytes <= 96.0e6 && L.ldm <= 8192);
+    const bool small_state = state_bytes <= 96.0e6 && L.ldm <= 8192;
+    const bool want_persistent = !sharded && !delayed && (prm->loop_mode == OSSCAR_LOOP_PERSISTENT || (prm->loop_mode == OSSCAR_LOOP_AUTO && small_state));
     size_t psmem = 0;
     const int pgrid = (fast && want_persistent && L.nJ > 0) ? persistent_grid(L, &psmem) : 0;
     if (prm->loop_mode == OSSCAR_LOOP_PERSISTENT && pgrid == 0) return OSSCAR_E_ARG;
@@ -1118,12 +1158,12 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     // idle during a search and, with the staged rows of the nested phase, larger than they are at every size); column shards
     // keep the step that writes them every time
     LazyPtrs lz = {};
-    const bool lazy = fast && !persistent && !sharded && L.nJ > 0;
+    const bool lazy = fast && !persistent && !delayed && !sharded && L.nJ > 0;
     if (lazy && lazy_layout(L, (char*)ctx->ws + L.off_big, &lz) > L.off_Hp - L.off_big) return OSSCAR_E_WORKSPACE;
     if (block) max_swaps /= bs;                   // from here on: iterations
     const int64_t npairs = (int64_t)L.k * (L.ng - L.k);
     if (sharded && !(g == 1 && !pair && !block)) return OSSCAR_E_ARG;
-    if (max_swaps > 0) CK(enqueue_scores(ctx, p, true, pair));
+    if (max_swaps > 0 && !delayed) CK(enqueue_scores(ctx, p, true, pair));
     if (max_swaps > 0 && sharded && shard_reduce(ctx, p.vnorm, L.d1, OSSCAR_FP32) != OSSCAR_OK) return OSSCAR_E_CUDA;
     const size_t inv_smem = ((size_t)g * g + 2 * (size_t)g) * sizeof(double);      // matrix under inversion + pivot row/column
     if (inv_smem > kFreeDynSmem) {
@@ -1188,7 +1228,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     if (g == 1 && !fast) ctx->hd_valid = false;          // these drivers move the fp32 inverse only
     if (max_swaps > 0 && fast) {
         if (!ctx->hd_valid) { const int rcd = build_hinv64(ctx, false); if (rcd != OSSCAR_OK) return rcd; }
-        CK(bootstrap_g1());
+        if (!delayed) CK(bootstrap_g1());
     }
 
     // Rebuild of the state inside a search.  It overwrites what a finished search still needs (pending terms, the inverse, V, R),
@@ -1342,7 +1382,8 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
             count_launches(1);
         }
     }
-    for (int it = 0; it < (persistent ? 0 : max_swaps) && rc == OSSCAR_OK; ++it) {
+    if (delayed) rc = delayed_search(ctx, p, dl, prm, tol, max_swaps, obj_trace, swap_trace, evb);
+    for (int it = 0; it < (persistent || delayed ? 0 : max_swaps) && rc == OSSCAR_OK; ++it) {
         if (it % batch == 0) {
             const int bi = it / batch;
             if (bi >= 2) {      // stay at most two batches ahead of the device, and stop feeding a finished loop
@@ -1513,7 +1554,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     res->obj_init = ctx->ctl_host->acc[2];
     res->obj_final = ctx->ctl_host->acc[3];
     res->ms_search = ms;
-    res->loop_driver = persistent ? OSSCAR_LOOP_PERSISTENT : OSSCAR_LOOP_LAUNCHES;
+    res->loop_driver = persistent || (delayed && small_state) ? OSSCAR_LOOP_PERSISTENT : OSSCAR_LOOP_LAUNCHES;
     // kernel times of the sampled steps that really swapped (a stopped loop runs empty kernels)
     int used = 0;
     for (int i = 0; i < nprof; ++i) {
