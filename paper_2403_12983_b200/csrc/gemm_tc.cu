@@ -41,12 +41,13 @@ enum { MODE_GEMM3 = 0,      // A fp32 split, K-major; B fp32 split; six term pai
        MODE_GRAM = 1,       // A = B = X (bf16, MN-major); one term; upper-triangle tiles
        MODE_CROSS = 2,      // A = X (MN-major), B = Y bf16; one term; all tiles
        MODE_CROSS3 = 3,     // A = X (MN-major), B = Y fp32 split in three terms
-       MODE_GRAM3 = 4 };    // A = B = X fp32 split in three terms (MN-major); six term pairs; upper-triangle tiles
+       MODE_GRAM3 = 4,      // A = B = X fp32 split in three terms (MN-major); six term pairs; upper-triangle tiles
+       MODE_GEMM3U = 5 };   // as MODE_GEMM3, upper-triangle tiles of a symmetric result
 template <int MODE> struct Traits {
-    static constexpr bool kAMN = MODE != MODE_GEMM3;
-    static constexpr bool kSixPairs = MODE == MODE_GEMM3 || MODE == MODE_GRAM3;
+    static constexpr bool kAMN = MODE != MODE_GEMM3 && MODE != MODE_GEMM3U;
+    static constexpr bool kSixPairs = MODE == MODE_GEMM3 || MODE == MODE_GRAM3 || MODE == MODE_GEMM3U;
     static constexpr int kTerms = kSixPairs ? 6 : (MODE == MODE_CROSS3 ? 3 : 1);
-    static constexpr bool kUpper = MODE == MODE_GRAM || MODE == MODE_GRAM3;
+    static constexpr bool kUpper = MODE == MODE_GRAM || MODE == MODE_GRAM3 || MODE == MODE_GEMM3U;
     // k-blocks per TMEM accumulation chain: short where small terms ride on large ones, 8 (32 MMAs) for plain bf16.  The drain of
     // one buffer (about a thousand cycles) hides behind the MMAs of the other even at one k-block of six pairs, and the
     // truncation bias of the accumulator shrinks with the chain
@@ -615,7 +616,7 @@ size_t gemm_tc_min_scratch(int64_t M, int64_t N)
 
 cudaError_t gemm_tc(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alpha, const float* A, int64_t lda,
                     const float* B, int64_t ldb, float beta, float* C, int64_t ldc,
-                    void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done)
+                    void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done, bool upper)
 {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (K <= 0 || scratch_bytes < gemm_tc_min_scratch(M, N) || ((uintptr_t)scratch & 255)) return cudaErrorInvalidValue;
@@ -639,10 +640,12 @@ cudaError_t gemm_tc(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alph
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_mma_pipe<MODE_GEMM3>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    const auto kernel = upper ? k_mma_pipe<MODE_GEMM3U> : k_mma_pipe<MODE_GEMM3>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
     const int TM = (int)((M + TILE_M - 1) / TILE_M), TN = (int)((N + TILE_N - 1) / TILE_N);
-    const int num_ids = TM * TN;
+    int num_ids = TM * TN;
+    if (upper) { num_ids = 0; for (int tm = 0; tm < TM; ++tm) num_ids += TN - tm / 2; }
     const int vec_ok = (((uintptr_t)C & 15) == 0 && (ldc % 4) == 0 && (N % 4) == 0) ? 1 : 0;
     for (int64_t k0 = 0; k0 < K; k0 += kc) {
         const int64_t kw = K - k0 < kc ? K - k0 : kc;
@@ -656,8 +659,7 @@ cudaError_t gemm_tc(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alph
             if (!encode_2d(enc, &maps.b[i], bp[i], (uint64_t)N, (uint64_t)kw, (uint64_t)ldn, 64, BLOCK_K)) return cudaErrorInvalidValue;
         }
         const int grid = num_ids < sms ? num_ids : sms;
-        k_mma_pipe<MODE_GEMM3><<<grid, NUM_THREADS, SMEM_BYTES, st>>>(maps, M, N, kw, alpha, k0 == 0 ? beta : 1.f, C, ldc, vec_ok,
-                                                                      num_ids, ctl_dev, done);
+        kernel<<<grid, NUM_THREADS, SMEM_BYTES, st>>>(maps, M, N, kw, alpha, k0 == 0 ? beta : 1.f, C, ldc, vec_ok, num_ids, ctl_dev, done);
         count_launches(3);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -680,8 +682,9 @@ __global__ void k_rownorm_sum(const float* __restrict__ part, int64_t rows, int 
 }
 }  // namespace
 
+struct RankTerms { void *u[3], *w[3]; int64_t k8, ldn; };
 // Where the bf16 terms of U (M x K, rows of round_up(K, 8)) and W (K x N, rows of round_up(N, 8)) lie in the scratch.
-bool rank_update_terms(int64_t M, int64_t N, int64_t K, void* scratch, size_t scratch_bytes, RankTerms* t)
+static bool rank_update_terms(int64_t M, int64_t N, int64_t K, void* scratch, size_t scratch_bytes, RankTerms* t)
 {
     if ((uintptr_t)scratch & 255) return false;
     t->k8 = round_up(K, 8); t->ldn = round_up(N, 8);
@@ -696,7 +699,7 @@ bool rank_update_terms(int64_t M, int64_t N, int64_t K, void* scratch, size_t sc
 }
 
 // C += alpha * U * W from terms already in place (K <= 128, N and ldc multiples of 4, C 16-byte aligned); see rank_update_tc.
-cudaError_t rank_update_run(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alpha, const RankTerms& t, float* C, int64_t ldc,
+static cudaError_t rank_update_run(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alpha, const RankTerms& t, float* C, int64_t ldc,
                             SearchCtl* ctl_dev, const int32_t* done, float* row_sq, float* sq_scratch)
 {
     PFN_encodeTiled enc = get_encode();

@@ -386,7 +386,7 @@ int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_t
     k_identity_perm<<<nbg, 256, 0, st>>>(p.perm, slotof, ng);
     k_copy_pad2<<<(unsigned)d1, 256, 0, st>>>(ctx->H, d1, d1, p.A, p.lda);
     count_launches(2);
-    // large layers: rank-64 updates on the tensor cores and one Newton-Schulz step from digits; else the fp32 pipes
+    // large layers: sweeps on the tensor cores and one Newton-Schulz step from digits; else the fp32 pipes
     const bool corrected = dense_inverse_correctable(ctx);
     int rc = invert_spd_inplace(ctx, p.A, p.lda, d1, ctx->H, d1, corrected);
     if (rc != OSSCAR_OK) return rc;

@@ -1,16 +1,16 @@
 // In-place inverse of an SPD matrix by the blocked exchange (Gauss-Jordan) scheme: per 64-wide pivot block P
 //   Dinv = A[P,P]^-1 (fp64),  T = A[:,P] Dinv,  Un = -Dinv A[P,:],  A -= T A[P,:],  A[:,P] = T, A[P,:] = Un, A[P,P] = Dinv.
 //
-// Bound: the chain of n / 64 steps.  Below kTensorRows rows a step is two launches, chained as programmatic dependents: the
+// Bound: the chain of n / 64 steps, about 26 us each.  A step is two launches, chained as programmatic dependents: the
 // panels, and the update of the whole matrix with the write-back in its epilogue, in which block 0 meanwhile inverts the
 // NEXT pivot block (from a copy that the panel kernel made, brought up to date by itself), so that the serial inverse
 // hides behind the update.  Before (pivot inverse, two panel products, two copies, update, write-back: seven launches a
-// step) the build of a state of 2304 rows took 4.0 ms with its correction, now 3.6 ms; 1777 rows 5.9 -> 3.1 ms with the digit
+// step) the build of a state of 2304 rows took 4.0 ms with its correction, then 3.6 ms; 1777 rows 5.9 -> 3.1 ms with the digit
 // products of the correction.
-// Larger matrices are streamed from HBM in every step; their update runs on the tensor cores (k_rank_update) between the
-// panel kernel, which also writes its bf16 terms, and a write-back beside which the next pivot block is inverted.
+// From kWideRows rows up the matrix is swept in blocks of 512 pivots on the tensor cores, and the scheme above inverts the 512 x 512
+// pivot blocks: the matrix is read and written n / 512 times instead of n / 64 times.  4096 rows 4.8 -> 3.1 ms, 8602 rows 42 -> 8.5 ms;
+// blocks of 256 at 2304 rows took as long as the steps of 64 (1.8 ms), which keep everything below.
 #include "osscar_internal.cuh"
-#include <cuda_bf16.h>
 #include <math.h>
 
 namespace osscar {
@@ -18,7 +18,6 @@ namespace {
 
 constexpr int NB = 64;
 constexpr double kPivotRelTol = 1e-7;
-constexpr int64_t kTensorRows = 4096;
 constexpr int GJ_T = 256;
 constexpr int UP_M = 64, UP_N = 128;                     // tile of the update
 
@@ -116,21 +115,11 @@ k_gj_pivot(const float* A, int64_t lda, int64_t p0, int nb, float* Dinv, const f
     pivot_block(A, lda, p0, nb, Dinv, ref, ldref, ctl);
 }
 
-__device__ __forceinline__ void split3(float x, __nv_bfloat16& a, __nv_bfloat16& b, __nv_bfloat16& c) {
-    a = __float2bfloat16_rn(x);
-    x -= __bfloat162float(a);
-    b = __float2bfloat16_rn(x);
-    x -= __bfloat162float(b);
-    c = __float2bfloat16_rn(x);
-}
-
 // Rows [32 b, 32 b + 32) of T = A[:,P] Dinv (zero in the pivot rows) and columns [32 b, 32 b + 32) of U = A[P,:] and
-// Un = -Dinv U; block 0 also copies the next pivot block, before the update changes it.  TERMS: T and U also as the three bf16
-// terms of the tensor-core update, zero beyond nb.
-template <bool TERMS>
+// Un = -Dinv U; block 0 also copies the next pivot block, before the update changes it.
 __global__ void __launch_bounds__(GJ_T)
 k_gj_panels(const float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* Dinv, float* T, float* U, float* Un, int64_t ldu,
-            float* next, RankTerms terms)
+            float* next)
 {
     pdl_wait_then_release();
     __shared__ float sD[NB][NB];
@@ -192,14 +181,6 @@ k_gj_panels(const float* A, int64_t lda, int64_t n, int64_t p0, int nb, const fl
             float4* dst = reinterpret_cast<float4*>(T + row * NB + c0);
             dst[0] = pivot ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(acc[0], acc[1], acc[2], acc[3]);
             dst[1] = pivot ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(acc[4], acc[5], acc[6], acc[7]);
-            if (TERMS) {
-                __align__(16) __nv_bfloat16 w[3][8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) split3(pivot ? 0.f : acc[c], w[0][c], w[1][c], w[2][c]);
-#pragma unroll
-                for (int i = 0; i < 3; ++i)
-                    *reinterpret_cast<uint4*>((__nv_bfloat16*)terms.u[i] + row * NB + c0) = *reinterpret_cast<const uint4*>(w[i]);
-            }
         }
     }
     {   // U and Un: a thread takes one column and 8 rows
@@ -216,18 +197,10 @@ k_gj_panels(const float* A, int64_t lda, int64_t n, int64_t p0, int nb, const fl
         if (i0 + c < n) {
 #pragma unroll
             for (int r = 0; r < 8; ++r)
-            {
                 if (r0 + r < nb) {
-                    if (!TERMS) U[(r0 + r) * ldu + i0 + c] = sU[r0 + r][c];
+                    U[(r0 + r) * ldu + i0 + c] = sU[r0 + r][c];
                     Un[(r0 + r) * ldu + i0 + c] = -acc[r];
                 }
-                if (TERMS) {                     // sU is zero beyond nb
-                    __nv_bfloat16 a, b, d;
-                    split3(sU[r0 + r][c], a, b, d);
-                    const int64_t o = (int64_t)(r0 + r) * terms.ldn + i0 + c;
-                    ((__nv_bfloat16*)terms.w[0])[o] = a; ((__nv_bfloat16*)terms.w[1])[o] = b; ((__nv_bfloat16*)terms.w[2])[o] = d;
-                }
-            }
         }
     }
 }
@@ -395,44 +368,151 @@ k_gj_update(float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* T
     }
 }
 
-// A[:, P] = T (rows outside P), A[P, :] = Un (columns outside P), A[P, P] = Dinv; block 0 inverts the next pivot block, which the
-// panels do not touch.
-__global__ void __launch_bounds__(GJ_T)
-k_gj_writeback(float* A, int64_t lda, int64_t n, int64_t p0, int nb, const float* T, const float* Un, int64_t ldu, const float* Dinv,
-               float* Dnext, const float* ref, int64_t ldref, SearchCtl* ctl)
+// Panel of a wide pivot block [p0, p0 + nb) of the upper triangle A: U (bw x n, rows of ldu) and Ut (n x bw), zero in the pivot rows and
+// beyond nb, and the pivot block itself in D (bw x bw, identity beyond nb).  Tiles of 32 x 32.
+__global__ void __launch_bounds__(256) k_sw_gather(const float* __restrict__ A, int64_t lda, int64_t n, int64_t p0, int nb, int bw, float* __restrict__ U, int64_t ldu,
+                                                   float* __restrict__ Ut, float* __restrict__ D)
 {
-    pdl_wait_then_release();
-    if (blockIdx.x == 0) {
-        if (p0 + NB < n) pivot_block(A, lda, p0 + NB, (int)(n - p0 - NB < NB ? n - p0 - NB : NB), Dnext, ref, ldref, ctl);
-        return;
+    __shared__ float tile[32][33];                   // [column of the panel][k] or the other way round
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t j0 = (int64_t)blockIdx.x * 32;
+    const int k0 = blockIdx.y * 32;
+    for (int i = ty; i < 32; i += 8) {
+        {   // columns left of the block lie transposed above it: read along k
+            const int64_t j = j0 + i;
+            const int k = k0 + tx;
+            if (j < n && j < p0) tile[i][tx] = k < nb ? A[j * lda + p0 + k] : 0.f;
+        }
     }
-    const int64_t total = n * nb;
-    for (int64_t idx = (int64_t)(blockIdx.x - 1) * GJ_T + threadIdx.x; idx < total; idx += (int64_t)(gridDim.x - 1) * GJ_T) {
-        {   // column panel: element (row, p0 + j)
-            const int64_t row = idx / nb; const int j = (int)(idx % nb);
-            if (row < p0 || row >= p0 + nb) A[row * lda + p0 + j] = T[row * NB + j];
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8) {               // the others: read along the columns; a thread writes what it alone reads
+        const int64_t j = j0 + tx;
+        const int k = k0 + i;
+        if (j >= p0) tile[tx][i] = j >= p0 + nb && j < n && k < nb ? A[(p0 + k) * lda + j] : 0.f;
+        if (j >= p0 && j < p0 + bw && k < bw) {
+            const int a = k, b = (int)(j - p0);
+            float v = a == b ? 1.f : 0.f;
+            if (a < nb && b < nb) v = a <= b ? A[(p0 + a) * lda + p0 + b] : A[(p0 + b) * lda + p0 + a];
+            D[(int64_t)a * bw + b] = v;
         }
-        {   // row panel: element (p0 + i, col)
-            const int i = (int)(idx / n); const int64_t col = idx % n;
-            A[(p0 + i) * lda + col] = col >= p0 && col < p0 + nb ? Dinv[i * NB + (col - p0)] : Un[i * ldu + col];
-        }
+    }
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8) {
+        if (j0 + i < n) Ut[(j0 + i) * bw + k0 + tx] = tile[i][tx];
+        if (j0 + tx < ldu) U[(int64_t)(k0 + i) * ldu + j0 + tx] = j0 + tx < n ? tile[tx][i] : 0.f;
+    }
+}
+// D = (D + D^T) / 2 where the two triangles differ by rounding (bw x bw).
+__global__ void __launch_bounds__(256) k_sw_sym(float* D, int bw)
+{
+    const int i = blockIdx.x;
+    for (int j = i + 1 + threadIdx.x; j < bw; j += 256) {
+        const float v = 0.5f * (D[(int64_t)i * bw + j] + D[(int64_t)j * bw + i]);
+        D[(int64_t)i * bw + j] = v; D[(int64_t)j * bw + i] = v;
+    }
+}
+// The swept panel: A[i, P] = T[i] above the block, A[P, j] = T[j]^T right of it, A[P, P] = -Dinv (upper triangle).
+__global__ void __launch_bounds__(256) k_sw_put(float* __restrict__ A, int64_t lda, int64_t n, int64_t p0, int nb, int bw, const float* __restrict__ T, const float* __restrict__ Dinv)
+{
+    __shared__ float tile[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t j0 = (int64_t)blockIdx.x * 32;
+    const int k0 = blockIdx.y * 32;
+    for (int i = ty; i < 32; i += 8) {
+        const int64_t j = j0 + i;
+        const int k = k0 + tx;
+        if (j >= n) continue;
+        tile[i][tx] = T[j * bw + k];
+        if (j < p0 && k < nb) A[j * lda + p0 + k] = tile[i][tx];
+    }
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8) {
+        const int64_t j = j0 + tx;
+        const int k = k0 + i;
+        if (j >= n || k >= nb || j < p0) continue;
+        if (j >= p0 + nb) A[(p0 + k) * lda + j] = tile[tx][i];
+        else if (j - p0 >= k) A[(p0 + k) * lda + j] = -Dinv[(int64_t)k * bw + (j - p0)];
+    }
+}
+// A = -A, the lower triangle as the mirror image of the upper one.
+__global__ void __launch_bounds__(256) k_sw_finish(float* A, int64_t lda, int64_t n)
+{
+    if (blockIdx.x < blockIdx.y) return;
+    __shared__ float tile[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t c = (int64_t)blockIdx.x * 32 + tx, r0 = (int64_t)blockIdx.y * 32;
+    for (int i = ty; i < 32; i += 8) {
+        const int64_t r = r0 + i;
+        if (r < n && c < n && c >= r) { const float v = -A[r * lda + c]; tile[i][tx] = v; A[r * lda + c] = v; }
+    }
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8) {               // row c' = block column + i, column r0 + tx
+        const int64_t r = (int64_t)blockIdx.x * 32 + i, cc = r0 + tx;
+        if (r < n && cc < r) A[r * lda + cc] = tile[tx][i];
     }
 }
 
 #define CK(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return OSSCAR_E_CUDA; } while (0)
 
+constexpr int64_t kWideRows = 3072;
+constexpr int kWide = 512;
+
+// Blocks of 512 pivots as symmetric sweeps of the upper triangle, A_ij -= A_iP A_PP^-1 A_Pj, A_iP := A_iP A_PP^-1, A_PP := -A_PP^-1:
+// the matrix is read and written once per block, on the tensor cores (three bf16 terms, half of the tiles), and the chain of
+// 64-wide pivot blocks runs inside the small A_PP.  The result is -A^-1.  0: not enough memory, 1: done.
+int invert_wide(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref, int* done)
+{
+    const Layout& L = ctx->L;
+    cudaStream_t st = ctx->stream;
+    *done = 0;
+    constexpr int bw = kWide;
+    char* base = (char*)ctx->ws + L.off_tc;
+    size_t off = 65536;                              // in front: what the inversion of the pivot block keeps here
+    auto take = [&](size_t floats) { float* q = (float*)(base + off); off += (floats * sizeof(float) + 1023) / 1024 * 1024; return q; };
+    float* D = take((size_t)bw * bw);
+    float* U = take((size_t)bw * lda);
+    float* Ut = take((size_t)bw * n);
+    float* T = take((size_t)bw * n);
+    if (off + gemm_tc_min_scratch(n, lda) * 4 > L.tc_bytes) return OSSCAR_OK;
+    void* scratch = base + off;
+    const size_t scratch_bytes = L.tc_bytes - off;
+    for (int64_t p0 = 0; p0 < n; p0 += bw) {
+        const int nb = (int)(n - p0 < bw ? n - p0 : bw);
+        const dim3 grid((unsigned)((lda + 31) / 32), (unsigned)(bw / 32));
+        k_sw_gather<<<grid, 256, 0, st>>>(A, lda, n, p0, nb, bw, U, lda, Ut, D);
+        const int rc = invert_spd_inplace(ctx, D, bw, nb, ref + p0 * (ldref + 1), ldref, false);
+        if (rc != OSSCAR_OK) return rc;
+        k_sw_sym<<<(unsigned)nb, 256, 0, st>>>(D, bw);
+        CK(gemm_tc(st, n, bw, bw, 1.f, Ut, bw, D, bw, 0.f, T, bw, scratch, scratch_bytes, ctx->ctl));
+        CK(gemm_tc(st, n, lda, bw, -1.f, T, bw, U, lda, 1.f, A, lda, scratch, scratch_bytes, ctx->ctl, nullptr, true));
+        k_sw_put<<<dim3((unsigned)((n + 31) / 32), (unsigned)(bw / 32)), 256, 0, st>>>(A, lda, n, p0, nb, bw, T, D);
+        count_launches(3);
+        CK(cudaGetLastError());
+    }
+    const unsigned nt = (unsigned)((n + 31) / 32);
+    k_sw_finish<<<dim3(nt, nt), 256, 0, st>>>(A, lda, n);
+    count_launches(1);
+    CK(cudaGetLastError());
+    *done = 1;
+    return OSSCAR_OK;
+}
+
 }  // namespace
 
 // In-place inverse of the n x n SPD matrix A (row stride lda, a multiple of 4; A 16-byte aligned).
 // `ref` (row stride ldref) supplies the original diagonal, the scale of the positive-definiteness test.
-// With `tensor_updates` the rank-64 updates of large matrices run on the tensor cores (three bf16 terms per operand,
-// k_rank_update): their accumulation chains are 64 products long, so the truncating accumulator costs nothing that
-// the correction of the inverse from a residual summed beyond fp32, which the caller then applies, does not remove.
+// With `tensor_updates` large matrices are swept on the tensor cores (three bf16 terms per operand): what their truncating accumulator
+// loses, the correction of the inverse from a residual summed beyond fp32, which the caller then applies, removes.
 int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref,
                        bool tensor_updates)
 {
     const Layout& L = ctx->L;
     cudaStream_t st = ctx->stream;
+    if (tensor_updates && n >= kWideRows) {
+        int done = 0;
+        const int rc = invert_wide(ctx, A, lda, n, ref, ldref, &done);
+        if (rc != OSSCAR_OK || done) return rc;
+    }
     float* T = (float*)((char*)ctx->ws + L.off_panel);
     float* U = T + L.d1 * NB;
     float* Un = U + NB * L.ldp;
@@ -441,24 +521,6 @@ int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const 
     const unsigned pgrid = (unsigned)((n + 31) / 32);
     k_gj_pivot<<<1, GJ_T, 0, st>>>(A, lda, 0, nb0, Dinv, ref, ldref, ctx->ctl);
     count_launches(1);
-    if (tensor_updates && n >= kTensorRows) {
-        // panels (with the bf16 terms of the update), update, write-back with the next pivot block beside it
-        float* Dbuf[2] = { Dinv, U };                  // U itself is not used: its terms are written directly
-        RankTerms terms;
-        if (!rank_update_terms(n, lda, NB, (char*)ctx->ws + L.off_tc, L.tc_bytes, &terms)) return OSSCAR_E_WORKSPACE;
-        for (int i = 0; i < 3; ++i) CK(cudaMemsetAsync(terms.w[i], 0, (size_t)NB * terms.ldn * 2, st));       // the pad columns stay zero
-        for (int64_t p0 = 0, s = 0; p0 < n; p0 += NB, ++s) {
-            const int nb = (int)(n - p0 < NB ? n - p0 : NB);
-            const float* D = Dbuf[s & 1];
-            CK(launch_pdl(p0 > 0, k_gj_panels<true>, dim3(pgrid), dim3(GJ_T), st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, (float*)nullptr, terms));
-            CK(rank_update_run(st, n, lda, NB, -1.f, terms, A, lda, ctx->ctl));
-            CK(launch_pdl(true, k_gj_writeback, dim3(1 + 4 * 148), dim3(GJ_T), st, A, lda, n, p0, nb, (const float*)T, (const float*)Un, lda, D,
-                          Dbuf[(s & 1) ^ 1], ref, ldref, ctx->ctl));
-            count_launches(2);
-        }
-        CK(cudaGetLastError());
-        return OSSCAR_OK;
-    }
     // the tensor-core region is idle here: the copy of the next pivot block and the second inverse live in it
     float* next = (float*)((char*)ctx->ws + L.off_tc);
     float* Dbuf[2] = { Dinv, next + NB * NB };
@@ -468,7 +530,7 @@ int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const 
     for (int64_t p0 = 0, s = 0; p0 < n; p0 += NB, ++s) {
         const int nb = (int)(n - p0 < NB ? n - p0 : NB);
         const float* D = Dbuf[s & 1];
-        CK(launch_pdl(true, k_gj_panels<false>, dim3(pgrid), dim3(GJ_T), st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, next, RankTerms{}));
+        CK(launch_pdl(true, k_gj_panels, dim3(pgrid), dim3(GJ_T), st, (const float*)A, lda, n, p0, nb, D, T, U, Un, lda, next));
         CK(launch_pdl_smem(true, k_gj_update, dim3(ugrid), dim3(GJ_T), UP_SMEM, st, A, lda, n, p0, nb, (const float*)T, (const float*)U, (const float*)Un, lda,
                             D, (const float*)next, Dbuf[(s & 1) ^ 1], ref, ldref, tiles_n, ctx->ctl));
         count_launches(2);

@@ -207,11 +207,13 @@ cudaError_t panel_dot_tc(cudaStream_t st, int64_t M, int64_t N, int64_t K, const
                          void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done = nullptr);
 
 // ---- gemm_tc.cu: the same product on the tensor cores (three-term bf16 split, fp32-accurate); A and B row-major.
-// `scratch` (256-byte aligned device memory, at least gemm_tc_min_scratch bytes) holds the bf16 terms of one K panel.
+// `scratch` (256-byte aligned device memory, at least gemm_tc_min_scratch bytes) holds the bf16 terms of one K panel.  `upper`: only the tiles
+// that reach the diagonal or lie above it.
 size_t gemm_tc_min_scratch(int64_t M, int64_t N);
 cudaError_t gemm_tc(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alpha, const float* A, int64_t lda,
                     const float* B, int64_t ldb, float beta, float* C, int64_t ldc,
-                    void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done = nullptr);
+                    void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done = nullptr,
+                    bool upper = false);
 
 // C += alpha * A * B for a short inner dimension (K <= 128 keeps the terms of A's row band in shared memory across a run
 // of column tiles; larger K goes through gemm_tc).  Same operands and scratch as gemm_tc.  With row_sq (M floats) and
@@ -220,12 +222,6 @@ cudaError_t rank_update_tc(cudaStream_t st, int64_t M, int64_t N, int64_t K, flo
                            const float* B, int64_t ldb, float* C, int64_t ldc,
                            void* scratch, size_t scratch_bytes, SearchCtl* ctl_dev, const int32_t* done = nullptr,
                            float* row_sq = nullptr, float* sq_scratch = nullptr);
-
-// The two halves of rank_update_tc for a caller that writes the bf16 terms itself.
-struct RankTerms { void *u[3], *w[3]; int64_t k8, ldn; };
-bool rank_update_terms(int64_t M, int64_t N, int64_t K, void* scratch, size_t scratch_bytes, RankTerms* t);
-cudaError_t rank_update_run(cudaStream_t st, int64_t M, int64_t N, int64_t K, float alpha, const RankTerms& t, float* C, int64_t ldc,
-                            SearchCtl* ctl_dev, const int32_t* done = nullptr, float* row_sq = nullptr, float* sq_scratch = nullptr);
 
 // H (+)= Xc^T Xc (upper-triangle tiles; Y null) or G (+)= Xc^T Yc with the drained-accumulator pipeline of gemm_tc.cu.
 cudaError_t gram_tc2(cudaStream_t st, const void* X, int64_t n_rows, int64_t d1, const void* Y, int y_fp32, int64_t m,
