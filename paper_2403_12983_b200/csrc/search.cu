@@ -274,30 +274,24 @@ k_small(Ptrs p, int accept_mode, double accept_tol, int max_swaps, double* __res
     __syncthreads();
     const double pivC = spd_inverse(Ms, Lws, Cinv, g);
     const double Ds = mat_trace_prod(Cinv, GV, g, red);               // Tr(C^-1 V_r V_r^T)
-    // R1 R1^T = GR + P (Cinv GX) + (P Cinv GX)^T + P Cinv GV Cinv P^T
-    mat_mul(Cinv, false, GX, false, T1, g);                           // K R_q^T
-    mat_mul(P, false, T1, false, T2, g);                              // P K R_q^T
+    // R1 R1^T = GR + P Cinv GX + (P Cinv GX)^T + P Cinv GV Cinv P^T.  Cinv and c1inv are symmetric: Q1 = Cinv P^T and M2 = c1inv P Cinv
+    // are transposes of products at hand (six products instead of nine; those with the left factor P Cinv go in one pass over the tiles).
     mat_mul(P, false, Cinv, false, T1, g);                            // P Cinv
-    mat_mul(T1, false, GV, false, T3, g);                             // P Cinv GV
+    mat_mul_jobs<3>({{T1, GX, false, T2}, {T1, GV, false, T3}, {T1, P, true, M2}}, g);       // P Cinv GX, P Cinv GV, P Cinv P^T
     mat_mul(T3, false, T1, true, Lw, g);                              // P Cinv GV Cinv P^T  (Lw reused as scratch)
     for (int idx = threadIdx.x; idx < gg; idx += blockDim.x) {
         const int i = idx / g, j = idx % g;
-        T3[idx] = GR[idx] + T2[idx] + T2[j * g + i] + Lw[idx];
-    }
-    __syncthreads();
-    mat_mul(T1, false, P, true, T2, g);                               // P Cinv P^T
-    for (int idx = threadIdx.x; idx < gg; idx += blockDim.x) {
-        const int i = idx / g, j = idx % g;
         const double cq = 0.5 * (p.c[tq * gg + idx] + p.c[tq * gg + j * g + i]);
-        Ms[idx] = cq + 0.5 * (T2[idx] + T2[j * g + i]);
+        Ms[idx] = cq + 0.5 * (M2[idx] + M2[j * g + i]);
+        T3[idx] = GR[idx] + T2[idx] + T2[j * g + i] + Lw[idx];
+        Q1[idx] = T1[j * g + i];
     }
     __syncthreads();
     const double pivc1 = spd_inverse(Ms, Lws, c1inv, g);
     const double gain = mat_trace_prod(c1inv, T3, g, red);
     const double delta = Ds - gain;
-    mat_mul(Cinv, false, P, true, Q1, g);                             // Q1 = Cinv y_r = Cinv P^T
     mat_mul(Q1, false, c1inv, false, Q1c, g);                         // Q1 c1inv
-    mat_mul(c1inv, false, T1, false, M2, g);                          // c1inv P Cinv
+    for (int idx = threadIdx.x; idx < gg; idx += blockDim.x) M2[idx] = Q1c[(idx % g) * g + idx / g];      // c1inv P Cinv
     if (threadIdx.x == 0) {
         const double obj = ctl->obj;
         bool stop = false; int reason = 0;
@@ -316,47 +310,75 @@ k_small(Ptrs p, int accept_mode, double accept_tol, int max_swaps, double* __res
     }
 }
 
-// Staged vectors of the step.  Part A (threads over kept rows s): b, bC = b C^-1, u2, u2c = u2 c1^-1.
-// Part B (threads over columns): K = C^-1 V_r, Vq = c1^-1 R_q + (c1^-1 P C^-1) V_r.
+// Staged vectors of the step, as products with the g x g matrices of the pair on the fp64 tensor path (mma m8n8k4), a warp per 8 x 8
+// entries: first [n_I x g] b, bC = b C^-1, u2 = y - b C^-1 y_r, u2c = u2 c1^-1 (zero on the leaving rows), then [g x ldm]
+// K = C^-1 V_r, Vq = c1^-1 R_q + (c1^-1 P C^-1) V_r.  With a thread per entry, each reading its row and column of the matrices
+// for itself, behind k_small 42 us for 32 heads of 80 rows, now 8.
 __global__ void __launch_bounds__(256) k_prep(Ptrs p)
 {
     pdl_wait_then_release();
     if (p.ctl->done) return;
-    const int g = p.g, gg = g * g;
+    const int g = p.g, gg = g * g, et = (g + 7) >> 3;
     const double* S = p.small;
     const double *Cinv = S + S_CINV * gg, *c1inv = S + S_C1INV * gg, *Q1 = S + S_Q1 * gg, *Q1c = S + S_Q1C * gg, *M2 = S + S_M2 * gg;
-    const int64_t r0 = (int64_t)p.ctl->sel_slot * g;
-    const int64_t q0 = (int64_t)p.ctl->sel_t * g;
-    const int64_t nA = p.nI * g, nB = p.ldm * g;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < nA + nB; idx += (int64_t)gridDim.x * blockDim.x) {
-        if (idx < nA) {
-            const int e = (int)(idx / p.nI); const int64_t s = idx % p.nI;
-            double bc = 0.0, bq = 0.0, bqc = 0.0, yc = 0.0;
-            for (int f = 0; f < g; ++f) {
-                const double bf = (double)p.Hinv[(r0 + f) * p.ldh + s];
-                bc += bf * Cinv[f * g + e];
-                bq += bf * Q1[f * g + e];
-                bqc += bf * Q1c[f * g + e];
-                yc += (double)p.y[(int64_t)f * p.ldh + s] * c1inv[f * g + e];
-            }
-            const bool in_r = s >= r0 && s < r0 + g;
-            p.b[(int64_t)e * p.ldh + s] = p.Hinv[(r0 + e) * p.ldh + s];
-            p.bC[(int64_t)e * p.ldh + s] = (float)bc;
-            p.u2[(int64_t)e * p.ldh + s] = in_r ? 0.f : (float)((double)p.y[(int64_t)e * p.ldh + s] - bq);
-            p.u2c[(int64_t)e * p.ldh + s] = in_r ? 0.f : (float)(yc - bqc);
-        } else {
-            const int64_t j = idx - nA;
-            const int e = (int)(j / p.ldm); const int64_t c = j % p.ldm;
-            double kk = 0.0, vq = 0.0;
-            for (int f = 0; f < g; ++f) {
-                const double vr = (double)p.V[(r0 + f) * p.ldm + c];
-                const double rq = (double)p.R[(q0 + f) * p.ldm + c];
-                kk += Cinv[e * g + f] * vr;
-                vq += c1inv[e * g + f] * rq + M2[e * g + f] * vr;
-            }
-            p.K[(int64_t)e * p.ldm + c] = (float)kk;
-            p.Vq[(int64_t)e * p.ldm + c] = (float)vq;
+    const int64_t r0 = (int64_t)p.ctl->sel_slot * g, q0 = (int64_t)p.ctl->sel_t * g;
+    const int lane = threadIdx.x & 31, fr = lane >> 2, fk = lane & 3;
+    int64_t id = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int64_t nA = (p.nI + 7) / 8 * et;
+    auto mma = [](double (&d)[2], double a, double b) {
+        asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
+    };
+    if (id < nA) {
+        const int e0 = (int)(id % et) * 8;
+        const int64_t s0 = id / et * 8, s = s0 + fr;
+        const bool row = s < p.nI, col = e0 + fr < g;
+        double bc[2] = {0.0, 0.0}, bq[2] = {0.0, 0.0}, bqc[2] = {0.0, 0.0}, yc[2] = {0.0, 0.0};
+#pragma unroll 4
+        for (int k0 = 0; k0 < g; k0 += 4) {
+            const int f = k0 + fk;
+            const bool on = f < g;
+            const double a = on && row ? (double)p.Hinv[(r0 + f) * p.ldh + s] : 0.0, y = on && row ? (double)p.y[(int64_t)f * p.ldh + s] : 0.0;
+            const int o = f * g + e0 + fr;
+            const bool in = on && col;
+            mma(bc, a, in ? Cinv[o] : 0.0);
+            mma(bq, a, in ? Q1[o] : 0.0);
+            mma(bqc, a, in ? Q1c[o] : 0.0);
+            mma(yc, y, in ? c1inv[o] : 0.0);
         }
+        if (!row) return;
+        const bool in_r = s >= r0 && s < r0 + g;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int e = e0 + 2 * fk + i;
+            if (e >= g) continue;
+            const int64_t o = (int64_t)e * p.ldh + s;
+            p.b[o] = p.Hinv[(r0 + e) * p.ldh + s];
+            p.bC[o] = (float)bc[i];
+            p.u2[o] = in_r ? 0.f : (float)((double)p.y[o] - bq[i]);
+            p.u2c[o] = in_r ? 0.f : (float)(yc[i] - bqc[i]);
+        }
+    } else {
+        id -= nA;
+        const int e0 = (int)(id % et) * 8;
+        const int64_t c0 = id / et * 8;
+        if (c0 >= p.ldm) return;
+        const bool row = e0 + fr < g;
+        double kk[2] = {0.0, 0.0}, vq[2] = {0.0, 0.0};
+#pragma unroll 4
+        for (int k0 = 0; k0 < g; k0 += 4) {
+            const int f = k0 + fk;
+            const bool on = f < g, in = on && row;
+            const double vr = on ? (double)p.V[(r0 + f) * p.ldm + c0 + fr] : 0.0, rq = on ? (double)p.R[(q0 + f) * p.ldm + c0 + fr] : 0.0;
+            const int o = (e0 + fr) * g + f;
+            mma(kk, in ? Cinv[o] : 0.0, vr);
+            mma(vq, in ? c1inv[o] : 0.0, rq);
+            mma(vq, in ? M2[o] : 0.0, vr);
+        }
+        if (!row) return;
+        float* K = p.K + (int64_t)(e0 + fr) * p.ldm + c0 + 2 * fk;
+        float* Q = p.Vq + (int64_t)(e0 + fr) * p.ldm + c0 + 2 * fk;
+        K[0] = (float)kk[0]; K[1] = (float)kk[1];
+        Q[0] = (float)vq[0]; Q[1] = (float)vq[1];
     }
 }
 
@@ -881,7 +903,7 @@ k_pair_delta(Ptrs p, const float* __restrict__ Pm, int64_t ldpm, const float* __
     double* Ms = smd; double* Lws = smd + gg;
     const int64_t npr = p.ng - p.k;
     double* S = p.pairScratch + (int64_t)blockIdx.x * kPairTemps * gg;
-    double *P = S, *GX = S + gg, *T1 = S + 2 * gg, *RR = S + 4 * gg, *TMP = S + 5 * gg, *OUT = S + 7 * gg;
+    double *P = S, *GX = S + gg, *T1 = S + 2 * gg, *TG = S + 3 * gg, *RR = S + 4 * gg, *TMP = S + 5 * gg, *OUT = S + 7 * gg;
     for (int64_t pair = blockIdx.x; pair < npairs; pair += gridDim.x) {
         const int64_t s = pair / npr, t = pair % npr;
         const double Ds = p.D[s], At = p.A[t];
@@ -897,19 +919,12 @@ k_pair_delta(Ptrs p, const float* __restrict__ Pm, int64_t ldpm, const float* __
             GX[idx] = (double)XG[(s * g + a) * ldxg + t * g + b];
         }
         __syncthreads();
-        mat_mul(P, false, Cinv, false, T1, g);                   // P C^-1
-        mat_mul(T1, false, P, true, TMP, g);                     // P C^-1 P^T
+        mat_mul_jobs<2>({{P, Cinv, false, T1}, {P, KK, false, OUT}}, g);                                  // P C^-1, P KK
+        mat_mul_jobs<3>({{T1, P, true, TMP}, {T1, GX, false, TG}, {OUT, P, true, RR}}, g);               // P C^-1 P^T, P C^-1 V_s R_t^T, P KK P^T
         for (int idx = threadIdx.x; idx < gg; idx += blockDim.x) {
             const int i = idx / g, j = idx % g;
             Ms[idx] = 0.5 * (p.c[t * gg + idx] + p.c[t * gg + j * g + i]) + 0.5 * (TMP[idx] + TMP[j * g + i]);
-        }
-        __syncthreads();
-        mat_mul(T1, false, GX, false, TMP, g);                   // P C^-1 V_s R_t^T
-        mat_mul(P, false, KK, false, OUT, g);                    // P KK
-        mat_mul(OUT, false, P, true, RR, g);                     // P KK P^T
-        for (int idx = threadIdx.x; idx < gg; idx += blockDim.x) {
-            const int i = idx / g, j = idx % g;
-            RR[idx] += p.gramR[t * gg + idx] + TMP[idx] + TMP[j * g + i];
+            RR[idx] += p.gramR[t * gg + idx] + TG[idx] + TG[j * g + i];
         }
         __syncthreads();
         const double piv = spd_inverse(Ms, Lws, OUT, g);
@@ -1287,7 +1302,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
         for (int R = 4; R > 1; R >>= 1) if ((int64_t)tile_blocks(rows, R) * gtiles >= 296) return R;
         return 1;
     };
-    const unsigned prep_blocks = (unsigned)(((L.nI + L.ldm) * g + 255) / 256);
+    const unsigned prep_blocks = (unsigned)((((L.nI + 7) / 8 + L.ldm / 8) * ((g + 7) / 8) + 7) / 8);      // a warp per 8 x 8 entries
     // threads per block of the three streaming kernels of the single-row step, by the length of the rows they stream
     const unsigned t_l1 = (unsigned)g1_threads(L.ldm > L.ldh ? L.ldm / 4 : L.ldh / 4), t_l2 = (unsigned)g1_threads(L.ldm / 4),
                    t_l4 = (unsigned)g1_threads(L.ldh / 2);

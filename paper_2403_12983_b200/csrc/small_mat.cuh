@@ -150,28 +150,44 @@ static __device__ double spd_inverse(double* M, double* Lw, double* Out, int g)
 // 8 x 8 tiles of C in turn and runs g / 4 steps of mma.m8n8k4 (A fragment: row lane / 4, column lane % 4; B fragment:
 // row lane % 4, column lane / 4; C fragment: row lane / 4, columns 2 (lane % 4) and + 1).  Entries beyond g read as 0.
 // C must not overlap A or B.  blockDim.x must be a multiple of 32.
+static __device__ __forceinline__ void mat_tile(const double* A, bool tA, const double* B, bool tB, double* C, int g, int tile)
+{
+    const int lane = threadIdx.x & 31, nt = (g + 7) >> 3;
+    const int r4 = lane >> 2, c4 = lane & 3;
+    const int i0 = (tile / nt) * 8, j0 = (tile % nt) * 8;
+    const int ai = i0 + r4, bj = j0 + r4;
+    double d0 = 0.0, d1 = 0.0;
+#pragma unroll 4
+    for (int k0 = 0; k0 < g; k0 += 4) {
+        const int kk = k0 + c4;
+        const bool ka = kk < g;
+        const double a = (ka && ai < g) ? (tA ? A[kk * g + ai] : A[ai * g + kk]) : 0.0;
+        const double b = (ka && bj < g) ? (tB ? B[bj * g + kk] : B[kk * g + bj]) : 0.0;
+        asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+                     : "+d"(d0), "+d"(d1) : "d"(a), "d"(b));
+    }
+    const int ci = i0 + r4, cj = j0 + 2 * c4;
+    if (ci < g) {
+        if (cj < g) C[ci * g + cj] = d0;
+        if (cj + 1 < g) C[ci * g + cj + 1] = d1;
+    }
+}
 static __device__ void mat_mul(const double* A, bool tA, const double* B, bool tB, double* C, int g)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int nt = (g + 7) >> 3;
-    const int r4 = lane >> 2, c4 = lane & 3;
-    for (int tile = warp; tile < nt * nt; tile += nwarps) {
-        const int i0 = (tile / nt) * 8, j0 = (tile % nt) * 8;
-        const int ai = i0 + r4, bj = j0 + r4;
-        double d0 = 0.0, d1 = 0.0;
-        for (int k0 = 0; k0 < g; k0 += 4) {
-            const int kk = k0 + c4;
-            const bool ka = kk < g;
-            const double a = (ka && ai < g) ? (tA ? A[kk * g + ai] : A[ai * g + kk]) : 0.0;
-            const double b = (ka && bj < g) ? (tB ? B[bj * g + kk] : B[kk * g + bj]) : 0.0;
-            asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-                         : "+d"(d0), "+d"(d1) : "d"(a), "d"(b));
-        }
-        const int ci = i0 + r4, cj = j0 + 2 * c4;
-        if (ci < g) {
-            if (cj < g) C[ci * g + cj] = d0;
-            if (cj + 1 < g) C[ci * g + cj + 1] = d1;
-        }
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, nt = (g + 7) >> 3;
+    for (int tile = warp; tile < nt * nt; tile += nwarps) mat_tile(A, tA, B, tB, C, g, tile);
+    __syncthreads();
+}
+// Several products at once, their tiles dealt to the warps together (a product of 80 x 80 has 100 tiles for 32 warps).
+struct MatJob { const double *A, *B; bool tB; double* C; };
+template <int N> static __device__ void mat_mul_jobs(const MatJob (&jobs)[N], int g)
+{
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, nt = (g + 7) >> 3, n = nt * nt;
+    for (int tile = warp; tile < N * n; tile += nwarps) {
+        MatJob j = jobs[0];
+#pragma unroll
+        for (int i = 1; i < N; ++i) if (tile >= i * n) j = jobs[i];
+        mat_tile(j.A, false, j.B, j.tB, j.C, g, tile % n);
     }
     __syncthreads();
 }
