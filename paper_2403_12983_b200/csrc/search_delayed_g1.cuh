@@ -200,29 +200,35 @@ __device__ __forceinline__ void dl_dmma(double& d0, double& d1, double a, double
     asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d0), "+d"(d1) : "d"(a), "d"(b));
 }
 
+__device__ __forceinline__ void dl_cp16(void* dst, const void* src, int bytes) {          // bytes of the 16 that exist; the rest is zero
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes) : "memory");
+}
+
 // out[z][c][row] = sum over slice z of k of A[row][k] B[k][c], c < BN, sums in fp64.  Block: 128 rows, 16 k a step, 8 warps of
-// 32 x 32 (BN = 64) or 16 x 32 (BN = 32); the global loads of the next step are in flight while the current one is multiplied.
-// A: rows [0, split) of A0, the others of A1 (all row starts 16-byte aligned, rows padded to whole pieces with zeros).
-// At d1 = 28672, m = 7168, k = 8602 the three products of a batch are 53 GFLOP.
+// 32 x 32 (BN = 64) or 16 x 32 (BN = 32); operands as they are through a ring of DL_PS steps of asynchronous copies, A converted when
+// its fragments are read.  A: rows [0, split) of A0, the others of A1 (row starts 16-byte aligned, whole pieces inside the matrix).
+// At d1 = 28672, m = 7168, k = 8602 the three products of a batch are 53 GFLOP; with one step of registers ahead and the operands
+// converted on their way into shared memory they took 3.7 ms, and 512 swaps 13 ms more of a solve (376 -> 362 ms; 31.8 -> 30.1 ms at 8192, 2048,
+// 7.20 -> 6.98 ms at 5000, 1283).
+constexpr int DL_PS = 4;
+template <typename TA, int BN> constexpr int dl_panel_smem() { return DL_PS * (128 * 20 * (int)sizeof(TA) + 16 * (BN + 4) * 8); }
 template <typename TA, int BN>
 __global__ void __launch_bounds__(256, 2)
 k_dl_panel(int64_t M, int64_t K, const TA* A0, const TA* A1, int64_t split, int64_t lda, const double* B, double* out, int slices, const SearchCtl* ctl)
 {
     if (ctl->done || ctl->dl_stop) return;
     constexpr int BM = 128, BK = 16, AS = BK + 4, BS = BN + 4, WN = BN / 32, WM = 8 / WN, TI = BM / WM / 8;
-    constexpr int AV = sizeof(TA) == 4 ? 2 : 4;                       // 16-byte pieces of the A tile per thread
-    extern __shared__ double dl_smem[];
-    double* As[2] = { dl_smem, dl_smem + BM * AS };
-    double* Bs[2] = { dl_smem + 2 * BM * AS, dl_smem + 2 * BM * AS + BK * BS };
+    constexpr int PE = 16 / (int)sizeof(TA), PR = BK / PE, AV = BM * PR / 256, BV = BK * BN / 2 / 256;      // elements of a piece, pieces of a row, per thread
+    extern __shared__ __align__(16) double dl_smem[];
+    TA* const As = reinterpret_cast<TA*>(dl_smem);
+    double* const Bs = reinterpret_cast<double*>(As + DL_PS * BM * AS);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wm = warp / WN, wn = warp % WN;
     const int64_t m0 = (int64_t)blockIdx.x * BM;
     const int64_t steps = (K + BK - 1) / BK, kb = steps * blockIdx.y / slices, ke = steps * (blockIdx.y + 1) / slices;
-    constexpr int PR = sizeof(TA) == 4 ? 4 : 8;                       // pieces per row and step
-    const TA* arow[AV]; int ac[AV], ar[AV];
+    const TA* arow[AV];
 #pragma unroll
     for (int q = 0; q < AV; ++q) {
-        ar[q] = (tid + q * 256) / PR; ac[q] = ((tid + q * 256) % PR) * (16 / (int)sizeof(TA));
-        int64_t r = m0 + ar[q];
+        int64_t r = m0 + (tid + q * 256) / PR;
         if (r >= M) r = M - 1;
         arow[q] = r < split ? A0 + r * lda : A1 + (r - split) * lda;
     }
@@ -231,51 +237,41 @@ k_dl_panel(int64_t M, int64_t K, const TA* A0, const TA* A1, int64_t split, int6
     for (int i = 0; i < TI; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) { acc[i][j][0] = 0.0; acc[i][j][1] = 0.0; }
-    float4 ra[AV];
-    double2 rb[BN / 32];
-    auto fetch = [&](int64_t kt) {
-        const int64_t k0 = kt * BK;
+    auto load = [&](int64_t kt) {
+        if (kt < ke) {
+            const int64_t k0 = kt * BK;
+            TA* a = As + (kt - kb) % DL_PS * (BM * AS);
+            double* b = Bs + (kt - kb) % DL_PS * (BK * BS);
 #pragma unroll
-        for (int q = 0; q < AV; ++q) {
-            ra[q] = k0 + ac[q] < K ? *reinterpret_cast<const float4*>(arow[q] + k0 + ac[q]) : make_float4(0.f, 0.f, 0.f, 0.f);
-            if (k0 + BK > K) {               // what lies behind the row's end is not part of the product, whatever it holds
-                TA* e = reinterpret_cast<TA*>(&ra[q]);
+            for (int q = 0; q < AV; ++q) {
+                const int i = tid + q * 256, c = (i % PR) * PE;
+                const int64_t left = K - k0 - c;          // what lies behind the row's end is not part of the product, whatever it holds
+                const int n = left >= PE ? 16 : (left > 0 ? (int)left * (int)sizeof(TA) : 0);
+                dl_cp16(a + (i / PR) * AS + c, n > 0 ? arow[q] + k0 + c : arow[q], n);
+            }
 #pragma unroll
-                for (int i = 0; i < 16 / (int)sizeof(TA); ++i) if (k0 + ac[q] + i >= K) e[i] = (TA)0;
+            for (int q = 0; q < BV; ++q) {
+                const int i = tid + q * 256, kr = i / (BN / 2), c = (i % (BN / 2)) * 2;
+                const bool in = k0 + kr < K;
+                dl_cp16(b + kr * BS + c, in ? B + (k0 + kr) * BN + c : B, in ? 16 : 0);
             }
         }
-#pragma unroll
-        for (int q = 0; q < BN / 32; ++q) {
-            const int i = tid + q * 256, kr = i / (BN / 2), c = (i % (BN / 2)) * 2;
-            rb[q] = k0 + kr < K ? *reinterpret_cast<const double2*>(B + (k0 + kr) * BN + c) : make_double2(0.0, 0.0);
-        }
-    };
-    auto stash = [&](int buf) {
-#pragma unroll
-        for (int q = 0; q < AV; ++q) {
-            double* a = As[buf] + ar[q] * AS + ac[q];
-            if (sizeof(TA) == 4) { a[0] = (double)ra[q].x; a[1] = (double)ra[q].y; a[2] = (double)ra[q].z; a[3] = (double)ra[q].w; }
-            else { const double2 d = *reinterpret_cast<const double2*>(&ra[q]); a[0] = d.x; a[1] = d.y; }
-        }
-#pragma unroll
-        for (int q = 0; q < BN / 32; ++q) {
-            const int i = tid + q * 256, kr = i / (BN / 2), c = (i % (BN / 2)) * 2;
-            Bs[buf][kr * BS + c] = rb[q].x; Bs[buf][kr * BS + c + 1] = rb[q].y;
-        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
     const int fr = lane >> 2, fk = lane & 3;
-    if (kb < ke) { fetch(kb); stash(0); }
-    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < DL_PS - 1; ++i) load(kb + i);
     for (int64_t kt = kb; kt < ke; ++kt) {
-        const int buf = (int)(kt - kb) & 1;
-        if (kt + 1 < ke) fetch(kt + 1);
-        const double* a = As[buf] + (wm * TI * 8) * AS;
-        const double* b = Bs[buf] + wn * 32;
+        asm volatile("cp.async.wait_group %0;" ::"n"(DL_PS - 2) : "memory");
+        __syncthreads();
+        load(kt + DL_PS - 1);                        // into the place that every warp has left behind
+        const TA* a = As + (kt - kb) % DL_PS * (BM * AS) + (wm * TI * 8) * AS;
+        const double* b = Bs + (kt - kb) % DL_PS * (BK * BS) + wn * 32;
 #pragma unroll
         for (int ks = 0; ks < BK; ks += 4) {
             double af[TI], bf[4];
 #pragma unroll
-            for (int i = 0; i < TI; ++i) af[i] = a[(i * 8 + fr) * AS + ks + fk];
+            for (int i = 0; i < TI; ++i) af[i] = (double)a[(i * 8 + fr) * AS + ks + fk];
 #pragma unroll
             for (int j = 0; j < 4; ++j) bf[j] = b[(ks + fk) * BS + j * 8 + fr];
 #pragma unroll
@@ -283,9 +279,8 @@ k_dl_panel(int64_t M, int64_t K, const TA* A0, const TA* A1, int64_t split, int6
 #pragma unroll
                 for (int j = 0; j < 4; ++j) dl_dmma(acc[i][j][0], acc[i][j][1], af[i], bf[j]);
         }
-        if (kt + 1 < ke) stash(buf ^ 1);
-        __syncthreads();
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < TI; ++i) {
         const int64_t row = m0 + wm * TI * 8 + i * 8 + fr;
@@ -1012,7 +1007,7 @@ inline bool dl_plan(osscar_ctx* ctx, DlPlan* d)
 }
 
 constexpr int DL_TERMS_SMEM = 4 * (128 * 20 + 16 * 68) * (int)sizeof(double);
-constexpr int DL_PANEL_SMEM = (2 * 128 * 20 + 2 * 16 * 68) * (int)sizeof(double), DL_PANEL_SMEM_Y = (2 * 128 * 20 + 2 * 16 * 36) * (int)sizeof(double);
+constexpr int DL_RANK_SMEM = (2 * 128 * 20 + 2 * 16 * 68) * (int)sizeof(double);
 
 // Base columns of a batch and its swaps.
 cudaError_t dl_batch(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, const DlArgs& args)
@@ -1025,11 +1020,11 @@ cudaError_t dl_batch(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, const DlAr
     k_dl_select<<<2, 1024, 0, st>>>(p, z);
     k_dl_stage<<<nbI + nbM + (unsigned)((z.kcap + 31) / 32), 256, 0, st>>>(p, z, nbI, nbM);
     k_dl_terms<<<tiles(L.d1, z.zt), 256, DL_TERMS_SMEM, st>>>(p, z);
-    k_dl_panel<double, DL_B><<<tiles(L.nI, z.zy), 256, DL_PANEL_SMEM_Y, st>>>(L.nI, L.nI, p.Hd, p.Hd, L.nI, L.ldh, z.By, z.py, z.zy, ctx->ctl);
-    k_dl_panel<float, DL_N><<<tiles(L.d1, z.zg), 256, DL_PANEL_SMEM, st>>>(L.d1, L.ldm, p.V, p.R, L.nI, L.ldm, z.Bg, z.pg, z.zg, ctx->ctl);
+    k_dl_panel<double, DL_B><<<tiles(L.nI, z.zy), 256, dl_panel_smem<double, DL_B>(), st>>>(L.nI, L.nI, p.Hd, p.Hd, L.nI, L.ldh, z.By, z.py, z.zy, ctx->ctl);
+    k_dl_panel<float, DL_N><<<tiles(L.d1, z.zg), 256, dl_panel_smem<float, DL_N>(), st>>>(L.d1, L.ldm, p.V, p.R, L.nI, L.ldm, z.Bg, z.pg, z.zg, ctx->ctl);
     k_dl_stage_y<<<nbI, 256, 0, st>>>(p, z);
     const float* HJI = p.Hp + L.nI * L.ldp;
-    k_dl_panel<float, DL_N><<<tiles(L.nJ, z.zh), 256, DL_PANEL_SMEM, st>>>(L.nJ, L.nI, HJI, HJI, L.nJ, L.ldp, z.Bh, z.ph, z.zh, ctx->ctl);
+    k_dl_panel<float, DL_N><<<tiles(L.nJ, z.zh), 256, dl_panel_smem<float, DL_N>(), st>>>(L.nJ, L.nI, HJI, HJI, L.nJ, L.ldp, z.Bh, z.ph, z.zh, ctx->ctl);
     k_dl_apply<<<dim3((unsigned)((L.d1 + 127) / 128), DL_N / DL_AC), 128, 0, st>>>(p, z);
     cudaError_t e = cudaMemsetAsync(&ctx->ctl->bar_count, 0, sizeof(unsigned long long) + sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
@@ -1043,10 +1038,10 @@ cudaError_t dl_batch(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, const DlAr
 cudaError_t dl_prepare(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d)
 {
     cudaError_t e = cudaFuncSetAttribute(k_dl_loop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_panel<double, DL_B>, cudaFuncAttributeMaxDynamicSharedMemorySize, DL_PANEL_SMEM_Y);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_panel<float, DL_N>, cudaFuncAttributeMaxDynamicSharedMemorySize, DL_PANEL_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_panel<double, DL_B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (dl_panel_smem<double, DL_B>()));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_panel<float, DL_N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (dl_panel_smem<float, DL_N>()));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_terms, cudaFuncAttributeMaxDynamicSharedMemorySize, DL_TERMS_SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, DL_PANEL_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_rank, cudaFuncAttributeMaxDynamicSharedMemorySize, DL_RANK_SMEM);
     if (e != cudaSuccess) return e;
     k_dl_init<<<(unsigned)((ctx->L.d1 + 7) / 8), 256, 0, ctx->stream>>>(p, d.z);
     count_launches(1);
@@ -1105,7 +1100,7 @@ cudaError_t dl_rewrite(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, int K, c
             } else e = gemm_f64acc(st, M, L.ldm, K, 1.0, A, kp, z.mk, L.ldm, 1.0, C, L.ldm, C, L.ldm, false);
             if (e != cudaSuccess) return e;
         }
-        k_dl_rank<<<dim3((unsigned)((L.nI + 63) / 64), (unsigned)((L.nI + 127) / 128)), 256, DL_PANEL_SMEM, st>>>(p, z, K);
+        k_dl_rank<<<dim3((unsigned)((L.nI + 63) / 64), (unsigned)((L.nI + 127) / 128)), 256, DL_RANK_SMEM, st>>>(p, z, K);
         count_launches(1);
     }
     k_dl_vectors<<<nbd, 256, 0, st>>>(p, z, d.perm0);
