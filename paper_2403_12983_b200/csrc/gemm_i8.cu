@@ -714,13 +714,14 @@ static cudaError_t gemm_i8_run(cudaStream_t st, const I8Gemm& p, I8Scratch& sc, 
         count_launches(2);
         for (int64_t m0 = 0; m0 < M; m0 += pl.mp) {
             const int64_t mw = M - m0 < pl.mp ? M - m0 : pl.mp;
-            // the digits of A from the product before serve again when the whole of A is there
-            const bool have = pl.mp >= M && sc.have_A == p.A && sc.have_rows == M && sc.have_K == K && sc.have_S == S;
+            // the digits of A from the product before serve again when the whole of A is there, in rows of the same length: that
+            // depends on the scratch left for B too (plan())
+            const bool have = pl.mp >= M && sc.have_A == p.A && sc.have_rows == M && sc.have_K == K && sc.have_S == S && sc.have_ldk == pl.ldk;
             if (!have) {
                 sc.have_A = nullptr;
                 k_i8_slice_rows<S><<<(unsigned)mw, 256, 0, st>>>(p.A + m0 * p.lda, p.lda, K, ck, ap, mw * pl.ldk, pl.ldk, sa, vecA, done);
                 count_launches(1);
-                if (pl.mp >= M) { sc.have_A = p.A; sc.have_rows = M; sc.have_K = K; sc.have_S = S; }
+                if (pl.mp >= M) { sc.have_A = p.A; sc.have_rows = M; sc.have_K = K; sc.have_S = S; sc.have_ldk = pl.ldk; }
             }
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;

@@ -165,7 +165,7 @@ cudaError_t gemm_f64out(cudaStream_t st, int64_t M, int64_t N, int64_t K, const 
 struct I8Scratch {                 // device memory for the digits of A and of B (256-byte aligned), and what A's part holds
     void* a = nullptr; size_t a_bytes = 0;
     void* b = nullptr; size_t b_bytes = 0;
-    const float* have_A = nullptr; int64_t have_rows = 0, have_K = 0; int have_S = 0;
+    const float* have_A = nullptr; int64_t have_rows = 0, have_K = 0, have_ldk = 0; int have_S = 0;
 };
 struct I8Gemm {                    // C = beta * C0 + alpha * A * B, A (M x K) and B (K x N) row-major
     int64_t M, N, K;
