@@ -88,6 +88,16 @@ __global__ void k_i8_balance(const float* __restrict__ diag, int64_t stride, int
     if (d > 0.f && isfinite(d)) frexpf(d, &e);
     ck[k] = flip ? -(e >> 1) : e >> 1;
 }
+// The same for an index that runs over pivots: half the binary exponent of |1 / S_kk|.
+__global__ void k_i8_balance_pivots(const double* __restrict__ alpha, int64_t K, int32_t* __restrict__ ck)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= K) return;
+    const double a = alpha[k];
+    int e = 0;
+    if (a != 0.0 && isfinite(a)) frexp(a, &e);
+    ck[k] = e >> 1;
+}
 
 // Digits of the rows of A (rows x K, row stride lda): plane s holds digit s + 1, rows ldk bytes apart.  One block per
 // row: a pass for the largest entry, a second one (from L1 / L2) for the digits, 16 per thread and plane store.
@@ -686,6 +696,9 @@ static cudaError_t gemm_i8_run(cudaStream_t st, const I8Gemm& p, I8Scratch& sc, 
     const int vecA = (((uintptr_t)p.A & 15) == 0 && (p.lda % 4) == 0) ? 1 : 0;
     if (p.diag) {
         k_i8_balance<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(p.diag, p.diag_stride, K, p.inverse_scale ? 1 : 0, ck);
+        count_launches(1);
+    } else if (p.pivots) {
+        k_i8_balance_pivots<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(p.pivots, K, ck);
         count_launches(1);
     } else {
         e = cudaMemsetAsync(ck, 0, sizeof(int32_t) * (size_t)K, st);

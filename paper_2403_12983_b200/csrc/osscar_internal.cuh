@@ -182,6 +182,7 @@ struct I8Gemm {                    // C = beta * C0 + alpha * A * B, A (M x K) a
     bool dot;                      // C (doubles, gemm_i8_dot_cols(N) per row) = partial sums of rows of A B times rows of C0 (- C0sub)
     const float* diag; int64_t diag_stride;            // diagonal of H_II: balances the contraction index (null: none)
     bool inverse_scale;            // the columns of A scale like those of the inverse of H, not like those of H
+    const double* pivots;          // or: K factors 1 / S_kk of pivots, columns of A scale with their square roots and rows of B with the inverses
 };
 bool gemm_i8_usable(int64_t M, int64_t N, int64_t K, int S, const I8Scratch& sc);
 cudaError_t gemm_i8(cudaStream_t st, const I8Gemm& p, int S, I8Scratch& sc, SearchCtl* ctl_dev, const int32_t* done);

@@ -1081,7 +1081,9 @@ cudaError_t dl_rewrite(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, int K, c
         }
         k_dl_coef<<<dim3((unsigned)((L.d1 + 31) / 32), (unsigned)(kp / 32)), 256, 0, st>>>(p, z, K, kp);
         count_launches(2);
-        // V and R: sums beyond fp32, as every other product that their values come from
+        // V and R: sums beyond fp32, as every other product that their values come from.  A leaving pivot has coefficients of the size of
+        // sqrt(H_pp) and a row M_p of its inverse, an entering one the other way round: digits below one scale per row and column need
+        // the index balanced, or the error grows with the units of H (1e-3 of V at 2600 rows whose activations have a size of 256).
         for (int side = 0; side < 2; ++side) {
             const int64_t M = side == 0 ? L.nI : L.nJ;
             float* C = side == 0 ? p.V : p.R;
@@ -1096,6 +1098,7 @@ cudaError_t dl_rewrite(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, int K, c
                 I8Gemm q = {};
                 q.M = M; q.N = L.ldm; q.K = K; q.alpha = 1.0; q.beta = 1.0;
                 q.A = A; q.lda = kp; q.B = z.mk; q.ldb = L.ldm; q.C0 = C; q.ldc0 = L.ldm; q.C = C; q.ldc = L.ldm;
+                q.pivots = z.alpha;
                 e = gemm_i8(st, q, 5, sc, ctx->ctl, nullptr);
             } else e = gemm_f64acc(st, M, L.ldm, K, 1.0, A, kp, z.mk, L.ldm, 1.0, C, L.ldm, C, L.ldm, false);
             if (e != cudaSuccess) return e;
