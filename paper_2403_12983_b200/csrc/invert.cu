@@ -7,7 +7,7 @@
 // hides behind the update.  Before (pivot inverse, two panel products, two copies, update, write-back: seven launches a
 // step) the build of a state of 2304 rows took 4.0 ms with its correction, then 3.6 ms; 1777 rows 5.9 -> 3.1 ms with the digit
 // products of the correction.
-// From kWideRows rows up the matrix is swept in blocks of 512 pivots on the tensor cores, and the scheme above inverts the 512 x 512
+// From kSweptRows rows up the matrix is swept in blocks of 512 pivots on the tensor cores, and the scheme above inverts the 512 x 512
 // pivot blocks: the matrix is read and written n / 512 times instead of n / 64 times.  4096 rows 4.8 -> 3.1 ms, 8602 rows 42 -> 8.5 ms;
 // blocks of 256 at 2304 rows took as long as the steps of 64 (1.8 ms), which keep everything below.
 #include "osscar_internal.cuh"
@@ -454,7 +454,6 @@ __global__ void __launch_bounds__(256) k_sw_finish(float* A, int64_t lda, int64_
 
 #define CK(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return OSSCAR_E_CUDA; } while (0)
 
-constexpr int64_t kWideRows = 3072;
 constexpr int kWide = 512;
 
 // Blocks of 512 pivots as symmetric sweeps of the upper triangle, A_ij -= A_iP A_PP^-1 A_Pj, A_iP := A_iP A_PP^-1, A_PP := -A_PP^-1:
@@ -508,7 +507,7 @@ int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const 
 {
     const Layout& L = ctx->L;
     cudaStream_t st = ctx->stream;
-    if (tensor_updates && n >= kWideRows) {
+    if (tensor_updates && n >= kSweptRows) {
         int done = 0;
         const int rc = invert_wide(ctx, A, lda, n, ref, ldref, &done);
         if (rc != OSSCAR_OK || done) return rc;

@@ -248,6 +248,10 @@ cudaError_t inverse_residual(osscar_ctx* ctx, float* E, bool v_free);
 // nothing happens where *skip (device, may be null) is set
 cudaError_t refine_v(osscar_ctx* ctx, const float* GI, float* rV, void* other, size_t other_bytes, const int32_t* skip = nullptr);
 // ---- invert.cu
+// Rows from which invert_spd_inplace sweeps on the tensor cores.  Sweeps against the steps of 64, ms: 2.25 / 3.05 at 3072 rows, 2.67 / 4.63 at 3584,
+// 3.17 / 6.14 at 4096, 10.1 / 49 at 8602; at 2304, with blocks of 256, they took the same time.  I - H Hinv has the same or a smaller norm, at condition 1e5 (scaled)
+// 8.4e-3 / 8.8e-3, but the largest error of an entry is 2.6e-4 against 1e-4 sqrt(Hinv_ii Hinv_jj) there.
+constexpr int64_t kSweptRows = 3072;
 int invert_spd_inplace(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* ref, int64_t ldref,
                        bool tensor_updates);
 // H^-1 of the whole layer in the place of Hp (nested phase): one Newton-Schulz step from digit products, in column panels, and

@@ -584,7 +584,7 @@ int build_state(osscar_ctx* ctx)
     // relative, and fp32 accumulation leaves cond(H_II) * 2^-24 in them.
     // (1) the inverse.  Single-row groups: fp64 copy by a third-order correction from one fp64 residual, and the fp32
     //     inverse rounded from it (build_hinv64).  Groups of several rows: one Newton-Schulz step, E = I - H_II Hinv in
-    //     fp64, Hinv := sym(Hinv + Hinv E) (E is tiny: any product will do)
+    //     fp64, Hinv := sym(Hinv + Hinv E) (E is tiny: any product will do), from kSweptRows rows up with E^2 as well
     ctx->hd_valid = false;
     if (L.g == 1) {
         const int rc_d = build_hinv64(ctx, true);
@@ -593,6 +593,10 @@ int build_state(osscar_ctx* ctx)
         float* E = big;
         float* Dlt = big + nI * L.ldh;
         CK(inverse_residual(ctx, E, true));
+        if (nI >= kSweptRows) {          // Hinv + Hinv (E + E^2): the sweeps leave more in single entries, see kSweptRows
+            CK(inverse_product(ctx, nI, E, E, L.ldh, 1.f, E, Dlt, L.ldh, 3, ws + L.off_Hd, L.off_y - L.off_Hd));
+            float* t = E; E = Dlt; Dlt = t;
+        }
         CK(inverse_product(ctx, nI, Hinv, E, L.ldh, 0.f, nullptr, Dlt, L.ldh, 3, ws + L.off_Hd, L.off_y - L.off_Hd));
         k_add_sym<<<dim3((unsigned)((nI + 31) / 32), (unsigned)((nI + 31) / 32)), dim3(32, 8), 0, st>>>(Hinv, L.ldh, Dlt, L.ldh, nI);
         count_launches(1);
