@@ -111,15 +111,14 @@ def reduce_over_ranks(values: dict, world: int, backend_device):
 LAZY_ROUND = 4     # steps between two writes of the matrices in the launch chain of single-row groups
 
 
-DELAYED_BATCH = 28  # swaps that a batch of candidate columns lasts (of 32), as measured on the layer shapes
 
-
-def swap_bytes(nI, nJ, m, fused_y=False, lazy=False, delayed=False):
+def swap_bytes(nI, nJ, m, fused_y=False, lazy=False, per_batch=0.0):
     """Algorithmic HBM bytes of one swap: V and R_J read+write and H[J,I] read once in fp32; the inverse read+write
     in fp64 with the next y fused into that pass (single-row groups), or in fp32 with a separate y pass.  `lazy`: V, R and
-    the inverse are read in every step and written in every LAZY_ROUND-th.  `delayed`: all of them are read once per batch."""
-    if delayed:
-        return (8 * nI * nI + 4 * (nI + nJ) * m + 4 * nJ * nI) // DELAYED_BATCH
+    the inverse are read in every step and written in every LAZY_ROUND-th.  `per_batch`: swaps per batch of the delayed loop, which reads all of
+    them once per batch."""
+    if per_batch:
+        return int((8 * nI * nI + 4 * (nI + nJ) * m + 4 * nJ * nI) / per_batch)
     if lazy:
         held = 8 * nI * nI + 4 * (nI + nJ) * m
         return held + 4 * nJ * nI + held // LAZY_ROUND
@@ -282,9 +281,9 @@ def other_configs(pkg, b, solver, dev, with_cpu):
         fused = wl.g == 1 and not pair
         loop_s = r.ms["search_loop"] * 1e-3
         rec = {"workload": workload_label(wl, wl.max_swaps), "layer_solve_s": f0.elapsed_time(f1) / 1e3, "swaps": r.n_swaps,
-               "stop_reason": r.stop_reason, "phases_ms": r.ms, "loop_driver": r.loop_driver,
+               "stop_reason": r.stop_reason, "phases_ms": r.ms, "loop_driver": r.loop_driver, "batches": r.n_batches,
                "swaps_per_s": r.n_swaps / max(loop_s, 1e-9) if r.n_swaps else 0.0,
-               "loop_gbs": swap_bytes(nI, nJ, wl.m, fused, delayed=fused) * r.n_swaps / max(loop_s, 1e-9) / 1e9 if r.n_swaps else 0.0}
+               "loop_gbs": swap_bytes(nI, nJ, wl.m, fused, fused and r.loop_driver == "launches", r.n_swaps / max(r.n_batches, 1) if r.loop_driver == "delayed" else 0.0) * r.n_swaps / max(loop_s, 1e-9) / 1e9 if r.n_swaps else 0.0}
         if name == "c3":        # no improving swap from the energy start: the paper's fixed-iteration form gives the step time
             rf = pkg.solve_layer(solver, x, W, wl.g, wl.k, 8, accept_mode=b.ACCEPT_ALWAYS, **kw)
             rec["forced_swaps"] = {"swaps": rf.n_swaps, "ms_per_swap": rf.ms["search_loop"] / max(rf.n_swaps, 1)}
@@ -467,8 +466,9 @@ def run_ours(args):
     dom = max(shares, key=shares.get) if shares else "gram_tcgen05"
     fused_path = wl.g == 1 and wl.score_mode != "pair_exact" and args.block_pairs <= 1
     loop_ms = phase["search_loop"] / K
-    # AUTO moves single-row groups with delayed updates: matrices are read once per batch, and the Gram is the largest kernel
-    delayed = fused_path and args.loop_mode == 0 and not (shard and world > 1)
+    # delayed updates: matrices are read once per batch, and the Gram is the largest kernel
+    delayed = fused_path and res.loop_driver == "delayed"
+    per_batch = res.n_swaps / max(res.n_batches, 1) if delayed else 0.0
     if fused_path and not delayed and loop_ms > 0 and loop_ms >= phase["gram"] / K:
         # the swap loop is the dominant kernel: one cooperative launch per solve (or its six-launch-per-step form),
         # timed by the library with CUDA events on its own stream around the loop
@@ -500,12 +500,12 @@ def run_ours(args):
     tiles = sum(tn_ - t // 2 for t in range(tm_))
     gram_exec_tflops = 2.0 * 128 * 256 * tiles * wl.n * gram_terms / max(phase["gram"] / K * 1e-3, 1e-12) / 1e12
     fused = wl.g == 1 and wl.score_mode != "pair_exact"
-    lazy = fused_path and not delayed and res.loop_driver == "launches" and not (shard and world > 1)
+    lazy = fused_path and res.loop_driver == "launches" and not (shard and world > 1)
     if args.block_pairs > 1:     # one pass over every matrix per ITERATION, plus the read of V and R for the scores
         it_bytes = swap_bytes(nI, nJ, m, False) + 4 * (nI + nJ) * m
         loop_gbs = it_bytes * (per_step_swaps / args.block_pairs) / max(phase["search_loop"] / K * 1e-3, 1e-12) / 1e9
     else:
-        loop_gbs = swap_bytes(nI, nJ, m, fused, lazy, delayed) * per_step_swaps / max(phase["search_loop"] / K * 1e-3, 1e-12) / 1e9
+        loop_gbs = swap_bytes(nI, nJ, m, fused, lazy, per_batch) * per_step_swaps / max(phase["search_loop"] / K * 1e-3, 1e-12) / 1e9
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_step, "higher_is_better": True, "scaling": "strong" if shard and world > 1 else "weak", "vs_baseline": None,
@@ -526,7 +526,7 @@ def run_ours(args):
                  "executed_mma_per_product": gram_terms,
                  "frac_of_bf16_peak": gram_exec_tflops / pk["bf16_tflops_sustained"], "peak": pk["bf16_tflops_sustained"],
                  "peak_source": pk["source"] + " (sustained)"},
-        "swap_loop": {"gbs": loop_gbs, "bytes_per_swap": swap_bytes(nI, nJ, m, fused, lazy, delayed), "frac_of_hbm": loop_gbs / pk["hbm_gbs"],
+        "swap_loop": {"gbs": loop_gbs, "bytes_per_swap": swap_bytes(nI, nJ, m, fused, lazy, per_batch), "swaps_per_batch": per_batch, "frac_of_hbm": loop_gbs / pk["hbm_gbs"],
                       "peak": pk["hbm_gbs"], "peak_source": pk["source"]},
         "roofline": roof,
         "gpu_launches": int(launches),

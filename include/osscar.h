@@ -52,9 +52,12 @@ enum { OSSCAR_ACCEPT_IMPROVING = 0, OSSCAR_ACCEPT_ALWAYS = 1 };
 enum { OSSCAR_STOP_MAX_SWAPS = 0, OSSCAR_STOP_NO_IMPROVEMENT = 1, OSSCAR_STOP_GUARD = 2 };
 /* Swap loop of single-row groups.  PERSISTENT = one cooperative kernel that runs all steps with bounded grid-wide
  * barriers between their phases (OSSCAR_E_ARG if the device cannot launch cooperatively); LAUNCHES = a chain of
- * dependent launches per step, enqueued ahead of the device; AUTO = PERSISTENT for states that fit the L2 cache (under 96 MB)
- * and have up to 8192 columns, LAUNCHES for wider ones and for states streamed from HBM. */
-enum { OSSCAR_LOOP_AUTO = 0, OSSCAR_LOOP_PERSISTENT = 1, OSSCAR_LOOP_LAUNCHES = 2 };
+ * dependent launches per step, enqueued ahead of the device; DELAYED = swaps on vectors only, in batches of candidate columns, the
+ * matrices of the state rewritten at the end (OSSCAR_E_ARG for column shards, for groups of several rows, pair scores and block exchanges, and
+ * where the device cannot launch cooperatively or the workspace has no room for its vectors); AUTO = DELAYED where it can run, else
+ * PERSISTENT for states that fit the L2 cache (under 96 MB) and have up to 8192 columns, LAUNCHES for wider ones and for
+ * states streamed from HBM. */
+enum { OSSCAR_LOOP_AUTO = 0, OSSCAR_LOOP_PERSISTENT = 1, OSSCAR_LOOP_LAUNCHES = 2, OSSCAR_LOOP_DELAYED = 3 };
 
 #define OSSCAR_MAX_GROUP 96   /* largest supported group size g */
 
@@ -191,7 +194,8 @@ typedef struct {
     float   ms_search;               /* device time of the swap loop                         */
     int32_t n_profiled;              /* steps that were timed kernel by kernel and did a swap */
     float   ms_kernel[OSSCAR_NUM_STEP_KERNELS]; /* mean device time of each kernel over those steps */
-    int32_t loop_driver;             /* OSSCAR_LOOP_PERSISTENT or OSSCAR_LOOP_LAUNCHES: what drove the loop  */
+    int32_t loop_driver;             /* OSSCAR_LOOP_PERSISTENT, _LAUNCHES or _DELAYED: what drove the loop  */
+    int32_t n_batches;               /* DELAYED: batches of candidate columns that were formed, else 0 */
 } osscar_search_result;
 
 /*

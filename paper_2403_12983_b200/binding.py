@@ -19,7 +19,8 @@ SCORE_INDEPENDENT, SCORE_PAIR_EXACT = 0, 1
 ACCEPT_IMPROVING, ACCEPT_ALWAYS = 0, 1
 STOP_MAX_SWAPS, STOP_NO_IMPROVEMENT, STOP_GUARD = 0, 1, 2
 STOP_NAMES = {0: "max_swaps", 1: "no_improvement", 2: "guard"}
-LOOP_AUTO, LOOP_PERSISTENT, LOOP_LAUNCHES = 0, 1, 2
+LOOP_AUTO, LOOP_PERSISTENT, LOOP_LAUNCHES, LOOP_DELAYED = 0, 1, 2, 3
+LOOP_NAMES = {1: "persistent", 2: "launches", 3: "delayed"}
 
 EXPORTS = ["osscar_create", "osscar_destroy", "osscar_workspace_bytes", "osscar_set_workspace",
            "osscar_gram", "osscar_init_support", "osscar_local_search", "osscar_objective",
@@ -36,7 +37,7 @@ class SearchParams(C.Structure):
 class SearchResult(C.Structure):
     _fields_ = [("n_swaps", C.c_int32), ("stop_reason", C.c_int32), ("n_refresh", C.c_int32), ("status", C.c_int32),
                 ("obj_init", C.c_double), ("obj_final", C.c_double), ("ms_search", C.c_float),
-                ("n_profiled", C.c_int32), ("ms_kernel", C.c_float * 12), ("loop_driver", C.c_int32)]
+                ("n_profiled", C.c_int32), ("ms_kernel", C.c_float * 12), ("loop_driver", C.c_int32), ("n_batches", C.c_int32)]
 
 
 STEP_KERNELS = ["select", "pair_grams", "y_pass", "small_algebra", "staging", "h_pass", "update_hinv", "update_v",
@@ -155,7 +156,8 @@ class SearchOutput:
     obj_final: float
     ms_search: float
     ms_kernel: dict              # mean device ms per kernel of a step over the profiled steps ({} if none)
-    loop_driver: str = "launches"  # "persistent" (one cooperative kernel) or "launches"
+    loop_driver: str = "launches"  # "persistent" (one cooperative kernel), "launches" or "delayed" (batches of candidate columns)
+    n_batches: int = 0           # of the delayed loop
 
 
 class Solver:
@@ -339,7 +341,7 @@ class Solver:
                             STOP_NAMES.get(res.stop_reason, str(res.stop_reason)), res.n_refresh,
                             res.obj_init, res.obj_final, res.ms_search,
                             {n: res.ms_kernel[i] for i, n in enumerate(STEP_KERNELS_BLOCK if block_pairs > 1 else STEP_KERNELS_G1 if g == 1 else STEP_KERNELS)}
-                            if res.n_profiled > 0 else {}, "persistent" if res.loop_driver == LOOP_PERSISTENT else "launches")
+                            if res.n_profiled > 0 else {}, LOOP_NAMES.get(res.loop_driver, str(res.loop_driver)), res.n_batches)
 
     def objective(self, H, W, Wt) -> float:
         _dev_f32(H, "H"); _dev_f32(W, "W"); _dev_f32(Wt, "Wt")

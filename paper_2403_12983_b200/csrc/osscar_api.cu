@@ -394,11 +394,11 @@ int osscar_local_search(osscar_ctx* ctx, const osscar_search_params* params,
     if (params->score_mode != OSSCAR_SCORE_INDEPENDENT && params->score_mode != OSSCAR_SCORE_PAIR_EXACT) return OSSCAR_E_ARG;
     if (params->accept_mode != OSSCAR_ACCEPT_IMPROVING && params->accept_mode != OSSCAR_ACCEPT_ALWAYS) return OSSCAR_E_ARG;
     if (params->refresh_every < 0 || params->profile_samples < 0 || params->profile_samples > 8 || params->block_pairs < 0) return OSSCAR_E_ARG;
-    if (params->loop_mode < OSSCAR_LOOP_AUTO || params->loop_mode > OSSCAR_LOOP_LAUNCHES || params->wait_limit_cycles > (uint64_t)1 << 62) return OSSCAR_E_ARG;
+    if (params->loop_mode < OSSCAR_LOOP_AUTO || params->loop_mode > OSSCAR_LOOP_DELAYED || params->wait_limit_cycles > (uint64_t)1 << 62) return OSSCAR_E_ARG;
     if (!ctx->have_state) return OSSCAR_E_STATE;
     if (params->score_mode == OSSCAR_SCORE_PAIR_EXACT && ctx->L.nJ > 0 && ctx->L.pair_capacity == 0) return OSSCAR_E_SHAPE;
     if (ctx->reduce && (ctx->L.g != 1 || params->score_mode != OSSCAR_SCORE_INDEPENDENT || params->block_pairs > 1 ||
-                        params->loop_mode == OSSCAR_LOOP_PERSISTENT)) return OSSCAR_E_ARG;      // what column shards support
+                        params->loop_mode == OSSCAR_LOOP_PERSISTENT || params->loop_mode == OSSCAR_LOOP_DELAYED)) return OSSCAR_E_ARG;      // what column shards support
     if (params->block_pairs > 1) {      // block exchanges: independent scores, s <= min(k, pruned groups), s g rows fit the panels
         const osscar::Layout& L = ctx->L;
         const int64_t s = params->block_pairs;

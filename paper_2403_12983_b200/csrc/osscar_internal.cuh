@@ -40,6 +40,7 @@ struct SearchCtl {
     int32_t y_due;           // the step in flight made a swap (search_lazy_g1.cuh)
     int32_t dl_terms;        // pivots whose terms the matrices do not have yet (search_delayed_g1.cuh)
     int32_t dl_stop;         // 1: the swaps of this part of the search are made, 2: the terms have filled their memory
+    int32_t dl_batches;      // batches of candidate columns of this search
     int32_t settled;         // the search made no swap: V is as refined as it was
     int32_t gram_skip[2];    // Gram of fp32 activations: the panel in flight skips the digits / the bf16 terms (gemm_i8.cu)
 };

@@ -851,7 +851,7 @@ __global__ void k_sorted_support(Ptrs p, int32_t* __restrict__ out)
 }
 __global__ void k_begin(SearchCtl* ctl, double* obj_trace, int32_t* done_host)
 {
-    ctl->done = 0; ctl->stop_reason = OSSCAR_STOP_MAX_SWAPS; ctl->n_swaps = 0; ctl->n_refresh = 0;
+    ctl->done = 0; ctl->stop_reason = OSSCAR_STOP_MAX_SWAPS; ctl->n_swaps = 0; ctl->n_refresh = 0; ctl->dl_batches = 0;
     obj_trace[0] = ctl->obj;
     ctl->acc[2] = ctl->obj;
     *done_host = 0;
@@ -1157,11 +1157,14 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     }
     BlockPtrs bp = make_block_ptrs(ctx, bs);
     const bool fast = g == 1 && !pair && !block;  // fused step for single-row groups
-    // AUTO: delayed updates (search_delayed_g1.cuh).  Asked for by name, or where that one does not fit: the cooperative loop for
-    // states that stay in L2, the launch chain for states streamed from HBM and for wide results (rows of V and R past 8192 floats: the
-    // chain deals a row to several blocks, the loop to one warp).  Column shards: their own chain.
+    // AUTO: delayed updates (search_delayed_g1.cuh).  Where they do not fit, the cooperative loop for states that stay in L2, and the
+    // launch chain for states streamed from HBM and for wide results (rows of V and R past 8192 floats: the chain deals a row to
+    // several blocks, the loop to one warp).  Column shards: their own chain.
     DlPlan dl = {};
-    const bool delayed = fast && !sharded && prm->loop_mode == OSSCAR_LOOP_AUTO && max_swaps > 0 && dl_plan(ctx, &dl);
+    const bool want_delayed = prm->loop_mode == OSSCAR_LOOP_DELAYED || prm->loop_mode == OSSCAR_LOOP_AUTO;
+    const bool fits = want_delayed && fast && !sharded && dl_plan(ctx, &dl);
+    if (prm->loop_mode == OSSCAR_LOOP_DELAYED && !fits) return OSSCAR_E_ARG;
+    const bool delayed = fits && max_swaps > 0;
     const double state_bytes = 8.0 * L.nI * L.ldh + 4.0 * (L.nI + L.nJ) * L.ldm + 4.0 * L.nJ * L.ldh;
     const bool small_state = state_bytes <= 96.0e6 && L.ldm <= 8192;
     const bool want_persistent = !sharded && !delayed && (prm->loop_mode == OSSCAR_LOOP_PERSISTENT || (prm->loop_mode == OSSCAR_LOOP_AUTO && small_state));
@@ -1569,7 +1572,8 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     res->obj_init = ctx->ctl_host->acc[2];
     res->obj_final = ctx->ctl_host->acc[3];
     res->ms_search = ms;
-    res->loop_driver = persistent || (delayed && small_state) ? OSSCAR_LOOP_PERSISTENT : OSSCAR_LOOP_LAUNCHES;
+    res->loop_driver = persistent ? OSSCAR_LOOP_PERSISTENT : delayed || prm->loop_mode == OSSCAR_LOOP_DELAYED ? OSSCAR_LOOP_DELAYED : OSSCAR_LOOP_LAUNCHES;
+    res->n_batches = delayed ? ctx->ctl_host->dl_batches : 0;
     // kernel times of the sampled steps that really swapped (a stopped loop runs empty kernels)
     int used = 0;
     for (int i = 0; i < nprof; ++i) {

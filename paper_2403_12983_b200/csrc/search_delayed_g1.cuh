@@ -689,7 +689,7 @@ __global__ void __launch_bounds__(DL_T, 1) k_dl_loop(const DlArgs a)
         z.val[r] = ok ? (kept[lr] ? v : -v) : INFINITY;
     }
     if (blockIdx.x == 0 && t == 0) {
-        ctl->dl_terms = K0 + nb; ctl->n_swaps = n_swaps; ctl->obj = obj;
+        ctl->dl_terms = K0 + nb; ctl->n_swaps = n_swaps; ctl->obj = obj; ctl->dl_batches += 1;
         if (stop != 3) ctl->dl_stop = stop;
     }
 }

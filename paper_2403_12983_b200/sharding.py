@@ -87,6 +87,6 @@ def solve_layer_sharded(solver: b.Solver, x_chunks_local: Sequence[torch.Tensor]
     ms["search_loop"] = out.ms_search
     res = LayerResult(out.support, out.W, out.obj_trace, out.swap_trace, out.n_swaps, out.stop_reason,
                       out.obj_init, out.obj_final, const_local, ms, out.ms_kernel, H, G)
-    res.loop_driver = out.loop_driver
+    res.loop_driver, res.n_batches = out.loop_driver, out.n_batches
     res.io = {"h2d": 0, "d2h": 0}
     return res

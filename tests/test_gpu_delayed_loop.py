@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("d1,m,k,swaps", [
-    (9, 5, 2, 6),                # fewer slots than candidates of a batch, groups that return
+    (9, 65, 2, 6),               # fewer slots than candidates of a batch, groups that return
+    (9, 5, 2, 6),                # no room for the vectors of the loop: AUTO takes another one
     (33, 16, 30, 40),            # three pruned slots: the same few groups again and again
     (65, 40, 20, 33),            # two blocks; one swap more than a batch can hold
     (200, 20, 80, 150),          # terms fill their memory: matrices rewritten inside the search, groups that moved before it move again
@@ -27,11 +28,12 @@ def test_forced_swaps_follow_the_oracle(d1, m, k, swaps):
     G = (H.double() @ W.double()).float()
     solver = pkg.Solver(0)
     S0, _ = solver.init_support(H, G, W, 1, k, b.INIT_MAGNITUDE)
-    out = solver.local_search(swaps, accept_mode=b.ACCEPT_ALWAYS)
+    fits = m > 5
+    out = solver.local_search(swaps, accept_mode=b.ACCEPT_ALWAYS, loop_mode=b.LOOP_DELAYED if fits else b.LOOP_AUTO)
     perm = solver.debug_state(4).long()
     Hinv, V, R, c = (solver.debug_state(i).double() for i in range(4))
     solver.close()
-    assert out.n_swaps == swaps and out.stop_reason == "max_swaps"
+    assert out.n_swaps == swaps and out.stop_reason == "max_swaps" and out.loop_driver == ("delayed" if fits else "persistent")
     H64, G64 = H.cpu().numpy().astype(np.float64), G.cpu().numpy().astype(np.float64)
     const = float(np.sum(W.cpu().numpy().astype(np.float64) * G64))
     trace = [tuple(int(v) for v in r) for r in out.swap_trace.cpu().numpy()]

@@ -27,7 +27,7 @@ def test_weights_do_not_depend_on_units(d1, m, k, swaps, spread):
         Hs, Gs = H * scale ** 2, G * scale ** 2
         solver.init_support(Hs, Gs, W, 1, k, b.INIT_MAGNITUDE)
         out = solver.local_search(swaps, accept_mode=b.ACCEPT_ALWAYS)
-        assert out.n_swaps == swaps
+        assert out.n_swaps == swaps and out.loop_driver == "delayed"
         perm = solver.debug_state(4).long()
         V, R = solver.debug_state(1).double(), solver.debug_state(2).double()
         I, J = perm[:k], perm[k:]

@@ -1,4 +1,4 @@
-"""The driver that AUTO picks on both sides of its limit of 8192 columns, and its result against a fresh fp64 solve."""
+"""The driver that ran, by name and under AUTO, for results on both sides of 8192 columns, and its result against a fresh fp64 solve."""
 import pytest
 import torch
 
@@ -8,8 +8,8 @@ from paper_2403_12983_b200 import binding as b
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("m,driver", [(8192, "persistent"), (8193, "launches"), (20001, "launches")])
-def test_auto_picks_the_chain_for_wide_results(m, driver):
+@pytest.mark.parametrize("m", [8192, 8193, 20001])
+def test_the_driver_that_ran_is_reported(m):
     d1, k = 90, 41
     gen = torch.Generator(device="cuda").manual_seed(m)
     X = torch.randn(300, d1, generator=gen, device="cuda", dtype=torch.float64) * torch.exp(0.5 * torch.randn(d1, generator=gen, device="cuda"))
@@ -19,11 +19,17 @@ def test_auto_picks_the_chain_for_wide_results(m, driver):
     G = (H.double() @ W.double()).float()
     solver = pkg.Solver(0)
     outs = []
-    for mode in (b.LOOP_AUTO, b.LOOP_PERSISTENT, b.LOOP_LAUNCHES):
+    for mode in (b.LOOP_AUTO, b.LOOP_DELAYED, b.LOOP_PERSISTENT, b.LOOP_LAUNCHES):
         solver.init_support(H, G, W, 1, k, b.INIT_MAGNITUDE)
         outs.append(solver.local_search(11, accept_mode=b.ACCEPT_ALWAYS, loop_mode=mode))
+    solver.init_support(H, G, W, 10, 4, b.INIT_MAGNITUDE)
+    with pytest.raises(pkg.OsscarError, match="osscar_local_search"):
+        solver.local_search(11, loop_mode=b.LOOP_DELAYED)              # single-row groups only
+    solver.init_support(H, G, W, 10, 4, b.INIT_MAGNITUDE)
+    assert solver.local_search(3).loop_driver == "launches"
     solver.close()
-    assert [o.loop_driver for o in outs] == [driver, "persistent", "launches"]
+    assert [o.loop_driver for o in outs] == ["delayed", "delayed", "persistent", "launches"]
+    assert [o.n_batches > 0 for o in outs] == [True, True, False, False]
     I = outs[0].support.long()
     ref = torch.linalg.solve(H.double()[I][:, I], G.double()[I])
     for o in outs:
