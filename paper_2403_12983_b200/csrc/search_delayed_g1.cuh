@@ -88,17 +88,40 @@ __global__ void __launch_bounds__(256) k_dl_init(Ptrs p, DlPtrs z)
     }
 }
 
+// Lane l has entry l of a list: score and group, ordered by score, then by group.
+__device__ __forceinline__ void dl_exchange(double& v, int& id, int j, bool low) {
+    const double ov = __shfl_xor_sync(0xffffffffu, v, j);
+    const int oid = __shfl_xor_sync(0xffffffffu, id, j);
+    const bool less = ov < v || (ov == v && oid < id), same = ov == v && oid == id;
+    if (less == low && !same) { v = ov; id = oid; }
+}
+__device__ __forceinline__ void dl_sort32(double& v, int& id, int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) dl_exchange(v, id, j, ((lane & j) == 0) == ((lane & k) == 0));
+}
+// The 32 first of two sorted lists of 32, sorted.
+__device__ __forceinline__ void dl_merge32(double& v, int& id, double ov, int oid, int lane) {
+    ov = __shfl_sync(0xffffffffu, ov, 31 - lane);
+    oid = __shfl_sync(0xffffffffu, oid, 31 - lane);
+    if (ov < v || (ov == v && oid < id)) { v = ov; id = oid; }
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) dl_exchange(v, id, j, (lane & j) == 0);
+}
 // Candidates: block 0 the kept slots with the smallest scores, block 1 the pruned ones with the largest: the first DL_B of the 2048 slots
 // that are among the two best of a thread's share.  The best slot is always there (the swap that comes next); a third one of the first 32
 // in one share is rare, and the set only decides how long a batch lasts.  (One per thread ended batches of 28 swaps after 24 at
-// d1 = 28672.)
+// d1 = 28672.)  Lists of 32 are sorted and merged by warps, in registers: a sort of all 2048 entries in shared memory, with a barrier for each
+// of its 66 steps, took 8 us longer, whatever the layer (51 swaps in 6 batches at d1 = 1024: 1.076 -> 1.034 ms).
 __global__ void __launch_bounds__(1024) k_dl_select(Ptrs p, DlPtrs z)
 {
+    static_assert(DL_B == 32, "a candidate per lane");
     if (p.ctl->done || p.ctl->dl_stop) return;
-    const int side = blockIdx.x, t = threadIdx.x;
+    const int side = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t d1 = p.nI + p.nJ;
-    __shared__ double sv[2048];
-    __shared__ int sx[2048];
+    __shared__ double sv[32][32];
+    __shared__ int sx[32][32];
     double v0 = INFINITY, v1 = INFINITY; int i0 = INT_MAX, i1 = INT_MAX;
     for (int64_t r = t; r < d1; r += 1024) {
         if ((z.kept[r] != 0) != (side == 0)) continue;
@@ -109,19 +132,16 @@ __global__ void __launch_bounds__(1024) k_dl_select(Ptrs p, DlPtrs z)
         if (v < v0 || (v == v0 && id < i0)) { v1 = v0; i1 = i0; v0 = v; i0 = id; }
         else if (v < v1 || id < i1) { v1 = v; i1 = id; }
     }
-    sv[t] = v0; sx[t] = i0; sv[t + 1024] = v1; sx[t + 1024] = i1;          // sorted by score, then by group
-    for (int k = 2; k <= 2048; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            __syncthreads();
-            const int a = 2 * t - (t & (j - 1)), b = a + j;
-            const double x = sv[a], y = sv[b];
-            const int ix = sx[a], iy = sx[b];
-            const bool after = y < x || (y == x && iy < ix);
-            if (after == ((a & k) == 0) && (x != y || ix != iy)) { sv[a] = y; sv[b] = x; sx[a] = iy; sx[b] = ix; }
-        }
-    __syncthreads();
+    dl_sort32(v0, i0, lane);
+    dl_sort32(v1, i1, lane);
+    dl_merge32(v0, i0, v1, i1, lane);
+    for (int n = 16; n > 0; n >>= 1) {               // the upper half of the lists into the lower one
+        if (warp >= n && warp < 2 * n) { sv[warp][lane] = v0; sx[warp][lane] = i0; }
+        __syncthreads();
+        if (warp < n) dl_merge32(v0, i0, sv[warp + n][lane], sx[warp + n][lane], lane);
+    }
     if (t < DL_B) {
-        const int x = sx[t] != INT_MAX ? p.slotof[sx[t]] : -1;
+        const int x = i0 != INT_MAX ? p.slotof[i0] : -1;
         z.cand[side * DL_B + t] = x;
         if (x >= 0) z.cidx[x] = side * DL_B + t;
     }
