@@ -54,9 +54,9 @@ enum { OSSCAR_STOP_MAX_SWAPS = 0, OSSCAR_STOP_NO_IMPROVEMENT = 1, OSSCAR_STOP_GU
  * barriers between their phases (OSSCAR_E_ARG if the device cannot launch cooperatively); LAUNCHES = a chain of
  * dependent launches per step, enqueued ahead of the device; DELAYED = swaps on vectors only, in batches of candidate columns, the
  * matrices of the state rewritten at the end (OSSCAR_E_ARG for column shards, for groups of several rows, pair scores and block exchanges, and
- * where the device cannot launch cooperatively or the workspace has no room for its vectors); AUTO = DELAYED where it can run, else
- * PERSISTENT for states that fit the L2 cache (under 96 MB) and have up to 8192 columns, LAUNCHES for wider ones and for
- * states streamed from HBM. */
+ * where the device cannot launch cooperatively or the workspace has no room for its vectors); AUTO = DELAYED where it can run and
+ * max_swaps is at least 10 (16 above 8192 columns), else PERSISTENT for states that fit the L2 cache (under 96 MB) and have up to
+ * 8192 columns, LAUNCHES for wider ones and for states streamed from HBM. */
 enum { OSSCAR_LOOP_AUTO = 0, OSSCAR_LOOP_PERSISTENT = 1, OSSCAR_LOOP_LAUNCHES = 2, OSSCAR_LOOP_DELAYED = 3 };
 
 #define OSSCAR_MAX_GROUP 96   /* largest supported group size g */

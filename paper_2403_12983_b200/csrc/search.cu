@@ -1157,14 +1157,15 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     }
     BlockPtrs bp = make_block_ptrs(ctx, bs);
     const bool fast = g == 1 && !pair && !block;  // fused step for single-row groups
-    // AUTO: delayed updates (search_delayed_g1.cuh).  Where they do not fit, the cooperative loop for states that stay in L2, and the
+    // AUTO: delayed updates (search_delayed_g1.cuh), unless so few swaps are asked for that the first batch and the rewrite cost more than
+    // a swap saves: DL_MIN_SWAPS.  For those, and where the vectors do not fit, the cooperative loop for states that stay in L2, and the
     // launch chain for states streamed from HBM and for wide results (rows of V and R past 8192 floats: the chain deals a row to
     // several blocks, the loop to one warp).  Column shards: their own chain.
     DlPlan dl = {};
     const bool want_delayed = prm->loop_mode == OSSCAR_LOOP_DELAYED || prm->loop_mode == OSSCAR_LOOP_AUTO;
     const bool fits = want_delayed && fast && !sharded && dl_plan(ctx, &dl);
     if (prm->loop_mode == OSSCAR_LOOP_DELAYED && !fits) return OSSCAR_E_ARG;
-    const bool delayed = fits && max_swaps > 0;
+    const bool delayed = fits && max_swaps > 0 && (prm->loop_mode == OSSCAR_LOOP_DELAYED || max_swaps >= (L.ldm > 8192 ? DL_MIN_SWAPS_WIDE : DL_MIN_SWAPS));
     const double state_bytes = 8.0 * L.nI * L.ldh + 4.0 * (L.nI + L.nJ) * L.ldm + 4.0 * L.nJ * L.ldh;
     const bool small_state = state_bytes <= 96.0e6 && L.ldm <= 8192;
     const bool want_persistent = !sharded && !delayed && (prm->loop_mode == OSSCAR_LOOP_PERSISTENT || (prm->loop_mode == OSSCAR_LOOP_AUTO && small_state));

@@ -29,6 +29,12 @@ constexpr int DL_KB = 2 * DL_B;                  // pivots (terms) of a batch
 constexpr int DL_T = 512;                        // threads of the loop
 constexpr int DL_MAX_BLOCKS = DL_T / 2;          // blocks of the loop: a thread for each of their candidates
 constexpr int DL_MAX_TERMS = 1024;               // terms between two rewrites of the matrices
+// Swaps asked for from which AUTO takes this loop.  Its fixed cost is the first batch and the rewrite, and AUTO cannot see how early a search stops.
+// Search of 4, 8, 12 and 16 swaps in us, this loop / the one AUTO took before it: 148 / 96, 168 / 152, 184 / 207, 199 / 264 at d1 = 64;
+// 207 / 117, 241 / 194, 268 / 268, 293 / 344 at 1024; 302 / 242, 325 / 411, 361 / 573, 389 / 744 at 5000, 1283; 569 / 444, 595 / 830, 654 / 1219,
+// 682 / 1600 at 8192, 2048; 5430 / 2350, 5510 / 4470, 5700 / 6690, 5700 / 8670 at 28672, 7168; 444 / 146, 475 / 263, 512 / 381, 537 / 506 at 90, 20001.
+// A search that may make hundreds and finds nothing to swap takes 113 / 41, 134 / 45, 212 / 72, 346 / 726, 3500 / 3100.
+constexpr int DL_MIN_SWAPS = 10, DL_MIN_SWAPS_WIDE = 16;
 
 // Best row of a block: score (smallest is best), diagonals, group, slot, last pivot on it, column in the batch.
 struct __align__(16) DlCand { double val, S, G; int32_t id, idx, last, col; double pad; };
