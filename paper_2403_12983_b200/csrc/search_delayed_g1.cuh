@@ -463,8 +463,8 @@ inline size_t dl_loop_smem(int rows, int kb) {
     return sizeof(double) * ((size_t)2 * kb * nrp + 3 * nrp + (size_t)(slices - 1) * 4 * nrp) + sizeof(int) * 4 * (size_t)nrp;
 }
 
-__device__ __forceinline__ uint64_t dl_ordered(double v) {              // whole numbers in the order of v
-    const uint64_t b = (uint64_t)__double_as_longlong(v);
+__device__ __forceinline__ uint64_t dl_ordered(double v) {              // whole numbers in the order of v; zeros of both signs alike, as in k_dl_select
+    const uint64_t b = (uint64_t)__double_as_longlong(v + 0.0);
     return b ^ ((uint64_t)((int64_t)b >> 63) | 0x8000000000000000ull);
 }
 // Lane of the warp with the smallest (val, id); -1 where no lane has one.
@@ -717,6 +717,8 @@ __global__ void __launch_bounds__(DL_T, 1) k_dl_loop(const DlArgs a)
     if (blockIdx.x == 0 && t == 0) {
         ctl->dl_terms = K0 + nb; ctl->n_swaps = n_swaps; ctl->obj = obj; ctl->dl_batches += 1;
         if (stop != 3) ctl->dl_stop = stop;
+        // the best slots are among the candidates, so that a batch makes a swap at least: one that does not would be followed by the same for ever
+        else if (nb == 0 && ctl->status == OSSCAR_OK) ctl->status = OSSCAR_E_TIMEOUT;
     }
 }
 // What the host looks at between batches: [0] stop (1: swaps of the segment made, search stopped or failed, 2: terms full), [1] terms,
