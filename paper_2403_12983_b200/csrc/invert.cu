@@ -402,11 +402,11 @@ __global__ void __launch_bounds__(256) k_sw_gather(const float* __restrict__ A, 
         if (j0 + tx < ldu) U[(int64_t)(k0 + i) * ldu + j0 + tx] = j0 + tx < n ? tile[tx][i] : 0.f;
     }
 }
-// D = (D + D^T) / 2 where the two triangles differ by rounding (bw x bw).
-__global__ void __launch_bounds__(256) k_sw_sym(float* D, int bw)
+// D = (D + D^T) / 2 where the two triangles differ by rounding (nb x nb, rows of bw).
+__global__ void __launch_bounds__(256) k_sw_sym(float* D, int nb, int bw)
 {
     const int i = blockIdx.x;
-    for (int j = i + 1 + threadIdx.x; j < bw; j += 256) {
+    for (int j = i + 1 + threadIdx.x; j < nb; j += 256) {
         const float v = 0.5f * (D[(int64_t)i * bw + j] + D[(int64_t)j * bw + i]);
         D[(int64_t)i * bw + j] = v; D[(int64_t)j * bw + i] = v;
     }
@@ -477,11 +477,12 @@ int invert_wide(osscar_ctx* ctx, float* A, int64_t lda, int64_t n, const float* 
     const size_t scratch_bytes = L.tc_bytes - off;
     for (int64_t p0 = 0; p0 < n; p0 += bw) {
         const int nb = (int)(n - p0 < bw ? n - p0 : bw);
-        const dim3 grid((unsigned)((lda + 31) / 32), (unsigned)(bw / 32));
+        const int64_t cols = lda > p0 + bw ? lda : p0 + bw;          // all of D, also where the last block reaches past the matrix
+        const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)(bw / 32));
         k_sw_gather<<<grid, 256, 0, st>>>(A, lda, n, p0, nb, bw, U, lda, Ut, D);
         const int rc = invert_spd_inplace(ctx, D, bw, nb, ref + p0 * (ldref + 1), ldref, false);
         if (rc != OSSCAR_OK) return rc;
-        k_sw_sym<<<(unsigned)nb, 256, 0, st>>>(D, bw);
+        k_sw_sym<<<(unsigned)nb, 256, 0, st>>>(D, nb, bw);
         CK(gemm_tc(st, n, bw, bw, 1.f, Ut, bw, D, bw, 0.f, T, bw, scratch, scratch_bytes, ctx->ctl));
         CK(gemm_tc(st, n, lda, bw, -1.f, T, bw, U, lda, 1.f, A, lda, scratch, scratch_bytes, ctx->ctl, nullptr, true));
         k_sw_put<<<dim3((unsigned)((n + 31) / 32), (unsigned)(bw / 32)), 256, 0, st>>>(A, lda, n, p0, nb, bw, T, D);
