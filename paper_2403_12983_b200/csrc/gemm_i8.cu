@@ -783,6 +783,7 @@ cudaError_t gemm_i8(cudaStream_t st, const I8Gemm& p, int S, I8Scratch& sc, Sear
     }
 }
 
+int64_t gemm_i8_row_bytes(int64_t K) { return digit_stride(K); }
 size_t gemm_i8_operand_bytes(int64_t rows, int64_t K, int S)
 {
     return (size_t)rows * ((size_t)S * digit_stride(K) + 16) + 4 * (size_t)K + 2048;

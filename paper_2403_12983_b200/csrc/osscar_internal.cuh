@@ -199,6 +199,7 @@ cudaError_t cross_term_tc(cudaStream_t st, const float* H, int64_t d1, const flo
 cudaError_t objective_i8(cudaStream_t st, const float* H, const float* W, const float* Wt, int64_t d1, int64_t m,
                          void* scratch, size_t scratch_bytes, double* partials, double* out_dev, SearchCtl* ctl_dev);
 size_t gemm_i8_operand_bytes(int64_t rows, int64_t K, int S);      // scratch that holds the digits of a whole operand
+int64_t gemm_i8_row_bytes(int64_t K);                              // one row of one digit, where whole operands fit
 
 // ---- panel_tc.cu: Y[i*so_row + e*so_col] = sum_k A[i][k] * P[e][k] on the tensor cores; A (M x K, streamed once) is split
 // into bf16 terms on the way (fp32-accurate); P is an N x K panel

@@ -493,7 +493,7 @@ static bool dense_panels(const osscar_ctx* ctx, DensePanels* d)
     char* ws = (char*)ctx->ws;
     const int64_t n = L.d1;
     d->digits = n <= 131071 / 5 ? 5 : 4;                             // contraction lengths that five (four) digits allow, see gemm_i8.cu
-    const size_t per_col = sizeof(float) * (size_t)n + (size_t)d->digits * round_up(n, 16) + 16, fixed = 4 * (size_t)n + 8192;
+    const size_t per_col = sizeof(float) * (size_t)n + (size_t)d->digits * gemm_i8_row_bytes(n) + 16, fixed = 4 * (size_t)n + 8192;
     int64_t np = L.tc_bytes > fixed ? (int64_t)((L.tc_bytes - fixed) / per_col) / 256 * 256 : 0;
     if (np > n) np = round_up(n, 4);
     if (n < 4096 || np < 256) return false;
