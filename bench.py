@@ -390,7 +390,8 @@ def run_ours(args):
     total_ms = e0.elapsed_time(e1)
     K = max(args.steps, 1)
     # phase / kernel times of a step come from one more solve outside the timed region (the launch-chain driver records
-    # events around sampled steps; the persistent loop reads the device clock at its barriers)
+    # events around sampled steps, the delayed loop around the parts of its first batches; the persistent loop reads the device
+    # clock at its barriers)
     prof_res = step(x_dev, W, prof=8)
     for key, val in prof_res.ms_kernel.items():
         kern[key] = val * K
@@ -461,7 +462,7 @@ def run_ours(args):
     # dominant kernel among the streaming kernels of a swap, and the Gram kernel, by share of the step
     kern_avg = {k2: v / K for k2, v in kern.items()}
     per_step_swaps = swaps / K
-    shares = {k2: v * per_step_swaps / max(args.block_pairs, 1) for k2, v in kern_avg.items()}
+    shares = {k2: v * (prof_res.n_batches or per_step_swaps / max(args.block_pairs, 1)) for k2, v in kern_avg.items()}
     shares["gram_tcgen05"] = phase["gram"] / K
     dom = max(shares, key=shares.get) if shares else "gram_tcgen05"
     fused_path = wl.g == 1 and wl.score_mode != "pair_exact" and args.block_pairs <= 1

@@ -178,7 +178,7 @@ typedef struct {
     int32_t accept_mode;      /* OSSCAR_ACCEPT_*                                             */
     int32_t refresh_every;    /* rebuild the state from H every this many steps (swaps, or iterations of a block exchange); 0 = never */
     double  accept_rel_tol;   /* IMPROVING: accept iff delta <= -tol * obj (1e-5 if < 0)     */
-    int32_t profile_samples;  /* time each kernel of this many evenly spaced steps (0..8)    */
+    int32_t profile_samples;  /* time each kernel of this many evenly spaced steps (0..8); DELAYED: the parts of this many first batches */
     int32_t block_pairs;      /* s: groups exchanged per iteration (0 or 1: one swap per step) */
     int32_t loop_mode;        /* OSSCAR_LOOP_*: how the swap loop of single-row groups is driven */
     int32_t reserved;         /* 0 */
@@ -186,13 +186,14 @@ typedef struct {
 } osscar_search_params;
 
 #define OSSCAR_NUM_STEP_KERNELS 12   /* select, pair Grams, y pass, small algebra, staging, H pass,
-                                        Hinv update, V update, R update, group scores, H row swap, H column swap */
+                                        Hinv update, V update, R update, group scores, H row swap, H column swap; DELAYED, per batch:
+                                        candidates and right-hand sides, panel products, columns, swaps */
 
 typedef struct {
     int32_t n_swaps, stop_reason, n_refresh, status;
     double  obj_init, obj_final;     /* obj_final is recomputed from the final state         */
     float   ms_search;               /* device time of the swap loop                         */
-    int32_t n_profiled;              /* steps that were timed kernel by kernel and did a swap */
+    int32_t n_profiled;              /* steps that were timed kernel by kernel and did a swap (DELAYED: batches) */
     float   ms_kernel[OSSCAR_NUM_STEP_KERNELS]; /* mean device time of each kernel over those steps */
     int32_t loop_driver;             /* OSSCAR_LOOP_PERSISTENT, _LAUNCHES or _DELAYED: what drove the loop  */
     int32_t n_batches;               /* DELAYED: batches of candidate columns that were formed, else 0 */

@@ -45,6 +45,8 @@ STEP_KERNELS = ["select", "pair_grams", "y_pass", "small_algebra", "staging", "h
 # single-row groups run a fused step: decide, H pass, rows of V and R, finish + select, inverse + next y (column shards and
 # the persistent loop: decide, H pass || V, R || slot exchange, select, inverse + next y)
 STEP_KERNELS_G1 = ["decide", "l1_hpass_update_v", "l2_update_r_swap", "select_in", "l4_update_hinv_y"]
+# delayed updates: parts of a batch of candidate columns
+STEP_KERNELS_DELAYED = ["candidates_staging_terms", "panel_products", "columns", "swaps"]
 # block exchanges (block_pairs > 1): stages of one iteration
 STEP_KERNELS_BLOCK = ["select", "gather_y", "grams_algebra_staging", "h_pass", "update_hinv", "update_v", "update_r",
                       "update_c_fix", "h_swap", "scores"]
@@ -155,7 +157,7 @@ class SearchOutput:
     obj_init: float
     obj_final: float
     ms_search: float
-    ms_kernel: dict              # mean device ms per kernel of a step over the profiled steps ({} if none)
+    ms_kernel: dict              # mean device ms per kernel of a step over the profiled steps, delayed loop: per part of a batch ({} if none)
     loop_driver: str = "launches"  # "persistent" (one cooperative kernel), "launches" or "delayed" (batches of candidate columns)
     n_batches: int = 0           # of the delayed loop
 
@@ -340,7 +342,7 @@ class Solver:
         return SearchOutput(support, W_out, obj_trace[:n_obj + 1], swap_trace[:2 * n].view(n, 2), n,
                             STOP_NAMES.get(res.stop_reason, str(res.stop_reason)), res.n_refresh,
                             res.obj_init, res.obj_final, res.ms_search,
-                            {n: res.ms_kernel[i] for i, n in enumerate(STEP_KERNELS_BLOCK if block_pairs > 1 else STEP_KERNELS_G1 if g == 1 else STEP_KERNELS)}
+                            {n: res.ms_kernel[i] for i, n in enumerate(STEP_KERNELS_BLOCK if block_pairs > 1 else STEP_KERNELS_DELAYED if res.loop_driver == LOOP_DELAYED else STEP_KERNELS_G1 if g == 1 else STEP_KERNELS)}
                             if res.n_profiled > 0 else {}, LOOP_NAMES.get(res.loop_driver, str(res.loop_driver)), res.n_batches)
 
     def objective(self, H, W, Wt) -> float:

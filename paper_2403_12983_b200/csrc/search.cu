@@ -1089,9 +1089,10 @@ cudaError_t score_pass(osscar_ctx* ctx)
 }
 
 // The delayed loop: batches of base columns and swaps, at most two of them ahead of the device, until the search ends; rewrites of the
-// matrices where the terms are full, rebuilds of the state every refresh_every swaps, and a rewrite at the end.
+// matrices where the terms are full, rebuilds of the state every refresh_every swaps, and a rewrite at the end.  The first `nprof` batches are
+// timed part by part.
 static int delayed_search(osscar_ctx* ctx, const Ptrs& p, const DlPlan& dl, const osscar_search_params* prm, double tol, int max_swaps,
-                          double* obj_trace, int32_t* swap_trace, cudaEvent_t* ev)
+                          double* obj_trace, int32_t* swap_trace, cudaEvent_t* ev, cudaEvent_t (*evp)[OSSCAR_NUM_STEP_KERNELS + 1], int nprof, int* profiled)
 {
     cudaStream_t st = ctx->stream;
     int made = 0, next_refresh = prm->refresh_every > 0 ? prm->refresh_every : INT_MAX;
@@ -1110,7 +1111,7 @@ static int delayed_search(osscar_ctx* ctx, const Ptrs& p, const DlPlan& dl, cons
                 rep = ctx->done_flag_host + 4 + 4 * (seen & 1);
                 if (rep[0]) break;
             }
-            CK(dl_batch(ctx, p, dl, a));
+            CK(dl_batch(ctx, p, dl, a, *profiled < nprof ? evp[(*profiled)++] : nullptr));
             k_dl_report<<<1, 1, 0, st>>>(ctx->ctl, ctx->done_flag_dev + 4 + 4 * (fed & 1));
             count_launches(1);
             CK(cudaEventRecord(ev[fed & 1], st));
@@ -1401,7 +1402,10 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
             count_launches(1);
         }
     }
-    if (delayed) rc = delayed_search(ctx, p, dl, prm, tol, max_swaps, obj_trace, swap_trace, evb);
+    if (delayed) {
+        rc = delayed_search(ctx, p, dl, prm, tol, max_swaps, obj_trace, swap_trace, evb, evp, nprof, &next_prof);
+        nmarks = DL_MARKS;
+    }
     for (int it = 0; it < (persistent || delayed ? 0 : max_swaps) && rc == OSSCAR_OK; ++it) {
         if (it % batch == 0) {
             const int bi = it / batch;
@@ -1575,10 +1579,10 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     res->ms_search = ms;
     res->loop_driver = persistent ? OSSCAR_LOOP_PERSISTENT : delayed || prm->loop_mode == OSSCAR_LOOP_DELAYED ? OSSCAR_LOOP_DELAYED : OSSCAR_LOOP_LAUNCHES;
     res->n_batches = delayed ? ctx->ctl_host->dl_batches : 0;
-    // kernel times of the sampled steps that really swapped (a stopped loop runs empty kernels)
+    // kernel times of the sampled steps that really swapped (a stopped loop runs empty kernels), or of the first batches
     int used = 0;
     for (int i = 0; i < nprof; ++i) {
-        if (i < next_prof && prof_it[i] < res->n_swaps / bs) {
+        if (i < next_prof && (delayed ? i < res->n_batches : prof_it[i] < res->n_swaps / bs)) {
             for (int j = 0; j + 1 < nmarks && j < NK; ++j) {
                 float t = 0.f;
                 if (cudaEventElapsedTime(&t, evp[i][j], evp[i][j + 1]) == cudaSuccess) res->ms_kernel[j] += t;

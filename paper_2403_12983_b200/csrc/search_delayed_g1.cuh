@@ -1037,28 +1037,35 @@ inline bool dl_plan(osscar_ctx* ctx, DlPlan* d)
 constexpr int DL_TERMS_SMEM = 4 * (128 * 20 + 16 * 68) * (int)sizeof(double);
 constexpr int DL_RANK_SMEM = (2 * 128 * 20 + 2 * 16 * 68) * (int)sizeof(double);
 
-// Base columns of a batch and its swaps.
-cudaError_t dl_batch(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, const DlArgs& args)
+// Base columns of a batch and its swaps.  `marks` (or null): DL_MARKS events around its four parts.
+constexpr int DL_MARKS = 5;
+cudaError_t dl_batch(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, const DlArgs& args, cudaEvent_t* marks)
 {
     const Layout& L = ctx->L;
     cudaStream_t st = ctx->stream;
     const DlPtrs& z = d.z;
     const unsigned nbI = (unsigned)((L.nI + 31) / 32), nbM = (unsigned)((L.ldm + 31) / 32);
     auto tiles = [](int64_t M, int n) { return dim3((unsigned)((M + 127) / 128), (unsigned)n); };
+    auto mark = [&](int i) { if (marks) cudaEventRecord(marks[i], st); };
+    mark(0);
     k_dl_select<<<2, 1024, 0, st>>>(p, z);
     k_dl_stage<<<nbI + nbM + (unsigned)((z.kcap + 31) / 32), 256, 0, st>>>(p, z, nbI, nbM);
     k_dl_terms<<<tiles(L.d1, z.zt), 256, DL_TERMS_SMEM, st>>>(p, z);
+    mark(1);
     k_dl_panel<double, DL_B><<<tiles(L.nI, z.zy), 256, dl_panel_smem<double, DL_B>(), st>>>(L.nI, L.nI, p.Hd, p.Hd, L.nI, L.ldh, z.By, z.py, z.zy, ctx->ctl);
     k_dl_panel<float, DL_N><<<tiles(L.d1, z.zg), 256, dl_panel_smem<float, DL_N>(), st>>>(L.d1, L.ldm, p.V, p.R, L.nI, L.ldm, z.Bg, z.pg, z.zg, ctx->ctl);
     k_dl_stage_y<<<nbI, 256, 0, st>>>(p, z);
     const float* HJI = p.Hp + L.nI * L.ldp;
     k_dl_panel<float, DL_N><<<tiles(L.nJ, z.zh), 256, dl_panel_smem<float, DL_N>(), st>>>(L.nJ, L.nI, HJI, HJI, L.nJ, L.ldp, z.Bh, z.ph, z.zh, ctx->ctl);
+    mark(2);
     k_dl_apply<<<dim3((unsigned)((L.d1 + 127) / 128), DL_N / DL_AC), 128, 0, st>>>(p, z);
+    mark(3);
     cudaError_t e = cudaMemsetAsync(&ctx->ctl->bar_count, 0, sizeof(unsigned long long) + sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     void* kargs[] = { (void*)&args };
     e = cudaLaunchCooperativeKernel((const void*)k_dl_loop, dim3((unsigned)d.grid), dim3(DL_T), kargs, d.smem, st);
     if (e != cudaSuccess) return e;
+    mark(4);
     count_launches(9);
     return cudaGetLastError();
 }

@@ -1,4 +1,4 @@
-"""How the swap loop with delayed updates ends: stops between rebuilds, a wait that runs out, scores that are not finite, ties."""
+"""How the swap loop with delayed updates ends: stops between rebuilds, a wait that runs out, scores that are not finite, ties; what it reports."""
 import pytest
 import torch
 
@@ -72,3 +72,15 @@ def test_ties_go_to_the_smaller_group():
         outs.append(solver.local_search(60, accept_mode=b.ACCEPT_ALWAYS, loop_mode=mode))
     solver.close()
     assert outs[0].n_swaps == 60 and torch.equal(outs[0].swap_trace, outs[1].swap_trace)
+
+
+def test_parts_of_the_first_batches_are_timed():
+    H, G, W = _problem(300, 64, 1)
+    solver = pkg.Solver(0)
+    for samples, swaps in ((2, 60), (8, 20), (0, 20)):
+        solver.init_support(H, G, W, 1, 150, b.INIT_MAGNITUDE)
+        out = solver.local_search(swaps, accept_mode=b.ACCEPT_ALWAYS, profile_samples=samples)
+        assert out.loop_driver == "delayed" and out.n_batches >= 1
+        assert list(out.ms_kernel) == (b.STEP_KERNELS_DELAYED if samples else [])
+        assert all(v > 0 for v in out.ms_kernel.values()) and sum(out.ms_kernel.values()) <= out.ms_search
+    solver.close()
