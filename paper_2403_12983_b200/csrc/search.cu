@@ -1143,8 +1143,6 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
 
     k_begin<<<1, 1, 0, st>>>(ctx->ctl, obj_trace, ctx->done_flag_dev);
     count_launches(1);
-    const bool own_limit = prm->wait_limit_cycles != 0;       // this search's budget for bounded waits; restored at the end
-    if (own_limit) { k_search_wait_limit<<<1, 1, 0, st>>>(ctx->ctl, (long long)prm->wait_limit_cycles); count_launches(1); }
     CK(cudaGetLastError());
     CK(cudaEventRecord(ctx->ev0, st));
     const bool pair = prm->score_mode == OSSCAR_SCORE_PAIR_EXACT;
@@ -1183,6 +1181,9 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     if (block) max_swaps /= bs;                   // from here on: iterations
     const int64_t npairs = (int64_t)L.k * (L.ng - L.k);
     if (sharded && !(g == 1 && !pair && !block)) return OSSCAR_E_ARG;
+    // this search's budget for bounded waits, set once nothing is refused any more; restored at the end
+    const bool own_limit = prm->wait_limit_cycles != 0;
+    if (own_limit) { k_search_wait_limit<<<1, 1, 0, st>>>(ctx->ctl, (long long)prm->wait_limit_cycles); count_launches(1); }
     if (max_swaps > 0 && !delayed) CK(enqueue_scores(ctx, p, true, pair));
     if (max_swaps > 0 && sharded && shard_reduce(ctx, p.vnorm, L.d1, OSSCAR_FP32) != OSSCAR_OK) return OSSCAR_E_CUDA;
     const size_t inv_smem = ((size_t)g * g + 2 * (size_t)g) * sizeof(double);      // matrix under inversion + pivot row/column

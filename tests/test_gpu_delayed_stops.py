@@ -29,6 +29,19 @@ def test_barrier_that_runs_out_is_a_status_and_the_context_goes_on():
     solver.close()
 
 
+def test_refused_search_leaves_the_wait_budget_as_it_was():
+    H, G, W = _problem(432, 64, 9)
+    solver = pkg.Solver(0)
+    for mode in (b.LOOP_PERSISTENT, b.LOOP_DELAYED):
+        solver.init_support(H, G, W, 9, 24, b.INIT_MAGNITUDE)
+        with pytest.raises(pkg.OsscarError) as e:                # loops of single-row groups
+            solver.local_search(4, loop_mode=mode, wait_limit_cycles=4)
+        assert e.value.status == b.E_ARG
+        solver.init_support(H, G, W, 1, 216, b.INIT_MAGNITUDE)
+        assert solver.local_search(12, accept_mode=b.ACCEPT_ALWAYS, loop_mode=mode).n_swaps == 12
+    solver.close()
+
+
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
 def test_groups_without_a_finite_score_stay_where_they_are(value):
     H, G, W = _problem(300, 64, 1)
