@@ -402,7 +402,7 @@ int greedy_support(osscar_ctx* ctx, int t_hat, int32_t* support, int32_t* drop_t
     count_launches(1);
 
     const size_t smem_score = 3 * (size_t)g * g * sizeof(double);
-    CK(cudaFuncSetAttribute(k_gr_score, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_score));
+    CK(cudaFuncSetAttribute(k_gr_score, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * kGroupBytes));
     CK(cudaFuncSetAttribute(k_gr_cinv, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     int n_live = (int)ng, iters = 0, trace_pos = 0;
     while (n_live > L.k) {

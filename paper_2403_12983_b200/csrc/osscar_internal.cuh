@@ -12,6 +12,9 @@ constexpr int64_t kMaxPairs = 1 << 20;     // PAIR_EXACT scores at most this man
 constexpr int kLoopMaxBlocks = 2048;   // most blocks the persistent swap loop is launched with (size of its candidate lists)
 constexpr double kTinyProduct = 16777216.0;   // multiply-adds (256^3) up to which a product is one launch on the fp64 pipe
 constexpr size_t kFreeDynSmem = 40 * 1024;   // dynamic shared memory above which a kernel asks for more (48 KB less its static arrays)
+// g x g doubles of the widest groups.  A kernel's limit of dynamic shared memory belongs to the process: it is set to the most any layer needs, never
+// to what this one needs, which another thread may be about to exceed.
+constexpr int kGroupBytes = OSSCAR_MAX_GROUP * OSSCAR_MAX_GROUP * (int)sizeof(double);
 constexpr int kPadF = 32;   // leading dimensions of internal fp32 matrices are padded to this many floats
 
 extern unsigned long long g_launches;      // kernels launched by the library (host-side count)

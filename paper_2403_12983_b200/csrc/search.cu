@@ -1010,7 +1010,7 @@ cudaError_t enqueue_scores(osscar_ctx* ctx, const Ptrs& p, bool norms, bool gene
         }
     } else {
         const size_t smem = 3 * (size_t)p.g * p.g * sizeof(double);
-        cudaError_t e = cudaFuncSetAttribute(k_scores_general, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(k_scores_general, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * kGroupBytes);
         if (e != cudaSuccess) return e;
         // kept and pruned groups together; inside a swap step (chain) the two are programmatic dependents
         launch_pdl(chain && dependent, k_group_gram, dim3((unsigned)p.ng, (unsigned)((p.g + GG_AT - 1) / GG_AT)), dim3(256), st, p);
@@ -1188,8 +1188,9 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     if (max_swaps > 0 && sharded && shard_reduce(ctx, p.vnorm, L.d1, OSSCAR_FP32) != OSSCAR_OK) return OSSCAR_E_CUDA;
     const size_t inv_smem = ((size_t)g * g + 2 * (size_t)g) * sizeof(double);      // matrix under inversion + pivot row/column
     if (inv_smem > kFreeDynSmem) {
-        CK(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem));
-        CK(cudaFuncSetAttribute(k_pair_delta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)inv_smem));
+        constexpr int most = kGroupBytes + 2 * OSSCAR_MAX_GROUP * (int)sizeof(double);
+        CK(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        CK(cudaFuncSetAttribute(k_pair_delta, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     }
     auto pair_scores = [&]() -> cudaError_t {      // PAIR_EXACT: exact change of obj of every (kept, pruned) pair
         float* Pm = (float*)((char*)ctx->ws + L.off_big);
@@ -1220,7 +1221,7 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
             e = sgemm(st, false, true, L.nI, L.nJ, L.m, 1.f, p.V, L.ldm, p.R, L.ldm, 0.f, XG, ldj, &ctx->ctl->done);
         if (e != cudaSuccess) return e;
         const size_t smem = 3 * (size_t)g * g * sizeof(double);
-        e = cudaFuncSetAttribute(k_pair_slots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k_pair_slots, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * kGroupBytes);
         if (e != cudaSuccess) return e;
         k_pair_slots<<<(unsigned)L.k, small_threads(g), smem, st>>>(p);
         k_pair_delta<<<(unsigned)(npairs < kPairBlocks ? npairs : kPairBlocks), small_threads(g), inv_smem, st>>>(p, Pm, L.ldh, XG, ldj, npairs);
@@ -1275,12 +1276,12 @@ int run_search(osscar_ctx* ctx, const osscar_search_params* prm, int32_t* suppor
     if (block) {
         CK(cudaMemsetAsync((char*)ctx->ws + L.off_block, 0, block_bytes_for(L, bs * g), st));
         const size_t smem = 2 * (size_t)g * bs * g * sizeof(double);
-        if (smem > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_update_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (smem > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_update_c, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kGroupBytes));
         const size_t smem2 = 2 * (size_t)bs * g * bs * g * sizeof(double);
-        if (smem2 > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
-        if (smem2 / 2 > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_update_c_g1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem2 / 2)));
+        if (smem2 > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kGroupBytes));
+        if (smem2 / 2 > kFreeDynSmem) CK(cudaFuncSetAttribute(k_blk_update_c_g1, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupBytes));
     }
-    if (g > 1) CK(cudaFuncSetAttribute(k_update_c, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * (size_t)g * g * sizeof(double))));
+    if (g > 1) CK(cudaFuncSetAttribute(k_update_c, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kGroupBytes));
 
     // Steps per host batch.  The host stays at most two batches ahead of the device, so a loop that stops has up to
     // three batches of launches behind it that return at once (about 2 us each): short batches for states whose step is

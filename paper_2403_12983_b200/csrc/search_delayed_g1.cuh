@@ -456,6 +456,7 @@ struct DlArgs {
     int accept_mode, max_swaps;      // the loop ends when ctl->n_swaps reaches max_swaps
     int rows, kb;                    // rows per block, terms this launch may add
 };
+constexpr size_t DL_SMEM_MAX = 219 * 1024;       // beside 7.4 KB of static arrays
 // dynamic shared memory of the loop: the batch's terms and the diagonals of the block's rows, partial sums of the k-slices
 inline size_t dl_loop_smem(int rows, int kb) {
     const int nrp = (rows + 31) / 32 * 32;
@@ -973,8 +974,7 @@ inline bool dl_plan(osscar_ctx* ctx, DlPlan* d)
     if (grid > DL_MAX_BLOCKS) grid = DL_MAX_BLOCKS;
     d->rows = (int)((L.d1 + grid - 1) / grid);
     d->grid = (int)((L.d1 + d->rows - 1) / d->rows);
-    constexpr size_t kMost = 220 * 1024;
-    for (d->kb = DL_KB; d->kb >= 8 && dl_loop_smem(d->rows, d->kb) > kMost; d->kb -= 2) {}
+    for (d->kb = DL_KB; d->kb >= 8 && dl_loop_smem(d->rows, d->kb) > DL_SMEM_MAX; d->kb -= 2) {}
     if (d->kb < 8) return false;
     d->smem = dl_loop_smem(d->rows, d->kb);
     DlPtrs& z = d->z;
@@ -1072,7 +1072,7 @@ cudaError_t dl_batch(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, const DlAr
 
 cudaError_t dl_prepare(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_dl_loop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.smem);
+    cudaError_t e = cudaFuncSetAttribute(k_dl_loop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DL_SMEM_MAX);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_panel<double, DL_B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (dl_panel_smem<double, DL_B>()));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_panel<float, DL_N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (dl_panel_smem<float, DL_N>()));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dl_terms, cudaFuncAttributeMaxDynamicSharedMemorySize, DL_TERMS_SMEM);
