@@ -10,15 +10,16 @@
 // needs entries (i, q) besides: diagonals and two columns per swap are all that the search reads.  So the matrices of the
 // state stay as they were (the base), every pivot leaves its vectors s and w, kept in fp64, and a column as it is now is its base
 // column less the terms.  Base columns are formed in batches for the DL_B best candidates of each side, one pass over
-// H_JI, Hinv, V and R for all of them; the swaps that follow almost always stay inside the batch (27 to 31 of 32), and the first one
-// that does not ends it: every choice is made from all scores, so the swaps are those of any other driver.  V, R, Hinv and Hp are
-// brought up to date once, at the end (or when the terms fill their memory).
+// H_JI, Hinv, V and R for all of them; the swaps that follow mostly stay inside the batch (27 to 31 of 32, or 8 to 9 where every swap moves the scores of many
+// groups, as from the energy start at d1 = 28672 and 1024), and the first one that does not ends it: every choice is made from all scores,
+// so the swaps are those of any other driver.  V, R, Hinv and Hp are brought up to date once, at the end (or when the terms fill
+// their memory).
 //
 // Bound: the panel products of a batch (fp64 tensor path) at large sizes, the latency of a swap at small ones: about 11000 cycles,
 // a third of them the grid barrier, the rest a chain of reductions, loads from L2 and fp64 operations.  A swap, its share of the
 // batches and of the rewrite included, took before (matrices streamed in every step, or kept in L2 with three barriers) and takes
 // now: 490 -> 160 us at d1 = 28672, m = 7168, k = 8602, 97 -> 30 us at 8192, 2048, 4096, 43 -> 16 us at 5000, 1283, 1777, 20 -> 11 us at
-// 1024, 1024, 512, 14 -> 8 us at 64, 64, 32.
+// 1024, 1024, 512, 14 -> 8 us at 64, 64, 32.  Where a batch lasts 8.6 swaps (28672, energy start) it is 490 -> 390 us.
 //   select     candidates of both sides          stage, panel     base columns: products with up to 64 columns on the fp64
 //   terms      sums over earlier pivots            apply              tensor path (mma m8n8k4), operands streamed once
 //   loop       the swaps                           history ... rank   the matrices after a search
