@@ -31,10 +31,10 @@ constexpr int DL_T = 512;                        // threads of the loop
 constexpr int DL_MAX_BLOCKS = DL_T / 2;          // blocks of the loop: a thread for each of their candidates
 constexpr int DL_MAX_TERMS = 1024;               // terms between two rewrites of the matrices
 // Swaps asked for from which AUTO takes this loop.  Its fixed cost is the first batch and the rewrite, and AUTO cannot see how early a search stops.
-// Search of 4, 8, 12 and 16 swaps in us, this loop / the one AUTO took before it: 148 / 96, 168 / 152, 184 / 207, 199 / 264 at d1 = 64;
-// 207 / 117, 241 / 194, 268 / 268, 293 / 344 at 1024; 302 / 242, 325 / 411, 361 / 573, 389 / 744 at 5000, 1283; 569 / 444, 595 / 830, 654 / 1219,
-// 682 / 1600 at 8192, 2048; 5430 / 2350, 5510 / 4470, 5700 / 6690, 5700 / 8670 at 28672, 7168; 444 / 146, 475 / 263, 512 / 381, 537 / 506 at 90, 20001.
-// A search that may make hundreds and finds nothing to swap takes 113 / 41, 134 / 45, 212 / 72, 346 / 726, 3500 / 3100.
+// Search of 4, 8, 12 and 16 swaps in us, this loop / the one AUTO took before it: 130 / 96, 145 / 152, 164 / 207, 179 / 264 at d1 = 64;
+// 187 / 117, 220 / 194, 246 / 268, 272 / 344 at 1024; 289 / 242, 317 / 411, 352 / 573, 378 / 744 at 5000, 1283; 557 / 444, 582 / 830, 640 / 1219,
+// 670 / 1600 at 8192, 2048; 5350 / 2350, 5380 / 4470, 5390 / 6690, 5590 / 8670 at 28672, 7168; 427 / 146, 456 / 263, 492 / 381, 518 / 506 at 90, 20001.
+// A search that may make hundreds and finds nothing to swap takes 105 / 41, 104 / 45, 182 / 72, 316 / 726, 3300 / 3100.
 constexpr int DL_MIN_SWAPS = 10, DL_MIN_SWAPS_WIDE = 16;
 
 // Best row of a block: score (smallest is best), diagonals, group, slot, last pivot on it, column in the batch.
@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(1024) k_dl_select(Ptrs p, DlPtrs z)
 {
     static_assert(DL_B == 32, "a candidate per lane");
     if (p.ctl->done || p.ctl->dl_stop) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) { p.ctl->bar_count = 0; p.ctl->abort = 0; }          // for the loop's grid barrier
     const int side = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t d1 = p.nI + p.nJ;
     __shared__ double sv[32][32];
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(1024) k_dl_select(Ptrs p, DlPtrs z)
 // the rest: s and w of 32 earlier terms at the candidates, less those that a candidate's own pivot has replaced.
 __global__ void __launch_bounds__(256) k_dl_stage(Ptrs p, DlPtrs z, unsigned nbI, unsigned nbM)
 {
+    pdl_wait_then_release();
     if (p.ctl->done || p.ctl->dl_stop) return;
     __shared__ double tile[DL_N][33];
     if (blockIdx.x >= nbI + nbM) {
@@ -201,6 +203,7 @@ __global__ void __launch_bounds__(256) k_dl_stage(Ptrs p, DlPtrs z, unsigned nbI
 // Hinv h of the pruned candidates from the slices of the product: right-hand sides of the H pass, and the kept rows of their columns.
 __global__ void __launch_bounds__(256) k_dl_stage_y(Ptrs p, DlPtrs z)
 {
+    pdl_wait_then_release();
     if (p.ctl->done || p.ctl->dl_stop) return;
     __shared__ double tile[DL_B][33];
     const int64_t k0 = (int64_t)blockIdx.x * 32;
@@ -243,6 +246,7 @@ template <typename TA, int BN>
 __global__ void __launch_bounds__(256, 2)
 k_dl_panel(int64_t M, int64_t K, const TA* A0, const TA* A1, int64_t split, int64_t lda, const double* B, double* out, int slices, const SearchCtl* ctl)
 {
+    pdl_wait_then_release();
     if (ctl->done || ctl->dl_stop) return;
     constexpr int BM = 128, BK = 16, AS = BK + 4, BS = BN + 4, WN = BN / 32, WM = 8 / WN, TI = BM / WM / 8;
     constexpr int PE = 16 / (int)sizeof(TA), PR = BK / PE, AV = BM * PR / 256, BV = BK * BN / 2 / 256;      // elements of a piece, pieces of a row, per thread
@@ -324,6 +328,7 @@ k_dl_panel(int64_t M, int64_t K, const TA* A0, const TA* A1, int64_t split, int6
 // (A thread per row with a loop over the terms took 55 us at d1 = 1024 and 650 us at d1 = 28672.)
 __global__ void __launch_bounds__(256, 1) k_dl_terms(Ptrs p, DlPtrs z)
 {
+    pdl_wait_then_release();
     const int K = p.ctl->dl_terms;
     if (p.ctl->done || p.ctl->dl_stop || K == 0) return;
     constexpr int BM = 128, BK = 16, AS = BK + 4, BS = DL_N + 4, ABUF = BM * AS, BBUF = BK * BS;
@@ -414,6 +419,7 @@ __global__ void __launch_bounds__(256, 1) k_dl_terms(Ptrs p, DlPtrs z)
 constexpr int DL_AC = 2;                         // columns per block
 __global__ void __launch_bounds__(128) k_dl_apply(Ptrs p, DlPtrs z)
 {
+    pdl_wait_then_release();
     if (p.ctl->done || p.ctl->dl_stop) return;
     const int K0 = p.ctl->dl_terms;
     const int64_t r = (int64_t)blockIdx.x * 128 + threadIdx.x, d1 = p.nI + p.nJ;
@@ -1050,18 +1056,23 @@ cudaError_t dl_batch(osscar_ctx* ctx, const Ptrs& p, const DlPlan& d, const DlAr
     auto mark = [&](int i) { if (marks) cudaEventRecord(marks[i], st); };
     mark(0);
     k_dl_select<<<2, 1024, 0, st>>>(p, z);
-    k_dl_stage<<<nbI + nbM + (unsigned)((z.kcap + 31) / 32), 256, 0, st>>>(p, z, nbI, nbM);
-    k_dl_terms<<<tiles(L.d1, z.zt), 256, DL_TERMS_SMEM, st>>>(p, z);
+    // the kernels up to the columns are programmatic dependents, each of the one before it (ordinary launches between events): a batch is 15 to 20 us
+    // shorter, 51 swaps in 6 batches at d1 = 1024 1.034 -> 0.924 ms
+    const bool dep = !marks;
+    const SearchCtl* ctl = ctx->ctl;
+    const float *Vc = p.V, *Rc = p.R, *HJI = p.Hp + L.nI * L.ldp;
+    const double* Hd = p.Hd;
+    launch_pdl(dep, k_dl_stage, dim3(nbI + nbM + (unsigned)((z.kcap + 31) / 32)), dim3(256), st, p, z, nbI, nbM);
+    launch_pdl_smem(dep, k_dl_terms, tiles(L.d1, z.zt), dim3(256), DL_TERMS_SMEM, st, p, z);
     mark(1);
-    k_dl_panel<double, DL_B><<<tiles(L.nI, z.zy), 256, dl_panel_smem<double, DL_B>(), st>>>(L.nI, L.nI, p.Hd, p.Hd, L.nI, L.ldh, z.By, z.py, z.zy, ctx->ctl);
-    k_dl_panel<float, DL_N><<<tiles(L.d1, z.zg), 256, dl_panel_smem<float, DL_N>(), st>>>(L.d1, L.ldm, p.V, p.R, L.nI, L.ldm, z.Bg, z.pg, z.zg, ctx->ctl);
-    k_dl_stage_y<<<nbI, 256, 0, st>>>(p, z);
-    const float* HJI = p.Hp + L.nI * L.ldp;
-    k_dl_panel<float, DL_N><<<tiles(L.nJ, z.zh), 256, dl_panel_smem<float, DL_N>(), st>>>(L.nJ, L.nI, HJI, HJI, L.nJ, L.ldp, z.Bh, z.ph, z.zh, ctx->ctl);
+    launch_pdl_smem(dep, k_dl_panel<double, DL_B>, tiles(L.nI, z.zy), dim3(256), dl_panel_smem<double, DL_B>(), st, L.nI, L.nI, Hd, Hd, L.nI, L.ldh, z.By, z.py, z.zy, ctl);
+    launch_pdl_smem(dep, k_dl_panel<float, DL_N>, tiles(L.d1, z.zg), dim3(256), dl_panel_smem<float, DL_N>(), st, L.d1, L.ldm, Vc, Rc, L.nI, L.ldm, z.Bg, z.pg, z.zg, ctl);
+    launch_pdl(dep, k_dl_stage_y, dim3(nbI), dim3(256), st, p, z);
+    launch_pdl_smem(dep, k_dl_panel<float, DL_N>, tiles(L.nJ, z.zh), dim3(256), dl_panel_smem<float, DL_N>(), st, L.nJ, L.nI, HJI, HJI, L.nJ, L.ldp, z.Bh, z.ph, z.zh, ctl);
     mark(2);
-    k_dl_apply<<<dim3((unsigned)((L.d1 + 127) / 128), DL_N / DL_AC), 128, 0, st>>>(p, z);
+    launch_pdl(dep, k_dl_apply, dim3((unsigned)((L.d1 + 127) / 128), DL_N / DL_AC), dim3(128), st, p, z);
     mark(3);
-    cudaError_t e = cudaMemsetAsync(&ctx->ctl->bar_count, 0, sizeof(unsigned long long) + sizeof(int32_t), st);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     void* kargs[] = { (void*)&args };
     e = cudaLaunchCooperativeKernel((const void*)k_dl_loop, dim3((unsigned)d.grid), dim3(DL_T), kargs, d.smem, st);
